@@ -82,7 +82,9 @@ typedef enum {
 } xtc_status;
 
 typedef enum {
-  XTC_PREC_FP64 = 0,   /* all four steps in FP64 (SIMT) */
+  XTC_PREC_FP64 = 0,   /* all four steps to FP64 accuracy: step (a) and (c) on the FP64 pipe, the
+                          contractions (b) and (d) on the tensor cores from eight 9-bit integer digits per
+                          value (71 bits below an operand row's maximum), summed in 64-bit integers */
   XTC_PREC_FP16X2 = 1, /* steps (b) and (d): range-exact 2-term FP16 split with power-of-2 scaling
                           (per pair column of rho in step b, per row of L and R in step d): per
                           accumulation range (range_stages blocks of 32 inner values, default 2)
@@ -282,9 +284,9 @@ XTC_API int xtc_three_body_L(xtc_ctx* ctx, int64_t n_grid, int n_orb, const doub
  *   dphi [n_grid][n_orb][3]  gradients of the orbitals at the grid points (bohr^-1), host or device
  *   K    [n_orb]^4 FP64, host or device memory (n_orb = 120: 1.66 GB)
  * The vector pair field V (steps a and b) is formed in the context's precision; the Laplacian
- * table, its product with the pair densities and the contraction are FP64 (SIMT).  Workspace:
- * n_orb^2 x n_pair doubles plus about 6 GB per chunk of outer points (the context's grid_chunk,
- * else chosen by that budget).  Synchronous.  Requires xtc_set_jastrow.  Errors: XTC_ERR_ARG,
+ * term, its product with the pair densities and the contraction are FP64 (as XTC_PREC_FP64).  Workspace:
+ * n_orb^2 x n_pair doubles, up to 32 GB of digits of the operands of the pair fields, and about 10 GB per
+ * chunk of outer points (the context's grid_chunk, else chosen by the budgets).  Synchronous.  Requires xtc_set_jastrow.  Errors: XTC_ERR_ARG,
  * XTC_ERR_STATE, XTC_ERR_NONFINITE (grid, weights, orbitals or their gradients), XTC_ERR_OOM,
  * XTC_ERR_CUDA and those of xtc_vfield. */
 #define XTC_TWO_BODY_K_MAX_ORB 200

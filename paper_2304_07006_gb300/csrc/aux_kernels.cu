@@ -1,4 +1,4 @@
-// Preparation kernels, the FP64 SIMT twins of steps (a)+(b) and (d), and the final kernels
+// Preparation kernels, the FP64 SIMT form of steps (a)+(b) (the allocation-free call), and the final kernels
 // (Delta U unpacking, the one-body correction and the constant of Appendix B).
 #include <algorithm>
 
@@ -423,56 +423,6 @@ __global__ void __launch_bounds__(256) vfield_f64_kernel(const double* __restric
   }
 }
 
-// ------------------------------------------------------------------ step (d), FP64 SIMT
-// M[pq][rs] += sum_k L[k][pq] R[k][rs]; 64 x 64 tiles, 16-deep K steps, 4 x 4 per thread.
-__global__ void __launch_bounds__(256) assemble_f64_kernel(const double* __restrict__ L,
-                                                            const double* __restrict__ R, int n_pair, int kdim,
-                                                            int ldm, double* __restrict__ M) {
-  __shared__ double Ls[16][64];
-  __shared__ double Rs[16][64];
-  const int t = threadIdx.x;
-  const int tx = t & 15, ty = t >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  double acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-  for (int k0 = 0; k0 < kdim; k0 += 16) {
-    for (int k = t; k < 16 * 64; k += 256) {
-      const int kk = k / 64, c = k % 64;
-      const int64_t row = static_cast<int64_t>(k0 + kk) * n_pair;
-      Ls[kk][c] = (k0 + kk < kdim && m0 + c < n_pair) ? L[row + m0 + c] : 0.0;
-      Rs[kk][c] = (k0 + kk < kdim && n0 + c < n_pair) ? R[row + n0 + c] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = Ls[kk][ty * 4 + u];
-        b[u] = Rs[kk][tx * 4 + u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int row = m0 + ty * 4 + u;
-    if (row >= n_pair) continue;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int col = n0 + tx * 4 + v;
-      if (col < n_pair) M[static_cast<int64_t>(row) * ldm + col] += acc[u][v];
-    }
-  }
-}
-
 // ------------------------------------------------------------------ final kernels
 // In place: M <- Delta U = -(M + M^T) (packed pairs), one CTA per pair of 32 x 32 tiles.
 __global__ void symmetrize_kernel(double* __restrict__ M, int n_pair, int ldm) {
@@ -701,12 +651,6 @@ void launch_vfield_f64_impl(const double* grid, const JastrowParams* jp, int n_n
   dim3 g(blocks_for(n_i, F64_TI), blocks_for(n_pair, F64_TP));
   vfield_f64_kernel<<<g, 256, smem, st>>>(grid, jp, jtab64, rho, n_pad, n_pair, i0, n_i, gcp, pair_p, pair_q, n_orb,
                                           V);
-}
-
-void launch_assemble_f64(const double* L, const double* R, int n_pair, int kdim, double* M, cudaStream_t st) {
-  const int ldm = static_cast<int>(m_stride(n_pair));
-  dim3 g(blocks_for(n_pair, 64), blocks_for(n_pair, 64));
-  assemble_f64_kernel<<<g, 256, 0, st>>>(L, R, n_pair, kdim, ldm, M);
 }
 
 void launch_unpack(const double* M, int n_orb, int n_pair, double* dU, float* dU32, cudaStream_t st) {

@@ -21,7 +21,7 @@
 // holds the whole N x N matrices of its points, a row p of them one contiguous run) and all orbital
 // pairs; lanes run over the points, so a warp reads whole 32-byte pieces of a row.  H for its
 // points lives in shared memory.  Outputs, per point and pair, are L = (rho, Vx, Vy, Vz) and R = (A, Bx, By, Bz), written
-// as the operands of step (d): FP32 rows [pq][4*gcp], FP64 [4*gcp][pq] or three bf16 parts
+// as the operands of step (d): FP32 or FP64 rows [pq][4*gcp] or three bf16 parts
 // [part][pq][4*gcp].  L does not depend on the density and R is linear in its factors, so a
 // density of more factors than one pass holds runs several passes: the first writes L and R, the
 // next ones add their R (FP32 and FP64 outputs).
@@ -101,12 +101,18 @@ template <typename TC, int OUT_PARTS>
 __device__ __forceinline__ void write4(void* base, int64_t n_pair, int64_t gcp, int q, int64_t il,
                                        const TC (&v)[4], bool add = false) {
   if (OUT_PARTS == 0) {
-    double* o = static_cast<double*>(base);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      double* e = o + (4 * il + c) * n_pair + q;
-      *e = add ? *e + static_cast<double>(v[c]) : static_cast<double>(v[c]);
+    // FP64 rows [pq][4*gcp] (cut into digits afterwards)
+    double2* o = reinterpret_cast<double2*>(static_cast<double*>(base) + static_cast<int64_t>(q) * 4 * gcp + 4 * il);
+    double2 w0 = make_double2(v[0], v[1]), w1 = make_double2(v[2], v[3]);
+    if (add) {
+      const double2 a0 = o[0], a1 = o[1];
+      w0.x += a0.x;
+      w0.y += a0.y;
+      w1.x += a1.x;
+      w1.y += a1.y;
     }
+    o[0] = w0;
+    o[1] = w1;
   } else if (OUT_PARTS == 1) {
     // FP32 rows [pq][4*gcp] (split afterwards with a per-row scale)
     float* o = static_cast<float*>(base) + static_cast<int64_t>(q) * 4 * gcp + 4 * il;

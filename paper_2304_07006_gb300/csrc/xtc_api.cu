@@ -97,7 +97,10 @@ struct xtc_ctx {
   DBuf Lv, T3;                 // explicit three-body L: V of the outer points, the packed T
   DBuf fc_U, fc_h, fc_hout, fc_Uout;  // frozen-core folding: staged host inputs and outputs
   DBuf G2;                     // second gradient table: step (a) of the next chunk on stream st2
-  DBuf k_dphi, k_V, k_Ft, k_W, k_S, k_P;  // two-body integrals K: staged gradients, V, F table, W, S, split-K slices
+  DBuf k_dphi, k_dphiT, k_W, k_S;  // two-body integrals K: staged and transposed gradients, rows of W and V, S
+  // digit planes and row exponents of the FP64 contractions: rho^T, the pair functions (with their
+  // scratch rows), and the operands of step (d) or of the contraction of K
+  DBuf d_rho, d_rhoe, d_sj, d_G, d_Ge, d_tmp, d_L, d_Le, d_R, d_Re;
   cudaStream_t st2 = nullptr;  // created on first use
   cudaEvent_t ev_g[2] = {nullptr, nullptr};  // gradient table b written
   cudaEvent_t ev_b[2] = {nullptr, nullptr};  // step (b) GEMM that read table b done
@@ -113,6 +116,7 @@ struct xtc_ctx {
   int vf_kd = 2;  // K-blocks per tensor-core accumulation range in step (b)
   int vf_flush = 8192;  // inner points (K values) between FP64 flushes of the running sums (0: FP32 only)
   int as_kd = 2;  // the same for step (d)
+  double d64_budget = 1.0;  // scale of the memory budgets of the FP64 contractions' blocks
   int x_period = 64;  // fp16 engine: K-blocks between drains of the cross-product accumulator
   // batched builds: lane contexts, each with its own stream (created on first use)
   std::vector<xtc_ctx*> lanes;
@@ -122,7 +126,8 @@ struct xtc_ctx {
     return {&jp_dev, &err_dev, &flag_dev, &grid, &w, &phi, &gamma, &phiT, &phi32, &pair_p, &pair_q, &jtab, &jtab64,
             &rho, &colmax, &colexp, &G, &V, &Vacc, &L, &R, &L32, &R32, &eL, &eR, &M, &evec, &lam, &dU_tmp,
             &dh_tmp, &e0_tmp, &vout, &r1, &r2, &lamd, &gamma_b, &M2, &M3, &lam2, &R2, &R32b, &eR2, &Lv, &T3,
-            &fc_U, &fc_h, &fc_hout, &fc_Uout, &G2, &k_dphi, &k_V, &k_Ft, &k_W, &k_S, &k_P};
+            &fc_U, &fc_h, &fc_hout, &fc_Uout, &G2, &k_dphi, &k_dphiT, &k_W, &k_S, &d_rho, &d_rhoe, &d_sj,
+            &d_G, &d_Ge, &d_tmp, &d_L, &d_Le, &d_R, &d_Re};
   }
 };
 
@@ -232,10 +237,10 @@ void jacobi_eigen(std::vector<double>& a, std::vector<double>& v, int n) {
 }
 
 int make_tmap_3d(xtc_ctx* ctx, CUtensorMap* tm, void* base, bool bf16, uint64_t d0, uint64_t d1, uint64_t d2,
-                 uint32_t b0, uint32_t b1, bool sw128 = false) {
+                 uint32_t b0, uint32_t b1, bool sw128 = false, uint32_t b2 = 1) {
   const cuuint64_t dims[3] = {d0, d1, d2};
   const cuuint64_t strides[2] = {d0 * 2, d0 * d1 * 2};
-  const cuuint32_t box[3] = {b0, b1, 1};
+  const cuuint32_t box[3] = {b0, b1, b2};
   const cuuint32_t es[3] = {1, 1, 1};
   CUresult r = ctx->encode(tm, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, base, dims,
                            strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -265,7 +270,19 @@ struct Plan {
   int splits;
   int parts_b;       // step (b) parts (2 fp16 / 3 bf16), 0 = FP64
   bool f64;
+  int64_t jb;        // FP64 contractions: inner points per block (the whole padded grid when it fits),
+  int64_t gb;        // outer points per block,
+  int comps;         // and rows per outer point: 3 (gradient), 4 (gradient and F), 1 (F), 0 (none)
 };
+
+// The digits of the FP64 contractions take 16 bytes a value; the operands are cut into digits in blocks
+// that keep within these budgets: rho^T, the pair functions, both operands of step (d).
+constexpr int64_t D64_BYTES = 2 * D64_PLANES;
+constexpr double D64_RHO_BYTES = 24.0e9, D64_G_BYTES = 8.0e9, D64_LR_BYTES = 6.0e9;
+// How many of `all` (in steps of 128) fit a budget at bytes_each.
+int64_t block_of(double budget, double bytes_each, int64_t all) {
+  return std::min(all, std::max<int64_t>(128, static_cast<int64_t>(budget / bytes_each) / 128 * 128));
+}
 
 // budget_scale < 1 shrinks the memory budgets (the autotuner's smaller candidates).
 int64_t auto_chunk(const xtc_ctx* c, int NP, int64_t NGp, int parts, int64_t n_outer, bool f64,
@@ -375,6 +392,7 @@ int xtc_create(xtc_ctx** out, const xtc_params* p) {
   if (const char* s = std::getenv("XTC_VF_KD")) ctx->vf_kd = std::max(1, std::atoi(s));
   if (const char* s = std::getenv("XTC_AS_KD")) ctx->as_kd = std::max(1, std::atoi(s));
   if (const char* s = std::getenv("XTC_VF_FLUSH")) ctx->vf_flush = std::max(0, std::atoi(s));
+  if (const char* s = std::getenv("XTC_D64_BUDGET")) ctx->d64_budget = std::atof(s);
   if (const char* s = std::getenv("XTC_X_PERIOD")) ctx->x_period = std::max(1, std::atoi(s));
   if (p->range_stages > 0) ctx->vf_kd = ctx->as_kd = p->range_stages;
   if (!ensure(ctx->jp_dev, sizeof(JastrowParams)) || !ensure(ctx->err_dev, 16) || !ensure(ctx->flag_dev, 16)) {
@@ -491,9 +509,95 @@ int check_device_error(xtc_ctx* ctx) {
   return XTC_OK;
 }
 
-// Common preparation of grid-wide tables.  Fills the plan.
+// Tables of the FP64 contractions over the inner points: per-point table, digits of rho^T when the whole
+// grid is one block (else they are formed block by block), room for the digits of `comps` pair functions.
+int prepare64(xtc_ctx* ctx, Plan& pl, int comps, const double* d_grid, const double* d_w) {
+  cudaStream_t st = ctx->st;
+  const int n_nuc = ctx->jp.n_nuc;
+  pl.comps = comps;
+  pl.jb = block_of(ctx->d64_budget * D64_RHO_BYTES, static_cast<double>(D64_BYTES) * pl.NP, pl.NGp);
+  pl.gb = block_of(ctx->d64_budget * D64_G_BYTES, static_cast<double>(D64_BYTES) * comps * pl.jb, pl.gc);
+  const size_t g_rows = static_cast<size_t>(comps) * pl.gb;
+  if (!ensure(ctx->jtab64, sizeof(double) * pl.NGp * (3 + n_nuc)) ||
+      !ensure(ctx->d_rho, static_cast<size_t>(D64_BYTES) * pl.NP * pl.jb) || !ensure(ctx->d_rhoe, 4ull * pl.NP) ||
+      !ensure(ctx->d_sj, 4ull * (pl.NGp + pl.N)) || !ensure(ctx->d_G, static_cast<size_t>(D64_BYTES) * g_rows * pl.jb) || !ensure(ctx->d_Ge, 4ull * g_rows) ||
+      !ensure(ctx->d_tmp, grad64_scratch_bytes(comps, pl.gb, pl.jb, ctx->n_sm)))
+    return fail(ctx, XTC_ERR_OOM, "FP64 grid tables (%.2f GB)", D64_BYTES * (pl.NP + 1.0 * g_rows) * pl.jb / 1e9);
+  timed(ctx, XTC_K_PREP, pl.jb >= pl.NGp ? 4 : 3, [&] {
+    launch_point_scale(ctx->phiT.as<double>(), pl.NGp, d_w, pl.NG, pl.N, ctx->d_sj.as<int>() + pl.NGp,
+                       ctx->d_sj.as<int>(), st);
+    launch_jtab64_soa(d_grid, pl.NG, pl.NGp, ctx->jp_dev.as<JastrowParams>(), n_nuc, ctx->jtab64.as<double>(), st);
+    if (pl.jb >= pl.NGp)
+      launch_digits_rho(ctx->phiT.as<double>(), pl.NGp, d_w, pl.NG, pl.jb, pl.N, ctx->pair_p.as<int>(),
+                        ctx->pair_q.as<int>(), ctx->d_sj.as<int>(), ctx->d_rho.as<uint16_t>(), ctx->d_rhoe.as<int>(),
+                        st);
+  });
+  return XTC_OK;
+}
+
+// One FP64 contraction of two digit operands (rows_a rows in `comps` components of c_rows, m_rows of each
+// valid; n_cols rows of B; kp values of k each) into `out`.
+int run_gemm64(xtc_ctx* ctx, int kind, const DBuf& A, const DBuf& Ae, int comps, int64_t c_rows, int64_t m_rows,
+               const DBuf& B, const DBuf& Be, int64_t n_cols, int64_t kp, const Gemm64Out& out, int mode) {
+  CUtensorMap ta{}, tb{};
+  int rc;
+  if ((rc = make_tmap_3d(ctx, &ta, A.p, false, kp, comps * c_rows, D64_PLANES, D64_BK, D64_BM, true))) return rc;
+  if ((rc = make_tmap_3d(ctx, &tb, B.p, false, kp, n_cols, D64_PLANES, D64_BK, D64_BN, true, D64_PLANES))) return rc;
+  Gemm64Args a{};
+  a.mt_per_c = static_cast<int>((m_rows + D64_BM - 1) / D64_BM);
+  a.m_tiles = comps * a.mt_per_c;
+  a.n_tiles = static_cast<int>((n_cols + D64_BN - 1) / D64_BN);
+  a.c_rows = c_rows;
+  a.m_rows = static_cast<int>(m_rows);
+  a.n_cols = static_cast<int>(n_cols);
+  a.n_ranges = static_cast<int>(kp / D64_BK);
+  a.exp_a = Ae.as<int>();
+  a.exp_b = Be.as<int>();
+  a.err = ctx->err_dev.as<int>();
+  const int splits = gemm64_splits(a.m_tiles, a.n_tiles, a.n_ranges, ctx->n_sm);
+  const size_t bytes = gemm64_tile_bytes(a.m_tiles, a.n_tiles, splits);
+  if (!ensure(ctx->Vacc, bytes)) return fail(ctx, XTC_ERR_OOM, "FP64 tile sums (%.2f GB)", bytes / 1e9);
+  a.C = ctx->Vacc.as<double>();
+  timed(ctx, kind, 2, [&] {
+    launch_gemm64(&ta, &tb, a, splits, ctx->st);
+    launch_gemm64_finalize(a, splits, out, mode, ctx->st);
+  });
+  return XTC_OK;
+}
+
+// Steps (a)+(b) in FP64 for outer points [i0, i0 + n_i): pl.comps pair functions against rho^T into `out`.
+int run_vfield64(xtc_ctx* ctx, const Plan& pl, const double* d_grid, const double* d_w, int64_t i0, int64_t n_i,
+                 Gemm64Out out, int mode) {
+  cudaStream_t st = ctx->st;
+  for (int64_t j0 = 0; j0 < pl.NGp; j0 += pl.jb) {
+    const int64_t kp = std::min(pl.jb, pl.NGp - j0), n_j = std::min(kp, pl.NG - j0);
+    if (pl.jb < pl.NGp)
+      timed(ctx, XTC_K_VFIELD, 1, [&] {
+        launch_digits_rho(ctx->phiT.as<double>() + j0, pl.NGp, d_w + j0, n_j, kp, pl.N, ctx->pair_p.as<int>(),
+                          ctx->pair_q.as<int>(), ctx->d_sj.as<int>() + j0, ctx->d_rho.as<uint16_t>(),
+                          ctx->d_rhoe.as<int>(), st);
+      });
+    out.add = j0 > 0;
+    for (int64_t b0 = 0; b0 < n_i; b0 += pl.gb) {
+      const int64_t n_b = std::min(pl.gb, n_i - b0);
+      timed(ctx, XTC_K_VFIELD, 1, [&] {
+        launch_grad64_digits(d_grid, ctx->jp_dev.as<JastrowParams>(), ctx->jp.n_nuc, ctx->jtab64.as<double>() + j0,
+                             ctx->d_sj.as<int>() + j0, pl.NGp, n_j, kp, i0 + b0, n_b, pl.gb, pl.comps, ctx->d_tmp.as<double>(),
+                             ctx->d_G.as<uint16_t>(), ctx->d_Ge.as<int>(), ctx->n_sm, st);
+      });
+      out.i0 = b0;
+      const int rc = run_gemm64(ctx, XTC_K_VFIELD, ctx->d_G, ctx->d_Ge, pl.comps, pl.gb, n_b, ctx->d_rho, ctx->d_rhoe,
+                                pl.NP, kp, out, mode);
+      if (rc) return rc;
+    }
+  }
+  return XTC_OK;
+}
+
+// Common preparation of grid-wide tables.  Fills the plan.  comps64: pair functions of the FP64
+// contractions (0: the gradient in FP64 contexts, none in the others).
 int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* grid_xyz, const double* weights,
-            const double* phi, const double** d_grid, const double** d_w, const double** d_phi) {
+            const double* phi, const double** d_grid, const double** d_w, const double** d_phi, int comps64 = 0) {
   if (!ctx->jastrow_set) return fail(ctx, XTC_ERR_STATE, "xtc_set_jastrow has not been called");
   if (n_grid < 1 || n_orb < 1 || n_orb > MAX_ORB || !grid_xyz || !weights || !phi)
     return fail(ctx, XTC_ERR_ARG, "bad sizes (n_grid=%lld, n_orb=%d) or null input", (long long)n_grid, n_orb);
@@ -552,25 +656,17 @@ int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* gri
   }
   if (!ensure(ctx->phiT, sizeof(double) * pl.NGp * n_orb)) return fail(ctx, XTC_ERR_OOM, "phiT");
   const int n_nuc = ctx->jp.n_nuc;
-  if (f64) {
-    if (!ensure(ctx->jtab64, sizeof(double) * pl.NGp * (3 + n_nuc)) ||
-        !ensure(ctx->rho, sizeof(double) * pl.NGp * pl.NP))
-      return fail(ctx, XTC_ERR_OOM, "FP64 grid tables (%.2f GB)", 8.0 * pl.NGp * pl.NP / 1e9);
-  } else {
+  if (!f64) {
     const int js = jtab_stride(n_nuc);
     if (!ensure(ctx->jtab, sizeof(float) * pl.NGp * js) ||
         !ensure(ctx->rho, 2ull * 3 * pl.NGp * pl.NP) || !ensure(ctx->colmax, 4ull * pl.NP) ||
         !ensure(ctx->colexp, 4ull * pl.NP) || !ensure(ctx->phi32, 8ull * (n_orb + 1) * pl.NGp))
       return fail(ctx, XTC_ERR_OOM, "grid tables (%.2f GB)", 2.0 * 3 * pl.NGp * pl.NP / 1e9);
   }
-  const int nprep = f64 ? 3 : (pl.parts_b == 2 ? 5 : 3);
+  const int nprep = f64 ? 1 : (pl.parts_b == 2 ? 5 : 3);
   timed(ctx, XTC_K_PREP, nprep, [&] {
     launch_transpose_phi(*d_phi, n_grid, pl.NGp, n_orb, ctx->phiT.as<double>(), st);
-    if (f64) {
-      launch_jtab64(*d_grid, n_grid, pl.NGp, ctx->jp_dev.as<JastrowParams>(), n_nuc, ctx->jtab64.as<double>(), st);
-      launch_rho_f64(*d_phi, *d_w, n_grid, pl.NGp, n_orb, ctx->pair_p.as<int>(), ctx->pair_q.as<int>(),
-                     ctx->rho.as<double>(), st);
-    } else {
+    if (!f64) {
       const int js = jtab_stride(n_nuc);
       launch_jtab(*d_grid, n_grid, pl.NGp, ctx->jp_dev.as<JastrowParams>(), n_nuc, js, ctx->jtab.as<float>(), st);
       launch_rho_split(ctx->phiT.as<double>(), *d_w, n_grid, pl.NGp, n_orb, pl.parts_b, f16_range_b(ctx->vf_kd),
@@ -578,7 +674,7 @@ int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* gri
                        ctx->colexp.as<int>(), ctx->phi32.as<float>(), ctx->rho.p, st);
     }
   });
-  const size_t vbytes = static_cast<size_t>(pl.splits) * v_slice(pl.gc, pl.N) * (f64 ? 8 : 4);
+  const size_t vbytes = comps64 && f64 ? 0 : static_cast<size_t>(pl.splits) * v_slice(pl.gc, pl.N) * (f64 ? 8 : 4);
   if (!ensure(ctx->V, vbytes)) return fail(ctx, XTC_ERR_OOM, "V chunk (%.2f GB)", vbytes / 1e9);
   if (!f64) {
     const size_t gbytes = 2ull * pl.parts_b * 3 * pl.gc * pl.NGp;
@@ -589,7 +685,8 @@ int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* gri
     const size_t abytes = ctx->vf_flush > 0 ? 8ull * pl.splits * tiles * VF_BM * bn : 0;
     if (!ensure(ctx->Vacc, abytes)) return fail(ctx, XTC_ERR_OOM, "step (b) FP64 sums (%.2f GB)", abytes / 1e9);
   }
-  return XTC_OK;
+  const int comps = comps64 ? comps64 : (f64 ? 3 : 0);
+  return comps ? prepare64(ctx, pl, comps, *d_grid, *d_w) : XTC_OK;
 }
 
 // Tensor maps of the step (b) operands: rho^T (box rows vf_bn) and the gradient table, as stored by
@@ -673,15 +770,16 @@ void run_gemm_b(xtc_ctx* ctx, const Plan& pl, int64_t n_i, const VfMaps& maps) {
 }
 
 // Steps (a)+(b) for outer points [i0, i0 + n_i) into ctx->V, on the context's stream.
-int run_vfield(xtc_ctx* ctx, const Plan& pl, const double* d_grid, int64_t i0, int64_t n_i, const VfMaps& maps) {
+int run_vfield(xtc_ctx* ctx, const Plan& pl, const double* d_grid, const double* d_w, int64_t i0, int64_t n_i,
+               const VfMaps& maps) {
   cudaStream_t st = ctx->st;
   if (pl.f64) {
-    timed(ctx, XTC_K_VFIELD, 1, [&] {
-      launch_vfield_f64_impl(d_grid, ctx->jp_dev.as<JastrowParams>(), ctx->jp.n_nuc, ctx->jtab64.as<double>(),
-                             ctx->rho.as<double>(), pl.NGp, pl.NP, i0, n_i, pl.gc, ctx->pair_p.as<int>(),
-                             ctx->pair_q.as<int>(), pl.N, ctx->V.as<double>(), st);
-    });
-    return XTC_OK;
+    Gemm64Out o{};
+    o.out = ctx->V.as<double>();
+    o.n_orb = pl.N;
+    o.pair_p = ctx->pair_p.as<int>();
+    o.pair_q = ctx->pair_q.as<int>();
+    return run_vfield64(ctx, pl, d_grid, d_w, i0, n_i, o, D64_TO_V);
   }
   run_grad(ctx, pl, d_grid, i0, n_i, maps, st);
   run_gemm_b(ctx, pl, n_i, maps);
@@ -844,6 +942,11 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
     CUDA_OK(cudaMemsetAsync(ctx->eR.p, 0, ebytes, st));
     if (spin) CUDA_OK(cudaMemsetAsync(ctx->eR2.p, 0, ebytes, st));
   }
+  const int64_t kblk = block_of(ctx->d64_budget * D64_LR_BYTES, 2.0 * D64_BYTES * NP, kdim);
+  if (pl.f64 && (!ensure(ctx->d_L, static_cast<size_t>(D64_BYTES) * kblk * NP) ||
+                 !ensure(ctx->d_R, static_cast<size_t>(D64_BYTES) * kblk * NP) || !ensure(ctx->d_Le, 4ull * NP) ||
+                 !ensure(ctx->d_Re, 4ull * NP)))
+    return fail(ctx, XTC_ERR_OOM, "step (d) digits (%.2f GB)", 2.0 * D64_BYTES * kblk * NP / 1e9);
   VfMaps maps{};
   CUtensorMap tm_L{}, tm_R{}, tm_R2{}, tm_R16{}, tm_R216{};
   if ((rc = make_vfield_maps(ctx, pl, maps))) return rc;
@@ -916,7 +1019,7 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
           CUDA_OK(cudaEventRecord(ctx->ev_g[1 - gb], ctx->st2));
         }
         gb = 1 - gb;
-      } else if ((rc = run_vfield(ctx, pl, d_grid, c0, n_i, maps))) {
+      } else if ((rc = run_vfield(ctx, pl, d_grid, d_w, c0, n_i, maps))) {
         return rc;
       }
     }
@@ -1004,10 +1107,26 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
           timed(ctx, XTC_K_AUX, 1, [&] { launch_vfield_tc_finalize(db, 2, 1, st); });
         }
       } else if (pl.f64) {
-        timed(ctx, XTC_K_ASSEMBLE, M2 ? 2 : 1, [&] {
-          launch_assemble_f64(ctx->L.as<double>(), ctx->R.as<double>(), NP, static_cast<int>(kdim), M, st);
-          if (M2) launch_assemble_f64(ctx->L.as<double>(), ctx->R2.as<double>(), NP, static_cast<int>(kdim), M2, st);
-        });
+        // per block of k: the digits of L once, those of R and the contraction for each accumulator
+        for (int64_t k0 = 0; k0 < kdim; k0 += kblk) {
+          const int64_t kp = std::min(kblk, kdim - k0);
+          timed(ctx, XTC_K_AUX, 1, [&] {
+            launch_digits_lr(ctx->L.as<double>(), NP, kdim, k0, kp, ctx->d_sj.as<int>() + c0, n_i, -1,
+                             ctx->d_L.as<uint16_t>(), ctx->d_Le.as<int>(), st);
+          });
+          for (int e = 0; e < (M2 ? 2 : 1); ++e) {
+            timed(ctx, XTC_K_AUX, 1, [&] {
+              launch_digits_lr((e ? ctx->R2 : ctx->R).as<double>(), NP, kdim, k0, kp, ctx->d_sj.as<int>() + c0, n_i,
+                               1, ctx->d_R.as<uint16_t>(), ctx->d_Re.as<int>(), st);
+            });
+            Gemm64Out o{};
+            o.out = e ? M2 : M;
+            o.ld = ldm;
+            if ((rc = run_gemm64(ctx, XTC_K_ASSEMBLE, ctx->d_L, ctx->d_Le, 1, NP, NP, ctx->d_R, ctx->d_Re, NP, kp, o,
+                                 D64_ADD)))
+              return rc;
+          }
+        }
       }
     }
   }
@@ -1156,7 +1275,7 @@ extern "C" int xtc_vfield(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double*
   const int64_t n_out = pl.oe - pl.ob;
   for (int64_t c0 = pl.ob; c0 < pl.oe; c0 += pl.gc) {
     const int64_t n_i = std::min<int64_t>(pl.gc, pl.oe - c0);
-    if ((rc = run_vfield(ctx, pl, d_grid, c0, n_i, maps))) return rc;
+    if ((rc = run_vfield(ctx, pl, d_grid, d_w, c0, n_i, maps))) return rc;
     double* dst = V + (c0 - pl.ob) * per_point;
     if (!out_dev) {
       if (!ensure(ctx->vout, n_i * per_point * 8)) return fail(ctx, XTC_ERR_OOM, "V staging");
@@ -1356,8 +1475,8 @@ extern "C" int xtc_three_body_L(xtc_ctx* ctx, int64_t n_grid, int n_orb, const d
 
 // ====================================================================== two-body integrals K
 // K_pr^qs of the Theory section on the grid: per chunk of outer points V (steps a+b, the
-// context's precision), the table w_j (lap_1 u + |grad_1 u|^2), W and the FP64 sum S of
-// two_body_k.cu; then K[p][q][r][s] = S[pq][rs] + S[rs][pq].
+// context's precision), W (the FP64 contraction with F = lap_1 u + |grad_1 u|^2) and the FP64 sum S
+// of two_body_k.cu; then K[p][q][r][s] = S[pq][rs] + S[rs][pq].
 extern "C" int xtc_two_body_K(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz,
                               const double* weights, const double* phi, const double* dphi, double* K) {
   if (!ctx) return XTC_ERR_ARG;
@@ -1379,40 +1498,58 @@ extern "C" int xtc_two_body_K(xtc_ctx* ctx, int64_t n_grid, int n_orb, const dou
   if (n_i == 0) {
     CUDA_OK(cudaMemsetAsync(Kd, 0, n4 * 8, st));
   } else {
-    // chunk of outer points: the caller's grid_chunk, else what keeps F table + V + W near 6 GB
-    const size_t per_point = static_cast<size_t>(n_grid) * 8 + static_cast<size_t>(4) * NP * 8;
-    int64_t ch = ctx->prm.grid_chunk > 0 ? ctx->prm.grid_chunk
-                                         : std::max<int64_t>(64, static_cast<int64_t>(6e9 / per_point));
-    ch = std::min<int64_t>(std::min<int64_t>(ch, n_i), int64_t{65535} * 64);  // grid.y of the W GEMM
-    const size_t s_bytes = static_cast<size_t>(N) * N * NP * 8;
-    if (!ensure(ctx->k_S, s_bytes) || !ensure(ctx->k_V, static_cast<size_t>(ch) * 3 * NP * 8) ||
-        !ensure(ctx->k_W, static_cast<size_t>(ch) * NP * 8) || !ensure(ctx->k_Ft, static_cast<size_t>(ch) * n_grid * 8) ||
-        !ensure(ctx->k_P, static_cast<size_t>(4) * ctx->n_sm * 4096 * 8))
-      return fail(ctx, XTC_ERR_OOM, "two_body_K workspace (%.2f GB)",
-                  (s_bytes + static_cast<size_t>(ch) * per_point) * 1e-9);
+    Plan pl{};
+    const double *d_grid = nullptr, *d_w = nullptr, *d_phi = nullptr, *d_dphi = nullptr;
+    const bool f64 = ctx->prm.precision == XTC_PREC_FP64;
+    reset_timers(ctx);
+    if ((rc = prepare(ctx, pl, n_grid, n_orb, grid_xyz, weights, phi, &d_grid, &d_w, &d_phi, f64 ? 4 : 1))) return rc;
+    if ((rc = stage_input(ctx, ctx->k_dphi, dphi, static_cast<size_t>(n_grid) * n_orb * 3, &d_dphi))) return rc;
+    CUDA_OK(cudaMemsetAsync(ctx->flag_dev.p, 0, 16, st));
+    launch_check_finite(d_dphi, n_grid * n_orb * 3, ctx->flag_dev.as<int>(), st);
+    int flag = 0;
+    CUDA_OK(cudaMemcpyAsync(&flag, ctx->flag_dev.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CUDA_OK(cudaStreamSynchronize(st));
+    if (flag) return fail(ctx, XTC_ERR_NONFINITE, "NaN or Inf in the orbital gradients");
+    // chunk of outer points: the plan's, and what keeps the rows of W and V and the digits of both
+    // operands of the contraction near 10 GB
+    const double per_point = 4.0 * (D64_BYTES * (static_cast<double>(N) * N + NP) + 8.0 * NP);
+    const int64_t ch = block_of(ctx->d64_budget * 10e9, per_point, pl.gc);
+    const int64_t NN = static_cast<int64_t>(N) * N;
+    const size_t s_bytes = static_cast<size_t>(NN) * NP * 8;
+    if (!ensure(ctx->k_S, s_bytes) || !ensure(ctx->k_W, static_cast<size_t>(4) * ch * NP * 8) ||
+        !ensure(ctx->k_dphiT, static_cast<size_t>(3) * N * pl.NGp * 8) ||
+        !ensure(ctx->d_L, static_cast<size_t>(D64_BYTES) * NN * 4 * ch) || !ensure(ctx->d_Le, 4ull * NN) ||
+        !ensure(ctx->d_R, static_cast<size_t>(D64_BYTES) * NP * 4 * ch) || !ensure(ctx->d_Re, 4ull * NP))
+      return fail(ctx, XTC_ERR_OOM, "two_body_K workspace (%.2f GB)", (s_bytes + ch * per_point) * 1e-9);
+    VfMaps maps{};
+    if ((rc = make_vfield_maps(ctx, pl, maps))) return rc;
+    launch_transpose_phi(d_dphi, n_grid, pl.NGp, 3 * N, ctx->k_dphiT.as<double>(), st);  // row 3 q + x
     CUDA_OK(cudaMemsetAsync(ctx->k_S.p, 0, s_bytes, st));
-    for (int64_t c0 = ob; c0 < oe; c0 += ch) {
-      const int64_t n_c = std::min<int64_t>(ch, oe - c0);
-      // steps (a)+(b) for the chunk; this also stages grid, weights and orbitals and checks them
-      if ((rc = xtc_vfield(ctx, n_grid, n_orb, grid_xyz, weights, phi, c0, c0 + n_c, ctx->k_V.as<double>())))
-        return rc;
-      const double *d_grid = nullptr, *d_w = nullptr, *d_phi = nullptr, *d_dphi = nullptr;
-      if ((rc = stage_input(ctx, ctx->grid, grid_xyz, static_cast<size_t>(n_grid) * 3, &d_grid))) return rc;
-      if ((rc = stage_input(ctx, ctx->w, weights, static_cast<size_t>(n_grid), &d_w))) return rc;
-      if ((rc = stage_input(ctx, ctx->phi, phi, static_cast<size_t>(n_grid) * n_orb, &d_phi))) return rc;
-      if ((rc = stage_input(ctx, ctx->k_dphi, dphi, static_cast<size_t>(n_grid) * n_orb * 3, &d_dphi))) return rc;
-      if (c0 == ob) {
-        CUDA_OK(cudaMemsetAsync(ctx->flag_dev.p, 0, 16, st));
-        launch_check_finite(d_dphi, n_grid * n_orb * 3, ctx->flag_dev.as<int>(), st);
-        int flag = 0;
-        CUDA_OK(cudaMemcpyAsync(&flag, ctx->flag_dev.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-        CUDA_OK(cudaStreamSynchronize(st));
-        if (flag) return fail(ctx, XTC_ERR_NONFINITE, "NaN or Inf in the orbital gradients");
+    for (int64_t c0 = pl.ob; c0 < pl.oe; c0 += ch) {
+      const int64_t n_c = std::min<int64_t>(ch, pl.oe - c0), ncp = round_up(n_c, D64_BK);
+      // rows[rs][c ncp + i]: W in component 0, V in 1..3 (zero past the chunk's points)
+      double* rows = ctx->k_W.as<double>();
+      if (ncp > n_c) CUDA_OK(cudaMemsetAsync(rows, 0, static_cast<size_t>(4) * ncp * NP * 8, st));
+      Gemm64Out o{};
+      o.out = rows;
+      o.ld = 4 * ncp;
+      o.ld_c = ncp;
+      o.c0 = f64 ? 1 : 0;  // FP64 contexts: components grad, F -> 1, 2, 3, 0; others F -> 0
+      if (!f64) {
+        if ((rc = run_vfield(ctx, pl, d_grid, d_w, c0, n_c, maps))) return rc;
+        launch_v_rows(ctx->V.as<float>(), pl.splits, NP, N, ctx->pair_p.as<int>(), ctx->pair_q.as<int>(), n_c, pl.gc,
+                      ncp, rows, st);
       }
-      launch_k_chunk(d_grid, d_w, d_phi, d_dphi, ctx->jp_dev.as<JastrowParams>(), n_grid, N, ctx->pair_p.as<int>(),
-                     ctx->pair_q.as<int>(), c0, n_c, ctx->k_V.as<double>(), ctx->k_Ft.as<double>(),
-                     ctx->k_W.as<double>(), ctx->k_S.as<double>(), ctx->k_P.as<double>(),
-                     static_cast<int64_t>(4) * ctx->n_sm * 4096, ctx->n_sm, st);
+      if ((rc = run_vfield64(ctx, pl, d_grid, d_w, c0, n_c, o, D64_TO_ROWS))) return rc;
+      launch_digits_rows(rows, NP, 4 * ncp, ctx->d_R.as<uint16_t>(), ctx->d_Re.as<int>(), st);
+      launch_digits_psi(ctx->phiT.as<double>(), ctx->k_dphiT.as<double>(), pl.NGp, d_w, c0, n_c, ncp, N,
+                        ctx->d_L.as<uint16_t>(), ctx->d_Le.as<int>(), st);
+      Gemm64Out so{};
+      so.out = ctx->k_S.as<double>();
+      so.ld = NP;
+      if ((rc = run_gemm64(ctx, XTC_K_ASSEMBLE, ctx->d_L, ctx->d_Le, 1, NN, NN, ctx->d_R, ctx->d_Re, NP, 4 * ncp, so,
+                           D64_ADD)))
+        return rc;
       CUDA_OK(cudaGetLastError());
     }
     launch_k_unpack(ctx->k_S.as<double>(), N, Kd, ctx->n_sm, st);

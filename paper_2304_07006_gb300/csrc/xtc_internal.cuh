@@ -49,6 +49,7 @@ static_assert(GEMM_BITS_A + gemm_bits_b(4) + 5 + 2 <= 24 && 2 * gemm_bits_lr(4) 
 constexpr int DEV_ERR_TIMEOUT_VF = 1;
 constexpr int DEV_ERR_TIMEOUT_AS = 2;
 constexpr int DEV_ERR_TIMEOUT_SELFTEST = 3;
+constexpr int DEV_ERR_TIMEOUT_G64 = 4;
 // Self-test of the bounded waits: one CTA waits on an mbarrier that nothing arrives on, with the
 // kernels' own wait routine and a limit of limit_ns, and records DEV_ERR_TIMEOUT_SELFTEST in err.
 void launch_wait_timeout_selftest(int* err, unsigned long long limit_ns, cudaStream_t st);
@@ -187,6 +188,68 @@ void launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const 
 // Then, with FP64 sums (a.flush > 0): mode 0 writes V from them, mode 1 adds the tiles into M.
 void launch_vfield_tc_finalize(const VfieldArgs& a, int parts, int splits, cudaStream_t st);
 
+// ---------------------------------------------------------------- FP64 contractions on the tensor cores
+// C[m][n] = sum_k A[m][k] B[n][k], both operands as eight planes of 9-bit digits in fp16,
+// planes[d][row][Kp], one exponent per row (digits64.cuh, gemm64_tc.cu).  Kp is a multiple of D64_BK,
+// zero past the operand's K.
+constexpr int D64_PLANES = 8;
+constexpr int D64_BM = 128, D64_BN = 32, D64_BK = 64;   // tile rows and columns, values of k per range
+constexpr int D64_NONFINITE = 1 << 20;                  // exponent of a row that holds an infinity or a NaN
+constexpr int D64_NO_SCALE = -(1 << 20);                // point scale of an inner point without density
+struct Gemm64Args {
+  int m_tiles, n_tiles;        // 128-row tiles of A (mt_per_c per component), 32-column tiles
+  int mt_per_c;                // row tiles per component of A; component c starts at row c * c_rows
+  int64_t c_rows;
+  int m_rows, n_cols;          // valid rows of a component, valid columns
+  int n_ranges;                // Kp / D64_BK
+  int ranges_per_split;        // set by the launcher
+  const int* exp_a;
+  const int* exp_b;
+  double* C;                   // [splits][tile][32][128]
+  int* err;
+};
+// Where the sum over the slices goes (gemm64_finalize_kernel).
+enum { D64_TO_V = 0, D64_TO_ROWS = 1, D64_ADD = 2 };
+struct Gemm64Out {
+  double* out;
+  int64_t ld, ld_c;
+  int c0, n_orb;
+  int add;
+  int64_t i0;                  // first point of the rows (D64_TO_V, D64_TO_ROWS)
+  const int* pair_p;
+  const int* pair_q;
+};
+int gemm64_splits(int m_tiles, int n_tiles, int n_ranges, int n_sm);
+size_t gemm64_tile_bytes(int m_tiles, int n_tiles, int splits);
+void launch_gemm64(const CUtensorMap* tm_a, const CUtensorMap* tm_b, const Gemm64Args& a, int splits,
+                   cudaStream_t st);
+void launch_gemm64_finalize(const Gemm64Args& a, int splits, const Gemm64Out& o, int mode, cudaStream_t st);
+// Digits: FP64 rows of L (sign -1) or R (+1) from value k0 on, K of them, with the point scales of rho and A
+// (gemm64_tc.cu; sj: launch_point_scale, of the chunk's first point); rows of K values as they are;
+// rho^T[pq][j] 2^-sj[j] of n_j inner points; the left operand of the contraction of K (rows p N + q,
+// k = c ncp + i; dphiT[3 q + x][j]).
+void launch_digits_lr(const double* src, int64_t rows, int64_t ld, int64_t k0, int64_t K, const int* sj, int64_t n_i,
+                      int sign, uint16_t* planes, int* exps, cudaStream_t st);
+void launch_digits_rows(const double* src, int64_t rows, int64_t K, uint16_t* planes, int* exps, cudaStream_t st);
+void launch_digits_rho(const double* phiT, int64_t ld, const double* w, int64_t n_j, int64_t Kp, int n_orb,
+                       const int* pair_p, const int* pair_q, const int* sj, uint16_t* planes, int* exps,
+                       cudaStream_t st);
+// sj[j]: exponent of |w_j| max_p (phi_p(j) / max phi_p)^2, the common scale of inner point j; orb[n_orb]: scratch.
+void launch_point_scale(const double* phiT, int64_t ld, const double* w, int64_t n_grid, int n_orb, int* orb, int* sj,
+                        cudaStream_t st);
+void launch_digits_psi(const double* phiT, const double* dphiT, int64_t ld, const double* w, int64_t i0, int64_t n_i,
+                       int64_t ncp, int n_orb, uint16_t* planes, int* exps, cudaStream_t st);
+// Pair functions of the Jastrow factor in FP64 as digit rows (grad64.cu): comps = 3: the three components
+// of grad_1 u, 4: those and F = lap_1 u + |grad_1 u|^2, 1: F alone; row c * c_rows + il for outer point
+// i0 + il, n_j inner points, values times 2^sj[j].  jt[3 + n_nuc][ld]: those points (launch_jtab64_soa); scratch:
+// grad64_scratch_bytes.
+size_t grad64_scratch_bytes(int comps, int64_t n_i, int64_t Kp, int n_sm);
+void launch_jtab64_soa(const double* grid, int64_t n_grid, int64_t n_pad, const JastrowParams* jp, int n_nuc,
+                       double* jt, cudaStream_t st);
+void launch_grad64_digits(const double* grid, const JastrowParams* jp, int n_nuc, const double* jt, const int* sj,
+                          int64_t ld, int64_t n_j, int64_t Kp, int64_t i0, int64_t n_i, int64_t c_rows, int comps, double* scratch,
+                          uint16_t* planes, int* exps, int n_sm, cudaStream_t st);
+
 // Steps (a)+(b), FP64 SIMT twin.  V in the layout of v_index (FP64).  jtab64[n_grid_pad][3 + n_nuc].
 void launch_jtab64(const double* grid, int64_t n_grid, int64_t n_pad, const JastrowParams* jp, int n_nuc,
                    double* jtab, cudaStream_t st);
@@ -199,8 +262,7 @@ void launch_jastrow_grad(const JastrowParams* jp, const double* r1, const double
                          cudaStream_t st);
 
 // Step (c).  Reads V (T = float or double, [splits] slices in the layout of v_index), writes L = (rho, Vx, Vy, Vz) and
-// R = (A, Bx, By, Bz) per outer point, either as split parts [part][pq][4*gcp] (fp16/bf16) or as FP64
-// [4*gcp][pq].
+// R = (A, Bx, By, Bz) per outer point as rows [pq][4*gcp], FP32, FP64 or split into bf16 parts.
 struct FieldsArgs {
   const void* V;
   int splits;
@@ -221,7 +283,7 @@ struct FieldsArgs {
   void* R;
   void* R2;                    // spin builds: R for electron-2 spin beta (R is alpha); nullptr otherwise
   const double* lam2;          // spin builds: beta exchange weights (lam holds the alpha ones)
-  int out_parts;               // 0 = FP64 [4*gcp][pq]; 1 = FP32 [pq][4*gcp]; 3 = bf16 x3 split [part][pq][4*gcp]
+  int out_parts;               // 0 = FP64 [pq][4*gcp]; 1 = FP32 [pq][4*gcp]; 3 = bf16 x3 split [part][pq][4*gcp]
   int write_L;                 // write L (the first pass over a density's factors)
   int add_R;                   // add R (and R2) to the buffer's contents (later passes; out_parts 0 or 1)
 };
@@ -242,9 +304,6 @@ void launch_lr_split(const float* src, int rows, int64_t kdim, int kc, int kd, u
 void launch_assemble_tc(const CUtensorMap* tm_L, const CUtensorMap* tm_R, int n_pair, int kdim, int kd, double* M,
                         int* err, cudaStream_t st);
 
-// Step (d), FP64 SIMT twin: M[pq][rs] += sum_k L[k][pq] R[k][rs].
-void launch_assemble_f64(const double* L, const double* R, int n_pair, int kdim, double* M, cudaStream_t st);
-
 // Final: M <- Delta U = -(M + M^T) in place; unpacking; Delta h; e0.  M row stride round_up(n_pair, AS_BN).
 void launch_symmetrize(double* M, int n_pair, cudaStream_t st);
 void launch_unpack(const double* M, int n_orb, int n_pair, double* dU, float* dU32, cudaStream_t st);
@@ -253,13 +312,9 @@ void launch_unpack(const double* M, int n_orb, int n_pair, double* dU, float* dU
 void launch_three_body_t(const double* phi, const double* w, int64_t i0, int64_t n_i, int n_orb, const int* pair_p,
                          const int* pair_q, const double* V, double* T, cudaStream_t st);
 void launch_three_body_unpack(const double* T, int n_orb, double* L, cudaStream_t st);
-// Two-body integrals K: one chunk of outer points [i0, i0 + n_i) adds into S (N^2 x n_pair, FP64)
-// from V of the chunk ([n_i][3][n_pair]); Ft (n_grid x n_i), W (n_i x n_pair) and partial
-// (split-K slices of small GEMMs, partial_elems doubles; 4 x n_sm x 4096 suffice) are workspace.
-void launch_k_chunk(const double* grid, const double* w, const double* phi, const double* dphi,
-                    const JastrowParams* jp_dev, int64_t n_grid, int n_orb, const int* pair_p, const int* pair_q,
-                    int64_t i0, int64_t n_i, const double* V, double* Ft, double* W, double* S, double* partial,
-                    int64_t partial_elems, int n_sm, cudaStream_t st);
+// Two-body integrals K: rows[pq][(1 + x) ncp + i] = V_x,pq(i) in FP64 from a chunk's V (FP32, slices added).
+void launch_v_rows(const float* V, int splits, int n_pair, int n_orb, const int* pair_p, const int* pair_q,
+                   int64_t n_i, int64_t gcp, int64_t ncp, double* rows, cudaStream_t st);
 // K[p][q][r][s] = S[pq][rs] + S[rs][pq].
 void launch_k_unpack(const double* S, int n_orb, double* K, int n_sm, cudaStream_t st);
 // Spin builds: U = Delta U^{ab} = -(Fb + Fa^T) (packed pairs, row stride m_stride(n_pair)).
