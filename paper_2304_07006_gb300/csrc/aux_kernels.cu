@@ -138,8 +138,8 @@ __global__ void rho_colmax_f32_kernel(const float* __restrict__ f32, int64_t n_g
 // accumulation range of the GEMM, points j0 + lane + 32 s (s < kd, j0 = 32 kd blockIdx.x); the
 // range shares one quantum (largest |value| of the range, `bits` bits).  rho = rh + rl in FP32
 // pairs (rho_pair_f32); hi = rh rounded to the quantum (exact), lo = fp16((rh - hi) + rl), whose
-// rounding error is far below fp16's.  Layout: the two parts of a 32-point block share one 128-byte
-// row, [pq][j / 32][part][j % 32]; then the plane [pq][j] of the value rounded to fp16.
+// rounding error is far below fp16's.  Layout: 128-byte runs of 64 points of one part,
+// [pq][j / 64][part][j % 64]; then the plane [pq][j] of the value rounded to fp16.
 __global__ void rho_split_f16_kernel(const float* __restrict__ f32, int64_t n_grid, int64_t n_pad, int n_orb,
                                      int n_pair, const int* __restrict__ pp, const int* __restrict__ pq_,
                                      const unsigned int* __restrict__ colmax, int kd, int bits,
@@ -175,9 +175,9 @@ __global__ void rho_split_f16_kernel(const float* __restrict__ f32, int64_t n_gr
     if (s >= kd || j >= n_pad) break;
     float h = 0.0f;
     if (qe >= -24) h = rintf(vh[s] * pow2f(-qe)) * pow2f(qe);  // both products exact (powers of 2)
-    const int64_t o = static_cast<int64_t>(pq) * 2 * n_pad + (j >> 5) * 64 + (j & 31);
+    const int64_t o = static_cast<int64_t>(pq) * 2 * n_pad + (j >> 6) * 128 + (j & 63);
     out[o] = __half_as_ushort(__float2half_rn(h));                      // exact: at most 10 bits
-    out[o + 32] = __half_as_ushort(__float2half_rn((vh[s] - h) + vl[s]));  // vh - h is exact
+    out[o + 64] = __half_as_ushort(__float2half_rn((vh[s] - h) + vl[s]));  // vh - h is exact
     out16[static_cast<int64_t>(pq) * n_pad + j] = __half_as_ushort(__float2half_rn(vh[s]));
   }
 }
@@ -273,9 +273,9 @@ __global__ void __launch_bounds__(256) lr_split_kernel(const float* __restrict__
         __half h, l;
         split_exact(v[t][c], qe, h, l);
         const int64_t kk = c * per_c + 32 * (kd * g + t);  // first value of the 32-value block
-        const int64_t blk = kk >> 5;
-        d[blk * 64 + lane] = __half_as_ushort(h);
-        d[blk * 64 + 32 + lane] = __half_as_ushort(l);
+        const int64_t o = (kk >> 6) * 128 + (kk & 63) + lane;
+        d[o] = __half_as_ushort(h);
+        d[o + 64] = __half_as_ushort(l);
         if (dst16) dst16[r * kdim + kk + lane] = __half_as_ushort(__float2half_rn(v[t][c]));
       }
     }

@@ -2,8 +2,8 @@
 // (outer point i, inner point j) pair of a chunk (section "Decomposition of two-body correction",
 // the factor that multiplies rho in V), split into fp16 (2 parts) or bf16 (3 parts) and stored
 // K-major as the A operand of the step (b) GEMM, row x * gcp + il (il = i - i0):
-//     fp16: G[row][j / 32][part][j % 32]  (both parts of a 32-point block in one 128-byte row,
-//           128-byte swizzle tiles, so that one TMA row request moves 128 bytes);
+//     fp16: G[row][j / 64][part][j % 64]  (128-byte runs of 64 points of one part, 128-byte swizzle
+//           tiles, so that one TMA row request moves 128 bytes);
 //     bf16: G[part][row][j]               (one plane per part, 64-byte swizzle tiles).
 // Computing G once per chunk, instead of inside every orbital-pair tile of the GEMM, removes the
 // gradient from the GEMM's critical path; the table costs one HBM write and is then read through L2
@@ -18,9 +18,9 @@
 // bytes) into shared memory in their swizzle (conflict-free 16-byte stores) and one lane stores
 // them with TMA.  The fp16 split is exact on a per-range quantum (simt_pack.cuh): for every row and
 // accumulation range of the GEMM (RB blocks of 32 inner points), hi = an integer of at most 9
-// bits times the range's quantum, lo = the fp16 remainder.  The lane first stages its RB x 32
-// FP32 values per component in its own tile rows, then splits them with the quantum of their
-// maximum; a warp then holds RB blocks of tiles, and a CTA GF_WARPS / RB warps.
+// bits times the range's quantum, lo = the fp16 remainder.  The lane first stages the FP32 values of
+// two blocks (64 points, a hi and a lo tile per component; four blocks when RB = 4) in its own tile rows,
+// then splits them with the quantum of their range's maximum; a CTA holds GF_WARPS / BB warps of BB blocks.
 // The gradient is taken with the pair formula of jastrow_coef.cuh: per-point coefficients times
 // polynomials in b = r12 / (1 + r12) and a_jI = |r_j - R_I| / (1 + |r_j - R_I|).
 #include "jastrow_coef.cuh"
@@ -57,8 +57,9 @@ __global__ void __launch_bounds__(GF_THREADS)
   constexpr bool BF16 = PARTS == 3;
   constexpr int JS = NNUC <= 4 ? 12 : 16;  // floats per inner point in the table (launch_jtab)
   constexpr int BLOCK_BYTES = 3 * PARTS * GF_TILE;  // the three component tiles of one block
-  constexpr int WARP_BYTES = RB * BLOCK_BYTES;       // RB blocks: one exact range of the GEMM
-  constexpr int WARPS = GF_WARPS / RB;
+  constexpr int BB = PARTS == 2 && RB < 2 ? 2 : RB;   // blocks staged together: whole pairs for the fp16 tiles
+  constexpr int WARP_BYTES = BB * BLOCK_BYTES;
+  constexpr int WARPS = GF_WARPS / BB;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -91,13 +92,17 @@ __global__ void __launch_bounds__(GF_THREADS)
     ZL = pk2(zl, zl);
   }
   const int row0 = tile * 32;
-  float gmax[3] = {0.0f, 0.0f, 0.0f};  // fp16: largest |G| of the range per component
+  constexpr int NQ = PARTS == 2 ? BB / RB : 1;   // exact ranges staged together
+  float gmax[NQ][3];                   // fp16: largest |G| of each range per component
+#pragma unroll
+  for (int v = 0; v < NQ; ++v) gmax[v][0] = gmax[v][1] = gmax[v][2] = 0.0f;
 
-  for (int kr = kb0; kr < kb1; kr += RB) {
+  for (int kr = kb0; kr < kb1; kr += BB) {
 #pragma unroll 1
-  for (int rb = 0; rb < RB; ++rb) {
+  for (int rb = 0; rb < BB; ++rb) {
     const int kb = kr + rb;
-    const uint32_t bbuf = buf + rb * BLOCK_BYTES;
+    // bf16: the block's own tiles; fp16: the hi and lo tiles of the block's pair
+    const uint32_t bbuf = buf + (PARTS == 2 ? (rb >> 1) * 2 : rb) * BLOCK_BYTES;
     // 16 records of two inner points each (the pair-interleaved table written by launch_jtab)
     const float* blk = args.jtab + static_cast<int64_t>(kb) * VF_BK * JS;
 #pragma unroll 1
@@ -198,15 +203,20 @@ __global__ void __launch_bounds__(GF_THREADS)
         __syncwarp();
       }
       if constexpr (PARTS == 2) {
-        // FP32 staging in the lane's own 128-byte rows of the block's component tiles (16-byte
-        // chunks b, b + 1 with b = 0, 4, 2, 6 for c = 0..3, so that the split below rewrites, for
-        // each half of the block, exactly the chunks it has read), and the range maxima
-        const int b = (c & 1) * 4 + (c >> 1) * 2;
+        // FP32 staging in the lane's own 128-byte rows of the pair's component tiles: points 8c .. 8c + 7 in
+        // the hi tile for even c, the lo tile for odd c, 16-byte chunks b and b + 1 with b = 4 (rb % 2) +
+        // 2 (c / 2), so that the split below rewrites, for each half of the block, exactly the chunks
+        // it has read; and the range maxima
+        const int b = (rb & 1) * 4 + (c >> 1) * 2;
 #pragma unroll
         for (int x = 0; x < 3; ++x) {
+          float m = 0.0f;
 #pragma unroll
-          for (int k = 0; k < 8; ++k) gmax[x] = fmaxf(gmax[x], fabsf(gv[x][k]));
-          const uint32_t row = bbuf + x * 2 * GF_TILE;
+          for (int k = 0; k < 8; ++k) m = fmaxf(m, fabsf(gv[x][k]));
+#pragma unroll
+          for (int v = 0; v < NQ; ++v)
+            if (NQ == 1 || rb == v) gmax[v][x] = fmaxf(gmax[v][x], m);
+          const uint32_t row = bbuf + (2 * x + (c & 1)) * 2 * GF_TILE;
           st_shared_v4(row + sw128_offset(lane, b), __float_as_uint(gv[x][0]), __float_as_uint(gv[x][1]),
                        __float_as_uint(gv[x][2]), __float_as_uint(gv[x][3]));
           st_shared_v4(row + sw128_offset(lane, b + 1), __float_as_uint(gv[x][4]), __float_as_uint(gv[x][5]),
@@ -226,54 +236,54 @@ __global__ void __launch_bounds__(GF_THREADS)
     }
   }
     if constexpr (PARTS == 2) {
-      // exact split of the lane's RB x 32 values per component on the range's quantum: hi of
-      // points 8c .. 8c + 7 of a block goes to chunk c, lo to chunk 4 + c (component tile x of 32
-      // rows x 128 bytes, the layout the GEMM loads)
+      // exact split of the lane's values per component on their range's quantum: hi of points 8c .. 8c + 7 of
+      // the pair's block rb goes to chunk 4 (rb % 2) + c of the hi tile, lo to the same chunk of the lo tile
+      // (tiles of 32 rows x 128 bytes, the layout the GEMM loads)
 #pragma unroll
       for (int x = 0; x < 3; ++x) {
-        const int q = exact_quantum(gmax[x], GF_EXACT_BITS);
-        gmax[x] = 0.0f;
 #pragma unroll
-        for (int rb = 0; rb < RB; ++rb) {
-          const uint32_t row = buf + rb * BLOCK_BYTES + x * 2 * GF_TILE;
+        for (int rb = 0; rb < BB; ++rb) {
+          const int q = exact_quantum(gmax[NQ == 1 ? 0 : rb][x], GF_EXACT_BITS);
+          const uint32_t hi = buf + (rb >> 1) * 2 * BLOCK_BYTES + 2 * x * 2 * GF_TILE, lo = hi + 2 * GF_TILE;
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            // sub-blocks c = 2h (staged in chunks 2h, 2h + 1) and 2h + 1 (chunks 4 + 2h, 5 + 2h)
+            const uint32_t c0 = sw128_offset(lane, 4 * (rb & 1) + 2 * h), c1 = sw128_offset(lane, 4 * (rb & 1) + 2 * h + 1);
             uint32_t f[16];
-            ld_shared_v4(row + sw128_offset(lane, 2 * h), f[0], f[1], f[2], f[3]);
-            ld_shared_v4(row + sw128_offset(lane, 2 * h + 1), f[4], f[5], f[6], f[7]);
-            ld_shared_v4(row + sw128_offset(lane, 4 + 2 * h), f[8], f[9], f[10], f[11]);
-            ld_shared_v4(row + sw128_offset(lane, 5 + 2 * h), f[12], f[13], f[14], f[15]);
+            ld_shared_v4(hi + c0, f[0], f[1], f[2], f[3]);
+            ld_shared_v4(hi + c1, f[4], f[5], f[6], f[7]);
+            ld_shared_v4(lo + c0, f[8], f[9], f[10], f[11]);
+            ld_shared_v4(lo + c1, f[12], f[13], f[14], f[15]);
             uint32_t w[8][2];
 #pragma unroll
             for (int k = 0; k < 8; ++k)
               split_pair_exact(__uint_as_float(f[2 * k]), __uint_as_float(f[2 * k + 1]), q, w[k]);
-            st_shared_v4(row + sw128_offset(lane, 2 * h), w[0][0], w[1][0], w[2][0], w[3][0]);
-            st_shared_v4(row + sw128_offset(lane, 2 * h + 1), w[4][0], w[5][0], w[6][0], w[7][0]);
-            st_shared_v4(row + sw128_offset(lane, 4 + 2 * h), w[0][1], w[1][1], w[2][1], w[3][1]);
-            st_shared_v4(row + sw128_offset(lane, 5 + 2 * h), w[4][1], w[5][1], w[6][1], w[7][1]);
+            st_shared_v4(hi + c0, w[0][0], w[1][0], w[2][0], w[3][0]);
+            st_shared_v4(hi + c1, w[4][0], w[5][0], w[6][0], w[7][0]);
+            st_shared_v4(lo + c0, w[0][1], w[1][1], w[2][1], w[3][1]);
+            st_shared_v4(lo + c1, w[4][1], w[5][1], w[6][1], w[7][1]);
           }
         }
       }
+#pragma unroll
+      for (int v = 0; v < NQ; ++v) gmax[v][0] = gmax[v][1] = gmax[v][2] = 0.0f;
     }
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) {
+      if constexpr (PARTS == 2) {
 #pragma unroll
-      for (int rb = 0; rb < RB; ++rb) {
-        const int kb = kr + rb;
-        const uint32_t bbuf = buf + rb * BLOCK_BYTES;
+        for (int pr = 0; pr < BB / 2; ++pr)
 #pragma unroll
-        for (int x = 0; x < 3; ++x) {
-          if (PARTS == 2) {
-            tma_store_3d(&tm_g, bbuf + x * 2 * GF_TILE, kb * 2 * VF_BK, static_cast<int>(x * args.gcp) + row0, 0);
-          } else {
+          for (int t = 0; t < 6; ++t)  // component t / 2, part t % 2
+            tma_store_3d(&tm_g, buf + (2 * pr) * BLOCK_BYTES + t * 2 * GF_TILE, (kr / 2 + pr) * 128 + (t & 1) * 64,
+                         static_cast<int>((t >> 1) * args.gcp) + row0, 0);
+      } else {
 #pragma unroll
-            for (int p = 0; p < PARTS; ++p)
-              tma_store_3d(&tm_g, bbuf + (x * PARTS + p) * GF_TILE, kb * VF_BK, static_cast<int>(x * args.gcp) + row0,
-                           p);
-          }
-        }
+        for (int rb = 0; rb < BB; ++rb)
+#pragma unroll
+          for (int t = 0; t < 3 * PARTS; ++t)  // component t / PARTS, part t % PARTS
+            tma_store_3d(&tm_g, buf + rb * BLOCK_BYTES + t * GF_TILE, (kr + rb) * VF_BK,
+                         static_cast<int>((t / PARTS) * args.gcp) + row0, t % PARTS);
       }
       bulk_commit();
     }
@@ -285,8 +295,8 @@ __global__ void __launch_bounds__(GF_THREADS)
 template <int PARTS, int NNUC, int RB>
 void launch_rb(const CUtensorMap* tm, const GfieldArgs& a, cudaStream_t st) {
   auto kern = gfield_kernel<PARTS, NNUC, RB>;
-  constexpr int warps = GF_WARPS / RB;
-  constexpr int smem = GF_WARPS * 3 * PARTS * GF_TILE + 1024;  // warps x RB blocks of three tiles
+  constexpr int warps = GF_WARPS / (PARTS == 2 && RB < 2 ? 2 : RB);
+  constexpr int smem = GF_WARPS * 3 * PARTS * GF_TILE + 1024;  // warps x staged blocks of three tiles
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const int64_t units = static_cast<int64_t>(a.n_tiles) * a.n_seg;
   const unsigned blocks = static_cast<unsigned>((units + warps - 1) / warps);

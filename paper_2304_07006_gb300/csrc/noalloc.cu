@@ -201,7 +201,7 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
     // rho^T (box rows vf_bn) and the gradient table [part][x * gc + il][j] (boxes 32 x 32
     // for the step (a) stores and 32 x 128 for the step (b) loads)
     auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(cv.encode_tiled);
-    // (fp16: both parts of a 32-point block in one 128-byte row; bf16: one plane per part)
+    // (fp16: 128-byte runs of 64 values of one part; bf16: one plane per part)
     const bool wide = parts == 2;
     const int64_t cols = wide ? 2 * NGp : NGp, planes = wide ? 1 : parts;
     auto map = [&](CUtensorMap* m, void* base, int64_t rows, uint32_t box_rows) {
@@ -218,13 +218,13 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
     if (!map(&tm, rho, NP, vf_bn(parts)) || !map(&tm_gs, G, 3 * gc, 32) || !map(&tm_gl, G, 3 * gc, VF_BM))
       return xtc_internal_fail(ctx, XTC_ERR_CUDA, "noalloc: cuTensorMapEncodeTiled failed");
     if (wide) {
-      // the fp16(rho^T) plane after the split rows: [pq][j], boxes 32 x vf_bn (64-byte swizzle)
+      // the fp16(rho^T) plane after the split rows: [pq][j], boxes 64 x vf_bn / 2
       const cuuint64_t dims[3] = {static_cast<cuuint64_t>(NGp), static_cast<cuuint64_t>(NP), 1};
       const cuuint64_t strides[2] = {static_cast<cuuint64_t>(NGp) * 2, static_cast<cuuint64_t>(NGp) * NP * 2};
-      const cuuint32_t box[3] = {static_cast<cuuint32_t>(VF_BK), static_cast<cuuint32_t>(vf_bn(2)), 1};
+      const cuuint32_t box[3] = {static_cast<cuuint32_t>(2 * VF_BK), static_cast<cuuint32_t>(vf_bn(2) / 2), 1};
       const cuuint32_t es[3] = {1, 1, 1};
       if (encode(&tm16, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, static_cast<uint16_t*>(rho) + 2 * static_cast<size_t>(NP) * NGp,
-                 dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                 dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return xtc_internal_fail(ctx, XTC_ERR_CUDA, "noalloc: cuTensorMapEncodeTiled failed");
     }

@@ -25,18 +25,23 @@
 // product where two would be needed.
 //
 // Tile 128 A rows x 128 columns, 32 K values per stage, both parts of a row of a block in one
-// 128-byte row (128-byte swizzle; one TMA box per operand part and stage).  Measured
-// on GB300: one thread issues a 128 x 128 x 16 MMA every ~50 cycles (the pipe takes 64), an MMA
-// and its commit round-trip in ~360 cycles, and a range's round trip (its MMAs complete, the
-// commit arrives, the drains read E, E is handed back) takes on the order of a thousand cycles.
-// So ranges span two stages (12 MMAs), and two issuers alternate ranges, each with its own
-// accumulator pair (TMEM: E0, X0, E1, X1 = 4 x 128 of 512 columns).  A stage holds 40 KB (A and B
-// hi/lo, fp16(B)); 5 stages.  Warp roles:
-//   * warp 0 (one lane): TMA loads; a slot is reloaded once the MMAs of its stage have completed;
-//   * warps 1 and 2 (one lane each): the MMAs of the even / odd ranges, a commit per stage (it
-//     frees the slot) and one per range (it starts the drains);
-//   * warps 3..18: after every range, drains of E_k, and every `xper` stages of X_k, into FP32
-//     running sums held in registers (four warps per TMEM lane quarter, 32 columns each).  The
+// 128-byte row of 64 values per part: [row][K / 64][hi, lo][64].
+//
+// Tile and split of the work.  With one CTA per 128 x 128 tile the engine was bound by shared
+// memory: per 32 values of K the six MMAs read 48 KB of operands and the loads wrote 40 KB, 704 cycles
+// at 128 bytes per clock (705 measured) for 384 cycles of tensor pipe.  Two things cut that: pairs of
+// CTAs share a 256 x 128 tile (tcgen05 cta_group::2: 256 rows of A, each CTA loads half of B), and
+// hi_a x hi_b and hi_a x lo_b are one MMA of 256 columns, [hi_b | lo_b], with hi_b in the leader's shared
+// memory and lo_b in the other's, writing the adjacent accumulators [E | X], so hi_a is read once.  Per
+// 64 values and CTA: 56 KB read, 56 KB written, 875 cycles for 768 of tensor pipe.
+//   * warp 0 of each CTA (one lane): TMA loads (4 stages of 56 KB: hi and lo of A, one part of B, half of
+//     fp16(B)), completing on the leader's barriers; a slot is reloaded once its MMAs have completed;
+//   * warps 1 and 2 of the leader: the MMAs of the even / odd ranges into the accumulator sets (E0, X0) and
+//     (E1, X1) (4 x 128 of 512 TMEM columns in each CTA), so that one set is drained while
+//     the other fills; commits (to both CTAs) after every stage and every range;
+//   * warps 3..18 of each CTA: after every range, drains of E_k, and every `xper` blocks of X_k, into FP32
+//     running sums held in registers (four warps per TMEM lane quarter, 32 columns each); what was
+//     read is set to zero, so that every MMA accumulates.  The
 //     sums move into an FP64 accumulator in HBM, private to the CTA and column-major in its tile,
 //     one column per range in turn (each column at least once per `flush` ranges; each element
 //     belongs to one thread); vfield_finalize_kernel writes V from it (MODE 0).
@@ -76,86 +81,87 @@ __device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t (&r)[16]) {
 struct TileXY {
   int m_tile, n_tile;
 };
+template <int G = GM>
 __device__ __forceinline__ TileXY grouped_tile(int L, int m_tiles, int n_tiles) {
-  const int group = L / (GM * n_tiles);
-  const int first_m = group * GM;
-  const int gm = min(GM, m_tiles - first_m);
-  const int rem = L - group * GM * n_tiles;
+  const int group = L / (G * n_tiles);
+  const int first_m = group * G;
+  const int gm = min(G, m_tiles - first_m);
+  const int rem = L - group * G * n_tiles;
   return {first_m + rem % gm, rem / gm};
 }
 
+// Tile of CTA L of the fp16 engine: consecutive CTAs are the two row tiles of a pair; groups of GM row
+// tiles x every column tile, pair row fastest.  With an odd number of row tiles the last pair's second
+// tile does not exist (m_tile == m_tiles).
+__device__ __forceinline__ TileXY pair_tile(int L, int m_tiles, int n_tiles) {
+  const TileXY t = grouped_tile<GM / 2>(L >> 1, (m_tiles + 1) >> 1, n_tiles);
+  return {2 * t.m_tile + (L & 1), t.n_tile};
+}
+
 // =================================================================== fp16 x2 engine
-constexpr int XB_BN = 128;                        // tile columns (TMEM accumulator width)
+constexpr int XB_BN = 128;                        // tile columns
+constexpr int XB_BK = 64;                         // K values per stage
 constexpr int XB_DRAIN_WARPS = 16;                // four per TMEM lane quarter, a quarter of the columns each
 constexpr int XB_HC = XB_BN / 4;                  // running-sum columns per drain thread
-constexpr int XB_A_BYTES = VF_BM * 128;           // 128 rows of 128 bytes (hi and lo of 32 values)
-constexpr int XB_B_BYTES = XB_BN * 128;
-constexpr int XB_B16_BYTES = XB_BN * 64;          // fp16(B) of the B rows, 64-byte rows
-// stage bytes and pipeline depth: 40 KB (A, B hi/lo, B fp16) x 5
-__host__ __device__ constexpr int xb_stage(int) { return XB_A_BYTES + XB_B_BYTES + XB_B16_BYTES; }
-__host__ __device__ constexpr int xb_stages(int) { return 5; }
-constexpr int XB_STAGES = 7;                      // the larger depth (barrier arrays)
-constexpr int XB_WARP_I0 = 1, XB_WARP_I1 = 2;      // issuers of the even / odd ranges; drains 3..18
+constexpr int XB_PART = VF_BM * XB_BK * 2;        // 128 rows of 128 bytes: hi or lo of A, hi (leader) or lo of B
+constexpr int XB_B16_BYTES = XB_BN / 2 * XB_BK * 2;  // fp16(B), half of the columns in each CTA
+constexpr int XB_STAGE = 3 * XB_PART + XB_B16_BYTES;
+constexpr int XB_STAGES = 4;
 constexpr int XB_THREADS = (3 + XB_DRAIN_WARPS) * 32;  // TMA warp, two MMA warps, drains
-__host__ __device__ constexpr int xb_smem(int mode) { return xb_stages(mode) * xb_stage(mode) + 1024 + 256; }
+constexpr int XB_SMEM = XB_STAGES * XB_STAGE + 1024 + 256;
+constexpr int XB_SET = 2 * XB_BN;                 // TMEM columns of an accumulator set (E, X)
 static_assert(XB_BN == vf_bn(2), "tile width of the fp16 engine");
-static_assert(4 * XB_BN <= 512, "E0, X0, E1, X1 in 512 TMEM columns");
+static_assert(2 * XB_SET <= 512, "E0, X0, E1, X1 in 512 TMEM columns");
 static_assert(XB_HC == 32, "drain columns per thread (one 32-column load)");
-static_assert(xb_smem(0) <= 232448 && xb_smem(1) <= 232448, "shared memory per CTA");
-static_assert(xb_stages(0) <= XB_STAGES && xb_stages(1) <= XB_STAGES, "barrier arrays");
-// a wait for range r must not alias range r + NRB: the producer waits for the range of stage
-// k - XB_STAGES before loading stage k, and range r + NRB starts past stage k
-static_assert(NRB > XB_STAGES, "range barriers");
-static_assert((XB_STAGES + NRB + 5) * 8 + 8 <= 256, "barrier area");
+static_assert(XB_SMEM <= 232448, "shared memory per CTA");
+static_assert((2 * XB_STAGES + 5) * 8 + 8 <= 256, "barrier area");
 
 // Shared-memory descriptor of a K-major operand in the 128-byte swizzle, for a shared address
 // below 2^18: the constant fields plus the address in 16-byte units (a plain add per stage and
 // K step, no re-encoding in the issue loop).
 __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) { return sdesc_kmajor_sw128(0) + (saddr >> 4); }
-// The same for 64-byte rows in the 64-byte swizzle.
-__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) { return sdesc_kmajor_sw64(0) + (saddr >> 4); }
 
 template <int MODE>
-__global__ void __launch_bounds__(XB_THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(XB_THREADS, 1)
     xgemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                  const __grid_constant__ CUtensorMap tm_b16, const VfieldArgs args) {
-  constexpr int XB_STAGE = xb_stage(MODE), STAGES = xb_stages(MODE);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * XB_STAGE);
-  uint64_t* tma_full = bars;                  // [XB_STAGES] the stage's loads landed
-  uint64_t* rdone = bars + XB_STAGES;         // [NRB] every MMA of range r (r % NRB) completed
-  uint64_t* e_free = rdone + NRB;             // [2] the drains released E_k (issuer k)
-  uint64_t* x_free = e_free + 2;              // [2] the drains released X_k
-  uint64_t* fin_bar = x_free + 2;             // every MMA of both issuers completed
-  uint64_t* sfree = fin_bar + 1;              // [XB_STAGES] the stage's MMAs completed (slot free)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sfree + XB_STAGES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + XB_STAGES * XB_STAGE);
+  uint64_t* full = bars;                 // [XB_STAGES] leader: the stage's loads of both CTAs landed
+  uint64_t* sfree = full + XB_STAGES;    // [XB_STAGES] the stage's MMAs completed (slot free)
+  uint64_t* rdone = sfree + XB_STAGES;   // [2] every MMA of the range in accumulator set k completed
+  uint64_t* e_free = rdone + 2;          // [2] leader: the drains of both CTAs released set k, zeroed
+  uint64_t* fin_bar = e_free + 2;        // leader: every MMA completed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp: uniform
+  const uint32_t rank = cluster_rank();
   const int m_tiles = MODE == 0 ? 3 * args.mt_per_x : (args.rows_a + VF_BM - 1) / VF_BM;
-  const TileXY t = grouped_tile(blockIdx.x, m_tiles, args.n_tiles);
+  const TileXY t = pair_tile(blockIdx.x, m_tiles, args.n_tiles);
+  const bool valid = t.m_tile < m_tiles;          // a tile that does not exist repeats the last one's rows
+  const int m_tile = valid ? t.m_tile : m_tiles - 1;
   // mode 0: rows x * gcp + outer point of component x; mode 1: rows pq
-  const int x = MODE == 0 ? t.m_tile / args.mt_per_x : 0;
-  const int ib = MODE == 0 ? (t.m_tile - x * args.mt_per_x) * VF_BM : t.m_tile * VF_BM;
+  const int x = MODE == 0 ? m_tile / args.mt_per_x : 0;
+  const int ib = MODE == 0 ? (m_tile - x * args.mt_per_x) * VF_BM : m_tile * VF_BM;
   const int row0 = MODE == 0 ? static_cast<int>(x * args.gcp) + ib : ib;
   const int split = blockIdx.y;
-  const int kb0 = split * args.kb_per_split;
-  const int kb1 = min(args.n_kb, kb0 + args.kb_per_split);
-  const int n_it = kb1 - kb0;
-  const int kd = args.kd;                                  // stages per exact range (1, 2 or 4)
+  const int kb0 = split * args.kb_per_split;               // multiple of 2 and of kd
+  const int n_it = min(args.n_kb, kb0 + args.kb_per_split) - kb0;  // blocks of 32 K values, even
+  const int n_st = (n_it + 1) >> 1;                        // stages
+  const int kd = args.kd;                                  // blocks per exact range (1, 2 or 4)
   const int n_ranges = (n_it + kd - 1) / kd;
-  const int xr = max(1, args.xper / (2 * kd));             // ranges of one issuer per X drain
+  const int xr = max(1, args.xper / (2 * kd));             // ranges of one set per X drain
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&tma_full[s], 1);
-      mbar_init(&sfree[s], 1);
+    for (int s = 0; s < XB_STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&sfree[s], args.kd == 1 ? 2 : 1);  // commits per stage: one of each issuer when they share it
     }
-    for (int r = 0; r < NRB; ++r) mbar_init(&rdone[r], 1);
     for (int k = 0; k < 2; ++k) {
-      mbar_init(&e_free[k], XB_DRAIN_WARPS);
-      mbar_init(&x_free[k], XB_DRAIN_WARPS);
+      mbar_init(&rdone[k], 1);
+      mbar_init(&e_free[k], 2 * XB_DRAIN_WARPS);
     }
     mbar_init(fin_bar, 2);
     *abort_flag = 0;
@@ -164,82 +170,94 @@ __global__ void __launch_bounds__(XB_THREADS, 1)
     tma_prefetch_desc(&tm_b);
     tma_prefetch_desc(&tm_b16);
   }
-  if (warp == 0) {
-    tmem_alloc(tmem_slot, 512);
-    tmem_relinquish();
-  }
+  if (warp == 0) tmem_alloc_pair(tmem_slot, 512);
   tc_fence_before();
   __syncthreads();
+  cluster_sync();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t smem_base = smem_u32(smem);
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (warp == 0) {
     if (lane == 0) {
-      // ---------------------------------------------------------------- TMA producer
-      // a slot is refilled as soon as the MMAs of the stage it held have completed (one commit
-      // per stage), not when the whole range has
+      // ---------------------------------------------------------------- TMA producer (both CTAs)
+      // own 128 rows of A (hi and lo), one part of B's 128 columns (hi in the leader, lo in the other
+      // CTA) and half of fp16(B); both CTAs' loads complete on the leader's barrier
       int issued = 0;
-      for (int it = 0; it < n_it; ++it) {
-        const int s = it % STAGES;
-        if (it >= STAGES &&
-            !mbar_wait(&sfree[s], ((it / STAGES) - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF))
+      for (int it = 0; it < n_st; ++it) {
+        const int s = it % XB_STAGES;
+        if (it >= XB_STAGES &&
+            !mbar_wait(&sfree[s], ((it / XB_STAGES) - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF))
           break;
-        mbar_arrive_expect_tx(&tma_full[s], XB_STAGE);
+        if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * XB_STAGE);
+        const uint32_t bar = cluster_addr(&full[s], 0);
         uint8_t* st = smem + s * XB_STAGE;
-        tma_load_3d(st, &tm_a, &tma_full[s], (kb0 + it) * 2 * VF_BK, row0, 0);
-        tma_load_3d(st + XB_A_BYTES, &tm_b, &tma_full[s], (kb0 + it) * 2 * VF_BK, t.n_tile * XB_BN, 0);
-        tma_load_3d(st + XB_A_BYTES + XB_B_BYTES, &tm_b16, &tma_full[s], (kb0 + it) * VF_BK, t.n_tile * XB_BN, 0);
+        const int k0 = kb0 * VF_BK + it * XB_BK;
+        tma_load_3d_pair(st, &tm_a, bar, 2 * k0, row0, 0);
+        tma_load_3d_pair(st + XB_PART, &tm_a, bar, 2 * k0 + XB_BK, row0, 0);
+        tma_load_3d_pair(st + 2 * XB_PART, &tm_b, bar, 2 * k0 + static_cast<int>(rank) * XB_BK, t.n_tile * XB_BN, 0);
+        tma_load_3d_pair(st + 3 * XB_PART, &tm_b16, bar, k0, t.n_tile * XB_BN + static_cast<int>(rank) * (XB_BN / 2), 0);
         issued = it + 1;
       }
-      // the copies still in flight land before the CTA may exit
+      // The last slots come free once their MMAs have read them, so every copy has landed and every
+      // arrival on this CTA's barriers has been made before the CTA exits.  After an abort the leader waits
+      // for the loads it announced instead, and the other CTA (whose loads complete on the leader's
+      // barriers) for a time no copy takes.
       int zero = 0;
-      for (int it = max(0, issued - STAGES); it < issued; ++it)
-        mbar_wait(&tma_full[it % STAGES], (it / STAGES) & 1, reinterpret_cast<volatile int*>(&zero),
-                  args.err, DEV_ERR_TIMEOUT_VF);
-    }
-  } else if (warp == XB_WARP_I0 || warp == XB_WARP_I1) {
-    if (lane == 0) {
-      // ---------------------------------------------------------------- MMA issuers
-      // Issuer k takes the ranges r = k, k + 2, ...: per stage the hi x hi products into E_k (a
-      // fresh, exact accumulation per range) and the cross products hi_a x lo_b, lo_a x fp16(b)
-      // into X_k (restarted every xr of its ranges); a commit after each stage frees
-      // its slot for the next load, one after each range starts the drains.  With two issuers
-      // one's waits and commits overlap the other's MMAs, and neither waits for the other's drains.
-      constexpr uint32_t idesc = idesc_f16(VF_BM, XB_BN, false);
-      const int k = warp == XB_WARP_I0 ? 0 : 1;
-      const uint32_t e_tmem = tmem + 2 * k * XB_BN, x_tmem = e_tmem + XB_BN;
-      for (int r = k, u = 0; r < n_ranges; r += 2, ++u) {
-        const int it0 = r * kd, it1 = min(n_it, it0 + kd);
-        const bool x_start = u % xr == 0;
-        if (u >= 1 && !mbar_spin(&e_free[k], (u - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF)) break;
-        if (x_start && u >= xr &&
-            !mbar_spin(&x_free[k], ((u / xr) - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF))
-          break;
-        bool alive = true;
-        for (int it = it0; it < it1; ++it) {
-          const int s = it % STAGES;
-          if (!(alive = mbar_spin(&tma_full[s], (it / STAGES) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF)))
-            break;
-          tc_fence_after();
-          const uint32_t sa = smem_base + s * XB_STAGE;
-          const uint64_t da = sw128_desc(sa), db = da + (XB_A_BYTES >> 4);
-          // K steps of 16 values advance 32 bytes (2 descriptor units); lo parts sit 64 bytes on
-          tc_mma_f16(e_tmem, da, db, idesc, it > it0 ? 1u : 0u);
-          tc_mma_f16(e_tmem, da + 2, db + 2, idesc, 1u);
-          tc_mma_f16(x_tmem, da, db + 4, idesc, (x_start && it == it0) ? 0u : 1u);   // hi_a x lo_b
-          tc_mma_f16(x_tmem, da + 2, db + 6, idesc, 1u);
-          // lo_a x fp16(b): lo_a x (hi_b + lo_b) to within fp16(b)'s rounding, one product
-          const uint64_t d16 = sw64_desc(sa + XB_A_BYTES + XB_B_BYTES);
-          tc_mma_f16(x_tmem, da + 4, d16, idesc, 1u);
-          tc_mma_f16(x_tmem, da + 6, d16 + 2, idesc, 1u);
-          tc_commit(&sfree[s]);
+      volatile int* no_abort = reinterpret_cast<volatile int*>(&zero);
+      for (int it = max(0, issued - XB_STAGES); it < issued; ++it)
+        if (!mbar_wait(&sfree[it % XB_STAGES], (it / XB_STAGES) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF)) break;
+      if (*abort_flag) {
+        if (rank == 0) {
+          for (int it = max(0, issued - XB_STAGES); it < issued; ++it)
+            mbar_wait(&full[it % XB_STAGES], (it / XB_STAGES) & 1, no_abort, args.err, DEV_ERR_TIMEOUT_VF);
+        } else {
+          const unsigned long long t0 = global_timer_ns();
+          while (global_timer_ns() - t0 < 50000000ull) {
+          }
         }
-        if (!alive) break;
-        tc_commit(&rdone[r % NRB]);
       }
-      // every MMA issued by both issuers has completed once fin_bar fires
-      tc_commit(fin_bar);
+    }
+  } else if (warp == 1 || warp == 2) {
+    if (rank == 0) {
+      // ---------------------------------------------------------------- MMA issuers (leader)
+      // Issuer k takes the ranges r = k, k + 2, ... into set k (one thread's waits and instructions for a
+      // range take about 1,500 cycles, twice its MMAs): per block of 32 values and k-step of 16, hi_a x [hi_b | lo_b] in
+      // one 256-column MMA into [E_k | X_k], then lo_a x fp16(b) into X_k (fp16(b): lo_a x (hi_b + lo_b)
+      // to within fp16's rounding).  The drains zero E_k after every range and X_k after its period, so
+      // that every MMA accumulates.
+      constexpr uint32_t idesc_hi = idesc_f16(2 * VF_BM, 2 * XB_BN, false);
+      constexpr uint32_t idesc_lo = idesc_f16(2 * VF_BM, XB_BN, false);
+      const uint32_t smem_base = smem_u32(smem);
+      bool alive = true;
+      const int k = warp - 1;
+      const uint32_t set = tmem + k * XB_SET;
+      const uint32_t sfree_bar = smem_base + XB_STAGES * XB_STAGE + XB_STAGES * 8, rdone_bar = sfree_bar + (XB_STAGES + k) * 8;
+      for (int r = k, u = 0; r < n_ranges && alive; r += 2, ++u) {
+        const int it0 = r * kd, it1 = min(n_it, it0 + kd);
+        const bool x_end = u % xr == xr - 1 || r + 2 >= n_ranges;
+        for (int it = it0; it < it1; ++it) {
+          const int s = (it >> 1) % XB_STAGES;
+          // the stage first: it landed long ago as a rule, the set is what the issuer waits for
+          if (!(it & 1) || it == it0)
+            alive = mbar_spin(&full[s], ((it >> 1) / XB_STAGES) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
+          if (it == it0) alive = alive && mbar_spin(&e_free[k], u & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
+          if (!alive) break;
+          tc_fence_after();
+          // the block's 32 values are half of the 128-byte rows; k-steps of 16 values advance 32 bytes
+          const uint64_t ah = sw128_desc(smem_base + s * XB_STAGE) + (it & 1) * 4;
+          const uint64_t al = ah + (XB_PART >> 4), b = ah + (2 * XB_PART >> 4), b16 = ah + (3 * XB_PART >> 4);
+          tc_mma_f16_pair(set, ah, b, idesc_hi);
+          tc_mma_f16_pair(set, ah + 2, b + 2, idesc_hi);
+          // E_k is complete here: its drain need not wait for the last cross products, unless it takes X_k too
+          if (it == it1 - 1 && !x_end) tc_commit_pair(rdone_bar);
+          tc_mma_f16_pair(set + XB_BN, al, b16, idesc_lo);
+          tc_mma_f16_pair(set + XB_BN, al + 2, b16 + 2, idesc_lo);
+          if ((it & 1) || it == it1 - 1) tc_commit_pair(sfree_bar + s * 8);
+        }
+        if (alive && x_end) tc_commit_pair(rdone_bar);
+      }
+      // every MMA of both issuers has completed once fin_bar fires
+      tc_commit_pair_local(smem_u32(fin_bar));
       int zero = 0;
       mbar_wait(fin_bar, 0, reinterpret_cast<volatile int*>(&zero), args.err, DEV_ERR_TIMEOUT_VF);
     }
@@ -247,19 +265,22 @@ __global__ void __launch_bounds__(XB_THREADS, 1)
     // ------------------------------------------------------------------ drains and epilogue
     const int quarter = warp & 3;               // TMEM lanes 32*quarter .. +31 (hardware rule)
     const int group = (warp - 3) >> 2;          // columns XB_HC*group .. +XB_HC-1
-    const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const uint32_t c_base = static_cast<uint32_t>(group * XB_HC);
+    const uint32_t my = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c_base;
+    const uint32_t free_bar[2] = {cluster_addr(&e_free[0], 0), cluster_addr(&e_free[1], 0)};
     float S[XB_HC];
 #pragma unroll
     for (int k = 0; k < XB_HC; ++k) S[k] = 0.0f;
-    // S += this thread's 32 columns of the accumulator at TMEM column col
-    auto add_acc = [&](uint32_t col) {
-      uint32_t d[32];
-      tmem_ld_32x32b_x32(tmem + lane_base + col + c_base, d);
-      tmem_wait_ld();
+    // the accumulators start at zero
 #pragma unroll
-      for (int k = 0; k < 32; ++k) S[k] += __uint_as_float(d[k]);
-    };
+    for (int a = 0; a < 4; ++a) tmem_zero_x32(my + a * XB_BN);
+    tmem_wait_st();
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive_cluster(free_bar[0]);
+      mbar_arrive_cluster(free_bar[1]);
+    }
     // The FP32 running sums move into the CTA-private FP64 accumulator, column-major in the tile:
     // Vacc[(split * gridDim.x + tile) * 128 * BN + column * 128 + row], column = c_base + c.  Column
     // c of every thread goes after range r when r % flush == c (staggered, so that no drain carries a
@@ -281,29 +302,39 @@ __global__ void __launch_bounds__(XB_THREADS, 1)
     bool ok = true;
     for (int r = 0; r < n_ranges && ok; ++r) {
       const int k = r & 1, u = r >> 1;
-      // X_k is drained at the end of each of its periods and after issuer k's last range
+      // X_k is drained at the end of each of its periods and after the set's last range
       const bool x_end = u % xr == xr - 1 || r + 2 >= n_ranges;
-      // a non-suspending wait: the drain's wake-up sits on the range round trip
-      ok = __all_sync(0xffffffffu,
-                      mbar_spin(&rdone[r % NRB], (r / NRB) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF));
-      __syncwarp();
+      // one lane waits, suspended: the board is at its power cap in these kernels, and 16 polling warps cost
+      // 10 % of the time (100.7 ms a 9,728-point launch with every lane polling, 95.3 with one, 90.7 so)
+      if (lane == 0) ok = mbar_wait(&rdone[k], u & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) break;
       tc_fence_after();
-      add_acc(2 * k * XB_BN);
-      if (x_end) add_acc((2 * k + 1) * XB_BN);
+      uint32_t d[32];
+      const uint32_t e_col = my + k * XB_SET;
+      tmem_ld_32x32b_x32(e_col, d);
+      tmem_wait_ld();
+      tmem_zero_x32(e_col);
+      if (x_end) {
+#pragma unroll
+        for (int c = 0; c < XB_HC; ++c) S[c] += __uint_as_float(d[c]);
+        tmem_ld_32x32b_x32(e_col + XB_BN, d);
+        tmem_wait_ld();
+        tmem_zero_x32(e_col + XB_BN);
+      }
+      tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&e_free[k]);
-        if (x_end) mbar_arrive(&x_free[k]);
-      }
-      // staggered FP64 flush (the accumulators are already handed back to the MMAs)
-      if (args.flush > 0 && r % args.flush < XB_HC) flush_col(r % args.flush, r < args.flush);
+      if (lane == 0) mbar_arrive_cluster(free_bar[k]);
+      // the sums and the staggered FP64 flush (the accumulators are already handed back to the MMAs)
+#pragma unroll
+      for (int c = 0; c < XB_HC; ++c) S[c] += __uint_as_float(d[c]);
+      if (valid && args.flush > 0 && r % args.flush < XB_HC) flush_col(r % args.flush, r < args.flush);
     }
     if (args.flush > 0) {
       // the remaining sums join the FP64 accumulator (columns never flushed in the loop are
       // stored); a finalize kernel writes V (mode 0) or adds the tile into M (mode 1)
-      if (ok) {
+      if (ok && valid) {
 #pragma unroll
         for (int c = 0; c < XB_HC; ++c) {
           if (c < min(n_ranges, args.flush))
@@ -317,7 +348,7 @@ __global__ void __launch_bounds__(XB_THREADS, 1)
       const int row = quarter * 32 + lane;
       const int64_t il = static_cast<int64_t>(ib) + row;
       const int pq0 = t.n_tile * XB_BN + static_cast<int>(c_base);
-      if (ok && !*abort_flag && il < args.n_i && n_it > 0) {
+      if (ok && valid && !*abort_flag && il < args.n_i && n_it > 0) {
         float* Vz = args.V + split * v_slice(args.gcp, args.n_orb);
 #pragma unroll
         for (int k = 0; k < XB_HC; ++k) {
@@ -335,10 +366,11 @@ __global__ void __launch_bounds__(XB_THREADS, 1)
 
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // the pair's MMAs, loads and remote arrivals are done
   if (warp == 0) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc_pair(tmem, 512);
   }
 }
 
@@ -560,7 +592,9 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
 // order is the GEMM's grouped order.
 template <int BN>
 __global__ void __launch_bounds__(VF_BM) vfield_finalize_kernel(const VfieldArgs args) {
-  const TileXY t = grouped_tile(blockIdx.x, 3 * args.mt_per_x, args.n_tiles);
+  const int m_tiles = 3 * args.mt_per_x;
+  const TileXY t = BN == XB_BN ? pair_tile(blockIdx.x, m_tiles, args.n_tiles) : grouped_tile(blockIdx.x, m_tiles, args.n_tiles);
+  if (t.m_tile >= m_tiles) return;
   const int x = t.m_tile / args.mt_per_x;
   const int row = threadIdx.x;
   const int64_t il = static_cast<int64_t>(t.m_tile - x * args.mt_per_x) * VF_BM + row;
@@ -585,7 +619,9 @@ __global__ void __launch_bounds__(VF_BM) vfield_finalize_kernel(const VfieldArgs
 template <int BN>
 __global__ void __launch_bounds__(VF_BM) assemble_finalize_kernel(const VfieldArgs args) {
   __shared__ double slab[32][VF_BM + 1];
-  const TileXY t = grouped_tile(blockIdx.x, (args.rows_a + VF_BM - 1) / VF_BM, args.n_tiles);
+  const int m_tiles = (args.rows_a + VF_BM - 1) / VF_BM;
+  const TileXY t = pair_tile(blockIdx.x, m_tiles, args.n_tiles);
+  if (t.m_tile >= m_tiles) return;
   const double* acc = args.Vacc + (static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * VF_BM * BN;
   const int ncol = min(BN, args.n_pair - t.n_tile * BN);
   const int row0 = t.m_tile * VF_BM, col0 = t.n_tile * BN;
@@ -608,7 +644,11 @@ __global__ void __launch_bounds__(VF_BM) assemble_finalize_kernel(const VfieldAr
   }
 }
 
-int m_tiles_of(const VfieldArgs& a) { return a.mode == 0 ? 3 * a.mt_per_x : (a.rows_a + VF_BM - 1) / VF_BM; }
+// CTAs along x: the fp16 engine's tiles come in pairs of row tiles.
+unsigned tile_ctas(const VfieldArgs& a, int parts) {
+  const int m = a.mode == 0 ? 3 * a.mt_per_x : (a.rows_a + VF_BM - 1) / VF_BM;
+  return static_cast<unsigned>((parts == 2 ? (m + 1) / 2 * 2 : m) * a.n_tiles);
+}
 
 }  // namespace
 
@@ -618,13 +658,13 @@ void launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const 
                       const VfieldArgs& a, int parts, int splits, cudaStream_t st) {
   if (a.n_tiles <= 0 || splits <= 0) return;
   if (a.mode == 1 ? a.rows_a <= 0 : a.mt_per_x <= 0) return;
-  dim3 grid(static_cast<unsigned>(m_tiles_of(a) * a.n_tiles), static_cast<unsigned>(splits));
+  dim3 grid(tile_ctas(a, parts), static_cast<unsigned>(splits));
   if (a.mode == 1) {
-    cudaFuncSetAttribute(xgemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, xb_smem(1));
-    xgemm_kernel<1><<<grid, XB_THREADS, xb_smem(1), st>>>(*tm_g, *tm_rho, *tm_rho16, a);
+    cudaFuncSetAttribute(xgemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, XB_SMEM);
+    xgemm_kernel<1><<<grid, XB_THREADS, XB_SMEM, st>>>(*tm_g, *tm_rho, *tm_rho16, a);
   } else if (parts == 2) {
-    cudaFuncSetAttribute(xgemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, xb_smem(0));
-    xgemm_kernel<0><<<grid, XB_THREADS, xb_smem(0), st>>>(*tm_g, *tm_rho, *tm_rho16, a);
+    cudaFuncSetAttribute(xgemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, XB_SMEM);
+    xgemm_kernel<0><<<grid, XB_THREADS, XB_SMEM, st>>>(*tm_g, *tm_rho, *tm_rho16, a);
   } else {
     cudaFuncSetAttribute(vfield_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BF_SMEM);
     vfield_bf16_kernel<<<grid, BF_THREADS, BF_SMEM, st>>>(*tm_g, *tm_rho, a);
@@ -634,7 +674,7 @@ void launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const 
 void launch_vfield_tc_finalize(const VfieldArgs& a, int parts, int splits, cudaStream_t st) {
   if (a.n_tiles <= 0 || splits <= 0 || a.flush <= 0) return;
   if (a.mode == 1 ? a.rows_a <= 0 : a.mt_per_x <= 0) return;
-  dim3 grid(static_cast<unsigned>(m_tiles_of(a) * a.n_tiles), static_cast<unsigned>(splits));
+  dim3 grid(tile_ctas(a, parts), static_cast<unsigned>(splits));
   if (a.mode == 1)
     assemble_finalize_kernel<XB_BN><<<grid, VF_BM, 0, st>>>(a);
   else if (parts == 2)

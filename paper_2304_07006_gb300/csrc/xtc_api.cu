@@ -267,7 +267,7 @@ struct Plan {
   int64_t NG, NGp;
   int64_t ob, oe;    // outer range
   int64_t gc;        // chunk length (multiple of 128)
-  int splits;
+  int splits, kb_per_split;
   int parts_b;       // step (b) parts (2 fp16 / 3 bf16), 0 = FP64
   bool f64;
   int64_t jb;        // FP64 contractions: inner points per block (the whole padded grid when it fits),
@@ -477,8 +477,9 @@ int xtc_set_outer_range(xtc_ctx* ctx, int64_t begin, int64_t end) {
 //    accumulator per issuer (128-column tiles);
 // 3: plus the fp16 plane of rho^T in step (b) and a commit per stage that frees its slot;
 // 4: step (d) on an fp16 plane of R as well (three products), drains waiting without suspending;
-// 5: tiles ordered in groups of 16 row tiles (8 before).
-int xtc_engine_revision(void) { return 5; }
+// 5: tiles ordered in groups of 16 row tiles (8 before);
+// 6: CTA pairs on 256 x 128 tiles, hi_a x [hi_b | lo_b] in one MMA, 64-value stages.
+int xtc_engine_revision(void) { return 6; }
 
 int xtc_get_timings(xtc_ctx* ctx, double* ms, int64_t* launches, int n) {
   if (!ctx || n < XTC_N_KERNELS) return XTC_ERR_ARG;
@@ -617,8 +618,10 @@ int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* gri
   pl.gc = ctx->prm.grid_chunk > 0 ? ctx->prm.grid_chunk
                                    : auto_chunk(ctx, pl.NP, pl.NGp, pl.parts_b, std::max<int64_t>(n_outer, 1), f64);
   const int n_kb = static_cast<int>(pl.NGp / VF_BK);
-  pl.splits = ctx->prm.split_k > 0 ? std::min(ctx->prm.split_k, n_kb) : 1;
-  if (f64) pl.splits = 1;
+  // slices of whole groups of 4 K-blocks (the fp16 stages and exact ranges do not straddle two slices)
+  pl.splits = !f64 && ctx->prm.split_k > 0 ? std::min(ctx->prm.split_k, n_kb / 4) : 1;
+  pl.kb_per_split = static_cast<int>(round_up((n_kb + pl.splits - 1) / pl.splits, 4));
+  pl.splits = (n_kb + pl.kb_per_split - 1) / pl.kb_per_split;  // every slice non-empty
 
   cudaStream_t st = ctx->st;
   int rc;
@@ -681,7 +684,7 @@ int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* gri
     if (!ensure(ctx->G, gbytes)) return fail(ctx, XTC_ERR_OOM, "gradient table (%.2f GB)", gbytes / 1e9);
     // FP64 partial sums of step (b): one 128 x vf_bn tile per CTA and split slice
     const int bn = vf_bn(pl.parts_b);
-    const size_t tiles = 3ull * ((pl.gc + VF_BM - 1) / VF_BM) * ((pl.NP + bn - 1) / bn);
+    const size_t tiles = round_up(3 * ((pl.gc + VF_BM - 1) / VF_BM), 2) * ((pl.NP + bn - 1) / bn);
     const size_t abytes = ctx->vf_flush > 0 ? 8ull * pl.splits * tiles * VF_BM * bn : 0;
     if (!ensure(ctx->Vacc, abytes)) return fail(ctx, XTC_ERR_OOM, "step (b) FP64 sums (%.2f GB)", abytes / 1e9);
   }
@@ -690,8 +693,8 @@ int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* gri
 }
 
 // Tensor maps of the step (b) operands: rho^T (box rows vf_bn) and the gradient table, as stored by
-// step (a) (box rows 32) and as loaded by the GEMM (box rows 128).  fp16: both parts of a 32-point
-// block in one 128-byte row (rows of 2 NGp values, boxes 64 wide, 128-byte swizzle); bf16: one
+// step (a) (box rows 32) and as loaded by the GEMM (box rows 128).  fp16: 128-byte runs of 64 values
+// of one part (rows of 2 NGp values, boxes 64 wide, 128-byte swizzle); bf16: one
 // plane per part (rows of NGp values, boxes 32 wide, 64-byte swizzle).
 struct VfMaps {
   CUtensorMap rho, rho16, g_store, g_load;
@@ -703,9 +706,9 @@ int make_vfield_maps(xtc_ctx* ctx, const Plan& pl, VfMaps& m) {
   const uint32_t bk = wide ? 2 * VF_BK : VF_BK;
   int rc;
   if ((rc = make_tmap_3d(ctx, &m.rho, ctx->rho.p, bf, cols, pl.NP, planes, bk, vf_bn(pl.parts_b), wide))) return rc;
-  // fp16: the plane of fp16(rho^T) after the split rows, boxes 32 wide (64-byte swizzle)
+  // fp16: the plane of fp16(rho^T) after the split rows, boxes of 64 values x half a column tile
   if (wide && (rc = make_tmap_3d(ctx, &m.rho16, ctx->rho.as<uint16_t>() + 2 * pl.NP * pl.NGp, false, pl.NGp, pl.NP, 1,
-                                 VF_BK, vf_bn(2))))
+                                 2 * VF_BK, vf_bn(2) / 2, true)))
     return rc;
   if ((rc = make_tmap_3d(ctx, &m.g_store, ctx->G.p, bf, cols, 3 * pl.gc, planes, bk, 32, wide))) return rc;
   return make_tmap_3d(ctx, &m.g_load, ctx->G.p, bf, cols, 3 * pl.gc, planes, bk, VF_BM, wide);
@@ -757,13 +760,13 @@ void run_gemm_b(xtc_ctx* ctx, const Plan& pl, int64_t n_i, const VfMaps& maps) {
   a.n_tiles = (pl.NP + vf_bn(pl.parts_b) - 1) / vf_bn(pl.parts_b);
   a.n_pair = pl.NP;
   a.n_kb = n_kb;
-  a.kb_per_split = (a.n_kb + pl.splits - 1) / pl.splits;
+  a.kb_per_split = pl.kb_per_split;
   a.kd = pl.parts_b == 2 ? f16_range_b(ctx->vf_kd) : std::min(ctx->vf_kd, 2);
   a.xper = ctx->x_period;
   a.flush = flush_ranges(ctx->vf_flush, a.kd);
   a.unscale_g = std::ldexp(1.0f, -gradient_scale(ctx, pl));
   a.err = ctx->err_dev.as<int>();
-  const int splits = (a.n_kb + a.kb_per_split - 1) / a.kb_per_split;  // every slice non-empty
+  const int splits = pl.splits;
   // the GEMM, then (FP64 flushes) the kernel that writes V from the FP64 sums
   timed(ctx, XTC_K_VFIELD, 1, [&] { launch_vfield_tc(&maps.g_load, &maps.rho, &maps.rho16, a, pl.parts_b, splits, st); });
   if (a.flush > 0) timed(ctx, XTC_K_AUX, 1, [&] { launch_vfield_tc_finalize(a, pl.parts_b, splits, st); });
@@ -932,7 +935,7 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
   if (d16) {
     const size_t ebytes = 4ull * m_stride(NP);
     const int bn = vf_bn(2);
-    const size_t tiles = static_cast<size_t>((NP + VF_BM - 1) / VF_BM) * ((NP + bn - 1) / bn);
+    const size_t tiles = static_cast<size_t>(round_up((NP + VF_BM - 1) / VF_BM, 2)) * ((NP + bn - 1) / bn);
     if (!ensure(ctx->L32, 4ull * kdim * NP) || !ensure(ctx->R32, 4ull * kdim * NP) || !ensure(ctx->eL, ebytes) ||
         !ensure(ctx->eR, ebytes) || !ensure(ctx->Vacc, std::max<size_t>(ctx->Vacc.n, 8ull * tiles * VF_BM * bn)) ||
         (spin && (!ensure(ctx->R32b, 4ull * kdim * NP) || !ensure(ctx->eR2, ebytes))))
@@ -955,11 +958,12 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
     if ((rc = make_tmap_3d(ctx, &tm_R, ctx->R.p, false, 2 * kdim, NP, 1, 2 * VF_BK, vf_bn(2), true))) return rc;
     if (spin && (rc = make_tmap_3d(ctx, &tm_R2, ctx->R2.p, false, 2 * kdim, NP, 1, 2 * VF_BK, vf_bn(2), true)))
       return rc;
-    // the fp16(R) planes, boxes 32 wide (64-byte swizzle)
-    if ((rc = make_tmap_3d(ctx, &tm_R16, ctx->R.as<uint16_t>() + 2 * kdim * NP, false, kdim, NP, 1, VF_BK, vf_bn(2))))
+    // the fp16(R) planes, boxes of 64 values x half a column tile
+    if ((rc = make_tmap_3d(ctx, &tm_R16, ctx->R.as<uint16_t>() + 2 * kdim * NP, false, kdim, NP, 1, 2 * VF_BK,
+                           vf_bn(2) / 2, true)))
       return rc;
-    if (spin &&
-        (rc = make_tmap_3d(ctx, &tm_R216, ctx->R2.as<uint16_t>() + 2 * kdim * NP, false, kdim, NP, 1, VF_BK, vf_bn(2))))
+    if (spin && (rc = make_tmap_3d(ctx, &tm_R216, ctx->R2.as<uint16_t>() + 2 * kdim * NP, false, kdim, NP, 1, 2 * VF_BK,
+                                   vf_bn(2) / 2, true)))
       return rc;
   } else if (!pl.f64) {
     if ((rc = make_tmap_3d(ctx, &tm_L, ctx->L.p, true, kdim, NP, 3, AS_BK, AS_BM))) return rc;

@@ -26,8 +26,8 @@ constexpr int PT_COEF = 14;     // x y z, K0[3] K1[3] K2[3], Hc1 Hc2
 
 // Tile shapes of the tensor-core kernels.
 constexpr int VF_BM = 128;      // outer points per tile (TMEM lanes)
-// orbital pairs per tensor-core tile (B rows): the fp16 engine keeps two pairs of TMEM accumulators
-// of 128 columns (exact hi x hi and cross products per issuer), 7 pipeline stages of 32 KB; the bf16
+// orbital pairs per tensor-core tile (B rows): the fp16 engine keeps two sets of TMEM accumulators
+// of 2 x 128 columns (exact hi x hi and cross products); the bf16
 // engine two accumulators of 160 columns, 4 stages of 54 KB; each drain thread holds a running sum
 // of half a tile row in registers
 __host__ __device__ constexpr int vf_bn(int parts) { return parts == 2 ? 128 : 160; }
@@ -110,8 +110,8 @@ void launch_jtab(const double* grid, int64_t n_grid, int64_t n_grid_pad, const J
 
 // Pair products rho^T[pq][j] = w_j phi_p(j) phi_q(j) split into parts.  fp16 (2 parts): each pair's
 // row scaled by a power of 2 (colexp[pq] receives the exponent; colmax is scratch) and split exactly
-// with one quantum per range of kd blocks of 32 points (gemm_bits_b(kd) bits), the two parts of a
-// block in one 128-byte row: [pq][j / 32][part][j % 32], followed by a plane of the scaled value
+// with one quantum per range of kd blocks of 32 points (gemm_bits_b(kd) bits), in 128-byte runs of one
+// part: [pq][j / 64][part][j % 64], followed by a plane of the scaled value
 // rounded to fp16, [pq][j] (2 x n_pair x n_pad values, then n_pair x n_pad); the products are
 // taken in FP32 pairs hi + lo from phi32, scratch of 2 (n_orb + 1) n_pad floats.  bf16 (3 parts):
 // per-element split, unscaled (colexp = 0), [part][pq][j].  n_pad must be a multiple of 32 kd.
@@ -131,7 +131,7 @@ void launch_transpose_phi(const double* phi, int64_t n_grid, int64_t n_grid_pad,
 void launch_check_finite(const double* x, int64_t n, int* flag, cudaStream_t st);
 
 // Step (a), tensor-core path: the split Jastrow gradient of the outer points [i0, i0 + n_i) and every
-// padded inner point, K-major, row x * gcp + il: fp16 (2 parts) G[row][j / 32][part][j % 32] stored
+// padded inner point, K-major, row x * gcp + il: fp16 (2 parts) G[row][j / 64][part][j % 64] stored
 // as 128-byte-swizzled TMA tiles (box 64 x 32); bf16 (3 parts) G[part][row][j] as 64-byte-swizzled
 // tiles (box 32 x 32).  Rows up to n_tiles * 32 are written (past n_i they repeat the last point).
 struct GfieldArgs {
@@ -163,7 +163,7 @@ struct VfieldArgs {
   int mt_per_x;                // 128-row tiles per component: ceil(n_i / 128)
   int n_tiles;                 // column tiles: ceil(n_pair / vf_bn(parts))
   int n_pair;
-  int kb_per_split, n_kb;      // inner K-blocks per split slice, total K-blocks
+  int kb_per_split, n_kb;      // inner K-blocks per split slice (a multiple of 4), total K-blocks
   int kd;                      // K-blocks per TMEM accumulation range (then added to the FP32 running sum);
                                // fp16 engine: 1, 2 or 4, the range of the operands' exact split
   int xper;                    // fp16 engine: K-blocks between drains of the cross-product accumulator
@@ -181,8 +181,7 @@ struct VfieldArgs {
 };
 bool vfield_tc_supported(int n_nuc);
 // Launches the GEMM.
-// tm_rho16: the fp16(rho^T) plane of the fp16 precision (box 32 x 128, 64-byte swizzle); step (d)
-// (mode 1) and the bf16 precision ignore it.
+// tm_rho16: the fp16(B) plane of the fp16 precision (box 64 x 64, 128-byte swizzle); the bf16 precision ignores it.
 void launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const CUtensorMap* tm_rho16,
                       const VfieldArgs& a, int parts, int splits, cudaStream_t st);
 // Then, with FP64 sums (a.flush > 0): mode 0 writes V from them, mode 1 adds the tiles into M.
@@ -292,8 +291,8 @@ void launch_fields(const FieldsArgs& a, bool f64, cudaStream_t st);  // f64: FP6
 
 // Step (d) operands in fp16 x2: each FP32 row src[r][0..kdim) is scaled by 2^exps[r] (largest
 // magnitude in [2^13, 2^14)) and split exactly into hi + lo fp16 with one quantum per range of kd
-// blocks of 32 values (gemm_bits_lr(kd) bits), both parts of a block in one 128-byte row:
-// dst[r][k' / 32][part][k' % 32].  kc = 4: the source holds 4 values per outer point (k = 4 i + c)
+// blocks of 32 values (gemm_bits_lr(kd) bits), in 128-byte runs of one part:
+// dst[r][k' / 64][part][k' % 64].  kc = 4: the source holds 4 values per outer point (k = 4 i + c)
 // and k' = c * kdim / 4 + i (component-major, so that a range never mixes components); kc = 1:
 // k' = k.  kdim / kc must be a multiple of 32 kd.  dst16 (or NULL): the scaled values rounded to
 // fp16, dst16[r][k'] (the plane of the B operand, for the lo x fp16(B) product).
