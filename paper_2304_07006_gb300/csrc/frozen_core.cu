@@ -61,25 +61,39 @@ __global__ void fc_core_energy_kernel(const double* __restrict__ dU, const doubl
 }
 
 constexpr int FC_G_THREADS = 256;
+constexpr int FC_U = 4;  // elements of a row per lane in flight
 
+// HBM-bound: 16 bytes per element.  A lane's loads of a row are issued before its stores (one load at a
+// time left 16 KB in flight per SM and half the bandwidth: 855 us for 118 active of 120 orbitals), and the
+// row number is split with 32-bit divisions (n_act^3 < 2^25).
 __global__ void __launch_bounds__(FC_G_THREADS) fc_gather_kernel(const double* __restrict__ dU, int N, FcIndex ix,
                                                                  double* __restrict__ dU_act) {
   __shared__ int act[FC_MAX_ORB];
   for (int t = threadIdx.x; t < ix.n_act; t += FC_G_THREADS) act[t] = ix.act[t];
   __syncthreads();
-  const int na = ix.n_act;
-  const int lane = threadIdx.x & 31;
+  const unsigned na = ix.n_act;
+  const unsigned lane = threadIdx.x & 31;
   const int64_t n = N;
-  const int64_t rows = static_cast<int64_t>(na) * na * na;
-  const int64_t warps = static_cast<int64_t>(gridDim.x) * (FC_G_THREADS / 32);
-  for (int64_t row = blockIdx.x * static_cast<int64_t>(FC_G_THREADS / 32) + (threadIdx.x >> 5); row < rows;
-       row += warps) {
-    const int r = static_cast<int>(row % na);
-    const int64_t pq = row / na;
-    const int q = static_cast<int>(pq % na), p = static_cast<int>(pq / na);
+  const unsigned rows = na * na * na;
+  const unsigned warps = gridDim.x * (FC_G_THREADS / 32);
+  for (unsigned row = blockIdx.x * (FC_G_THREADS / 32) + (threadIdx.x >> 5); row < rows; row += warps) {
+    const unsigned pq = row / na, r = row - pq * na;
+    const unsigned p = pq / na, q = pq - p * na;
     const double* src = dU + ((act[p] * n + act[q]) * n + act[r]) * n;
-    double* dst = dU_act + row * na;
-    for (int s = lane; s < na; s += 32) dst[s] = __ldcs(src + act[s]);
+    double* dst = dU_act + static_cast<int64_t>(row) * na;
+    for (unsigned s0 = lane; s0 < na; s0 += 32 * FC_U) {
+      double v[FC_U];
+#pragma unroll
+      for (int u = 0; u < FC_U; ++u) {
+        const unsigned s = s0 + 32 * u;
+        if (s < na) v[u] = __ldcs(src + act[s]);
+      }
+#pragma unroll
+      for (int u = 0; u < FC_U; ++u) {
+        const unsigned s = s0 + 32 * u;
+        if (s < na) __stcs(dst + s, v[u]);
+      }
+    }
   }
 }
 
