@@ -103,11 +103,8 @@ __global__ void split_phi_f32_kernel(const double* __restrict__ phiT, const doub
 
 // w phi_p phi_q from the FP32 pairs of split_phi_f32_kernel as an unevaluated sum rh + rl (error-
 // free products by fma, then one renormalisation): about 2^-44 of the value, on the FP32 pipes.
-__device__ __forceinline__ void rho_pair_f32(const float* __restrict__ f32, int64_t total, int64_t n_pad, int n_orb,
-                                             int p, int q, int64_t j, float& rh, float& rl) {
-  const float ah = f32[p * n_pad + j], al = f32[total + p * n_pad + j];
-  const float bh = f32[q * n_pad + j], bl = f32[total + q * n_pad + j];
-  const float wh = f32[n_orb * n_pad + j], wl = f32[total + n_orb * n_pad + j];
+__device__ __forceinline__ void rho_pair_f32(float ah, float al, float bh, float bl, float wh, float wl, float& rh,
+                                             float& rl) {
   const float xh = ah * bh;
   const float xl = fmaf(ah, bh, -xh) + fmaf(ah, bl, al * bh);
   const float yh = xh * wh;
@@ -116,69 +113,124 @@ __device__ __forceinline__ void rho_pair_f32(const float* __restrict__ f32, int6
   rl = yl - (rh - yh);
 }
 
-// Largest |rho| of each pair over the grid (FP32; it only picks the pair's power-of-2 scale).
-__global__ void rho_colmax_f32_kernel(const float* __restrict__ f32, int64_t n_grid, int64_t n_pad, int n_orb,
-                                      const int* __restrict__ pp, const int* __restrict__ pq_,
-                                      unsigned int* __restrict__ colmax) {
-  const int pq = blockIdx.y;
-  const int p = pp[pq], q = pq_[pq];
+// The pair products are taken with p fixed in a CTA and a run over q >= p: phi_p and w stay in registers
+// and each product loads phi_q alone (16 bytes a point pair).  With one warp per pair and 64 points, every
+// value loaded all three factors and wrote 2 bytes per lane: 20 ms for N = 200 and 200,000 points (24 GB),
+// 4 bytes per lane and these loops 5 ms, against 3.7 ms at the copy rate.
+
+// Largest |rho| of each pair over the grid (FP32; it only picks the pair's power-of-2 scale): CTA p =
+// blockIdx.y, four points per thread.
+constexpr int RC_POINTS = 1024;
+__global__ void __launch_bounds__(256) rho_colmax_f32_kernel(const float* __restrict__ f32, int64_t n_pad, int n_orb,
+                                                             unsigned int* __restrict__ colmax) {
+  extern __shared__ unsigned int cmax[];  // [n_orb]
+  const int p = blockIdx.y;
+  const int64_t j = static_cast<int64_t>(blockIdx.x) * RC_POINTS + 4 * threadIdx.x;
   const int64_t total = (static_cast<int64_t>(n_orb) + 1) * n_pad;
-  float m = 0.0f;
-  for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j < n_grid;
-       j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    float rh, rl;
-    rho_pair_f32(f32, total, n_pad, n_orb, p, q, j, rh, rl);
-    m = fmaxf(m, fabsf(rh));
+  const bool in = j < n_pad;   // n_pad is a multiple of 4; padded points have zero weight
+  const int64_t jj = in ? j : 0;
+  auto load = [&](int64_t row, float4& hi, float4& lo) {
+    hi = __ldg(reinterpret_cast<const float4*>(f32 + row * n_pad + jj));
+    lo = __ldg(reinterpret_cast<const float4*>(f32 + total + row * n_pad + jj));
+  };
+  for (int q = p + threadIdx.x; q < n_orb; q += 256) cmax[q] = 0;
+  __syncthreads();
+  float4 ah, al, wh, wl;
+  load(p, ah, al);
+  load(n_orb, wh, wl);
+#pragma unroll 2
+  for (int q = p; q < n_orb; ++q) {
+    float4 bh, bl;
+    load(q, bh, bl);
+    float rh[4], rl;
+    rho_pair_f32(ah.x, al.x, bh.x, bl.x, wh.x, wl.x, rh[0], rl);
+    rho_pair_f32(ah.y, al.y, bh.y, bl.y, wh.y, wl.y, rh[1], rl);
+    rho_pair_f32(ah.z, al.z, bh.z, bl.z, wh.z, wl.z, rh[2], rl);
+    rho_pair_f32(ah.w, al.w, bh.w, bl.w, wh.w, wl.w, rh[3], rl);
+    const float m = fmaxf(fmaxf(fabsf(rh[0]), fabsf(rh[1])), fmaxf(fabsf(rh[2]), fabsf(rh[3])));
+    const unsigned int bits = __reduce_max_sync(0xffffffffu, in ? __float_as_uint(m) : 0u);
+    if ((threadIdx.x & 31) == 0) atomicMax(cmax + q, bits);
   }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(colmax + pq, __float_as_uint(m));
+  __syncthreads();
+  const int base = p * n_orb - p * (p - 1) / 2 - p;
+  for (int q = p + threadIdx.x; q < n_orb; q += 256)
+    if (cmax[q]) atomicMax(colmax + base + q, cmax[q]);
 }
 
-// fp16 (2 parts, exact split): warp w of the CTA handles pair pq = 8 * blockIdx.y + w over one
-// accumulation range of the GEMM, points j0 + lane + 32 s (s < kd, j0 = 32 kd blockIdx.x); the
-// range shares one quantum (largest |value| of the range, `bits` bits).  rho = rh + rl in FP32
-// pairs (rho_pair_f32); hi = rh rounded to the quantum (exact), lo = fp16((rh - hi) + rl), whose
+__global__ void rho_colexp_kernel(const unsigned int* __restrict__ colmax, int n_pair, int* __restrict__ colexp) {
+  const int pq = blockIdx.x * blockDim.x + threadIdx.x;
+  if (pq < n_pair) colexp[pq] = col_exponent(colmax, pq, true);
+}
+
+// fp16 (2 parts, exact split): a warp takes two runs of 64 points (KD = 4: one of 128) and, with p =
+// blockIdx.y fixed, the pairs (p, q), q >= p; lane t holds points 2 t and 2 t + 1 of every 64.  An accumulation
+// range of the GEMM (32 KD points: half a warp's points, a warp's, or two runs) shares one quantum (largest
+// |value| of the range, `bits` bits).  rho = rh + rl in FP32 pairs (rho_pair_f32); hi = rh rounded to the
+// quantum (exact), lo = fp16((rh - hi) + rl), whose
 // rounding error is far below fp16's.  Layout: 128-byte runs of 64 points of one part,
 // [pq][j / 64][part][j % 64]; then the plane [pq][j] of the value rounded to fp16.
-__global__ void rho_split_f16_kernel(const float* __restrict__ f32, int64_t n_grid, int64_t n_pad, int n_orb,
-                                     int n_pair, const int* __restrict__ pp, const int* __restrict__ pq_,
-                                     const unsigned int* __restrict__ colmax, int kd, int bits,
-                                     int* __restrict__ colexp, uint16_t* __restrict__ out) {
+constexpr int RS_POINTS = 8 * 128;  // points per CTA of 8 warps
+template <int KD>
+__global__ void __launch_bounds__(256) rho_split_f16_kernel(const float* __restrict__ f32, int64_t n_pad, int n_orb,
+                                                            int n_pair, const int* __restrict__ colexp, int bits,
+                                                            uint16_t* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  const int pq = blockIdx.y * 8 + (threadIdx.x >> 5);
-  if (pq >= n_pair) return;  // whole warp
-  const int e = col_exponent(colmax, pq, true);
-  if (blockIdx.x == 0 && lane == 0) colexp[pq] = e;
-  const int p = pp[pq], q = pq_[pq];
-  const int64_t j0 = static_cast<int64_t>(blockIdx.x) * 32 * kd;
+  const int p = blockIdx.y;
+  const int64_t j0 = static_cast<int64_t>(blockIdx.x) * RS_POINTS + (threadIdx.x >> 5) * 128;
+  if (j0 >= n_pad) return;  // whole warp: n_pad is a multiple of 128
   const int64_t total = (static_cast<int64_t>(n_orb) + 1) * n_pad;
-  const float sc = pow2f(e);  // |e| <= 60: exact scaling
-  float vh[4] = {0.0f, 0.0f, 0.0f, 0.0f}, vl[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  float m = 0.0f;
+  const float* base = f32 + j0 + 2 * lane;
+  float2 ah[2], al[2], wh[2], wl[2];
 #pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int64_t j = j0 + 32 * s + lane;
-    if (s < kd && j < n_grid) {
-      float rh, rl;
-      rho_pair_f32(f32, total, n_pad, n_orb, p, q, j, rh, rl);
-      vh[s] = rh * sc;
-      vl[s] = rl * sc;
-    }
-    m = fmaxf(m, fabsf(vh[s]));
+  for (int g = 0; g < 2; ++g) {
+    ah[g] = __ldg(reinterpret_cast<const float2*>(base + p * n_pad + 64 * g));
+    al[g] = __ldg(reinterpret_cast<const float2*>(base + total + p * n_pad + 64 * g));
+    wh[g] = __ldg(reinterpret_cast<const float2*>(base + n_orb * n_pad + 64 * g));
+    wl[g] = __ldg(reinterpret_cast<const float2*>(base + total + n_orb * n_pad + 64 * g));
   }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  const int qe = exact_quantum(m, bits);
   uint16_t* out16 = out + static_cast<int64_t>(n_pair) * 2 * n_pad;  // the fp16(rho) plane
+  const int64_t pair0 = p * n_orb - static_cast<int64_t>(p) * (p - 1) / 2 - p;
+#pragma unroll 2
+  for (int q = p; q < n_orb; ++q) {
+    const int64_t pq = pair0 + q;
+    const float sc = pow2f(__ldg(colexp + pq));  // |e| <= 60: exact scaling
+    float2 vh[2], vl[2];
+    unsigned int m[2];
 #pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int64_t j = j0 + 32 * s + lane;
-    if (s >= kd || j >= n_pad) break;
-    float h = 0.0f;
-    if (qe >= -24) h = rintf(vh[s] * pow2f(-qe)) * pow2f(qe);  // both products exact (powers of 2)
-    const int64_t o = static_cast<int64_t>(pq) * 2 * n_pad + (j >> 6) * 128 + (j & 63);
-    out[o] = __half_as_ushort(__float2half_rn(h));                      // exact: at most 10 bits
-    out[o + 64] = __half_as_ushort(__float2half_rn((vh[s] - h) + vl[s]));  // vh - h is exact
-    out16[static_cast<int64_t>(pq) * n_pad + j] = __half_as_ushort(__float2half_rn(vh[s]));
+    for (int g = 0; g < 2; ++g) {
+      const float2 bh = __ldg(reinterpret_cast<const float2*>(base + q * n_pad + 64 * g));
+      const float2 bl = __ldg(reinterpret_cast<const float2*>(base + total + q * n_pad + 64 * g));
+      float rh, rl;
+      rho_pair_f32(ah[g].x, al[g].x, bh.x, bl.x, wh[g].x, wl[g].x, rh, rl);
+      vh[g].x = rh * sc;
+      vl[g].x = rl * sc;
+      rho_pair_f32(ah[g].y, al[g].y, bh.y, bl.y, wh[g].y, wl[g].y, rh, rl);
+      vh[g].y = rh * sc;
+      vl[g].y = rl * sc;
+      m[g] = __float_as_uint(fmaxf(fabsf(vh[g].x), fabsf(vh[g].y)));
+    }
+    if (KD == 4) {
+      m[0] = m[1] = __reduce_max_sync(0xffffffffu, max(m[0], m[1]));
+    } else {
+#pragma unroll
+      for (int g = 0; g < 2; ++g) m[g] = __reduce_max_sync(KD == 2 ? 0xffffffffu : (lane < 16 ? 0xffffu : 0xffff0000u), m[g]);
+    }
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      const int qe = exact_quantum(__uint_as_float(m[g]), bits);
+      float hx = 0.0f, hy = 0.0f;
+      if (qe >= -24) {  // both products exact (powers of 2)
+        const float up = pow2f(-qe), down = pow2f(qe);
+        hx = rintf(vh[g].x * up) * down;
+        hy = rintf(vh[g].y * up) * down;
+      }
+      const int64_t o = pq * 2 * n_pad + 2 * (j0 + 64 * g) + 2 * lane;
+      const __half2 h = __floats2half2_rn(hx, hy);                                      // exact: at most 10 bits
+      const __half2 l = __floats2half2_rn((vh[g].x - hx) + vl[g].x, (vh[g].y - hy) + vl[g].y);  // v - h is exact
+      *reinterpret_cast<__half2*>(out + o) = h;
+      *reinterpret_cast<__half2*>(out + o + 64) = l;
+      *reinterpret_cast<__half2*>(out16 + pq * n_pad + j0 + 64 * g + 2 * lane) = __floats2half2_rn(vh[g].x, vh[g].y);
+    }
   }
 }
 
@@ -210,17 +262,19 @@ __global__ void rho_split_bf16_kernel(const double* __restrict__ phiT, const dou
 }
 
 // One CTA per row of a step (d) operand: the row maximum sets a power-of-2 scale, then the scaled
-// row is split exactly into fp16 hi + lo (simt_pack.cuh), one quantum per accumulation range of kd
-// blocks of 32 values (`bits` bits).  With kc = 4 the source row holds kc values per outer point
-// (k = kc * i + c) and the split row is written component-major (k' = c * (kdim / kc) + i), so that
-// a range never mixes components; with kc = 1 the order is kept.
-__global__ void __launch_bounds__(256) lr_split_kernel(const float* __restrict__ src, int64_t kdim, int kc, int kd,
-                                                       int bits, uint16_t* __restrict__ dst, int* __restrict__ exps,
+// row is split exactly into fp16 hi + lo (simt_pack.cuh), one quantum per accumulation range of 32 KD
+// values (`bits` bits).  The source row holds 4 values per outer point (k = 4 i + c); the split row is
+// component-major (k' = c * (kdim / 4) + i), so that a range never mixes components.  Lane t holds points 2 t and
+// 2 t + 1 of every 64, so that a warp writes whole 128-byte runs of one part.
+template <int KD>
+__global__ void __launch_bounds__(256) lr_split_kernel(const float* __restrict__ src, int64_t kdim, int bits,
+                                                       uint16_t* __restrict__ dst, int* __restrict__ exps,
                                                        uint16_t* __restrict__ dst16) {
   __shared__ float red[8];
   const int64_t r = blockIdx.x;
   const float* s = src + r * kdim;
   float m = 0.0f;
+#pragma unroll 4
   for (int64_t k = threadIdx.x * 4; k < kdim; k += blockDim.x * 4) {
     const float4 v = *reinterpret_cast<const float4*>(s + k);
     m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
@@ -240,43 +294,37 @@ __global__ void __launch_bounds__(256) lr_split_kernel(const float* __restrict__
   const float scale = ldexpf(1.0f, e);  // exact power of 2 (|e| <= 100)
   uint16_t* d = dst + r * 2 * kdim;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t per_c = kdim / kc;           // outer points (kc = 4) or values (kc = 1) per component
-  // warp g handles the source points 32 kd g .. 32 kd (g + 1) - 1 (all kc components of each)
-  for (int64_t g = warp; g < per_c / (32 * kd); g += 8) {
-    float v[4][4];
+  const int64_t per_c = kdim / 4;            // outer points, a multiple of 128
+  constexpr int G = KD == 4 ? 2 : 1;         // runs of 64 points per step
+  for (int64_t i0 = 64 * G * warp; i0 < per_c; i0 += 64 * G * 8) {
+    float v[G][2][4];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int64_t i = 32 * (kd * g + t) + lane;
-      v[t][0] = v[t][1] = v[t][2] = v[t][3] = 0.0f;
-      if (t >= kd) continue;
-      if (kc == 4) {
-        const float4 q4 = *reinterpret_cast<const float4*>(s + 4 * i);
-        v[t][0] = q4.x * scale;
-        v[t][1] = q4.y * scale;
-        v[t][2] = q4.z * scale;
-        v[t][3] = q4.w * scale;
-      } else {
-        v[t][0] = s[i] * scale;
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        const float4 q4 = *reinterpret_cast<const float4*>(s + 4 * (i0 + 64 * g + 2 * lane + t));
+        v[g][t][0] = q4.x * scale;
+        v[g][t][1] = q4.y * scale;
+        v[g][t][2] = q4.z * scale;
+        v[g][t][3] = q4.w * scale;
       }
-    }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      if (c >= kc) break;
       float bm = 0.0f;
 #pragma unroll
-      for (int t = 0; t < 4; ++t) bm = fmaxf(bm, fabsf(v[t][c]));
-      for (int o = 16; o > 0; o >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, o));
+      for (int g = 0; g < G; ++g) bm = fmaxf(bm, fmaxf(fabsf(v[g][0][c]), fabsf(v[g][1][c])));
+      bm = __uint_as_float(__reduce_max_sync(KD >= 2 ? 0xffffffffu : (lane < 16 ? 0xffffu : 0xffff0000u), __float_as_uint(bm)));
       const int qe = exact_quantum(bm, bits);
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        if (t >= kd) break;
-        __half h, l;
-        split_exact(v[t][c], qe, h, l);
-        const int64_t kk = c * per_c + 32 * (kd * g + t);  // first value of the 32-value block
-        const int64_t o = (kk >> 6) * 128 + (kk & 63) + lane;
-        d[o] = __half_as_ushort(h);
-        d[o + 64] = __half_as_ushort(l);
-        if (dst16) dst16[r * kdim + kk + lane] = __half_as_ushort(__float2half_rn(v[t][c]));
+      for (int g = 0; g < G; ++g) {
+        __half2 h, l;
+        split_exact(v[g][0][c], qe, h.x, l.x);
+        split_exact(v[g][1][c], qe, h.y, l.y);
+        const int64_t kk = c * per_c + i0 + 64 * g;  // first value of the run
+        *reinterpret_cast<__half2*>(d + 2 * kk + 2 * lane) = h;
+        *reinterpret_cast<__half2*>(d + 2 * kk + 64 + 2 * lane) = l;
+        if (dst16)
+          *reinterpret_cast<__half2*>(dst16 + r * kdim + kk + 2 * lane) = __floats2half2_rn(v[g][0][c], v[g][1][c]);
       }
     }
   }
@@ -445,41 +493,109 @@ __global__ void symmetrize_kernel(double* __restrict__ M, int n_pair, int ldm) {
   }
 }
 
-// dU[p][q][r][s] = U[pair(p,q)][pair(r,s)]
-__global__ void unpack_kernel(const double* __restrict__ U, int N, int ldm, double* __restrict__ dU,
-                              float* __restrict__ dU32) {
+// dU[p][q][r][s] = U[pair(p,q)][pair(r,s)]: one CTA per (p, q), p <= q, reads its row of U once (the part s < r
+// again from L1 / L2) and writes rows (p, q) and (q, p); a warp takes rows r, lanes run over s, so no
+// index needs a division.  HBM-bound: 8 (or 4) bytes written per element; one thread per element with two
+// divisions took 12.8 ms for N = 200 in FP32 (6.4 GB).
+__global__ void __launch_bounds__(256) unpack_kernel(const double* __restrict__ U, int N, int ldm,
+                                                     double* __restrict__ dU, float* __restrict__ dU32) {
+  const int p = blockIdx.y, q = blockIdx.x;
+  if (q < p) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t n2 = static_cast<int64_t>(N) * N;
-  const int64_t rs = blockIdx.y * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  const int64_t pqi = blockIdx.x;
-  if (rs >= n2) return;
-  const int p = static_cast<int>(pqi / N), q = static_cast<int>(pqi % N);
-  const int r = static_cast<int>(rs / N), s = static_cast<int>(rs % N);
-  const double v = U[static_cast<int64_t>(pair_of(p, q, N)) * ldm + pair_of(r, s, N)];
-  const int64_t o = pqi * n2 + rs;
-  if (dU) dU[o] = v;
-  if (dU32) dU32[o] = static_cast<float>(v);
+  const double* src = U + static_cast<int64_t>(pair_of(p, q, N)) * ldm;
+  const int64_t o1 = (static_cast<int64_t>(p) * N + q) * n2, o2 = (static_cast<int64_t>(q) * N + p) * n2;
+  const bool two = p != q;
+  for (int r = warp; r < N; r += 8) {
+    const int base_r = r * N - r * (r - 1) / 2 - r;
+#pragma unroll 4
+    for (int s = lane; s < N; s += 32) {
+      const double v = __ldg(src + (s >= r ? base_r + s : s * N - s * (s - 1) / 2 - s + r));
+      const int64_t o = static_cast<int64_t>(r) * N + s;
+      if (dU) {
+        __stcs(dU + o1 + o, v);
+        if (two) __stcs(dU + o2 + o, v);
+      }
+      if (dU32) {
+        __stcs(dU32 + o1 + o, static_cast<float>(v));
+        if (two) __stcs(dU32 + o2 + o, static_cast<float>(v));
+      }
+    }
+  }
 }
 
-// Delta h_pq = -1/2 (2 sum_rs U(pq|rs) gamma_rs - sum_rs U(ps|rq) gamma_rs), one CTA per (p, q).
-__global__ void onebody_kernel(const double* __restrict__ U, const double* __restrict__ gamma, int N, int ldm,
-                               double* __restrict__ dh) {
-  const int p = blockIdx.y, q = blockIdx.x;
-  const int pq = pair_of(p, q, N);
-  double acc = 0.0;
-  for (int k = threadIdx.x; k < N * N; k += blockDim.x) {
-    const int r = k / N, s = k % N;
-    const double g = gamma[k];
-    acc += g * (2.0 * U[static_cast<int64_t>(pq) * ldm + pair_of(r, s, N)] -
-                U[static_cast<int64_t>(pair_of(p, s, N)) * ldm + pair_of(r, q, N)]);
+// Delta h_pq = -1/2 (2 sum_rs U(pq|rs) gamma_rs - sum_rs U(ps|rq) gamma_rs).  One CTA per row (p, s) of U gives
+//   D[ps]      = sum_rt U(ps|rt) gamma_rt   (packed, gpk: gamma_rr, gamma_rt + gamma_tr)
+//   Z[p][s][q] = sum_r U(ps|rq) gamma_rs  and  Z[s][p][q] = sum_r U(ps|rq) gamma_rp,
+// the latter over the nonzero entries of a column of gamma (lists of gamma_lists_kernel; nothing for an
+// empty column), so U is read once, not N^2 gathers per entry of Delta h (16.3 ms for N = 200).  Then
+// onebody_sum_kernel adds the columns in order.
+__global__ void gamma_lists_kernel(const double* __restrict__ gamma, int N, double* __restrict__ gpk,
+                                   int* __restrict__ idx, int* __restrict__ cnt) {
+  const int c = blockIdx.x, lane = threadIdx.x;
+  int n = 0;
+  for (int r0 = 0; r0 < N; r0 += 32) {
+    const int r = r0 + lane;
+    const double g = r < N ? gamma[r * N + c] : 0.0;
+    const unsigned m = __ballot_sync(0xffffffffu, g != 0.0);
+    if (g != 0.0) idx[c * N + n + __popc(m & ((1u << lane) - 1))] = r;
+    n += __popc(m);
+    if (r < c) gpk[pair_of(r, c, N)] = g + gamma[c * N + r];
+    if (r == c) gpk[pair_of(r, c, N)] = g;
   }
+  if (lane == 0) cnt[c] = n;
+}
+
+__device__ __forceinline__ double block_sum_256(double v) {
   __shared__ double red[256];
-  red[threadIdx.x] = acc;
+  red[threadIdx.x] = v;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+  for (int o = 128; o > 0; o >>= 1) {
     if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) dh[p * N + q] = -0.5 * red[0];
+  return red[0];
+}
+
+__global__ void __launch_bounds__(256) onebody_rows_kernel(const double* __restrict__ U, const double* __restrict__ gamma,
+                                                           const double* __restrict__ gpk, const int* __restrict__ idx,
+                                                           const int* __restrict__ cnt, int N, int NP, int ldm,
+                                                           double* __restrict__ D, double* __restrict__ Z) {
+  const int p = blockIdx.y, s = blockIdx.x;
+  if (s < p) return;
+  const int ps = pair_of(p, s, N);
+  const double* row = U + static_cast<int64_t>(ps) * ldm;
+  double acc = 0.0;
+#pragma unroll 4
+  for (int k = threadIdx.x; k < NP; k += 256) acc += row[k] * gpk[k];
+  const double d = block_sum_256(acc);
+  if (threadIdx.x == 0) D[ps] = d;
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const int a = side ? s : p, c = side ? p : s;   // Z[a][c][.] with column c of gamma
+    if (side && p == s) break;
+    const int n = cnt[c];
+    if (n == 0) continue;
+    for (int q = threadIdx.x; q < N; q += 256) {
+      double z = 0.0;
+      for (int k = 0; k < n; ++k) {
+        const int r = idx[c * N + k];
+        z += gamma[r * N + c] * row[pair_of(r, q, N)];
+      }
+      Z[(static_cast<int64_t>(a) * N + c) * N + q] = z;
+    }
+  }
+}
+
+__global__ void onebody_sum_kernel(const double* __restrict__ D, const double* __restrict__ Z,
+                                   const int* __restrict__ cnt, int N, double* __restrict__ dh) {
+  const int p = blockIdx.y, q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= N) return;
+  double x = 0.0;
+#pragma unroll 4
+  for (int s = 0; s < N; ++s)
+    if (cnt[s]) x += Z[(static_cast<int64_t>(p) * N + s) * N + q];
+  dh[p * N + q] = -0.5 * (2.0 * D[pair_of(p, q, N)] - x);
 }
 
 // Spin builds (Appendix A): U[pq][rs] = -(Fb[pq][rs] + Fa[rs][pq]) = Delta U^{ab}(pq|rs), where
@@ -547,11 +663,12 @@ __global__ void constant_spin_kernel(const double* __restrict__ dh_a, const doub
 }
 
 // e0 = -2/3 sum_pq Delta h_pq gamma_pq
-__global__ void constant_kernel(const double* __restrict__ dh, const double* __restrict__ gamma, int n2,
-                                double* __restrict__ e0) {
+__global__ void __launch_bounds__(1024) constant_kernel(const double* __restrict__ dh, const double* __restrict__ gamma,
+                                                        int n2, double* __restrict__ e0) {
   double acc = 0.0;
+#pragma unroll 4
   for (int k = threadIdx.x; k < n2; k += blockDim.x) acc += dh[k] * gamma[k];
-  __shared__ double red[256];
+  __shared__ double red[1024];
   red[threadIdx.x] = acc;
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {
@@ -608,11 +725,17 @@ void launch_rho_split(const double* phiT, const double* w, int64_t n_grid, int64
     split_phi_f32_kernel<<<std::min<unsigned int>(blocks_for(total, 256), 8192u), 256, 0, st>>>(phiT, w, n_grid,
                                                                                                 n_pad, n_orb, phi32);
     cudaMemsetAsync(colmax, 0, sizeof(unsigned int) * n_pair, st);
-    dim3 g(std::min<unsigned int>(blocks_for(n_grid, 256), 64u), n_pair);
-    rho_colmax_f32_kernel<<<g, 256, 0, st>>>(phi32, n_grid, n_pad, n_orb, pp, pq, colmax);
-    dim3 g2(static_cast<unsigned int>(n_pad / (32 * kd)), blocks_for(n_pair, 8));
-    rho_split_f16_kernel<<<g2, 256, 0, st>>>(phi32, n_grid, n_pad, n_orb, n_pair, pp, pq, colmax, kd,
-                                              gemm_bits_b(kd), colexp, static_cast<uint16_t*>(out));
+    rho_colmax_f32_kernel<<<dim3(blocks_for(n_pad, RC_POINTS), n_orb), 256, n_orb * sizeof(unsigned int), st>>>(
+        phi32, n_pad, n_orb, colmax);
+    rho_colexp_kernel<<<blocks_for(n_pair, 256), 256, 0, st>>>(colmax, n_pair, colexp);
+    const dim3 g2(blocks_for(n_pad, RS_POINTS), n_orb);
+    uint16_t* o = static_cast<uint16_t*>(out);
+    if (kd >= 4)
+      rho_split_f16_kernel<4><<<g2, 256, 0, st>>>(phi32, n_pad, n_orb, n_pair, colexp, gemm_bits_b(kd), o);
+    else if (kd >= 2)
+      rho_split_f16_kernel<2><<<g2, 256, 0, st>>>(phi32, n_pad, n_orb, n_pair, colexp, gemm_bits_b(kd), o);
+    else
+      rho_split_f16_kernel<1><<<g2, 256, 0, st>>>(phi32, n_pad, n_orb, n_pair, colexp, gemm_bits_b(kd), o);
   } else {
     dim3 g2(blocks_for(n_pad, 256), blocks_for(n_pair, 8));
     rho_split_bf16_kernel<<<g2, 256, 0, st>>>(phiT, w, n_grid, n_pad, n_pair, pp, pq, colexp,
@@ -620,10 +743,15 @@ void launch_rho_split(const double* phiT, const double* w, int64_t n_grid, int64
   }
 }
 
-void launch_lr_split(const float* src, int rows, int64_t kdim, int kc, int kd, uint16_t* dst, int* exps,
-                     uint16_t* dst16, cudaStream_t st) {
+void launch_lr_split(const float* src, int rows, int64_t kdim, int kd, uint16_t* dst, int* exps, uint16_t* dst16,
+                     cudaStream_t st) {
   if (rows <= 0) return;
-  lr_split_kernel<<<rows, 256, 0, st>>>(src, kdim, kc, kd, gemm_bits_lr(kd), dst, exps, dst16);
+  if (kd >= 4)
+    lr_split_kernel<4><<<rows, 256, 0, st>>>(src, kdim, gemm_bits_lr(kd), dst, exps, dst16);
+  else if (kd >= 2)
+    lr_split_kernel<2><<<rows, 256, 0, st>>>(src, kdim, gemm_bits_lr(kd), dst, exps, dst16);
+  else
+    lr_split_kernel<1><<<rows, 256, 0, st>>>(src, kdim, gemm_bits_lr(kd), dst, exps, dst16);
 }
 
 void launch_rho_f64(const double* phi, const double* w, int64_t n_grid, int64_t n_pad, int n_orb, const int* pp,
@@ -656,8 +784,7 @@ void launch_vfield_f64_impl(const double* grid, const JastrowParams* jp, int n_n
 void launch_unpack(const double* M, int n_orb, int n_pair, double* dU, float* dU32, cudaStream_t st) {
   const int ldm = static_cast<int>(m_stride(n_pair));
   if (dU || dU32) {
-    dim3 g(static_cast<unsigned int>(n_orb) * n_orb, blocks_for(static_cast<int64_t>(n_orb) * n_orb, 256));
-    unpack_kernel<<<g, 256, 0, st>>>(M, n_orb, ldm, dU, dU32);
+    unpack_kernel<<<dim3(n_orb, n_orb), 256, 0, st>>>(M, n_orb, ldm, dU, dU32);
   }
 }
 
@@ -667,11 +794,23 @@ void launch_symmetrize(double* M, int n_pair, cudaStream_t st) {
   symmetrize_kernel<<<g, dim3(32, 8), 0, st>>>(M, n_pair, ldm);
 }
 
-void launch_onebody(const double* M, const double* gamma, int n_orb, int n_pair, double* dh, double* e0,
+size_t onebody_bytes(int n_orb) {
+  const size_t n = n_orb, np = n * (n + 1) / 2;
+  return 8 * (n * n * n + 2 * np) + 4 * (n * n + n);
+}
+
+void launch_onebody(const double* M, const double* gamma, int n_orb, int n_pair, void* tmp, double* dh, double* e0,
                     cudaStream_t st) {
   const int ldm = static_cast<int>(m_stride(n_pair));
-  onebody_kernel<<<dim3(n_orb, n_orb), 256, 0, st>>>(M, gamma, n_orb, ldm, dh);
-  constant_kernel<<<1, 256, 0, st>>>(dh, gamma, n_orb * n_orb, e0);
+  double* Z = static_cast<double*>(tmp);
+  double* D = Z + static_cast<size_t>(n_orb) * n_orb * n_orb;
+  double* gpk = D + n_pair;
+  int* idx = reinterpret_cast<int*>(gpk + n_pair);
+  int* cnt = idx + n_orb * n_orb;
+  gamma_lists_kernel<<<n_orb, 32, 0, st>>>(gamma, n_orb, gpk, idx, cnt);
+  onebody_rows_kernel<<<dim3(n_orb, n_orb), 256, 0, st>>>(M, gamma, gpk, idx, cnt, n_orb, n_pair, ldm, D, Z);
+  onebody_sum_kernel<<<dim3(blocks_for(n_orb, 64), n_orb), 64, 0, st>>>(D, Z, cnt, n_orb, dh);
+  constant_kernel<<<1, 1024, 0, st>>>(dh, gamma, n_orb * n_orb, e0);
 }
 
 void launch_spin_cross(const double* Fb, const double* Fa, int n_pair, double* U, cudaStream_t st) {

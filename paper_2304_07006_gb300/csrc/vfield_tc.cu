@@ -588,8 +588,9 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
 }
 
 // =================================================================== finalize kernels
-// V from the FP64 accumulator of the GEMM: one CTA per (tile, split), thread = tile row; the tile
+// V from the FP64 accumulator of the GEMM: one CTA per (tile, split, 32 columns), thread = tile row; the tile
 // order is the GEMM's grouped order.
+constexpr int FIN_COLS = 32;
 template <int BN>
 __global__ void __launch_bounds__(VF_BM) vfield_finalize_kernel(const VfieldArgs args) {
   const int m_tiles = 3 * args.mt_per_x;
@@ -602,7 +603,9 @@ __global__ void __launch_bounds__(VF_BM) vfield_finalize_kernel(const VfieldArgs
   const double* acc = args.Vacc + (static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * VF_BM * BN + row;
   float* v = args.V + blockIdx.y * v_slice(args.gcp, args.n_orb);
   const int ncol = min(BN, args.n_pair - t.n_tile * BN);
-  for (int c = 0; c < ncol; ++c) {
+  const int c1 = min(ncol, static_cast<int>(blockIdx.z + 1) * FIN_COLS);
+#pragma unroll 4
+  for (int c = blockIdx.z * FIN_COLS; c < c1; ++c) {
     const int pq = t.n_tile * BN + c;
     const int p = __ldg(args.pair_p + pq), q = __ldg(args.pair_q + pq);
     const float val =
@@ -613,8 +616,7 @@ __global__ void __launch_bounds__(VF_BM) vfield_finalize_kernel(const VfieldArgs
 }
 
 // M[pq][rs] += tile sum * 2^-(exp_a[pq] + exp_b[rs]) for one tile of the step (d) GEMM (mode 1);
-// one CTA per tile (each M element is owned by one tile), through shared memory in slabs of 32
-// columns: read column-major from the tile sums (thread = row), added row-major into M (warp =
+// one CTA per tile and slab of 32 columns (each M element is owned by one), through shared memory: read column-major from the tile sums (thread = row), added row-major into M (warp =
 // row, lane = column), both coalesced.
 template <int BN>
 __global__ void __launch_bounds__(VF_BM) assemble_finalize_kernel(const VfieldArgs args) {
@@ -626,21 +628,21 @@ __global__ void __launch_bounds__(VF_BM) assemble_finalize_kernel(const VfieldAr
   const int ncol = min(BN, args.n_pair - t.n_tile * BN);
   const int row0 = t.m_tile * VF_BM, col0 = t.n_tile * BN;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int c0 = 0; c0 < ncol; c0 += 32) {
-    for (int c = 0; c < 32; ++c)
-      slab[c][threadIdx.x] = c0 + c < ncol ? acc[static_cast<int64_t>(c0 + c) * VF_BM + threadIdx.x] : 0.0;
-    __syncthreads();
-    const int c = c0 + lane;
-    if (c < ncol) {
-      const int eb = __ldg(args.exp_b + col0 + c);
-      for (int r = warp; r < VF_BM && row0 + r < args.rows_a; r += VF_BM / 32) {
-        const int pq = row0 + r;
-        const int e = __ldg(args.exp_a + pq) + eb;
-        double* m = args.M + static_cast<int64_t>(pq) * args.ldm + col0 + c;
-        *m += slab[lane][r] * __longlong_as_double(static_cast<long long>(1023 - e) << 52);
-      }
-    }
-    __syncthreads();
+  const int c0 = blockIdx.z * FIN_COLS;
+#pragma unroll 8
+  for (int c = 0; c < 32; ++c)
+    slab[c][threadIdx.x] = c0 + c < ncol ? acc[static_cast<int64_t>(c0 + c) * VF_BM + threadIdx.x] : 0.0;
+  __syncthreads();
+  const int c = c0 + lane;
+  if (c >= ncol) return;
+  const int eb = __ldg(args.exp_b + col0 + c);
+#pragma unroll 4
+  for (int r = warp; r < VF_BM; r += VF_BM / 32) {
+    if (row0 + r >= args.rows_a) break;
+    const int pq = row0 + r;
+    const int e = __ldg(args.exp_a + pq) + eb;
+    double* m = args.M + static_cast<int64_t>(pq) * args.ldm + col0 + c;
+    *m += slab[lane][r] * __longlong_as_double(static_cast<long long>(1023 - e) << 52);
   }
 }
 
@@ -675,6 +677,7 @@ void launch_vfield_tc_finalize(const VfieldArgs& a, int parts, int splits, cudaS
   if (a.n_tiles <= 0 || splits <= 0 || a.flush <= 0) return;
   if (a.mode == 1 ? a.rows_a <= 0 : a.mt_per_x <= 0) return;
   dim3 grid(tile_ctas(a, parts), static_cast<unsigned>(splits));
+  grid.z = (parts == 2 ? XB_BN : BF_BN) / FIN_COLS;
   if (a.mode == 1)
     assemble_finalize_kernel<XB_BN><<<grid, VF_BM, 0, st>>>(a);
   else if (parts == 2)

@@ -95,6 +95,7 @@ struct xtc_ctx {
   DBuf lamd, gamma_b, M2, M3;  // direct weights; spin builds: beta density, f^b, Delta U^{ab}
   DBuf lam2, R2, R32b, eR2;    // spin builds: beta exchange weights, R for electron-2 beta
   DBuf Lv, T3;                 // explicit three-body L: V of the outer points, the packed T
+  DBuf h_tmp;                         // one-body kernel's partial sums
   DBuf fc_U, fc_h, fc_hout, fc_Uout;  // frozen-core folding: staged host inputs and outputs
   DBuf G2;                     // second gradient table: step (a) of the next chunk on stream st2
   DBuf k_dphi, k_dphiT, k_W, k_S;  // two-body integrals K: staged and transposed gradients, rows of W and V, S
@@ -126,7 +127,7 @@ struct xtc_ctx {
     return {&jp_dev, &err_dev, &flag_dev, &grid, &w, &phi, &gamma, &phiT, &phi32, &pair_p, &pair_q, &jtab, &jtab64,
             &rho, &colmax, &colexp, &G, &V, &Vacc, &L, &R, &L32, &R32, &eL, &eR, &M, &evec, &lam, &dU_tmp,
             &dh_tmp, &e0_tmp, &vout, &r1, &r2, &lamd, &gamma_b, &M2, &M3, &lam2, &R2, &R32b, &eR2, &Lv, &T3,
-            &fc_U, &fc_h, &fc_hout, &fc_Uout, &G2, &k_dphi, &k_dphiT, &k_W, &k_S, &d_rho, &d_rhoe, &d_sj,
+            &h_tmp, &fc_U, &fc_h, &fc_hout, &fc_Uout, &G2, &k_dphi, &k_dphiT, &k_W, &k_S, &d_rho, &d_rhoe, &d_sj,
             &d_G, &d_Ge, &d_tmp, &d_L, &d_Le, &d_R, &d_Re};
   }
 };
@@ -666,7 +667,7 @@ int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* gri
         !ensure(ctx->colexp, 4ull * pl.NP) || !ensure(ctx->phi32, 8ull * (n_orb + 1) * pl.NGp))
       return fail(ctx, XTC_ERR_OOM, "grid tables (%.2f GB)", 2.0 * 3 * pl.NGp * pl.NP / 1e9);
   }
-  const int nprep = f64 ? 1 : (pl.parts_b == 2 ? 5 : 3);
+  const int nprep = f64 ? 1 : (pl.parts_b == 2 ? 6 : 3);
   timed(ctx, XTC_K_PREP, nprep, [&] {
     launch_transpose_phi(*d_phi, n_grid, pl.NGp, n_orb, ctx->phiT.as<double>(), st);
     if (!f64) {
@@ -1093,12 +1094,12 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
         da.exp_b = ctx->eR.as<int>();
         da.err = ctx->err_dev.as<int>();
         timed(ctx, XTC_K_AUX, M2 ? 3 : 2, [&] {
-          launch_lr_split(ctx->L32.as<float>(), NP, kdim, 4, da.kd, ctx->L.as<uint16_t>(), ctx->eL.as<int>(), nullptr,
+          launch_lr_split(ctx->L32.as<float>(), NP, kdim, da.kd, ctx->L.as<uint16_t>(), ctx->eL.as<int>(), nullptr,
                           st);
-          launch_lr_split(ctx->R32.as<float>(), NP, kdim, 4, da.kd, ctx->R.as<uint16_t>(), ctx->eR.as<int>(),
+          launch_lr_split(ctx->R32.as<float>(), NP, kdim, da.kd, ctx->R.as<uint16_t>(), ctx->eR.as<int>(),
                           ctx->R.as<uint16_t>() + 2 * kdim * NP, st);
           if (M2)
-            launch_lr_split(ctx->R32b.as<float>(), NP, kdim, 4, da.kd, ctx->R2.as<uint16_t>(), ctx->eR2.as<int>(),
+            launch_lr_split(ctx->R32b.as<float>(), NP, kdim, da.kd, ctx->R2.as<uint16_t>(), ctx->eR2.as<int>(),
                             ctx->R2.as<uint16_t>() + 2 * kdim * NP, st);
         });
         timed(ctx, XTC_K_ASSEMBLE, 1, [&] { launch_vfield_tc(&tm_L, &tm_R, &tm_R16, da, 2, 1, st); });
@@ -1139,7 +1140,8 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
   NvtxRange nvtx_final("final");
   const size_t n4 = static_cast<size_t>(N) * N * N * N;
   const size_t n2b = static_cast<size_t>(N) * N * 8;
-  if (!ensure(ctx->dh_tmp, 2 * n2b) || !ensure(ctx->e0_tmp, 8)) return fail(ctx, XTC_ERR_OOM, "dh staging");
+  if (!ensure(ctx->dh_tmp, 2 * n2b) || !ensure(ctx->e0_tmp, 8) || (!spin && !ensure(ctx->h_tmp, onebody_bytes(N))))
+    return fail(ctx, XTC_ERR_OOM, "dh staging");
   double* dh_d[2] = {nullptr, nullptr};
   for (int sp = 0; sp < out.n_spin; ++sp)
     dh_d[sp] = is_device_ptr(out.dh[sp]) ? out.dh[sp] : ctx->dh_tmp.as<double>() + static_cast<size_t>(sp) * N * N;
@@ -1158,10 +1160,10 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
   float* u32dst = out.dU32 ? (u32_dev ? out.dU32 : ctx->vout.as<float>()) : nullptr;
   if (!spin) {
     double* udst = out.dU[0] ? (u_dev[0] ? out.dU[0] : ctx->dU_tmp.as<double>()) : nullptr;
-    timed(ctx, XTC_K_FINAL, (udst || u32dst) ? 4 : 3, [&] {
+    timed(ctx, XTC_K_FINAL, (udst || u32dst) ? 6 : 5, [&] {
       launch_symmetrize(ctx->M.as<double>(), NP, st);
       launch_unpack(ctx->M.as<double>(), N, NP, udst, u32dst, st);
-      launch_onebody(ctx->M.as<double>(), ctx->gamma.as<double>(), N, NP, dh_d[0], e0_d, st);
+      launch_onebody(ctx->M.as<double>(), ctx->gamma.as<double>(), N, NP, ctx->h_tmp.p, dh_d[0], e0_d, st);
     });
     CUDA_OK(cudaGetLastError());
     if (out.dU[0] && !u_dev[0]) CUDA_OK(cudaMemcpyAsync(out.dU[0], udst, n4 * 8, cudaMemcpyDeviceToHost, st));

@@ -292,12 +292,12 @@ void launch_fields(const FieldsArgs& a, bool f64, cudaStream_t st);  // f64: FP6
 // Step (d) operands in fp16 x2: each FP32 row src[r][0..kdim) is scaled by 2^exps[r] (largest
 // magnitude in [2^13, 2^14)) and split exactly into hi + lo fp16 with one quantum per range of kd
 // blocks of 32 values (gemm_bits_lr(kd) bits), in 128-byte runs of one part:
-// dst[r][k' / 64][part][k' % 64].  kc = 4: the source holds 4 values per outer point (k = 4 i + c)
-// and k' = c * kdim / 4 + i (component-major, so that a range never mixes components); kc = 1:
-// k' = k.  kdim / kc must be a multiple of 32 kd.  dst16 (or NULL): the scaled values rounded to
+// dst[r][k' / 64][part][k' % 64].  The source holds 4 values per outer point (k = 4 i + c)
+// and k' = c * kdim / 4 + i (component-major, so that a range never mixes components); kdim / 4 is a
+// multiple of 128.  dst16 (or NULL): the scaled values rounded to
 // fp16, dst16[r][k'] (the plane of the B operand, for the lo x fp16(B) product).
-void launch_lr_split(const float* src, int rows, int64_t kdim, int kc, int kd, uint16_t* dst, int* exps,
-                     uint16_t* dst16, cudaStream_t st);
+void launch_lr_split(const float* src, int rows, int64_t kdim, int kd, uint16_t* dst, int* exps, uint16_t* dst16,
+                     cudaStream_t st);
 
 // Step (d), tensor cores, bf16 x3: M[pq][rs] += sum_k L[pq][k] R[rs][k] over k < kdim (FP64 accumulator).
 void launch_assemble_tc(const CUtensorMap* tm_L, const CUtensorMap* tm_R, int n_pair, int kdim, int kd, double* M,
@@ -321,7 +321,9 @@ void launch_spin_cross(const double* Fb, const double* Fa, int n_pair, double* U
 // Spin builds: Delta h^a, Delta h^b and e0 from Delta U^{aa}, ^{ab}, ^{bb} and the two densities.
 void launch_onebody_spin(const double* Uaa, const double* Uab, const double* Ubb, const double* ga, const double* gb,
                          int n_orb, int n_pair, double* dh_a, double* dh_b, double* e0, cudaStream_t st);
-void launch_onebody(const double* M, const double* gamma, int n_orb, int n_pair, double* dh, double* e0,
+// tmp: onebody_bytes(n_orb) of workspace.
+size_t onebody_bytes(int n_orb);
+void launch_onebody(const double* M, const double* gamma, int n_orb, int n_pair, void* tmp, double* dh, double* e0,
                     cudaStream_t st);
 
 // V (FP32 or FP64, [splits] slices in the layout of v_index) -> FP64 [n_i][3][pq] (for xtc_vfield).
