@@ -275,6 +275,7 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
       a.kd = parts == 2 ? kd_b : std::min(cv.vf_kd, 2);
       a.xper = 64;
       a.unscale_g = std::ldexp(1.0f, -sg);
+      a.n_sm = cv.n_sm;
       a.err = err;
       launch_vfield_tc(&tm_gl, &tm, &tm16, a, parts, 1, st);
     }

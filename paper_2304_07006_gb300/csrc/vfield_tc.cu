@@ -52,6 +52,8 @@
 // operand (64-byte swizzle), six products (i + j <= 2) into one of two TMEM accumulators per range
 // of `kd` stages, small cross products first, drained into FP32 running sums after every range.
 // Its accumulation is not exact: the truncation bias is only kept small by the short ranges.
+#include <algorithm>
+
 #include "ptx_sm100.cuh"
 #include "xtc_internal.cuh"
 
@@ -139,7 +141,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(XB_THREADS, 1)
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp: uniform
   const uint32_t rank = cluster_rank();
   const int m_tiles = MODE == 0 ? 3 * args.mt_per_x : (args.rows_a + VF_BM - 1) / VF_BM;
-  const TileXY t = pair_tile(blockIdx.x, m_tiles, args.n_tiles);
+  const TileXY t = pair_tile(args.cta0 + blockIdx.x, m_tiles, args.n_tiles);
   const bool valid = t.m_tile < m_tiles;          // a tile that does not exist repeats the last one's rows
   const int m_tile = valid ? t.m_tile : m_tiles - 1;
   // mode 0: rows x * gcp + outer point of component x; mode 1: rows pq
@@ -286,7 +288,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(XB_THREADS, 1)
     // c of every thread goes after range r when r % flush == c (staggered, so that no drain carries a
     // whole tile of FP64 adds at once): a store the first time (r < flush), then a fire-and-forget
     // reduction; every column is flushed at least once per `flush` ranges.
-    double* acc = args.Vacc + (static_cast<int64_t>(split) * gridDim.x + blockIdx.x) * VF_BM * XB_BN +
+    double* acc = args.Vacc + (static_cast<int64_t>(split) * args.n_cta + args.cta0 + blockIdx.x) * VF_BM * XB_BN +
                   static_cast<int64_t>(c_base) * VF_BM + quarter * 32 + lane;
     auto flush_col = [&](int c, bool first) {
 #pragma unroll
@@ -406,7 +408,7 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const TileXY t = grouped_tile(blockIdx.x, 3 * args.mt_per_x, args.n_tiles);
+  const TileXY t = grouped_tile(args.cta0 + blockIdx.x, 3 * args.mt_per_x, args.n_tiles);
   const int x = t.m_tile / args.mt_per_x;
   const int ib = (t.m_tile - x * args.mt_per_x) * VF_BM;
   const int row0 = static_cast<int>(x * args.gcp) + ib;
@@ -521,7 +523,7 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
     for (int k = 0; k < BF_HC; ++k) S[k] = 0.0f;
     int nflush = 0;
     auto flush_sums = [&]() {
-      double* acc = args.Vacc + (static_cast<int64_t>(split) * gridDim.x + blockIdx.x) * VF_BM * BF_BN +
+      double* acc = args.Vacc + (static_cast<int64_t>(split) * args.n_cta + args.cta0 + blockIdx.x) * VF_BM * BF_BN +
                     static_cast<int64_t>(c_base) * VF_BM + quarter * 32 + lane;
       if (nflush == 0) {
 #pragma unroll
@@ -652,25 +654,49 @@ unsigned tile_ctas(const VfieldArgs& a, int parts) {
   return static_cast<unsigned>((parts == 2 ? (m + 1) / 2 * 2 : m) * a.n_tiles);
 }
 
+// CTAs per launch of a GEMM of n CTAs along x.  The CTAs resident at one time stream the same panels of A and
+// B and meet in L2 only while they are at about the same k.  Nothing keeps them there: each new tile starts when
+// some other one ends, and after ten waves of the N = 120 build the starts are spread over a third of a tile's time,
+// with 58.6 GB read from HBM where the panels of its waves are 17 GB.  The board is at its power cap, so that
+// traffic is paid for in clock rate.  Launches of whole waves line the CTAs up again: step (b) of that build 1,060 -> 925 ms,
+// of a piece of the N = 200 build 169 -> 134 ms (one wave a launch; two 134, four 139).  A launch costs a few
+// microseconds and the tail of its last wave, so it lasts at least LAUNCH_RANGES ranges of 64 values (2 ms;
+// at 376 ranges a tile, eight waves a launch are as fast as all of them in one).  Tiles do not depend on each other.
+constexpr int LAUNCH_RANGES = 3000;
+int launch_ctas(const VfieldArgs& a, int n, int splits) {
+  if (splits > 1 || a.n_sm < 2) return n;
+  const int64_t ranges = std::max(1, a.n_kb / 2);
+  const int64_t step = (LAUNCH_RANGES + ranges - 1) / ranges * (a.n_sm & ~1);
+  return static_cast<int>(std::min<int64_t>(std::max(n, 1), step));
+}
+
 }  // namespace
 
 bool vfield_tc_supported(int n_nuc) { return n_nuc >= 1 && n_nuc <= 8; }
 
-void launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const CUtensorMap* tm_rho16,
-                      const VfieldArgs& a, int parts, int splits, cudaStream_t st) {
-  if (a.n_tiles <= 0 || splits <= 0) return;
-  if (a.mode == 1 ? a.rows_a <= 0 : a.mt_per_x <= 0) return;
+int launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const CUtensorMap* tm_rho16,
+                     const VfieldArgs& a, int parts, int splits, cudaStream_t st) {
+  if (a.n_tiles <= 0 || splits <= 0) return 0;
+  if (a.mode == 1 ? a.rows_a <= 0 : a.mt_per_x <= 0) return 0;
   dim3 grid(tile_ctas(a, parts), static_cast<unsigned>(splits));
-  if (a.mode == 1) {
-    cudaFuncSetAttribute(xgemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, XB_SMEM);
-    xgemm_kernel<1><<<grid, XB_THREADS, XB_SMEM, st>>>(*tm_g, *tm_rho, *tm_rho16, a);
-  } else if (parts == 2) {
-    cudaFuncSetAttribute(xgemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, XB_SMEM);
-    xgemm_kernel<0><<<grid, XB_THREADS, XB_SMEM, st>>>(*tm_g, *tm_rho, *tm_rho16, a);
+  VfieldArgs w = a;
+  w.n_cta = static_cast<int>(grid.x);
+  const int step = launch_ctas(a, w.n_cta, splits);
+  auto each_launch = [&](auto&& launch) {
+    for (w.cta0 = 0; w.cta0 < w.n_cta; w.cta0 += step) {
+      grid.x = static_cast<unsigned>(std::min(step, w.n_cta - w.cta0));
+      launch(w);
+    }
+  };
+  if (parts == 2) {
+    auto kern = a.mode == 1 ? xgemm_kernel<1> : xgemm_kernel<0>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, XB_SMEM);
+    each_launch([&](const VfieldArgs& v) { kern<<<grid, XB_THREADS, XB_SMEM, st>>>(*tm_g, *tm_rho, *tm_rho16, v); });
   } else {
     cudaFuncSetAttribute(vfield_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BF_SMEM);
-    vfield_bf16_kernel<<<grid, BF_THREADS, BF_SMEM, st>>>(*tm_g, *tm_rho, a);
+    each_launch([&](const VfieldArgs& v) { vfield_bf16_kernel<<<grid, BF_THREADS, BF_SMEM, st>>>(*tm_g, *tm_rho, v); });
   }
+  return (w.n_cta + step - 1) / step;
 }
 
 void launch_vfield_tc_finalize(const VfieldArgs& a, int parts, int splits, cudaStream_t st) {

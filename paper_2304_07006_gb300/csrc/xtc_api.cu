@@ -766,10 +766,13 @@ void run_gemm_b(xtc_ctx* ctx, const Plan& pl, int64_t n_i, const VfMaps& maps) {
   a.xper = ctx->x_period;
   a.flush = flush_ranges(ctx->vf_flush, a.kd);
   a.unscale_g = std::ldexp(1.0f, -gradient_scale(ctx, pl));
+  a.n_sm = ctx->n_sm;
   a.err = ctx->err_dev.as<int>();
   const int splits = pl.splits;
   // the GEMM, then (FP64 flushes) the kernel that writes V from the FP64 sums
-  timed(ctx, XTC_K_VFIELD, 1, [&] { launch_vfield_tc(&maps.g_load, &maps.rho, &maps.rho16, a, pl.parts_b, splits, st); });
+  timed(ctx, XTC_K_VFIELD, 0, [&] {
+    ctx->launches[XTC_K_VFIELD] += launch_vfield_tc(&maps.g_load, &maps.rho, &maps.rho16, a, pl.parts_b, splits, st);
+  });
   if (a.flush > 0) timed(ctx, XTC_K_AUX, 1, [&] { launch_vfield_tc_finalize(a, pl.parts_b, splits, st); });
 }
 
@@ -1092,6 +1095,7 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
         da.ldm = m_stride(NP);
         da.exp_a = ctx->eL.as<int>();
         da.exp_b = ctx->eR.as<int>();
+        da.n_sm = ctx->n_sm;
         da.err = ctx->err_dev.as<int>();
         timed(ctx, XTC_K_AUX, M2 ? 3 : 2, [&] {
           launch_lr_split(ctx->L32.as<float>(), NP, kdim, da.kd, ctx->L.as<uint16_t>(), ctx->eL.as<int>(), nullptr,
@@ -1102,13 +1106,17 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
             launch_lr_split(ctx->R32b.as<float>(), NP, kdim, da.kd, ctx->R2.as<uint16_t>(), ctx->eR2.as<int>(),
                             ctx->R2.as<uint16_t>() + 2 * kdim * NP, st);
         });
-        timed(ctx, XTC_K_ASSEMBLE, 1, [&] { launch_vfield_tc(&tm_L, &tm_R, &tm_R16, da, 2, 1, st); });
+        timed(ctx, XTC_K_ASSEMBLE, 0, [&] {
+          ctx->launches[XTC_K_ASSEMBLE] += launch_vfield_tc(&tm_L, &tm_R, &tm_R16, da, 2, 1, st);
+        });
         timed(ctx, XTC_K_AUX, 1, [&] { launch_vfield_tc_finalize(da, 2, 1, st); });
         if (M2) {  // the tile sums buffer is reused after the finalize above, in stream order
           VfieldArgs db = da;
           db.M = M2;
           db.exp_b = ctx->eR2.as<int>();
-          timed(ctx, XTC_K_ASSEMBLE, 1, [&] { launch_vfield_tc(&tm_L, &tm_R2, &tm_R216, db, 2, 1, st); });
+          timed(ctx, XTC_K_ASSEMBLE, 0, [&] {
+            ctx->launches[XTC_K_ASSEMBLE] += launch_vfield_tc(&tm_L, &tm_R2, &tm_R216, db, 2, 1, st);
+          });
           timed(ctx, XTC_K_AUX, 1, [&] { launch_vfield_tc_finalize(db, 2, 1, st); });
         }
       } else if (pl.f64) {

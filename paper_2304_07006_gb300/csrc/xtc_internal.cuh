@@ -161,6 +161,8 @@ struct VfieldArgs {
   int64_t n_i;                 // outer points of this chunk
   int64_t gcp;                 // padded chunk length (row stride of V and of G per component)
   int mt_per_x;                // 128-row tiles per component: ceil(n_i / 128)
+  int n_sm;
+  int cta0, n_cta;             // first CTA of this launch and CTAs of the whole GEMM (set by the launcher)
   int n_tiles;                 // column tiles: ceil(n_pair / vf_bn(parts))
   int n_pair;
   int kb_per_split, n_kb;      // inner K-blocks per split slice (a multiple of 4), total K-blocks
@@ -180,10 +182,10 @@ struct VfieldArgs {
   const int* exp_b;
 };
 bool vfield_tc_supported(int n_nuc);
-// Launches the GEMM.
+// Launches the GEMM; returns the number of launches.
 // tm_rho16: the fp16(B) plane of the fp16 precision (box 64 x 64, 128-byte swizzle); the bf16 precision ignores it.
-void launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const CUtensorMap* tm_rho16,
-                      const VfieldArgs& a, int parts, int splits, cudaStream_t st);
+int launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const CUtensorMap* tm_rho16,
+                     const VfieldArgs& a, int parts, int splits, cudaStream_t st);
 // Then, with FP64 sums (a.flush > 0): mode 0 writes V from them, mode 1 adds the tiles into M.
 void launch_vfield_tc_finalize(const VfieldArgs& a, int parts, int splits, cudaStream_t st);
 
