@@ -9,20 +9,29 @@
 // gradient from the GEMM's critical path; the table costs one HBM write and is then read through L2
 // by the GEMM's tiles.
 //
-// One warp owns a unit of 32 outer points (one per lane, its per-point coefficients in registers)
-// and a run of inner-point blocks of 32.  For each block it evaluates the gradient in FP32 (two
+// One warp owns a unit of 16 outer points (two lanes each, one per half of a block, its per-point coefficients
+// in registers) and a run of inner-point blocks of 32.  For each block it evaluates the gradient in FP32 (two
 // inner points per packed FP32 instruction for up to two Jastrow centres; reciprocal square roots
 // and reciprocals refined by a Newton-Raphson step, so that no one-signed error of the hardware
 // approximations enters the gradient), splits
-// it, writes the tiles of the three components (32 rows x 128 bytes, or 3 parts x 32 rows x 64
+// it, writes the tiles of the three components (16 rows x 128 bytes, or 3 parts x 16 rows x 64
 // bytes) into shared memory in their swizzle (conflict-free 16-byte stores) and one lane stores
 // them with TMA.  The fp16 split is exact on a per-range quantum (simt_pack.cuh): for every row and
 // accumulation range of the GEMM (RB blocks of 32 inner points), hi = an integer of at most 9
-// bits times the range's quantum, lo = the fp16 remainder.  The lane first stages the FP32 values of
-// two blocks (64 points, a hi and a lo tile per component; four blocks when RB = 4) in its own tile rows,
-// then splits them with the quantum of their range's maximum; a CTA holds GF_WARPS / BB warps of BB blocks.
+// bits times the range's quantum, lo = the fp16 remainder.  The lanes first stage the FP32 values of
+// two blocks (64 points, a hi and a lo tile per component; four blocks when RB = 4) in their tile rows,
+// then split them with the quantum of their range's maximum.
+//
+// What bounds it: the latency of the table loads and of the dependent FP32 chain, so warps in flight count, and
+// the staging limits those: with 32 rows a warp (24 KB) an SM held 8 warps and issued in 28 % of its cycles,
+// with 16 rows (12 KB) it holds 16.  The FP64 arithmetic of the coefficients (about 250 operations a
+// nucleus on a pipe of two per clock, a third of a unit's time) runs once per outer point, in gcoef_kernel, not once per
+// unit.  Measured (one GB300), before -> now: 4,000 x 4,000 points and 3 nuclei 253 -> 119 us (with units of 16 blocks, see
+// launch_rb), 20,000 x 20,000 and 3 nuclei 3.35 -> 1.75 ms, the bf16 parts of 40,000 x 40,000 points 14.0 -> 9.0 ms.
 // The gradient is taken with the pair formula of jastrow_coef.cuh: per-point coefficients times
 // polynomials in b = r12 / (1 + r12) and a_jI = |r_j - R_I| / (1 + |r_j - R_I|).
+#include <algorithm>
+
 #include "jastrow_coef.cuh"
 #include "ptx_sm100.cuh"
 #include "simt_pack.cuh"
@@ -31,9 +40,9 @@
 namespace xtc {
 namespace {
 
-constexpr int GF_WARPS = 8;
-constexpr int GF_THREADS = GF_WARPS * 32;
-constexpr int GF_TILE = 32 * 64;   // one part's share of a component tile: 32 rows of 64 bytes
+constexpr int GF_ROWS = GFIELD_ROWS;       // outer points of a warp
+constexpr int GF_WARPS = 4;                // warps of a CTA
+constexpr int GF_TILE = GF_ROWS * 64;      // one part's share of a component tile: 16 rows of 64 bytes
 // fp16: bits of the integer hi part of G on its range's quantum (|k| <= 2^9, exact in fp16)
 constexpr int GF_EXACT_BITS = GEMM_BITS_A;
 
@@ -51,35 +60,60 @@ __device__ __forceinline__ void bulk_wait_read_all() {
 // Waits until every committed bulk store has completed.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
+// Nuclei of the kernel's template for n nuclei, and CTAs of an SM (registers: 128 up to 3 nuclei).
+constexpr int nuc_slots(int n) { return n <= 4 ? n : 8; }
+constexpr int gf_ctas(int nnuc) { return nnuc <= 3 ? 4 : (nnuc == 4 ? 3 : 2); }
+
+// Coefficients of the outer points [i0, i0 + rows), rows past the chunk's n_i repeating its last point:
+// coef[k][row], k = 0..13 the point's, 14..16 the low parts of its coordinates (the pair difference is taken
+// in hi/lo FP32), then NUC_COEF per nucleus.
+template <int NNUC>
+__global__ void __launch_bounds__(128) gcoef_kernel(const GfieldArgs args) {
+  const int64_t il = blockIdx.x * 128ll + threadIdx.x;
+  if (il >= args.rows) return;
+  const int64_t ig = args.i0 + (il < args.n_i ? il : args.n_i - 1);
+  float pc[PT_COEF];
+  float nc[NNUC * NUC_COEF];
+  const double gx = args.grid[3 * ig], gy = args.grid[3 * ig + 1], gz = args.grid[3 * ig + 2];
+  point_coefs_fixed<float, NNUC>(*args.jp, gx, gy, gz, static_cast<double>(args.g_scale), pc, nc);
+  float* o = args.coef + il;
+#pragma unroll
+  for (int k = 0; k < PT_COEF; ++k) o[k * args.rows] = pc[k];
+  o[(PT_COEF + 0) * args.rows] = static_cast<float>(gx - static_cast<double>(pc[0]));
+  o[(PT_COEF + 1) * args.rows] = static_cast<float>(gy - static_cast<double>(pc[1]));
+  o[(PT_COEF + 2) * args.rows] = static_cast<float>(gz - static_cast<double>(pc[2]));
+#pragma unroll
+  for (int k = 0; k < NNUC * NUC_COEF; ++k) o[(PT_COEF + 3 + k) * args.rows] = nc[k];
+}
+
 template <int PARTS, int NNUC, int RB>
-__global__ void __launch_bounds__(GF_THREADS)
+__global__ void __launch_bounds__(GF_WARPS * 32, gf_ctas(NNUC))
     gfield_kernel(const __grid_constant__ CUtensorMap tm_g, const GfieldArgs args) {
   constexpr bool BF16 = PARTS == 3;
   constexpr int JS = NNUC <= 4 ? 12 : 16;  // floats per inner point in the table (launch_jtab)
   constexpr int BLOCK_BYTES = 3 * PARTS * GF_TILE;  // the three component tiles of one block
   constexpr int BB = PARTS == 2 && RB < 2 ? 2 : RB;   // blocks staged together: whole pairs for the fp16 tiles
   constexpr int WARP_BYTES = BB * BLOCK_BYTES;
-  constexpr int WARPS = GF_WARPS / BB;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t unit = static_cast<int64_t>(blockIdx.x) * WARPS + warp;
-  if (unit >= static_cast<int64_t>(args.n_tiles) * args.n_seg) return;  // whole warp; no block barrier below
+  const int row = lane & (GF_ROWS - 1), half = lane / GF_ROWS;  // this lane: points 16 half .. 16 half + 15 of each block
+  const int64_t unit = static_cast<int64_t>(blockIdx.x) * GF_WARPS + warp;
+  if (unit >= static_cast<int64_t>(args.rows / GF_ROWS) * args.n_seg) return;  // whole warp; no block barrier below
   const int tile = static_cast<int>(unit / args.n_seg), seg = static_cast<int>(unit % args.n_seg);
   const int kb0 = seg * args.kb_per_seg, kb1 = min(args.n_kb, kb0 + args.kb_per_seg);
   const uint32_t buf = smem_u32(smem) + warp * WARP_BYTES;
 
-  // coefficients of this lane's outer point (rows past the chunk repeat its last point)
-  const int64_t il = static_cast<int64_t>(tile) * 32 + lane;
-  const int64_t ig = args.i0 + (il < args.n_i ? il : args.n_i - 1);
+  const int row0 = tile * GF_ROWS;
   float pc[PT_COEF];
   float nc[NNUC * NUC_COEF];
-  const double gx = args.grid[3 * ig], gy = args.grid[3 * ig + 1], gz = args.grid[3 * ig + 2];
-  point_coefs_fixed<float, NNUC>(*args.jp, gx, gy, gz, static_cast<double>(args.g_scale), pc, nc);
-  // low parts of the outer coordinates (the pair difference is taken in hi/lo FP32)
-  const float xl = static_cast<float>(gx - static_cast<double>(pc[0]));
-  const float yl = static_cast<float>(gy - static_cast<double>(pc[1]));
-  const float zl = static_cast<float>(gz - static_cast<double>(pc[2]));
+  const float* cf0 = args.coef + row0 + row;
+#pragma unroll
+  for (int k = 0; k < PT_COEF; ++k) pc[k] = __ldg(cf0 + k * args.rows);
+  const float xl = __ldg(cf0 + (PT_COEF + 0) * args.rows), yl = __ldg(cf0 + (PT_COEF + 1) * args.rows),
+              zl = __ldg(cf0 + (PT_COEF + 2) * args.rows);
+#pragma unroll
+  for (int k = 0; k < NNUC * NUC_COEF; ++k) nc[k] = __ldg(cf0 + (PT_COEF + 3 + k) * args.rows);
   // the same constants duplicated in both halves of a packed pair (paired FP32 path, <= 2 nuclei)
   f32x2 PC[NNUC <= 2 ? PT_COEF : 1], NC[NNUC <= 2 ? NNUC * NUC_COEF : 1], XL = 0, YL = 0, ZL = 0;
   if constexpr (NNUC <= 2) {
@@ -91,7 +125,6 @@ __global__ void __launch_bounds__(GF_THREADS)
     YL = pk2(yl, yl);
     ZL = pk2(zl, zl);
   }
-  const int row0 = tile * 32;
   constexpr int NQ = PARTS == 2 ? BB / RB : 1;   // exact ranges staged together
   float gmax[NQ][3];                   // fp16: largest |G| of each range per component
 #pragma unroll
@@ -106,7 +139,8 @@ __global__ void __launch_bounds__(GF_THREADS)
     // 16 records of two inner points each (the pair-interleaved table written by launch_jtab)
     const float* blk = args.jtab + static_cast<int64_t>(kb) * VF_BK * JS;
 #pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
+    for (int c2 = 0; c2 < 2; ++c2) {
+      const int c = 2 * half + c2;   // points 8c .. 8c + 7 of the block
       float gv[3][8];
 #pragma unroll
       for (int v2 = 0; v2 < 4; ++v2) {
@@ -198,16 +232,16 @@ __global__ void __launch_bounds__(GF_THREADS)
         }
       }
       // the previous range's tiles must have been read by their TMA stores before they are overwritten
-      if (c == 0 && rb == 0 && kr > kb0) {
+      if (c2 == 0 && rb == 0 && kr > kb0) {
         if (lane == 0) bulk_wait_read_all();
         __syncwarp();
       }
       if constexpr (PARTS == 2) {
-        // FP32 staging in the lane's own 128-byte rows of the pair's component tiles: points 8c .. 8c + 7 in
+        // FP32 staging in the row's 128-byte rows of the pair's component tiles: points 8c .. 8c + 7 in
         // the hi tile for even c, the lo tile for odd c, 16-byte chunks b and b + 1 with b = 4 (rb % 2) +
-        // 2 (c / 2), so that the split below rewrites, for each half of the block, exactly the chunks
-        // it has read; and the range maxima
-        const int b = (rb & 1) * 4 + (c >> 1) * 2;
+        // 2 half, so that the split below rewrites, for the lane's half of the block, exactly the chunks
+        // that the lane itself has written and read; and the range maxima
+        const int b = (rb & 1) * 4 + half * 2;
 #pragma unroll
         for (int x = 0; x < 3; ++x) {
           float m = 0.0f;
@@ -216,10 +250,10 @@ __global__ void __launch_bounds__(GF_THREADS)
 #pragma unroll
           for (int v = 0; v < NQ; ++v)
             if (NQ == 1 || rb == v) gmax[v][x] = fmaxf(gmax[v][x], m);
-          const uint32_t row = bbuf + (2 * x + (c & 1)) * 2 * GF_TILE;
-          st_shared_v4(row + sw128_offset(lane, b), __float_as_uint(gv[x][0]), __float_as_uint(gv[x][1]),
+          const uint32_t trow = bbuf + (2 * x + c2) * 2 * GF_TILE;
+          st_shared_v4(trow + sw128_offset(row, b), __float_as_uint(gv[x][0]), __float_as_uint(gv[x][1]),
                        __float_as_uint(gv[x][2]), __float_as_uint(gv[x][3]));
-          st_shared_v4(row + sw128_offset(lane, b + 1), __float_as_uint(gv[x][4]), __float_as_uint(gv[x][5]),
+          st_shared_v4(trow + sw128_offset(row, b + 1), __float_as_uint(gv[x][4]), __float_as_uint(gv[x][5]),
                        __float_as_uint(gv[x][6]), __float_as_uint(gv[x][7]));
         }
       } else {
@@ -230,38 +264,39 @@ __global__ void __launch_bounds__(GF_THREADS)
           for (int h = 0; h < 4; ++h) split_pair<BF16>(gv[x][2 * h], gv[x][2 * h + 1], w[h]);
 #pragma unroll
           for (int p = 0; p < PARTS; ++p)
-            st_shared_v4(bbuf + (x * PARTS + p) * GF_TILE + sw64_offset(lane, c), w[0][p], w[1][p], w[2][p], w[3][p]);
+            st_shared_v4(bbuf + (x * PARTS + p) * GF_TILE + sw64_offset(row, c), w[0][p], w[1][p], w[2][p], w[3][p]);
         }
       }
     }
   }
     if constexpr (PARTS == 2) {
-      // exact split of the lane's values per component on their range's quantum: hi of points 8c .. 8c + 7 of
-      // the pair's block rb goes to chunk 4 (rb % 2) + c of the hi tile, lo to the same chunk of the lo tile
-      // (tiles of 32 rows x 128 bytes, the layout the GEMM loads)
+      // exact split of the lane's values per component on their range's quantum (the maximum over both of the
+      // row's lanes): hi of points 8c .. 8c + 7 of the pair's block rb goes to chunk 4 (rb % 2) + c of the hi tile, lo to the
+      // same chunk of the lo tile (tiles of 16 rows x 128 bytes, the layout the GEMM loads)
 #pragma unroll
       for (int x = 0; x < 3; ++x) {
 #pragma unroll
         for (int rb = 0; rb < BB; ++rb) {
+          if (NQ > 1 || rb == 0) {
+            float& m = gmax[NQ == 1 ? 0 : rb][x];
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, GF_ROWS));
+          }
           const int q = exact_quantum(gmax[NQ == 1 ? 0 : rb][x], GF_EXACT_BITS);
           const uint32_t hi = buf + (rb >> 1) * 2 * BLOCK_BYTES + 2 * x * 2 * GF_TILE, lo = hi + 2 * GF_TILE;
+          const uint32_t c0 = sw128_offset(row, 4 * (rb & 1) + 2 * half), c1 = sw128_offset(row, 4 * (rb & 1) + 2 * half + 1);
+          uint32_t f[16];
+          ld_shared_v4(hi + c0, f[0], f[1], f[2], f[3]);
+          ld_shared_v4(hi + c1, f[4], f[5], f[6], f[7]);
+          ld_shared_v4(lo + c0, f[8], f[9], f[10], f[11]);
+          ld_shared_v4(lo + c1, f[12], f[13], f[14], f[15]);
+          uint32_t w[8][2];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t c0 = sw128_offset(lane, 4 * (rb & 1) + 2 * h), c1 = sw128_offset(lane, 4 * (rb & 1) + 2 * h + 1);
-            uint32_t f[16];
-            ld_shared_v4(hi + c0, f[0], f[1], f[2], f[3]);
-            ld_shared_v4(hi + c1, f[4], f[5], f[6], f[7]);
-            ld_shared_v4(lo + c0, f[8], f[9], f[10], f[11]);
-            ld_shared_v4(lo + c1, f[12], f[13], f[14], f[15]);
-            uint32_t w[8][2];
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-              split_pair_exact(__uint_as_float(f[2 * k]), __uint_as_float(f[2 * k + 1]), q, w[k]);
-            st_shared_v4(hi + c0, w[0][0], w[1][0], w[2][0], w[3][0]);
-            st_shared_v4(hi + c1, w[4][0], w[5][0], w[6][0], w[7][0]);
-            st_shared_v4(lo + c0, w[0][1], w[1][1], w[2][1], w[3][1]);
-            st_shared_v4(lo + c1, w[4][1], w[5][1], w[6][1], w[7][1]);
-          }
+          for (int k = 0; k < 8; ++k)
+            split_pair_exact(__uint_as_float(f[2 * k]), __uint_as_float(f[2 * k + 1]), q, w[k]);
+          st_shared_v4(hi + c0, w[0][0], w[1][0], w[2][0], w[3][0]);
+          st_shared_v4(hi + c1, w[4][0], w[5][0], w[6][0], w[7][0]);
+          st_shared_v4(lo + c0, w[0][1], w[1][1], w[2][1], w[3][1]);
+          st_shared_v4(lo + c1, w[4][1], w[5][1], w[6][1], w[7][1]);
         }
       }
 #pragma unroll
@@ -293,14 +328,28 @@ __global__ void __launch_bounds__(GF_THREADS)
 }
 
 template <int PARTS, int NNUC, int RB>
-void launch_rb(const CUtensorMap* tm, const GfieldArgs& a, cudaStream_t st) {
+void launch_rb(const CUtensorMap* tm, const GfieldArgs& in, cudaStream_t st) {
   auto kern = gfield_kernel<PARTS, NNUC, RB>;
-  constexpr int warps = GF_WARPS / (PARTS == 2 && RB < 2 ? 2 : RB);
-  constexpr int smem = GF_WARPS * 3 * PARTS * GF_TILE + 1024;  // warps x staged blocks of three tiles
+  constexpr int bb = PARTS == 2 && RB < 2 ? 2 : RB;
+  constexpr int smem = GF_WARPS * bb * 3 * PARTS * GF_TILE + 1024;  // warps x staged blocks of three tiles
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  const int64_t units = static_cast<int64_t>(a.n_tiles) * a.n_seg;
-  const unsigned blocks = static_cast<unsigned>((units + warps - 1) / warps);
-  kern<<<blocks, warps * 32, smem, st>>>(*tm, a);
+  GfieldArgs a = in;
+  // Blocks per unit (a multiple of 4: whole staged groups): the length with the least (rounds of resident warps) x
+  // (blocks + 1 for the coefficients), the longest of equals.  124 blocks of 248 tiles: 16 (one round), not 32.
+  const int64_t tiles = a.rows / GF_ROWS, slots = static_cast<int64_t>(std::max(a.n_sm, 1)) * gf_ctas(NNUC) * GF_WARPS;
+  int64_t best_cost = -1;
+  for (int seg = 4; seg <= 64; seg += 4) {
+    const int64_t units = tiles * ((a.n_kb + seg - 1) / seg), cost = (units + slots - 1) / slots * (seg + 1);
+    if (best_cost < 0 || cost <= best_cost) {
+      best_cost = cost;
+      a.kb_per_seg = seg;
+    }
+  }
+  a.n_seg = (a.n_kb + a.kb_per_seg - 1) / a.kb_per_seg;
+  const int64_t units = tiles * a.n_seg;
+  const unsigned blocks = static_cast<unsigned>((units + GF_WARPS - 1) / GF_WARPS);
+  gcoef_kernel<NNUC><<<static_cast<unsigned>((a.rows + 127) / 128), 128, 0, st>>>(a);
+  kern<<<blocks, GF_WARPS * 32, smem, st>>>(*tm, a);
 }
 template <int PARTS, int NNUC>
 void launch_t(const CUtensorMap* tm, const GfieldArgs& a, cudaStream_t st) {
@@ -314,8 +363,12 @@ void launch_t(const CUtensorMap* tm, const GfieldArgs& a, cudaStream_t st) {
 
 }  // namespace
 
+size_t gfield_coef_floats(int n_nuc, int64_t rows) {
+  return static_cast<size_t>(PT_COEF + 3 + nuc_slots(n_nuc) * NUC_COEF) * rows;
+}
+
 void launch_gfield(const CUtensorMap* tm_g_store, const GfieldArgs& a, int parts, cudaStream_t st) {
-  if (a.n_tiles <= 0 || a.n_seg <= 0) return;
+  if (a.rows <= 0 || a.n_kb <= 0) return;
   if (parts == 2) {
     switch (a.n_nuc) {
       case 1: launch_t<2, 1>(tm_g_store, a, st); break;

@@ -131,6 +131,10 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
   const int64_t n_outer = outer_end - outer_begin;
   const int parts = f64 ? 0 : (cv.precision == XTC_PREC_FP16X2 ? 2 : 3);
   const int kd_b = cv.vf_kd >= 2 ? 2 : 1;  // exact range of the fp16 step (b) engine
+  // the orbitals; once rho is split, step (a)'s coefficients of the outer points
+  auto phiT_doubles = [&](int64_t gc) {
+    return std::max(static_cast<size_t>(N) * NGp, (gfield_coef_floats(n_nuc, gc) + 1) / 2);
+  };
   // bytes the layout below carves for a chunk of gc outer points (same order and rounding)
   auto need = [&](int64_t gc) {
     Carver c{nullptr};
@@ -142,7 +146,7 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
       c.take<double>(static_cast<size_t>(NGp) * NP);
       c.take<double>(static_cast<size_t>(v_slice(gc, N)));
     } else {
-      c.take<double>(static_cast<size_t>(N) * NGp);
+      c.take<double>(phiT_doubles(gc));
       c.take<float>(static_cast<size_t>(NGp) * jtab_stride(n_nuc));
       c.take<uint16_t>(static_cast<size_t>(3) * NP * NGp);
       c.take<unsigned int>(NP);
@@ -176,6 +180,7 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
   CUtensorMap tm{}, tm16{}, tm_gs{}, tm_gl{};
   double* jtab64 = nullptr;
   double* rho64 = nullptr;
+  double* phiT = nullptr;
   float* jtab = nullptr;
   void* rho = nullptr;
   int* colexp = nullptr;
@@ -187,7 +192,7 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
     launch_jtab64(grid_xyz, n_grid, NGp, cv.jp_dev, n_nuc, jtab64, st);
     launch_rho_f64(phi, weights, n_grid, NGp, N, pair_p, pair_q, rho64, st);
   } else {
-    double* phiT = cz.take<double>(static_cast<size_t>(N) * NGp);
+    phiT = cz.take<double>(phiT_doubles(gc));
     jtab = cz.take<float>(static_cast<size_t>(NGp) * jtab_stride(n_nuc));
     rho = cz.take<uint16_t>(static_cast<size_t>(3) * NP * NGp);  // fp16: split rows + fp16 plane
     unsigned int* colmax = cz.take<unsigned int>(NP);
@@ -215,7 +220,7 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
                     wide ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    if (!map(&tm, rho, NP, vf_bn(parts)) || !map(&tm_gs, G, 3 * gc, 32) || !map(&tm_gl, G, 3 * gc, VF_BM))
+    if (!map(&tm, rho, NP, vf_bn(parts)) || !map(&tm_gs, G, 3 * gc, GFIELD_ROWS) || !map(&tm_gl, G, 3 * gc, VF_BM))
       return xtc_internal_fail(ctx, XTC_ERR_CUDA, "noalloc: cuTensorMapEncodeTiled failed");
     if (wide) {
       // the fp16(rho^T) plane after the split rows: [pq][j], boxes 64 x vf_bn / 2
@@ -249,10 +254,10 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
       g.i0 = c0;
       g.n_i = n_i;
       g.gcp = gc;
-      g.n_tiles = mt_per_x * (VF_BM / 32);
+      g.rows = round_up(n_i, VF_BM);
+      g.coef = reinterpret_cast<float*>(phiT);  // read for the last time by the rho split
+      g.n_sm = cv.n_sm;
       g.n_kb = n_kb;
-      g.kb_per_seg = 32;
-      g.n_seg = (n_kb + g.kb_per_seg - 1) / g.kb_per_seg;
       g.n_nuc = n_nuc;
       g.g_scale = std::ldexp(1.0f, sg);
       g.range_blocks = kd_b;

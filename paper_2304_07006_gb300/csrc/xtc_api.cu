@@ -90,7 +90,7 @@ struct xtc_ctx {
   // device workspace
   DBuf jp_dev, err_dev, flag_dev;
   DBuf grid, w, phi, gamma, phiT, phi32, pair_p, pair_q;
-  DBuf jtab, jtab64, rho, colmax, colexp, G;
+  DBuf jtab, jtab64, rho, colmax, colexp, G, gcoef;
   DBuf V, Vacc, L, R, L32, R32, eL, eR, M, evec, lam, dU_tmp, dh_tmp, e0_tmp, vout, r1, r2;
   DBuf lamd, gamma_b, M2, M3;  // direct weights; spin builds: beta density, f^b, Delta U^{ab}
   DBuf lam2, R2, R32b, eR2;    // spin builds: beta exchange weights, R for electron-2 beta
@@ -125,7 +125,7 @@ struct xtc_ctx {
 
   std::vector<DBuf*> buffers() {
     return {&jp_dev, &err_dev, &flag_dev, &grid, &w, &phi, &gamma, &phiT, &phi32, &pair_p, &pair_q, &jtab, &jtab64,
-            &rho, &colmax, &colexp, &G, &V, &Vacc, &L, &R, &L32, &R32, &eL, &eR, &M, &evec, &lam, &dU_tmp,
+            &rho, &colmax, &colexp, &G, &gcoef, &V, &Vacc, &L, &R, &L32, &R32, &eL, &eR, &M, &evec, &lam, &dU_tmp,
             &dh_tmp, &e0_tmp, &vout, &r1, &r2, &lamd, &gamma_b, &M2, &M3, &lam2, &R2, &R32b, &eR2, &Lv, &T3,
             &h_tmp, &fc_U, &fc_h, &fc_hout, &fc_Uout, &G2, &k_dphi, &k_dphiT, &k_W, &k_S, &d_rho, &d_rhoe, &d_sj,
             &d_G, &d_Ge, &d_tmp, &d_L, &d_Le, &d_R, &d_Re};
@@ -682,6 +682,7 @@ int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* gri
   if (!ensure(ctx->V, vbytes)) return fail(ctx, XTC_ERR_OOM, "V chunk (%.2f GB)", vbytes / 1e9);
   if (!f64) {
     const size_t gbytes = 2ull * pl.parts_b * 3 * pl.gc * pl.NGp;
+    if (!ensure(ctx->gcoef, 4 * gfield_coef_floats(n_nuc, pl.gc))) return fail(ctx, XTC_ERR_OOM, "outer-point coefficients");
     if (!ensure(ctx->G, gbytes)) return fail(ctx, XTC_ERR_OOM, "gradient table (%.2f GB)", gbytes / 1e9);
     // FP64 partial sums of step (b): one 128 x vf_bn tile per CTA and split slice
     const int bn = vf_bn(pl.parts_b);
@@ -694,7 +695,7 @@ int prepare(xtc_ctx* ctx, Plan& pl, int64_t n_grid, int n_orb, const double* gri
 }
 
 // Tensor maps of the step (b) operands: rho^T (box rows vf_bn) and the gradient table, as stored by
-// step (a) (box rows 32) and as loaded by the GEMM (box rows 128).  fp16: 128-byte runs of 64 values
+// step (a) (box rows GFIELD_ROWS) and as loaded by the GEMM (box rows 128).  fp16: 128-byte runs of 64 values
 // of one part (rows of 2 NGp values, boxes 64 wide, 128-byte swizzle); bf16: one
 // plane per part (rows of NGp values, boxes 32 wide, 64-byte swizzle).
 struct VfMaps {
@@ -711,7 +712,7 @@ int make_vfield_maps(xtc_ctx* ctx, const Plan& pl, VfMaps& m) {
   if (wide && (rc = make_tmap_3d(ctx, &m.rho16, ctx->rho.as<uint16_t>() + 2 * pl.NP * pl.NGp, false, pl.NGp, pl.NP, 1,
                                  2 * VF_BK, vf_bn(2) / 2, true)))
     return rc;
-  if ((rc = make_tmap_3d(ctx, &m.g_store, ctx->G.p, bf, cols, 3 * pl.gc, planes, bk, 32, wide))) return rc;
+  if ((rc = make_tmap_3d(ctx, &m.g_store, ctx->G.p, bf, cols, 3 * pl.gc, planes, bk, GFIELD_ROWS, wide))) return rc;
   return make_tmap_3d(ctx, &m.g_load, ctx->G.p, bf, cols, 3 * pl.gc, planes, bk, VF_BM, wide);
 }
 
@@ -726,7 +727,6 @@ int gradient_scale(const xtc_ctx* ctx, const Plan& pl) {
 void run_grad(xtc_ctx* ctx, const Plan& pl, const double* d_grid, int64_t i0, int64_t n_i, const VfMaps& maps,
               cudaStream_t st) {
   const int n_kb = static_cast<int>(pl.NGp / VF_BK);
-  const int mt_per_x = static_cast<int>((n_i + VF_BM - 1) / VF_BM);
   GfieldArgs g{};
   g.grid = d_grid;
   g.jp = ctx->jp_dev.as<JastrowParams>();
@@ -734,14 +734,14 @@ void run_grad(xtc_ctx* ctx, const Plan& pl, const double* d_grid, int64_t i0, in
   g.i0 = i0;
   g.n_i = n_i;
   g.gcp = pl.gc;
-  g.n_tiles = mt_per_x * (VF_BM / 32);
+  g.rows = round_up(n_i, VF_BM);
+  g.coef = ctx->gcoef.as<float>();
+  g.n_sm = ctx->n_sm;
   g.n_kb = n_kb;
-  g.kb_per_seg = 32;
-  g.n_seg = (n_kb + g.kb_per_seg - 1) / g.kb_per_seg;
   g.n_nuc = ctx->jp.n_nuc;
   g.g_scale = std::ldexp(1.0f, gradient_scale(ctx, pl));
   g.range_blocks = f16_range_b(ctx->vf_kd);
-  timed(ctx, XTC_K_GRAD, 1, [&] { launch_gfield(&maps.g_store, g, pl.parts_b, st); }, st);
+  timed(ctx, XTC_K_GRAD, 2, [&] { launch_gfield(&maps.g_store, g, pl.parts_b, st); }, st);
 }
 
 // Step (b) for outer points [i0, i0 + n_i) from the gradient table behind `maps`, into ctx->V.
@@ -1002,7 +1002,7 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
     }
     if (pipe) {
       const uint64_t cols = 2 * pl.NGp;
-      if ((rc = make_tmap_3d(ctx, &maps2.g_store, ctx->G2.p, false, cols, 3 * pl.gc, 1, 2 * VF_BK, 32, true))) return rc;
+      if ((rc = make_tmap_3d(ctx, &maps2.g_store, ctx->G2.p, false, cols, 3 * pl.gc, 1, 2 * VF_BK, GFIELD_ROWS, true))) return rc;
       if ((rc = make_tmap_3d(ctx, &maps2.g_load, ctx->G2.p, false, cols, 3 * pl.gc, 1, 2 * VF_BK, VF_BM, true)))
         return rc;
     }

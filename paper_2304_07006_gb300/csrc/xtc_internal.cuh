@@ -140,12 +140,18 @@ struct GfieldArgs {
   const float* jtab;           // pair-interleaved inner-point table (launch_jtab, 12 floats per point)
   int64_t i0, n_i;             // outer range of this chunk
   int64_t gcp;                 // padded chunk length (rows per component)
-  int n_tiles;                 // 32-row outer tiles to write (multiple of 4)
-  int n_kb, kb_per_seg, n_seg; // inner K-blocks (32 points), K-blocks per warp unit, units along K
+  int64_t rows;                // rows to write per component: n_i rounded up to 128
+  float* coef;                 // workspace: gfield_coef_floats(n_nuc, rows)
+  int n_sm;
+  int n_kb;                    // inner K-blocks (32 points, a multiple of 4)
+  int kb_per_seg, n_seg;       // K-blocks per warp unit, units along K (set by the launcher)
   int n_nuc;
   float g_scale;               // 2^sG folded into the gradient
   int range_blocks;            // fp16: K-blocks per exact range of the step (b) GEMM (1 or 2)
 };
+constexpr int GFIELD_ROWS = 16;  // box rows of tm_g_store
+size_t gfield_coef_floats(int n_nuc, int64_t rows);
+// Two kernels: the outer points' coefficients, then the table.
 void launch_gfield(const CUtensorMap* tm_g_store, const GfieldArgs& a, int parts, cudaStream_t st);
 
 // Step (b), tensor cores.  V[z][pq][x][il] (FP32, il = i - i0 < gcp) for the outer points of the
