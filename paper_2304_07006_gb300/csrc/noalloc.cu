@@ -220,7 +220,7 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
                     wide ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    if (!map(&tm, rho, NP, vf_bn(parts)) || !map(&tm_gs, G, 3 * gc, GFIELD_ROWS) || !map(&tm_gl, G, 3 * gc, VF_BM))
+    if (!map(&tm, rho, NP, wide ? vf_bn(2) : vf_bn(3) / 2) || !map(&tm_gs, G, 3 * gc, GFIELD_ROWS) || !map(&tm_gl, G, 3 * gc, VF_BM))
       return xtc_internal_fail(ctx, XTC_ERR_CUDA, "noalloc: cuTensorMapEncodeTiled failed");
     if (wide) {
       // the fp16(rho^T) plane after the split rows: [pq][j], boxes 64 x vf_bn / 2

@@ -208,14 +208,15 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 }
 // The issuing warp runs its loop with all lanes (uniform control flow, so that descriptors stay in uniform
 // registers) and these let one elected lane, always the same one, issue.
-// D[tmem] += A[smem] * B[smem]^T over the pair.
-__device__ __forceinline__ void tc_mma_f16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
+// D[tmem] (+)= A[smem] * B[smem]^T over the pair.
+__device__ __forceinline__ void tc_mma_f16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                uint32_t accumulate = 1u) {
   asm volatile(
       "{\n\t.reg .pred p, e;\n\t"
-      "setp.ne.b32 p, 1, 0;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
       "elect.sync _|e, 0xffffffff;\n\t"
       "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc)
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // Arrives on the barrier at this offset in both CTAs once every MMA issued so far has completed.

@@ -377,138 +377,145 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(XB_THREADS, 1)
 }
 
 // =================================================================== bf16 x3 engine (step (b))
+// CTA pairs share a 256 x 160 tile (tcgen05 cta_group::2): each CTA loads its 128 rows of A and 80 of B's
+// columns.  One CTA per 128 x 160 tile was bound by shared memory: per 64 values of K the 24 MMAs read 216 KB and the
+// loads wrote 108 KB, 2,531 cycles at 128 bytes a clock (3,360 measured) for 1,920 of tensor pipe; a pair's
+// CTA reads 156 KB and writes 78 KB, 1,828 (2,410 measured).  Step (b) of a water-sized build (40,000 points, 58
+// orbitals, one GB300): 71.6 -> 51.4 ms.
 constexpr int BF_BN = 160;
 constexpr int BF_HC = BF_BN / 2;
 constexpr int BF_PARTS = 3;
 constexpr int BF_A_TILE = VF_BM * 64;             // bytes per part of an A tile (128 rows of 64 B)
-constexpr int BF_B_TILE = BF_BN * 64;
-constexpr int BF_A_BYTES = BF_PARTS * BF_A_TILE;
-constexpr int BF_B_BYTES = BF_PARTS * BF_B_TILE;
-constexpr int BF_STAGE = ((BF_A_BYTES + BF_B_BYTES + 1023) / 1024) * 1024;
-constexpr int BF_STAGES = 4;
-constexpr int BF_MMA_WARPS = 2;                   // issuers of the even / odd ranges
-constexpr int BF_THREADS = (1 + BF_MMA_WARPS + DRAIN_WARPS) * 32;
+constexpr int BF_B_TILE = BF_BN / 2 * 64;         // bytes per part of a CTA's half of the B tile
+constexpr int BF_STAGE = BF_PARTS * (BF_A_TILE + BF_B_TILE);
+constexpr int BF_STAGES = 5;
+constexpr int BF_THREADS = (2 + DRAIN_WARPS) * 32;
 constexpr int BF_SMEM = BF_STAGES * BF_STAGE + 1024 + 256;
 static_assert(BF_BN == vf_bn(3), "tile width of the bf16 engine");
+static_assert(BF_STAGE % 1024 == 0 && BF_B_TILE % 512 == 0, "swizzle atoms");
 static_assert(BF_SMEM <= 232448, "shared memory per CTA");
 static_assert(NRB > BF_STAGES, "range barriers");
 static_assert(2 * BF_BN <= 512 && BF_BN % 32 == 0, "two accumulators, drain halves of 16-column chunks");
 
-__global__ void __launch_bounds__(BF_THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(BF_THREADS, 1)
     vfield_bf16_kernel(const __grid_constant__ CUtensorMap tm_g, const __grid_constant__ CUtensorMap tm_rho,
                        const VfieldArgs args) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + BF_STAGES * BF_STAGE);
-  uint64_t* tma_full = bars;                  // [BF_STAGES] the stage's loads landed
-  uint64_t* rdone = bars + BF_STAGES;         // [NRB] the MMAs of range r (r % NRB) completed
-  uint64_t* d_free = bars + BF_STAGES + NRB;  // [2] the drains released accumulator b
-  uint64_t* fin_bar = bars + BF_STAGES + NRB + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + BF_STAGES + NRB + 3);
+  uint64_t* full = bars;                      // [BF_STAGES] leader: the stage's loads of both CTAs landed
+  uint64_t* rdone = full + BF_STAGES;         // [NRB] the MMAs of range r (r % NRB) completed
+  uint64_t* d_free = rdone + NRB;             // [2] leader: the drains of both CTAs released accumulator b
+  uint64_t* fin_bar = d_free + 2;             // leader: every MMA completed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const TileXY t = grouped_tile(args.cta0 + blockIdx.x, 3 * args.mt_per_x, args.n_tiles);
-  const int x = t.m_tile / args.mt_per_x;
-  const int ib = (t.m_tile - x * args.mt_per_x) * VF_BM;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp: uniform
+  const uint32_t rank = cluster_rank();
+  const int m_tiles = 3 * args.mt_per_x;
+  const TileXY t = pair_tile(args.cta0 + blockIdx.x, m_tiles, args.n_tiles);
+  const bool valid = t.m_tile < m_tiles;          // a tile that does not exist repeats the last one's rows
+  const int m_tile = valid ? t.m_tile : m_tiles - 1;
+  const int x = m_tile / args.mt_per_x;
+  const int ib = (m_tile - x * args.mt_per_x) * VF_BM;
   const int row0 = static_cast<int>(x * args.gcp) + ib;
   const int split = blockIdx.y;
   const int kb0 = split * args.kb_per_split;
-  const int kb1 = min(args.n_kb, kb0 + args.kb_per_split);
-  const int n_it = kb1 - kb0;
+  const int n_it = min(args.n_kb, kb0 + args.kb_per_split) - kb0;
   const int kd = args.kd;
   const int n_ranges = (n_it + kd - 1) / kd;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < BF_STAGES; ++s) mbar_init(&tma_full[s], 1);
+    for (int s = 0; s < BF_STAGES; ++s) mbar_init(&full[s], 1);
     for (int r = 0; r < NRB; ++r) mbar_init(&rdone[r], 1);
-    for (int b = 0; b < 2; ++b) mbar_init(&d_free[b], DRAIN_WARPS);
-    mbar_init(fin_bar, BF_MMA_WARPS);
+    for (int b = 0; b < 2; ++b) mbar_init(&d_free[b], 2 * DRAIN_WARPS);
+    mbar_init(fin_bar, 1);
     *abort_flag = 0;
     fence_mbar_init();
     tma_prefetch_desc(&tm_g);
     tma_prefetch_desc(&tm_rho);
   }
-  if (warp == 0) {
-    tmem_alloc(tmem_slot, 512);
-    tmem_relinquish();
-  }
+  if (warp == 0) tmem_alloc_pair(tmem_slot, 512);
   tc_fence_before();
   __syncthreads();
+  cluster_sync();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const uint32_t smem_base = smem_u32(smem);
 
   if (warp == 0) {
     if (lane == 0) {
-      // ---------------------------------------------------------------- TMA producer
+      // ---------------------------------------------------------------- TMA producer (both CTAs)
       int seen = 0;  // ranges known to have completed (their slots are free again)
-      int issued_end = kb0;
-      for (int kb = kb0; kb < kb1; ++kb) {
-        const int it = kb - kb0, s = it % BF_STAGES;
+      bool ok = true;
+      const int n0 = t.n_tile * BF_BN + static_cast<int>(rank) * (BF_BN / 2);
+      for (int it = 0; it < n_it && ok; ++it) {
+        const int s = it % BF_STAGES;
         if (it >= BF_STAGES) {
           const int need = (it - BF_STAGES) / kd;  // range holding the slot's previous stage
-          bool ok = true;
           for (; seen <= need && ok; ++seen)
             ok = mbar_wait(&rdone[seen % NRB], (seen / NRB) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
           if (!ok) break;
         }
-        mbar_arrive_expect_tx(&tma_full[s], BF_A_BYTES + BF_B_BYTES);
+        if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * BF_STAGE);
+        const uint32_t bar = cluster_addr(&full[s], 0);
         uint8_t* st = smem + s * BF_STAGE;
         for (int p = 0; p < BF_PARTS; ++p) {
-          tma_load_3d(st + p * BF_A_TILE, &tm_g, &tma_full[s], kb * VF_BK, row0, p);
-          tma_load_3d(st + BF_A_BYTES + p * BF_B_TILE, &tm_rho, &tma_full[s], kb * VF_BK, t.n_tile * BF_BN, p);
+          tma_load_3d_pair(st + p * BF_A_TILE, &tm_g, bar, (kb0 + it) * VF_BK, row0, p);
+          tma_load_3d_pair(st + BF_PARTS * BF_A_TILE + p * BF_B_TILE, &tm_rho, bar, (kb0 + it) * VF_BK, n0, p);
         }
-        issued_end = kb + 1;
       }
-      int zero = 0;
-      for (int kb = max(kb0, issued_end - BF_STAGES); kb < issued_end; ++kb) {
-        const int it = kb - kb0;
-        mbar_wait(&tma_full[it % BF_STAGES], (it / BF_STAGES) & 1, reinterpret_cast<volatile int*>(&zero), args.err,
-                  DEV_ERR_TIMEOUT_VF);
+      // Every range completes before the CTA exits, so every copy has landed and every arrival on this CTA's
+      // barriers has been made.  After an abort: a time no copy takes.
+      for (; ok && seen < n_ranges; ++seen)
+        ok = mbar_wait(&rdone[seen % NRB], (seen / NRB) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
+      if (!ok || *abort_flag) {
+        const unsigned long long t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 50000000ull) {
+        }
       }
     }
-  } else if (warp == 1 || warp == 2 + DRAIN_WARPS) {
-    if (lane == 0) {
-      // ---------------------------------------------------------------- MMA issuers
+  } else if (warp == 1) {
+    if (rank == 0) {
+      // ---------------------------------------------------------------- MMA issuer (leader)
       // A range of kd stages goes into one TMEM accumulator: first the cross products of each
       // stage as it lands (the accumulator is still small), then the hi x hi product of every
-      // stage; one commit per range.  Warp 1 issues the even ranges (accumulator 0), the last warp
-      // the odd ones (accumulator 1).
-      constexpr uint32_t idesc = idesc_f16(VF_BM, BF_BN, true);
+      // stage; one commit per range.  The even and odd ranges alternate between two accumulators.
+      constexpr uint32_t idesc = idesc_f16(2 * VF_BM, BF_BN, true);
       constexpr int pa_of[5] = {1, 0, 2, 0, 1};   // (A part, B part) of the products before hi x hi
       constexpr int pb_of[5] = {1, 2, 0, 1, 0};
+      const uint32_t rdone_bar = smem_u32(rdone);
+      const uint64_t desc0 = sdesc_kmajor_sw64(0);
       bool alive = true;
-      for (int r = warp == 1 ? 0 : 1; r < n_ranges && alive; r += BF_MMA_WARPS) {
+      for (int r = 0; r < n_ranges && alive; ++r) {
         const int it0 = r * kd, it1 = min(n_it, it0 + kd);
         const int b = r & 1, u = r >> 1;
         const uint32_t d_tmem = tmem + b * BF_BN;
-        if (u >= 1 && !mbar_wait(&d_free[b], (u - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF)) break;
+        if (u >= 1 && !mbar_spin(&d_free[b], (u - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF)) break;
         for (int it = it0; it < it1; ++it) {
           const int s = it % BF_STAGES;
-          if (!(alive = mbar_wait(&tma_full[s], (it / BF_STAGES) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF))) break;
+          if (!(alive = mbar_spin(&full[s], (it / BF_STAGES) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF))) break;
           tc_fence_after();
-          const uint32_t sa = smem_base + s * BF_STAGE;
-          const uint32_t sb = sa + BF_A_BYTES;
+          const uint64_t sa = desc0 + ((smem_base + s * BF_STAGE) >> 4);
+          const uint64_t sb = sa + (BF_PARTS * BF_A_TILE >> 4);
 #pragma unroll
           for (int p = 0; p < 5; ++p)
 #pragma unroll
             for (int ks = 0; ks < 2; ++ks)
-              tc_mma_f16(d_tmem, sdesc_kmajor_sw64(sa + pa_of[p] * BF_A_TILE + ks * 32),
-                         sdesc_kmajor_sw64(sb + pb_of[p] * BF_B_TILE + ks * 32), idesc,
-                         (it == it0 && p == 0 && ks == 0) ? 0u : 1u);
+              tc_mma_f16_pair(d_tmem, sa + ((pa_of[p] * BF_A_TILE + ks * 32) >> 4),
+                              sb + ((pb_of[p] * BF_B_TILE + ks * 32) >> 4), idesc,
+                              it == it0 && p == 0 && ks == 0 ? 0u : 1u);
         }
         if (!alive) break;
         for (int it = it0; it < it1; ++it) {
-          const uint32_t sa = smem_base + (it % BF_STAGES) * BF_STAGE;
-          const uint32_t sb = sa + BF_A_BYTES;
+          const uint64_t sa = desc0 + ((smem_base + (it % BF_STAGES) * BF_STAGE) >> 4);
+          const uint64_t sb = sa + (BF_PARTS * BF_A_TILE >> 4);
 #pragma unroll
-          for (int ks = 0; ks < 2; ++ks)
-            tc_mma_f16(d_tmem, sdesc_kmajor_sw64(sa + ks * 32), sdesc_kmajor_sw64(sb + ks * 32), idesc, 1u);
+          for (int ks = 0; ks < 2; ++ks) tc_mma_f16_pair(d_tmem, sa + 2 * ks, sb + 2 * ks, idesc);
         }
-        tc_commit(&rdone[r % NRB]);
+        tc_commit_pair(rdone_bar + 8 * (r % NRB));
       }
-      tc_commit(fin_bar);
+      tc_commit_pair_local(smem_u32(fin_bar));
       int zero = 0;
       mbar_wait(fin_bar, 0, reinterpret_cast<volatile int*>(&zero), args.err, DEV_ERR_TIMEOUT_VF);
     }
@@ -518,6 +525,7 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
     const int half = (warp - 2) >> 2;
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     const uint32_t c_base = static_cast<uint32_t>(half * BF_HC);
+    const uint32_t free_bar = cluster_addr(&d_free[0], 0);
     float S[BF_HC];
 #pragma unroll
     for (int k = 0; k < BF_HC; ++k) S[k] = 0.0f;
@@ -525,23 +533,25 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
     auto flush_sums = [&]() {
       double* acc = args.Vacc + (static_cast<int64_t>(split) * args.n_cta + args.cta0 + blockIdx.x) * VF_BM * BF_BN +
                     static_cast<int64_t>(c_base) * VF_BM + quarter * 32 + lane;
-      if (nflush == 0) {
+      if (valid) {
+        if (nflush == 0) {
 #pragma unroll
-        for (int k = 0; k < BF_HC; ++k) acc[k * VF_BM] = static_cast<double>(S[k]);
-      } else {
+          for (int k = 0; k < BF_HC; ++k) acc[k * VF_BM] = static_cast<double>(S[k]);
+        } else {
 #pragma unroll
-        for (int k = 0; k < BF_HC; ++k) red_add_f64(acc + k * VF_BM, static_cast<double>(S[k]));
+          for (int k = 0; k < BF_HC; ++k) red_add_f64(acc + k * VF_BM, static_cast<double>(S[k]));
+        }
       }
 #pragma unroll
       for (int k = 0; k < BF_HC; ++k) S[k] = 0.0f;
       ++nflush;
     };
     bool ok = true;
-    for (int r = 0; r < n_ranges && ok; ++r) {
+    for (int r = 0; r < n_ranges; ++r) {
       const int b = r & 1;
-      ok = __all_sync(0xffffffffu,
-                      mbar_wait(&rdone[r % NRB], (r / NRB) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF));
-      __syncwarp();
+      // one lane waits, suspended: the board's power is better spent on the MMAs
+      if (lane == 0) ok = mbar_wait(&rdone[r % NRB], (r / NRB) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) break;
       tc_fence_after();
       const uint32_t src = tmem + lane_base + b * BF_BN + c_base;
@@ -550,12 +560,14 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
         uint32_t d0[16];
         tmem_ld_x16(src + c, d0);
         tmem_wait_ld();
+        if (c + 16 == BF_HC) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(free_bar + 8 * b);
+        }
 #pragma unroll
         for (int k = 0; k < 16; ++k) S[c + k] += __uint_as_float(d0[k]);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&d_free[b]);
       if (args.flush > 0 && (r + 1) % args.flush == 0) flush_sums();
     }
     if (args.flush > 0) {
@@ -564,7 +576,7 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
       const int row = quarter * 32 + lane;
       const int64_t il = static_cast<int64_t>(ib) + row;
       const int pq0 = t.n_tile * BF_BN + static_cast<int>(c_base);
-      if (ok && !*abort_flag && il < args.n_i && n_it > 0) {
+      if (ok && valid && !*abort_flag && il < args.n_i && n_it > 0) {
         float* Vz = args.V + split * v_slice(args.gcp, args.n_orb);
 #pragma unroll
         for (int k = 0; k < BF_HC; ++k) {
@@ -582,10 +594,11 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
 
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // the pair's MMAs, loads and remote arrivals are done
   if (warp == 0) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc_pair(tmem, 512);
   }
 }
 
@@ -596,7 +609,7 @@ constexpr int FIN_COLS = 32;
 template <int BN>
 __global__ void __launch_bounds__(VF_BM) vfield_finalize_kernel(const VfieldArgs args) {
   const int m_tiles = 3 * args.mt_per_x;
-  const TileXY t = BN == XB_BN ? pair_tile(blockIdx.x, m_tiles, args.n_tiles) : grouped_tile(blockIdx.x, m_tiles, args.n_tiles);
+  const TileXY t = pair_tile(blockIdx.x, m_tiles, args.n_tiles);
   if (t.m_tile >= m_tiles) return;
   const int x = t.m_tile / args.mt_per_x;
   const int row = threadIdx.x;
@@ -648,10 +661,10 @@ __global__ void __launch_bounds__(VF_BM) assemble_finalize_kernel(const VfieldAr
   }
 }
 
-// CTAs along x: the fp16 engine's tiles come in pairs of row tiles.
-unsigned tile_ctas(const VfieldArgs& a, int parts) {
+// CTAs along x: tiles come in pairs of row tiles.
+unsigned tile_ctas(const VfieldArgs& a) {
   const int m = a.mode == 0 ? 3 * a.mt_per_x : (a.rows_a + VF_BM - 1) / VF_BM;
-  return static_cast<unsigned>((parts == 2 ? (m + 1) / 2 * 2 : m) * a.n_tiles);
+  return static_cast<unsigned>((m + 1) / 2 * 2 * a.n_tiles);
 }
 
 // CTAs per launch of a GEMM of n CTAs along x.  The CTAs resident at one time stream the same panels of A and
@@ -678,7 +691,7 @@ int launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const C
                      const VfieldArgs& a, int parts, int splits, cudaStream_t st) {
   if (a.n_tiles <= 0 || splits <= 0) return 0;
   if (a.mode == 1 ? a.rows_a <= 0 : a.mt_per_x <= 0) return 0;
-  dim3 grid(tile_ctas(a, parts), static_cast<unsigned>(splits));
+  dim3 grid(tile_ctas(a), static_cast<unsigned>(splits));
   VfieldArgs w = a;
   w.n_cta = static_cast<int>(grid.x);
   const int step = launch_ctas(a, w.n_cta, splits);
@@ -702,7 +715,7 @@ int launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const C
 void launch_vfield_tc_finalize(const VfieldArgs& a, int parts, int splits, cudaStream_t st) {
   if (a.n_tiles <= 0 || splits <= 0 || a.flush <= 0) return;
   if (a.mode == 1 ? a.rows_a <= 0 : a.mt_per_x <= 0) return;
-  dim3 grid(tile_ctas(a, parts), static_cast<unsigned>(splits));
+  dim3 grid(tile_ctas(a), static_cast<unsigned>(splits));
   grid.z = (parts == 2 ? XB_BN : BF_BN) / FIN_COLS;
   if (a.mode == 1)
     assemble_finalize_kernel<XB_BN><<<grid, VF_BM, 0, st>>>(a);

@@ -707,7 +707,9 @@ int make_vfield_maps(xtc_ctx* ctx, const Plan& pl, VfMaps& m) {
   const uint64_t cols = wide ? 2 * pl.NGp : pl.NGp, planes = wide ? 1 : pl.parts_b;
   const uint32_t bk = wide ? 2 * VF_BK : VF_BK;
   int rc;
-  if ((rc = make_tmap_3d(ctx, &m.rho, ctx->rho.p, bf, cols, pl.NP, planes, bk, vf_bn(pl.parts_b), wide))) return rc;
+  if ((rc = make_tmap_3d(ctx, &m.rho, ctx->rho.p, bf, cols, pl.NP, planes, bk,
+                         wide ? vf_bn(2) : vf_bn(3) / 2, wide)))
+    return rc;
   // fp16: the plane of fp16(rho^T) after the split rows, boxes of 64 values x half a column tile
   if (wide && (rc = make_tmap_3d(ctx, &m.rho16, ctx->rho.as<uint16_t>() + 2 * pl.NP * pl.NGp, false, pl.NGp, pl.NP, 1,
                                  2 * VF_BK, vf_bn(2) / 2, true)))
