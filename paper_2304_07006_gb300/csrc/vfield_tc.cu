@@ -150,7 +150,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(XB_THREADS, 1)
   const int row0 = MODE == 0 ? static_cast<int>(x * args.gcp) + ib : ib;
   const int split = blockIdx.y;
   const int kb0 = split * args.kb_per_split;               // multiple of 2 and of kd
-  const int n_it = min(args.n_kb, kb0 + args.kb_per_split) - kb0;  // blocks of 32 K values, even
+  // MODE 1: slices of the chain, each but the last running XB_HC ranges into the next one (chain_slices)
+  const int kb_over = MODE == 1 && args.slices > 1 ? XB_HC * args.kd : 0;
+  const int n_it = min(args.n_kb, kb0 + args.kb_per_split + kb_over) - kb0;  // blocks of 32 K values, even
   const int n_st = (n_it + 1) >> 1;                        // stages
   const int kd = args.kd;                                  // blocks per exact range (1, 2 or 4)
   const int n_ranges = (n_it + kd - 1) / kd;
@@ -301,6 +303,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(XB_THREADS, 1)
           S[k] = 0.0f;
         }
     };
+    // A later slice of the chain starts where column 0 was flushed: column c's sums up to range c belong to the
+    // slice before, and its first flush is at range flush + c.
+    const int first = MODE == 1 && split > 0 ? args.flush : 0;
+    const bool last = MODE == 0 || split + 1 >= args.slices;
     bool ok = true;
     for (int r = 0; r < n_ranges && ok; ++r) {
       const int k = r & 1, u = r >> 1;
@@ -331,15 +337,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(XB_THREADS, 1)
       // the sums and the staggered FP64 flush (the accumulators are already handed back to the MMAs)
 #pragma unroll
       for (int c = 0; c < XB_HC; ++c) S[c] += __uint_as_float(d[c]);
-      if (valid && args.flush > 0 && r % args.flush < XB_HC) flush_col(r % args.flush, r < args.flush);
+      if (valid && args.flush > 0 && r % args.flush < XB_HC) {
+        if (MODE == 1 && r < first) {
+#pragma unroll
+          for (int c = 0; c < XB_HC; ++c)
+            if (c == r) S[c] = 0.0f;
+        } else {
+          flush_col(r % args.flush, r < first + args.flush);
+        }
+      }
     }
-    if (args.flush > 0) {
+    if (MODE == 1 && !last) {
+      // what is left belongs to the next slice
+    } else if (args.flush > 0) {
       // the remaining sums join the FP64 accumulator (columns never flushed in the loop are
       // stored); a finalize kernel writes V (mode 0) or adds the tile into M (mode 1)
       if (ok && valid) {
 #pragma unroll
         for (int c = 0; c < XB_HC; ++c) {
-          if (c < min(n_ranges, args.flush))
+          if (c < min(n_ranges - first, args.flush))
             red_add_f64(acc + c * VF_BM, static_cast<double>(S[c]));
           else
             acc[c * VF_BM] = static_cast<double>(S[c]);
@@ -639,14 +655,25 @@ __global__ void __launch_bounds__(VF_BM) assemble_finalize_kernel(const VfieldAr
   const int m_tiles = (args.rows_a + VF_BM - 1) / VF_BM;
   const TileXY t = pair_tile(blockIdx.x, m_tiles, args.n_tiles);
   if (t.m_tile >= m_tiles) return;
-  const double* acc = args.Vacc + (static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x) * VF_BM * BN;
+  const double* acc = args.Vacc + static_cast<int64_t>(blockIdx.x) * VF_BM * BN;
+  const int64_t slice = static_cast<int64_t>(gridDim.x) * VF_BM * BN;
   const int ncol = min(BN, args.n_pair - t.n_tile * BN);
   const int row0 = t.m_tile * VF_BM, col0 = t.n_tile * BN;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c0 = blockIdx.z * FIN_COLS;
-#pragma unroll 8
-  for (int c = 0; c < 32; ++c)
-    slab[c][threadIdx.x] = c0 + c < ncol ? acc[static_cast<int64_t>(c0 + c) * VF_BM + threadIdx.x] : 0.0;
+#pragma unroll
+  for (int c = 0; c < 32; c += 8) {
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      v[k] = c0 + c + k < ncol ? acc[static_cast<int64_t>(c0 + c + k) * VF_BM + threadIdx.x] : 0.0;
+    for (int z = 1; z < args.slices; ++z)
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (c0 + c + k < ncol) v[k] += acc[z * slice + static_cast<int64_t>(c0 + c + k) * VF_BM + threadIdx.x];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) slab[c + k][threadIdx.x] = v[k];
+  }
   __syncthreads();
   const int c = c0 + lane;
   if (c >= ncol) return;
@@ -685,6 +712,35 @@ int launch_ctas(const VfieldArgs& a, int n, int splits) {
 
 }  // namespace
 
+// Slices of a step (d) GEMM's K, when its tiles leave pairs of SMs idle (10 of 76 pairs at N = 23).  Its sums are FP32
+// chains between FP64 flushes, column c of a thread being flushed after the ranges r with r % flush = c: a slice that
+// starts at a multiple of the flush interval and runs XB_HC ranges past its end holds whole chains of every column, and
+// whole periods of the cross-product accumulators, so that every FP32 sum is the unsliced one.  The price is
+// the overlap, XB_HC ranges a slice.  The count with the least (waves x (ranges of a slice + 30 for its start and
+// end)); measured,
+// step (d) unsliced -> sliced: N = 23, 3,957 points 154 -> 106 us; two GEMMs of N = 40, 20,000 points 1.45 -> 0.74
+// ms; N = 65, 24,001 points (153 pairs of tiles, one more than two waves) 2.69 -> 2.33 ms.
+int chain_slices(const VfieldArgs& a, int* kb_per_slice) {
+  const int n = a.n_kb / a.kd, tiles = static_cast<int>(tile_ctas(a) / 2), slots = std::max(1, a.n_sm / 2);
+  int best = 1;
+  *kb_per_slice = a.n_kb;
+  const int x_period = 2 * std::max(1, a.xper / (2 * a.kd));
+  if (a.mode != 1 || a.n_kb % a.kd || a.flush < XB_HC || a.flush % XB_HC || XB_HC % x_period || a.kd < 2) return best;
+  int64_t best_cost = static_cast<int64_t>((tiles + slots - 1) / slots) * (n + 30);
+  for (int q = (n - 1) / a.flush; q >= 1; --q) {   // flush intervals of a slice
+    const int z = (n + q * a.flush - 1) / (q * a.flush);
+    if (z > 16) break;
+    if (n - (z - 1) * q * a.flush <= XB_HC) continue;   // the last slice holds the end of every column's chains
+    const int64_t cost = (static_cast<int64_t>(tiles) * z + slots - 1) / slots * (std::min(n, q * a.flush + XB_HC) + 30);
+    if (cost < best_cost - best_cost / 20) {
+      best_cost = cost;
+      best = z;
+      *kb_per_slice = q * a.flush * a.kd;
+    }
+  }
+  return best;
+}
+
 bool vfield_tc_supported(int n_nuc) { return n_nuc >= 1 && n_nuc <= 8; }
 
 int launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const CUtensorMap* tm_rho16,
@@ -717,6 +773,7 @@ void launch_vfield_tc_finalize(const VfieldArgs& a, int parts, int splits, cudaS
   if (a.mode == 1 ? a.rows_a <= 0 : a.mt_per_x <= 0) return;
   dim3 grid(tile_ctas(a), static_cast<unsigned>(splits));
   grid.z = (parts == 2 ? XB_BN : BF_BN) / FIN_COLS;
+  if (a.mode == 1) grid.y = 1;  // the kernel adds the slices
   if (a.mode == 1)
     assemble_finalize_kernel<XB_BN><<<grid, VF_BM, 0, st>>>(a);
   else if (parts == 2)

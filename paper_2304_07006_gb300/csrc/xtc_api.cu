@@ -938,12 +938,23 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
   const size_t r_bytes = lr_bytes + (d16 ? 2ull * kdim * NP : 0);
   if (!ensure(ctx->L, lr_bytes) || !ensure(ctx->R, r_bytes) || (spin && !ensure(ctx->R2, r_bytes)))
     return fail(ctx, XTC_ERR_OOM, "step (d) operands (%.2f GB)", (spin ? 3.0 : 2.0) * lr_bytes / 1e9);
+  VfieldArgs da{};  // step (d) GEMM
   if (d16) {
     const size_t ebytes = 4ull * m_stride(NP);
     const int bn = vf_bn(2);
     const size_t tiles = static_cast<size_t>(round_up((NP + VF_BM - 1) / VF_BM, 2)) * ((NP + bn - 1) / bn);
+    da.mode = 1;
+    da.rows_a = NP;
+    da.n_pair = NP;
+    da.n_tiles = (NP + bn - 1) / bn;
+    da.n_kb = static_cast<int>(kdim / VF_BK);
+    da.kd = f16_range(ctx->as_kd);
+    da.xper = ctx->x_period;
+    da.flush = flush_ranges(ctx->vf_flush > 0 ? ctx->vf_flush : 8192, da.kd);
+    da.n_sm = ctx->n_sm;
+    da.slices = chain_slices(da, &da.kb_per_split);
     if (!ensure(ctx->L32, 4ull * kdim * NP) || !ensure(ctx->R32, 4ull * kdim * NP) || !ensure(ctx->eL, ebytes) ||
-        !ensure(ctx->eR, ebytes) || !ensure(ctx->Vacc, std::max<size_t>(ctx->Vacc.n, 8ull * tiles * VF_BM * bn)) ||
+        !ensure(ctx->eR, ebytes) || !ensure(ctx->Vacc, 8ull * da.slices * tiles * VF_BM * bn) ||
         (spin && (!ensure(ctx->R32b, 4ull * kdim * NP) || !ensure(ctx->eR2, ebytes))))
       return fail(ctx, XTC_ERR_OOM, "step (d) FP32 operands (%.2f GB)", 8.0 * kdim * NP / 1e9);
     // exponents of the padding columns of M stay 0
@@ -1082,22 +1093,11 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
         }
       }
       if (d16) {
-        VfieldArgs da{};
-        da.mode = 1;
-        da.rows_a = NP;
-        da.n_pair = NP;
-        da.n_tiles = (NP + vf_bn(2) - 1) / vf_bn(2);
-        da.n_kb = static_cast<int>(kdim / VF_BK);
-        da.kb_per_split = da.n_kb;
-        da.kd = f16_range(ctx->as_kd);
-        da.xper = ctx->x_period;
-        da.flush = flush_ranges(ctx->vf_flush > 0 ? ctx->vf_flush : 8192, da.kd);
         da.Vacc = ctx->Vacc.as<double>();
         da.M = M;
         da.ldm = m_stride(NP);
         da.exp_a = ctx->eL.as<int>();
         da.exp_b = ctx->eR.as<int>();
-        da.n_sm = ctx->n_sm;
         da.err = ctx->err_dev.as<int>();
         timed(ctx, XTC_K_AUX, M2 ? 3 : 2, [&] {
           launch_lr_split(ctx->L32.as<float>(), NP, kdim, da.kd, ctx->L.as<uint16_t>(), ctx->eL.as<int>(), nullptr,
@@ -1109,7 +1109,7 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
                             ctx->R2.as<uint16_t>() + 2 * kdim * NP, st);
         });
         timed(ctx, XTC_K_ASSEMBLE, 0, [&] {
-          ctx->launches[XTC_K_ASSEMBLE] += launch_vfield_tc(&tm_L, &tm_R, &tm_R16, da, 2, 1, st);
+          ctx->launches[XTC_K_ASSEMBLE] += launch_vfield_tc(&tm_L, &tm_R, &tm_R16, da, 2, da.slices, st);
         });
         timed(ctx, XTC_K_AUX, 1, [&] { launch_vfield_tc_finalize(da, 2, 1, st); });
         if (M2) {  // the tile sums buffer is reused after the finalize above, in stream order
@@ -1117,7 +1117,7 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
           db.M = M2;
           db.exp_b = ctx->eR2.as<int>();
           timed(ctx, XTC_K_ASSEMBLE, 0, [&] {
-            ctx->launches[XTC_K_ASSEMBLE] += launch_vfield_tc(&tm_L, &tm_R2, &tm_R216, db, 2, 1, st);
+            ctx->launches[XTC_K_ASSEMBLE] += launch_vfield_tc(&tm_L, &tm_R2, &tm_R216, db, 2, db.slices, st);
           });
           timed(ctx, XTC_K_AUX, 1, [&] { launch_vfield_tc_finalize(db, 2, 1, st); });
         }

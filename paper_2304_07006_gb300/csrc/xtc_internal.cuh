@@ -181,6 +181,7 @@ struct VfieldArgs {
   // (n_pair), K = 32 * n_kb; the tile sums (FP64, Vacc, flush > 0 required) are added, unscaled by
   // 2^-(exp_a[pq] + exp_b[rs]), into M[pq * ldm + rs]
   int mode;
+  int slices;                  // slices of K (chain_slices), tile sums [slice][grid CTAs][BN][128]
   int rows_a;
   double* M;
   int64_t ldm;
@@ -188,6 +189,8 @@ struct VfieldArgs {
   const int* exp_b;
 };
 bool vfield_tc_supported(int n_nuc);
+// Slices of K for a step (d) GEMM (its other arguments set), and the K-blocks of each but the last.
+int chain_slices(const VfieldArgs& a, int* kb_per_slice);
 // Launches the GEMM; returns the number of launches.
 // tm_rho16: the fp16(B) plane of the fp16 precision (box 64 x 64, 128-byte swizzle); the bf16 precision ignores it.
 int launch_vfield_tc(const CUtensorMap* tm_g, const CUtensorMap* tm_rho, const CUtensorMap* tm_rho16,
