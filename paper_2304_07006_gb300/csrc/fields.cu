@@ -28,6 +28,11 @@
 // Points past the chunk end are written as zeros.
 #include <cuda_bf16.h>
 
+//
+// What bounds it: instructions, shared loads first (the V traffic is a quarter of the time at rank 16).  So
+// the factor loops are unrolled to the rank's bucket (4, 8, 16), phase 1 loads four factors of c in one access, and
+// phase 2 keeps lam H_p of a row in registers.  Step (c), before -> now (one GB300): N = 65, 24,001 points, 65 factors
+// 10.1 -> 8.7 ms; N = 120, 100,000 points, 7 factors 26 -> 19 ms; N = 23, 3,957 points 52 -> 43 us.
 #include "xtc_internal.cuh"
 
 namespace xtc {
@@ -36,13 +41,16 @@ namespace {
 constexpr int THREADS = 256;
 constexpr int RMAX = 16;
 constexpr int U1 = 4;  // phase 1: columns per group (3 V loads each in flight)
-constexpr int U2 = 2;  // phase 2: pairs per iteration
+constexpr int U2 = 2;  // phase 2: pairs per iteration (spin builds)
+
+// Register bucket of the rank: the factor loops of the kernel are unrolled to it.
+__host__ __device__ constexpr int rank_slots(int R) { return R <= 4 ? 4 : (R <= 8 ? 8 : RMAX); }
 
 template <typename TC>
 struct FieldsSmem {
   TC* phis;  // [N][P]
   TC* ws;    // [P]
-  TC* cs;    // [R][N]
+  TC* cs;    // [N][rank_slots(R)], zero past the rank
   TC* lam;   // [R]
   TC* lamd;  // [R]
   TC* cph;   // [R][P]
@@ -61,7 +69,7 @@ __host__ __device__ inline size_t carve(FieldsSmem<TC>* s, uint8_t* base, int N,
   TC* p[13];
   const size_t n[13] = {static_cast<size_t>(N) * P,
                         static_cast<size_t>(P),
-                        static_cast<size_t>(R) * N,
+                        static_cast<size_t>(rank_slots(R)) * N,
                         static_cast<size_t>(R),
                         static_cast<size_t>(R),
                         static_cast<size_t>(R) * P,
@@ -146,7 +154,7 @@ __device__ __forceinline__ void write4(void* base, int64_t n_pair, int64_t gcp, 
   }
 }
 
-template <typename TV, typename TC, int OUT_PARTS, bool SPIN>
+template <typename TV, typename TC, int OUT_PARTS, bool SPIN, int RM>
 __global__ void __launch_bounds__(THREADS) fields_kernel(const FieldsArgs a) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   const int N = a.n_orb, R = a.rank, P = a.pts;
@@ -169,7 +177,10 @@ __global__ void __launch_bounds__(THREADS) fields_kernel(const FieldsArgs a) {
     const int64_t i = static_cast<int64_t>(blockIdx.x) * P + k;
     sm.ws[k] = i < a.n_i ? static_cast<TC>(a.w[a.i0 + i]) : TC(0);
   }
-  for (int k = t; k < R * N; k += THREADS) sm.cs[k] = static_cast<TC>(a.evec[k]);
+  for (int k = t; k < RM * N; k += THREADS) {
+    const int p = k / RM, kk = k % RM;
+    sm.cs[k] = kk < R ? static_cast<TC>(a.evec[kk * N + p]) : TC(0);
+  }
   for (int k = t; k < R; k += THREADS) {
     sm.lam[k] = static_cast<TC>(a.lam[k]);
     sm.lamd[k] = static_cast<TC>(a.lamd[k]);
@@ -179,7 +190,7 @@ __global__ void __launch_bounds__(THREADS) fields_kernel(const FieldsArgs a) {
   for (int k = t; k < R * P; k += THREADS) {
     const int kk = k / P, q = k % P;
     TC acc = 0;
-    for (int p = 0; p < N; ++p) acc += sm.cs[kk * N + p] * sm.phis[p * P + q];
+    for (int p = 0; p < N; ++p) acc += sm.cs[p * RM + kk] * sm.phis[p * P + q];
     sm.cph[k] = acc;
   }
   __syncthreads();
@@ -194,11 +205,11 @@ __global__ void __launch_bounds__(THREADS) fields_kernel(const FieldsArgs a) {
   // (v_index), U1 columns s at a time (their loads issued before the products), s = 0..N-1 in order.
   const TV* vrow0 = V + (il / VB) * static_cast<int64_t>(N) * N * 3 * VB + (il % VB);
   for (int p = sub; p < N; p += nsub) {
-    TC acc[3][RMAX];
+    TC acc[3][RM];
 #pragma unroll
     for (int x = 0; x < 3; ++x)
 #pragma unroll
-      for (int kk = 0; kk < RMAX; ++kk) acc[x][kk] = 0;
+      for (int kk = 0; kk < RM; ++kk) acc[x][kk] = 0;
     const TV* vrow = vrow0 + static_cast<int64_t>(p) * N * 3 * VB;
     for (int s0 = 0; s0 < N; s0 += U1) {
       TC v[U1][3];
@@ -212,20 +223,23 @@ __global__ void __launch_bounds__(THREADS) fields_kernel(const FieldsArgs a) {
 #pragma unroll
       for (int u = 0; u < U1; ++u) {
         const int s = min(s0 + u, N - 1);  // v[u] = 0 past the last orbital
+        constexpr int W = 16 / sizeof(TC);   // factors of a 16-byte load
 #pragma unroll
-        for (int kk = 0; kk < RMAX; ++kk)
-          if (kk < R) {
-            const TC c = sm.cs[kk * N + s];
+        for (int k0 = 0; k0 < RM; k0 += W) {
+          TC c[W];
+          *reinterpret_cast<uint4*>(c) = *reinterpret_cast<const uint4*>(sm.cs + s * RM + k0);
 #pragma unroll
-            for (int x = 0; x < 3; ++x) acc[x][kk] += v[u][x] * c;
-          }
+          for (int kk = 0; kk < W; ++kk)
+#pragma unroll
+            for (int x = 0; x < 3; ++x) acc[x][k0 + kk] += v[u][x] * c[kk];
+        }
       }
     }
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
       TC h = 0, h2 = 0;
 #pragma unroll
-      for (int kk = 0; kk < RMAX; ++kk)
+      for (int kk = 0; kk < RM; ++kk)
         if (kk < R) {
           sm.Hs[((x * R + kk) * N + p) * P + pt] = acc[x][kk];
           h += sm.lam[kk] * sm.cph[kk * P + pt] * acc[x][kk];
@@ -240,7 +254,7 @@ __global__ void __launch_bounds__(THREADS) fields_kernel(const FieldsArgs a) {
   for (int k = t; k < 3 * R * P; k += THREADS) {
     const int q = k % P, xk = k / P, kk = xk % R;
     TC acc = 0;
-    for (int p = 0; p < N; ++p) acc += sm.cs[kk * N + p] * sm.Hs[(xk * N + p) * P + q];
+    for (int p = 0; p < N; ++p) acc += sm.cs[p * RM + kk] * sm.Hs[(xk * N + p) * P + q];
     sm.part[k] = sm.lamd[kk] * acc;
   }
   __syncthreads();
@@ -256,6 +270,61 @@ __global__ void __launch_bounds__(THREADS) fields_kernel(const FieldsArgs a) {
   const TC w = sm.ws[pt];
   const TC wt = sm.Wt[pt];
   const TC W0 = sm.Wv[pt], W1 = sm.Wv[P + pt], W2 = sm.Wv[2 * P + pt];
+  if constexpr (!SPIN) {
+    // A thread takes row p of its point, lam H_p in registers (two shared loads and two products a factor and
+    // pair become one of each), and the pairs (p, s >= p) in order.  The four rows of a warp are neighbours, so that their
+    // lengths are alike; every other round of rows goes the other way, so that a warp gets long and short ones.
+    for (int base = 0, round = 0; base < N; base += nsub, ++round) {
+      const int p = base + (round & 1 ? nsub - 1 - sub : sub);
+      if (p >= N) continue;
+      TC g[3][RM];
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int kk = 0; kk < RM; ++kk) g[x][kk] = kk < R ? sm.lam[kk] * sm.Hs[((x * R + kk) * N + p) * P + pt] : TC(0);
+      const TC php = sm.phis[p * P + pt];
+      const TC hp0 = sm.hs[p * P + pt], hp1 = sm.hs[(N + p) * P + pt], hp2 = sm.hs[(2 * N + p) * P + pt];
+      const int q0 = p * N - p * (p - 1) / 2 - p;   // pair (p, s) is q0 + s
+      const TV* vrow = vrow0 + static_cast<int64_t>(p) * N * 3 * VB;
+      TC vn[3];
+#pragma unroll
+      for (int x = 0; x < 3; ++x) vn[x] = live ? static_cast<TC>(vload<TV>(vrow, a.splits, sstride, (p * 3 + x) * VB)) : TC(0);
+      for (int s = p; s < N; ++s) {
+        const TC v[3] = {vn[0], vn[1], vn[2]};
+        const int sn = min(s + 1, N - 1);   // the next pair's V in flight
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+          vn[x] = live ? static_cast<TC>(vload<TV>(vrow, a.splits, sstride, (sn * 3 + x) * VB)) : TC(0);
+        TC Lv[4] = {0, 0, 0, 0}, Rv[4] = {0, 0, 0, 0};
+        if (live) {
+          TC zt = 0;
+#pragma unroll
+          for (int x = 0; x < 3; ++x) {
+            const TC* Hq = sm.Hs + (x * R * N + s) * P + pt;
+#pragma unroll
+            for (int kk = 0; kk < RM; ++kk)
+              if (kk < R) zt += g[x][kk] * Hq[kk * N * P];
+          }
+          const TC vt = W0 * v[0] + W1 * v[1] + W2 * v[2];
+          const TC phs = sm.phis[s * P + pt];
+          Lv[0] = w * php * phs;
+          Lv[1] = v[0];
+          Lv[2] = v[1];
+          Lv[3] = v[2];
+          Rv[0] = vt - zt;
+          const TC hp[3] = {hp0, hp1, hp2};
+#pragma unroll
+          for (int x = 0; x < 3; ++x) {
+            const TC zx = w * (php * sm.hs[(x * N + s) * P + pt] + hp[x] * phs);
+            Rv[1 + x] = TC(0.5) * wt * v[x] - zx;
+          }
+        }
+        if (a.write_L) write4<TC, OUT_PARTS>(a.L, a.n_pair, a.gcp, q0 + s, il, Lv);
+        write4<TC, OUT_PARTS>(a.R, a.n_pair, a.gcp, q0 + s, il, Rv, a.add_R);
+      }
+    }
+    return;
+  }
   // U2 pairs per iteration, their V loads issued first
   for (int q0 = sub; q0 < a.n_pair; q0 += U2 * nsub) {
     TC v[U2][3];
@@ -324,7 +393,9 @@ __global__ void __launch_bounds__(THREADS) fields_kernel(const FieldsArgs a) {
 template <typename TV, typename TC, int OUT, bool SPIN>
 void launch_t(const FieldsArgs& a, cudaStream_t st) {
   const size_t smem = fields_smem_bytes(a.n_orb, a.rank, a.pts, sizeof(TC) == 8, SPIN);
-  auto kern = fields_kernel<TV, TC, OUT, SPIN>;
+  const int rm = rank_slots(a.rank);
+  auto kern = rm == 4 ? fields_kernel<TV, TC, OUT, SPIN, 4>
+                      : (rm == 8 ? fields_kernel<TV, TC, OUT, SPIN, 8> : fields_kernel<TV, TC, OUT, SPIN, RMAX>);
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn_smem());
   const int blocks = static_cast<int>(a.gcp / a.pts);
   kern<<<blocks, THREADS, smem, st>>>(a);
