@@ -5,13 +5,13 @@
 //
 // CTA tile 128 x 128, 32-element K stages with both operands TMA-loaded in the 64-byte swizzle,
 // three bf16 parts per operand and six split products (i + j <= 2, smallest first).  Warp 0 issues
-// the TMA loads, warp 1 the MMAs into one of two TMEM accumulators; every `kd` stages warps 2..5
+// the TMA loads, warp 1 the MMAs into one of two TMEM accumulators; every `kd` stages warps 2..17
 // add the finished accumulator into a compensated FP32 running sum (sum and error term, Knuth's
-// TwoSum, both in TMEM) while the MMA fills the other one, which keeps the tensor-core
+// TwoSum, in registers, 32 columns a thread) while the MMA fills the other one, which keeps the tensor-core
 // accumulation (truncating at each MMA) to short ranges.  A tcgen05.commit stalls the tensor pipe
 // for a few hundred cycles, so each range ends with one commit, whose arrival both frees the
 // range's stage slots (the TMA producer counts finished ranges in order) and starts the drain.
-// At the end warps 2..5 add sum + error into the FP64 accumulator M in HBM (read-modify-write;
+// At the end warps 2..17 add sum + error into the FP64 accumulator M in HBM (read-modify-write;
 // every tile of M is owned by exactly one CTA).
 #include "ptx_sm100.cuh"
 #include "xtc_internal.cuh"
@@ -26,27 +26,36 @@ constexpr int A_TILE = AS_BM * 64;
 constexpr int B_TILE = AS_BN * 64;
 constexpr int STAGE_BYTES = PARTS * (A_TILE + B_TILE);
 constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256;
-constexpr int THREADS = 192;
-constexpr int DRAIN_WARPS = 4;
-constexpr uint32_t S_COL = 2 * AS_BN;  // running sum
-constexpr uint32_t C_COL = 3 * AS_BN;  // its rounding-error term
+constexpr int DRAIN_WARPS = 16;        // four per TMEM lane quarter, a quarter of the columns each
+constexpr int THREADS = (2 + DRAIN_WARPS) * 32;
+constexpr int HC = AS_BN / 4;          // running-sum columns per drain thread
+constexpr int TMEM_COLS = 2 * AS_BN;
+static_assert(HC == 32 && TMEM_COLS == 256, "drain columns; TMEM allocation (a power of 2)");
 constexpr int NRB = 8;                 // range barriers (range r uses r % NRB)
 // a wait for range r must not alias range r + NRB (the producer waits for the range of stage
 // k - STAGES before loading stage k)
 static_assert(NRB > STAGES, "range barriers");
 
-__device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-      "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),
-      "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
-      "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// *p += s + c in FP64.  The conversions stay beside the access: hoisted out of a row of these, they would not
+// fit the registers.
+__device__ __forceinline__ void add_f64(double* p, float s, float c) {
+  asm volatile(
+      "{\n\t.reg .f64 a, b;\n\t"
+      "cvt.f64.f32 a, %1;\n\tcvt.f64.f32 b, %2;\n\tadd.rn.f64 a, a, b;\n\t"
+      "ld.global.f64 b, [%0];\n\tadd.rn.f64 b, b, a;\n\tst.global.f64 [%0], b;\n\t}" ::"l"(p),
+      "f"(s), "f"(c)
+      : "memory");
+}
 
 __global__ void __launch_bounds__(THREADS, 1)
     assemble_tc_kernel(const __grid_constant__ CUtensorMap tm_L, const __grid_constant__ CUtensorMap tm_R,
@@ -61,7 +70,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + STAGES + NRB + 3);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp: uniform
   const int m_tile = blockIdx.x, n_tile = blockIdx.y;
   const int n_ranges = (n_kb + kd - 1) / kd;
 
@@ -76,7 +85,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     tma_prefetch_desc(&tm_R);
   }
   if (warp == 0) {
-    tmem_alloc(tmem_slot, 512);
+    tmem_alloc(tmem_slot, TMEM_COLS);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -112,114 +121,90 @@ __global__ void __launch_bounds__(THREADS, 1)
                   DEV_ERR_TIMEOUT_AS);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_f16(AS_BM, AS_BN, true);
-      // small cross products first, hi x hi last, over all stages of a range (the early
-      // truncations then act on a small accumulator)
-      constexpr int pa_of[6] = {1, 0, 2, 0, 1, 0};
-      constexpr int pb_of[6] = {1, 2, 0, 1, 0, 0};
-      bool alive = true;
-      for (int r = 0; r < n_ranges && alive; ++r) {
-        const int kb0 = r * kd, kb1 = min(n_kb, kb0 + kd);
-        const int b = r & 1, u = r >> 1;
-        if (u >= 1 && !mbar_wait(&d_free[b], (u - 1) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS)) break;
-        // cross products of each stage as it lands, then the hi x hi products of the range
-        for (int pass = 0; pass < 2 && alive; ++pass) {
-          for (int kb = kb0; kb < kb1; ++kb) {
-            if (pass == 0) {
-              if (!(alive = mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS)))
-                break;
-              tc_fence_after();
-            }
-            const uint32_t sa = smem_base + (kb % STAGES) * STAGE_BYTES;
-            const uint32_t sb = sa + PARTS * A_TILE;
+    // The whole warp runs the loop, so that descriptors stay in uniform registers: one thread encoding and
+    // spilling them took 4,350 cycles for the 24 MMAs of a range (1,536 cycles of tensor pipe), and that bound the kernel.
+    // Step (d) of a water-sized build (58 orbitals, 40,000 points): 17.9 -> 11.4 ms.
+    constexpr uint32_t idesc = idesc_f16(AS_BM, AS_BN, true);
+    // small cross products first, hi x hi last, over all stages of a range (the early
+    // truncations then act on a small accumulator)
+    constexpr int pa_of[5] = {1, 0, 2, 0, 1};
+    constexpr int pb_of[5] = {1, 2, 0, 1, 0};
+    const uint64_t desc0 = sdesc_kmajor_sw64(0);
+    const uint32_t rdone_bar = smem_u32(rdone);
+    bool alive = true;
+    for (int r = 0; r < n_ranges && alive; ++r) {
+      const int kb0 = r * kd, kb1 = min(n_kb, kb0 + kd);
+      const int b = r & 1, u = r >> 1;
+      const uint32_t d = tmem + b * AS_BN;
+      if (u >= 1 && !mbar_spin(&d_free[b], (u - 1) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS)) break;
+      // cross products of each stage as it lands, then the hi x hi products of the range
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!(alive = mbar_spin(&full[kb % STAGES], (kb / STAGES) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS))) break;
+        tc_fence_after();
+        const uint64_t sa = desc0 + ((smem_base + (kb % STAGES) * STAGE_BYTES) >> 4), sb = sa + (PARTS * A_TILE >> 4);
 #pragma unroll
-            for (int p = 0; p < NPROD; ++p) {
-              if ((p == NPROD - 1) != (pass == 1)) continue;
+        for (int p = 0; p < NPROD - 1; ++p)
 #pragma unroll
-              for (int ks = 0; ks < 2; ++ks) {
-                const uint64_t ad = sdesc_kmajor_sw64(sa + pa_of[p] * A_TILE + ks * 32);
-                const uint64_t bd = sdesc_kmajor_sw64(sb + pb_of[p] * B_TILE + ks * 32);
-                tc_mma_f16(tmem + b * AS_BN, ad, bd, idesc, (kb == kb0 && p == 0 && ks == 0) ? 0u : 1u);
-              }
-            }
-          }
-        }
-        if (!alive) break;
-        tc_commit(&rdone[r % NRB]);
+          for (int ks = 0; ks < 2; ++ks)
+            tc_mma_f16_warp(d, sa + ((pa_of[p] * A_TILE + ks * 32) >> 4), sb + ((pb_of[p] * B_TILE + ks * 32) >> 4),
+                            idesc, kb == kb0 && p == 0 && ks == 0 ? 0u : 1u);
       }
-      tc_commit(fin_bar);
-      int zero = 0;
-      mbar_wait(fin_bar, 0, reinterpret_cast<volatile int*>(&zero), err, DEV_ERR_TIMEOUT_AS);
+      if (!alive) break;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        const uint64_t sa = desc0 + ((smem_base + (kb % STAGES) * STAGE_BYTES) >> 4), sb = sa + (PARTS * A_TILE >> 4);
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) tc_mma_f16_warp(d, sa + 2 * ks, sb + 2 * ks, idesc, 1u);
+      }
+      tc_commit_warp(rdone_bar + 8 * (r % NRB));
     }
+    tc_commit_warp(smem_u32(fin_bar));
+    int zero = 0;
+    mbar_wait(fin_bar, 0, reinterpret_cast<volatile int*>(&zero), err, DEV_ERR_TIMEOUT_AS);
   } else {
-    const int quarter = warp & 3;
-    const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
+    const int quarter = warp & 3;               // TMEM lanes 32*quarter .. +31 (hardware rule)
+    const int c_base = ((warp - 2) >> 2) * HC;  // columns c_base .. +HC-1
+    const uint32_t my = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c_base;
+    float S[HC], C[HC];
+#pragma unroll
+    for (int k = 0; k < HC; ++k) S[k] = C[k] = 0.0f;
     bool ok = true;
-    for (int r = 0; r < n_ranges && ok; ++r) {
+#pragma unroll 1
+    for (int r = 0; r < n_ranges; ++r) {
       const int b = r & 1;
-      ok = __all_sync(0xffffffffu, mbar_wait(&rdone[r % NRB], (r / NRB) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS));
-      __syncwarp();
+      // one lane waits, suspended (the board's power is better spent on the MMAs)
+      if (lane == 0) ok = mbar_wait(&rdone[r % NRB], (r / NRB) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) break;
       tc_fence_after();
-#pragma unroll 1
-      for (int c0 = 0; c0 < AS_BN; c0 += 32) {
-        uint32_t d[32], sacc[32], cacc[32];
-        tmem_ld_32x32b_x32(tmem + lane_base + b * AS_BN + c0, d);
-        if (r > 0) {
-          tmem_ld_32x32b_x32(tmem + lane_base + S_COL + c0, sacc);
-          tmem_ld_32x32b_x32(tmem + lane_base + C_COL + c0, cacc);
-        }
+#pragma unroll
+      for (int c0 = 0; c0 < HC; c0 += 16) {
+        uint32_t d[16];
+        tmem_ld_x16(my + b * AS_BN + c0, d);
         tmem_wait_ld();
-        if (r > 0) {
-#pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            // TwoSum: s1 + e == x + y exactly
-            const float x = __uint_as_float(sacc[k]), y = __uint_as_float(d[k]);
-            const float s1 = __fadd_rn(x, y);
-            const float yp = __fsub_rn(s1, x);
-            const float xp = __fsub_rn(s1, yp);
-            const float e = __fadd_rn(__fsub_rn(x, xp), __fsub_rn(y, yp));
-            sacc[k] = __float_as_uint(s1);
-            cacc[k] = __float_as_uint(__fadd_rn(__uint_as_float(cacc[k]), e));
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            sacc[k] = d[k];
-            cacc[k] = 0u;
-          }
+        if (c0 + 16 == HC) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&d_free[b]);
         }
-        tmem_st_32x32b_x32(tmem + lane_base + S_COL + c0, sacc);
-        tmem_st_32x32b_x32(tmem + lane_base + C_COL + c0, cacc);
-      }
-      tmem_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&d_free[b]);
-    }
-    const int row = m_tile * AS_BM + quarter * 32 + lane;
-    const bool valid = ok && !*abort_flag && row < n_pair && n_kb > 0;
-    double* Mrow = M + static_cast<int64_t>(row) * ldm;
-    tc_fence_after();
-#pragma unroll 1
-    for (int c0 = 0; c0 < AS_BN; c0 += 32) {
-      uint32_t sacc[32], cacc[32];
-      tmem_ld_32x32b_x32(tmem + lane_base + S_COL + c0, sacc);
-      tmem_ld_32x32b_x32(tmem + lane_base + C_COL + c0, cacc);
-      tmem_wait_ld();
-      const int col0 = n_tile * AS_BN + c0;
-      if (valid && col0 < n_pair) {
-        double2* dst = reinterpret_cast<double2*>(Mrow + col0);
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-          double2 v = dst[k];
-          v.x += static_cast<double>(__uint_as_float(sacc[2 * k])) + static_cast<double>(__uint_as_float(cacc[2 * k]));
-          v.y += static_cast<double>(__uint_as_float(sacc[2 * k + 1])) +
-                 static_cast<double>(__uint_as_float(cacc[2 * k + 1]));
-          dst[k] = v;
+          // TwoSum: s1 + e == x + y exactly (the first range gives s1 = y, e = 0)
+          const float x = S[c0 + k], y = __uint_as_float(d[k]);
+          const float s1 = __fadd_rn(x, y);
+          const float yp = __fsub_rn(s1, x);
+          const float xp = __fsub_rn(s1, yp);
+          const float e = __fadd_rn(__fsub_rn(x, xp), __fsub_rn(y, yp));
+          S[c0 + k] = s1;
+          C[c0 + k] = __fadd_rn(C[c0 + k], e);
         }
       }
+    }
+    const int row = m_tile * AS_BM + quarter * 32 + lane;
+    const int col0 = n_tile * AS_BN + c_base;
+    if (ok && !*abort_flag && row < n_pair && n_kb > 0 && col0 < n_pair) {
+      double* dst = M + static_cast<int64_t>(row) * ldm + col0;
+#pragma unroll
+      for (int k = 0; k < HC; ++k) add_f64(dst + k, S[k], C[k]);
     }
   }
 
@@ -228,7 +213,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 0) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc(tmem, TMEM_COLS);
   }
 }
 
