@@ -10,12 +10,19 @@
 // nucleus), b' = (1 + r12)^-2, b'' = -2 b'/(1 + r12).  A zero-length unit vector (a point on a nucleus,
 // r12 = 0) and the 1/r terms that go with it contribute zero; everything else is kept.
 //
-// Bound by the FP64 pipe (2 instructions per SM and clock): about 60 FP64 instructions a pair for the
-// gradient with two nuclei, 100 with F, where summing F term by term took ten times that.  So 1/r12
-// and 1/(1+r12) come from the FP32 approximations by one third-order step (error of the step below
-// 2^-60, then FP64 rounding), conversions and digits are integer operations on bit patterns, and the
+// Bound by the FP64 pipe (2 instructions per SM and clock; with every term in FP64 130 instructions a pair for F
+// with three nuclei).  The polynomials in a2 and b, nine tenths of the arithmetic, have arguments in
+// [0, 1) and coefficients that are fixed for an outer point, so they are evaluated in 64-bit fixed point on the
+// integer pipe: coefficients scaled per outer point so that the sum of all magnitudes stays below 2^58 to 2^61, products
+// as the upper half of 64 x 64 bits.  Their error is a few units of that scale, at most 2^-55 of that sum, less
+// than FP64's rounding of as many terms.  What is left in FP64 are the distances, b' and the last products, about 35 instructions.
+// 1/r12 and 1/(1+r12) come from the FP32 approximations by one third-order step (error of the step below
+// 2^-60, then FP64 rounding), comparisons, conversions and digits are integer operations on bit patterns, and the
 // values are formed once per pair, not once per tile of orbital pairs.  A CTA takes one outer point at
 // a time: the row in FP64 into its scratch row (L2) with the row maximum, then the digits.
+// Calls, all FP64 -> fixed point (one GB300): K with 30 orbitals, 8,000 points and 3 nuclei 18.8 -> 10.6 ms, K on an H2-sized input
+// 1,168 -> 770 us, its FP64 build 847 -> 659 us, 512 points of a water-sized build 9.7 -> 8.3 ms; their errors against
+// 64 bits are those of the FP64 pipe.
 #include <algorithm>
 
 #include "digits64.cuh"
@@ -100,6 +107,119 @@ __device__ __forceinline__ void nuc_coef(const JastrowParams& jp, int I, double 
   }
 }
 
+// ------------------------------------------------------------------ fixed point
+// x 2^s as an integer, rounded to nearest (|x| 2^s < 2^63).
+__device__ __forceinline__ long long to_fixed(double x, int s) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int ex = static_cast<int>(b >> 52) & 0x7ff;
+  const unsigned long long m = (b & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
+  const int sh = max(ex, 1) - 1075 + s;
+  const unsigned long long u = sh >= 0 ? m << min(sh, 63) : (sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull);
+  return static_cast<long long>(b) < 0 ? -static_cast<long long>(u) : static_cast<long long>(u);
+}
+// A factor t as t_h 2^32 + t_l with both halves signed 32-bit (|t_l| <= 2^31), so that a product takes three signed
+// 32 x 32 multiplications; packed as (t_h, t_l).
+__device__ __forceinline__ long long halves(long long t) {
+  const int l = static_cast<int>(t);
+  const unsigned h = static_cast<unsigned>(t >> 32) + (static_cast<unsigned>(l) >> 31);
+  return static_cast<long long>((static_cast<unsigned long long>(h) << 32) | static_cast<unsigned>(l));
+}
+// x t / 2^64 for |x|, |t| < 2^62 (t in halves), to within two units: the product of the low halves is left out.
+__device__ __forceinline__ long long mulh(long long x, long long t) {
+  const long long xb = halves(x);
+  const long long xh = static_cast<int>(xb >> 32), xl = static_cast<int>(xb), th = static_cast<int>(t >> 32), tl = static_cast<int>(t);
+  return xh * th + ((xh * tl + xl * th) >> 32);
+}
+// x in [0, 1] as x 2^62, truncated, in halves.
+__device__ __forceinline__ long long unit_fixed(double x) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int sh = static_cast<int>(b >> 52) - 1013;   // at most 10
+  const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+  return halves(static_cast<long long>(sh >= 0 ? m << min(sh, 10) : m >> min(-sh, 63)));
+}
+// The rare forms out of line: inlined they are predicated, and their FP64 instructions issue for every pair (45 of
+// 81 a pair before).
+__device__ __noinline__ double from_fixed_rare(long long v, int s) { return scalbn(static_cast<double>(v), -s); }
+__device__ __noinline__ double sqrt_rare(double x) { return sqrt(x); }
+__device__ __noinline__ double rsqrt_rare(double x) { return 1.0 / sqrt(x); }
+__device__ __noinline__ double rcp_rare(double x) { return 1.0 / x; }
+// v 2^-s in FP64, rounded to nearest.
+__device__ __forceinline__ double from_fixed(long long v, int s) {
+  const unsigned long long u = v < 0 ? 0ull - static_cast<unsigned long long>(v) : static_cast<unsigned long long>(v);
+  const int lz = __clzll(static_cast<long long>(u));
+  const int ex = 1085 - lz - s;   // biased exponent less one
+  if (static_cast<unsigned>(ex) > 2044u) return from_fixed_rare(v, s);
+  const unsigned long long m = u << (lz & 63);
+  const unsigned long long r = (static_cast<unsigned long long>(ex) << 52) + (m >> 11) + ((m >> 10) & 1);
+  return u ? __longlong_as_double(static_cast<long long>(r | (static_cast<unsigned long long>(v) & 0x8000000000000000ull)))
+           : 0.0;
+}
+// x t, t a fraction from unit_fixed.
+__device__ __forceinline__ long long mulf(long long x, long long t) { return mulh(x, t) * 4; }
+// Exponent e with |x| < 2^e (x finite).
+__device__ __forceinline__ int exponent_above(double x) {
+  return max(static_cast<int>((__double_as_longlong(x) >> 52) & 0x7ff), 1) - 1022;
+}
+
+// The fixed-point coefficients of an outer point.  Scales: a.. of nucleus I by 2^(61 - e_I), e_I bounding the sum of their
+// magnitudes; g of nucleus I so that their products' upper halves, and K, carry 2^sE; b.. and Hc 2^sH, L 2^sL.
+struct NucFix {
+  long long a01, a02, a11, a12, a21, a22, g[3];
+  long long b11, b12, b21, b22;
+  long long L[3][2];
+};
+struct PointFix {
+  long long K[3][3], Hc1, Hc2, L[3];
+  int sE, sH, sL;
+};
+__device__ __forceinline__ double bound_a(const NucCoef& q) {
+  return fabs(q.a01) + fabs(q.a02) + fabs(q.a11) + fabs(q.a12) + 2.0 * (fabs(q.a21) + fabs(q.a22));
+}
+// Threads 0, 1, 2: the scales of E, H and L.
+__device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef* nuc, int n_nuc, int k, PointFix& f) {
+  double s = 0.0, s2 = 0.0, s3 = 0.0;
+  if (k == 0) {
+    for (int x = 0; x < 3; ++x) s = fmax(s, fabs(pt.K[0][x]) + fabs(pt.K[1][x]) + 2.0 * fabs(pt.K[2][x]));
+    for (int I = 0; I < n_nuc; ++I)
+      s += bound_a(nuc[I]) * fmax(fabs(nuc[I].g[0]), fmax(fabs(nuc[I].g[1]), fabs(nuc[I].g[2])));
+    f.sE = 58 - exponent_above(s);
+  } else if (k == 1) {
+    s = fabs(pt.Hc1);
+    s2 = fabs(pt.Hc2);
+    for (int I = 0; I < n_nuc; ++I) {
+      s += fabs(nuc[I].b11) + fabs(nuc[I].b12);
+      s2 += fabs(nuc[I].b21) + fabs(nuc[I].b22);
+    }
+    f.sH = 60 - exponent_above(fmax(s, s2));
+  } else {
+    s = fabs(pt.L[0]);
+    s2 = fabs(pt.L[1]);
+    s3 = fabs(pt.L[2]);
+    for (int I = 0; I < n_nuc; ++I) {
+      s += fabs(nuc[I].L[0][0]) + fabs(nuc[I].L[0][1]);
+      s2 += fabs(nuc[I].L[1][0]) + fabs(nuc[I].L[1][1]);
+      s3 += fabs(nuc[I].L[2][0]) + fabs(nuc[I].L[2][1]);
+    }
+    f.sL = 59 - exponent_above(fmax(s, fmax(s2, s3)));
+  }
+}
+__device__ __forceinline__ void nuc_fix(const NucCoef& q, const PointFix& p, NucFix& f) {
+  const int eI = exponent_above(bound_a(q)), sa = 61 - eI, sg = p.sE + 3 + eI;  // 61 + e_I - e_E, at g / 2^64: sE
+  f.a01 = to_fixed(q.a01, sa);
+  f.a02 = to_fixed(q.a02, sa);
+  f.a11 = to_fixed(q.a11, sa);
+  f.a12 = to_fixed(q.a12, sa);
+  f.a21 = to_fixed(q.a21, sa);
+  f.a22 = to_fixed(q.a22, sa);
+  for (int x = 0; x < 3; ++x) f.g[x] = halves(to_fixed(q.g[x], sg));
+  f.b11 = to_fixed(q.b11, p.sH);
+  f.b12 = to_fixed(q.b12, p.sH);
+  f.b21 = to_fixed(q.b21, p.sH);
+  f.b22 = to_fixed(q.b22, p.sH);
+  for (int o = 0; o < 3; ++o)
+    for (int k = 0; k < 2; ++k) f.L[o][k] = to_fixed(q.L[o][k], p.sL);
+}
+
 // FP32 value of a normal FP64 number in [2^-126, 2^127) (truncated) and back (exact), by the bit patterns.
 __device__ __forceinline__ float narrow(double x) {
   return __uint_as_float(__funnelshift_l(static_cast<uint32_t>(__double2loint(x)),
@@ -111,14 +231,14 @@ __device__ __forceinline__ double widen(float y) {
 }
 // 1/sqrt(x), x > 0: y0 + y0 e (1/2 + 3/8 e) with e = 1 - x y0^2 (third order).
 __device__ __forceinline__ double rsqrt64(double x) {
-  if (!(x > 1e-36 && x < 1e36)) return 1.0 / sqrt(x);
+  if (static_cast<unsigned>((__double2hiint(x) >> 20) - 904) > 238u) return rsqrt_rare(x);   // outside 2^-119 .. 2^120
   const double y = widen(rsqrt_approx(narrow(x)));
   const double e = fma(-(x * y), y, 1.0);
   return fma(fma(0.375, e, 0.5), e * y, y);
 }
 // 1/x, x >= 1: y0 + y0 (e + e^2) with e = 1 - x y0.
 __device__ __forceinline__ double rcp64(double x) {
-  if (!(x < 1e36)) return 1.0 / x;
+  if (static_cast<unsigned>(__double2hiint(x) >> 20) > 1142u) return rcp_rare(x);
   const double y = widen(rcp_approx(narrow(x)));
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
@@ -134,7 +254,9 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
   extern __shared__ __align__(16) uint8_t smem_raw[];
   __shared__ PointCoef pt;
   __shared__ int red[32];
+  __shared__ PointFix pf;
   NucCoef* nuc = reinterpret_cast<NucCoef*>(smem_raw);
+  NucFix* nf = reinterpret_cast<NucFix*>(nuc + n_nuc);
   double* rows = scratch + static_cast<int64_t>(blockIdx.x) * NC * Kp;
   for (int64_t il = blockIdx.x; il < n_i; il += gridDim.x) {
     const double px = grid[3 * (i0 + il)], py = grid[3 * (i0 + il) + 1], pz = grid[3 * (i0 + il) + 2];
@@ -152,6 +274,20 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
       (k < 9 ? pt.K[k / 3][k % 3] : (k == 9 ? pt.Hc1 : (k == 10 ? pt.Hc2 : pt.L[k - 11]))) = s;
     }
     __syncthreads();
+    if (threadIdx.x < 3) point_scales(pt, nuc, n_nuc, threadIdx.x, pf);
+    __syncthreads();
+    for (int I = threadIdx.x; I < n_nuc; I += THREADS) nuc_fix(nuc[I], pf, nf[I]);
+    if (threadIdx.x < 14) {
+      const int k = threadIdx.x;
+      if (k < 9)
+        pf.K[k / 3][k % 3] = to_fixed(pt.K[k / 3][k % 3], pf.sE);
+      else if (k < 11)
+        (k == 9 ? pf.Hc1 : pf.Hc2) = to_fixed(k == 9 ? pt.Hc1 : pt.Hc2, pf.sH);
+      else
+        pf.L[k - 11] = to_fixed(pt.L[k - 11], pf.sL);
+    }
+    __syncthreads();
+    const int sE = pf.sE, sH = pf.sH, sL = pf.sL;
     // ------------------------------------------------------------ the row in FP64, and its largest exponents
     int mx[NC];
 #pragma unroll
@@ -159,54 +295,50 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
     for (int64_t j = threadIdx.x; j < n_j; j += THREADS) {
       const double dx = px - __ldg(jt + j), dy = py - __ldg(jt + ld + j), dz = pz - __ldg(jt + 2 * ld + j);
       const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-      const double i12 = r2 > EPS2 ? rsqrt64(r2) : 0.0;
+      const bool apart = __double_as_longlong(r2) > __double_as_longlong(EPS2);   // r2 > EPS2
+      const double i12 = apart ? rsqrt64(r2) : 0.0;
       // below 1e-14 bohr the distance still enters b (the unit vector does not)
-      const double r = r2 > EPS2 ? r2 * i12 : sqrt(r2);
+      const double r = apart ? r2 * i12 : sqrt_rare(r2);
       const double s12 = rcp64(1.0 + r);
       const double b = r * s12, bp = s12 * s12;
-      double ex = fma(b, fma(b, pt.K[2][0], pt.K[1][0]), pt.K[0][0]);
-      double ey = fma(b, fma(b, pt.K[2][1], pt.K[1][1]), pt.K[0][1]);
-      double ez = fma(b, fma(b, pt.K[2][2], pt.K[1][2]), pt.K[0][2]);
-      double h1 = pt.Hc1, h2 = pt.Hc2;
-      double fx = 0.0, fy = 0.0, fz = 0.0, l0 = 0.0, l1 = 0.0, l2 = 0.0;
-      if (LAP) {
-        const double b2 = b + b;
-        fx = fma(b2, pt.K[2][0], pt.K[1][0]);
-        fy = fma(b2, pt.K[2][1], pt.K[1][1]);
-        fz = fma(b2, pt.K[2][2], pt.K[1][2]);
-        l0 = pt.L[0];
-        l1 = pt.L[1];
-        l2 = pt.L[2];
+      const long long B = unit_fixed(b);
+      long long e[3], fe[3];   // E and dE/db
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        const long long kb = mulf(pf.K[2][x], B);
+        e[x] = pf.K[0][x] + mulf(pf.K[1][x] + kb, B);
+        fe[x] = pf.K[1][x] + 2 * kb;
       }
+      long long h1 = pf.Hc1, h2 = pf.Hc2, l0 = pf.L[0], l1 = pf.L[1], l2 = pf.L[2];
       for (int I = 0; I < n_nuc; ++I) {
-        const NucCoef& q = nuc[I];
-        const double a = __ldg(jt + (3 + I) * ld + j);
-        const double u1 = fma(a, q.a12, q.a11), u2 = b * fma(a, q.a22, q.a21);
-        const double at = a * fma(b, u1 + u2, fma(a, q.a02, q.a01));
-        ex = fma(at, q.g[0], ex);
-        ey = fma(at, q.g[1], ey);
-        ez = fma(at, q.g[2], ez);
-        h1 = fma(a, fma(a, q.b12, q.b11), h1);
-        h2 = fma(a, fma(a, q.b22, q.b21), h2);
+        const NucFix& q = nf[I];
+        const long long A = __ldg(reinterpret_cast<const long long*>(jt) + (3 + I) * ld + j);   // a2
+        const long long u1 = q.a11 + mulf(q.a12, A), u2 = mulf(q.a21 + mulf(q.a22, A), B);
+        const long long at = mulf(q.a01 + mulf(q.a02, A) + mulf(u1 + u2, B), A);
+#pragma unroll
+        for (int x = 0; x < 3; ++x) e[x] += mulh(at, q.g[x]);
+        h1 += mulf(q.b11 + mulf(q.b12, A), A);
+        h2 += mulf(q.b21 + mulf(q.b22, A), A);
         if (LAP) {
-          const double ad = a * fma(2.0, u2, u1);
-          fx = fma(ad, q.g[0], fx);
-          fy = fma(ad, q.g[1], fy);
-          fz = fma(ad, q.g[2], fz);
-          l0 = fma(a, fma(a, q.L[0][1], q.L[0][0]), l0);
-          l1 = fma(a, fma(a, q.L[1][1], q.L[1][0]), l1);
-          l2 = fma(a, fma(a, q.L[2][1], q.L[2][0]), l2);
+          const long long ad = mulf(u1 + 2 * u2, A);
+#pragma unroll
+          for (int x = 0; x < 3; ++x) fe[x] += mulh(ad, q.g[x]);
+          l0 += mulf(q.L[0][0] + mulf(q.L[0][1], A), A);
+          l1 += mulf(q.L[1][0] + mulf(q.L[1][1], A), A);
+          l2 += mulf(q.L[2][0] + mulf(q.L[2][1], A), A);
         }
       }
-      const double h = fma(b, h2, h1);
+      const double h = from_fixed(h1 + mulf(h2, B), sH);
       const double s = bp * i12, hs = h * s;   // b' e12 = s d
-      const double gx = fma(hs, dx, ex), gy = fma(hs, dy, ey), gz = fma(hs, dz, ez);
+      const double gx = fma(hs, dx, from_fixed(e[0], sE)), gy = fma(hs, dy, from_fixed(e[1], sE)),
+                   gz = fma(hs, dz, from_fixed(e[2], sE));
       double v[4] = {gx, gy, gz, 0.0};
       if (LAP) {
-        double f = fma(b, fma(b, l2, l1), l0);
-        f = fma(h2 * bp, bp, f);
-        f = fma(2.0 * (h * bp), i12 - s12, f);
-        f = fma(2.0 * s, fma(dx, fx, fma(dy, fy, dz * fz)), f);
+        const double fx = from_fixed(fe[0], sE), fy = from_fixed(fe[1], sE), fz = from_fixed(fe[2], sE);
+        double f = from_fixed(l0 + mulf(l1 + mulf(l2, B), B), sL);
+        f = fma(from_fixed(h2, sH) * bp, bp, f);
+        const double t = fma(s, fma(dx, fx, fma(dy, fy, dz * fz)), (h * bp) * (i12 - s12));
+        f = fma(2.0, t, f);
         f = fma(gx, gx, fma(gy, gy, fma(gz, gz, f)));
         v[NC == 1 ? 0 : 3] = f;
       }
@@ -253,7 +385,7 @@ __global__ void jtab64_soa_kernel(const double* __restrict__ grid, int64_t n_gri
   for (int I = 0; I < n_nuc; ++I) {
     const double dx = x - jp->nuc[I][0], dy = y - jp->nuc[I][1], dz = z - jp->nuc[I][2];
     const double d = sqrt(dx * dx + dy * dy + dz * dz);
-    jt[(3 + I) * n_pad + j] = d / (1.0 + d);
+    reinterpret_cast<long long*>(jt)[(3 + I) * n_pad + j] = unit_fixed(d / (1.0 + d));
   }
 }
 
@@ -277,7 +409,7 @@ void launch_grad64_digits(const double* grid, const JastrowParams* jp, int n_nuc
                           uint16_t* planes, int* exps, int n_sm, cudaStream_t st) {
   if (n_i <= 0) return;
   const unsigned ctas = grad_ctas(n_i, n_sm);
-  const size_t smem = sizeof(NucCoef) * n_nuc;   // at most 64 nuclei: 14 KB
+  const size_t smem = (sizeof(NucCoef) + sizeof(NucFix)) * n_nuc;   // at most 64 nuclei: 24 KB
   const int64_t plane = comps * c_rows * Kp;
   if (comps == 3)
     grad64_kernel<3><<<ctas, THREADS, smem, st>>>(grid, jp, n_nuc, jt, sj, ld, n_j, Kp, i0, n_i, c_rows, scratch, planes,
