@@ -112,11 +112,11 @@ class Clocks:
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": mx, "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# dram__bytes_read.sum + dram__bytes_write.sum of one step (b) GEMM launch (fp16x2) captured with
+# dram__bytes_read.sum + dram__bytes_write.sum of one step (b) GEMM (fp16x2, the sum over its launches) captured with
 # ncu on the first VFIELD_CAPTURE_OUTER outer points of the workload (`--ncu-case`), for GEMM
 # engine revision VFIELD_CAPTURE_REVISION; with another revision the traffic is reported as null
-VFIELD_CAPTURE_REVISION = 5
-VFIELD_DRAM_BYTES_CAPTURED = 21_219_623_424 + 2_889_048_320
+VFIELD_CAPTURE_REVISION = 7
+VFIELD_DRAM_BYTES_CAPTURED = 21_236_646_656 + 2_783_462_656
 VFIELD_CAPTURE_OUTER = 1184
 
 
@@ -494,9 +494,10 @@ def main():
     # roofline of the dominant kernel: step (b), per-launch algorithmic flops / mean launch time
     per_kernel = {name: {"ms_per_step": kern_ms[k] / args.steps, "launches_per_step": int(kern_n[k] // args.steps)}
                   for k, name in enumerate(KERNEL_NAMES)}
-    # one gradient-table launch per chunk; "vfield" and "assemble" time the step (b) and step (d)
-    # GEMMs alone, "aux" the kernels around them (V and M from the FP64 tile sums, row splits)
-    n_vf = kern_n[KERNEL_NAMES.index("grad")] / args.steps
+    # two step (a) launches per chunk (coefficients, table); "vfield" and "assemble" time the step (b) and step
+    # (d) GEMMs alone (each as launches of whole waves), "aux" the kernels around them (V and M from the FP64 tile
+    # sums, row splits); the figures below are per chunk
+    n_vf = kern_n[KERNEL_NAMES.index("grad")] / 2 / args.steps
     vf_ms = kern_ms[1] / args.steps / n_vf
     vf_flops_launch = F["b"] / n_vf
     peaks, peak_src = measured_peaks()
