@@ -13,9 +13,8 @@
 // Bound by the FP64 pipe (2 instructions per SM and clock; with every term in FP64 130 instructions a pair for F
 // with three nuclei).  The polynomials in a2 and b, nine tenths of the arithmetic, have arguments in
 // [0, 1) and coefficients that are fixed for an outer point, so they are evaluated in 64-bit fixed point on the
-// integer pipe: coefficients scaled per outer point so that the sum of all magnitudes stays below 2^58 to 2^61, products
-// as the upper half of 64 x 64 bits.  Their error is a few units of that scale, at most 2^-55 of that sum, less
-// than FP64's rounding of as many terms.  What is left in FP64 are the distances, b' and the last products, about 35 instructions.
+// integer pipe: coefficients scaled per outer point so that the sum of all magnitudes stays below 2^59 to 2^61, products
+// rounded to units of that scale, 2^-59 of that sum or less, where FP64 rounds every term to 2^-53 of itself.  What is left in FP64 are the distances, b' and the last products, about 35 instructions.
 // 1/r12 and 1/(1+r12) come from the FP32 approximations by one third-order step (error of the step below
 // 2^-60, then FP64 rounding), comparisons, conversions and digits are integer operations on bit patterns, and the
 // values are formed once per pair, not once per tile of orbital pairs.  A CTA takes one outer point at
@@ -124,11 +123,13 @@ __device__ __forceinline__ long long halves(long long t) {
   const unsigned h = static_cast<unsigned>(t >> 32) + (static_cast<unsigned>(l) >> 31);
   return static_cast<long long>((static_cast<unsigned long long>(h) << 32) | static_cast<unsigned>(l));
 }
-// x t / 2^64 for |x|, |t| < 2^62 (t in halves), to within two units: the product of the low halves is left out.
+// x t / 2^(64 - UP) for |x|, |t| < 2^62 (t in halves), rounded; the product of the low halves is left out (at most
+// 2^(UP - 2) units, either sign).
+template <int UP>
 __device__ __forceinline__ long long mulh(long long x, long long t) {
   const long long xb = halves(x);
   const long long xh = static_cast<int>(xb >> 32), xl = static_cast<int>(xb), th = static_cast<int>(t >> 32), tl = static_cast<int>(t);
-  return xh * th + ((xh * tl + xl * th) >> 32);
+  return xh * th * (1 << UP) + ((xh * tl + xl * th + (1ll << (31 - UP))) >> (32 - UP));
 }
 // x in [0, 1] as x 2^62, truncated, in halves.
 __device__ __forceinline__ long long unit_fixed(double x) {
@@ -155,14 +156,14 @@ __device__ __forceinline__ double from_fixed(long long v, int s) {
            : 0.0;
 }
 // x t, t a fraction from unit_fixed.
-__device__ __forceinline__ long long mulf(long long x, long long t) { return mulh(x, t) * 4; }
+__device__ __forceinline__ long long mulf(long long x, long long t) { return mulh<2>(x, t); }
 // Exponent e with |x| < 2^e (x finite).
 __device__ __forceinline__ int exponent_above(double x) {
   return max(static_cast<int>((__double_as_longlong(x) >> 52) & 0x7ff), 1) - 1022;
 }
 
 // The fixed-point coefficients of an outer point.  Scales: a.. of nucleus I by 2^(61 - e_I), e_I bounding the sum of their
-// magnitudes; g of nucleus I so that their products' upper halves, and K, carry 2^sE; b.. and Hc 2^sH, L 2^sL.
+// magnitudes; g of nucleus I so that their products, and K, carry 2^sE; b.. and Hc 2^sH, L 2^sL.
 struct NucFix {
   long long a01, a02, a11, a12, a21, a22, g[3];
   long long b11, b12, b21, b22;
@@ -182,7 +183,7 @@ __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef*
     for (int x = 0; x < 3; ++x) s = fmax(s, fabs(pt.K[0][x]) + fabs(pt.K[1][x]) + 2.0 * fabs(pt.K[2][x]));
     for (int I = 0; I < n_nuc; ++I)
       s += bound_a(nuc[I]) * fmax(fabs(nuc[I].g[0]), fmax(fabs(nuc[I].g[1]), fabs(nuc[I].g[2])));
-    f.sE = 58 - exponent_above(s);
+    f.sE = 61 - exponent_above(s);
   } else if (k == 1) {
     s = fabs(pt.Hc1);
     s2 = fabs(pt.Hc2);
@@ -204,7 +205,7 @@ __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef*
   }
 }
 __device__ __forceinline__ void nuc_fix(const NucCoef& q, const PointFix& p, NucFix& f) {
-  const int eI = exponent_above(bound_a(q)), sa = 61 - eI, sg = p.sE + 3 + eI;  // 61 + e_I - e_E, at g / 2^64: sE
+  const int eI = exponent_above(bound_a(q)), sa = 61 - eI, sg = p.sE + eI;  // at g / 2^61 then carries sE
   f.a01 = to_fixed(q.a01, sa);
   f.a02 = to_fixed(q.a02, sa);
   f.a11 = to_fixed(q.a11, sa);
@@ -316,13 +317,13 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
         const long long u1 = q.a11 + mulf(q.a12, A), u2 = mulf(q.a21 + mulf(q.a22, A), B);
         const long long at = mulf(q.a01 + mulf(q.a02, A) + mulf(u1 + u2, B), A);
 #pragma unroll
-        for (int x = 0; x < 3; ++x) e[x] += mulh(at, q.g[x]);
+        for (int x = 0; x < 3; ++x) e[x] += mulh<3>(at, q.g[x]);
         h1 += mulf(q.b11 + mulf(q.b12, A), A);
         h2 += mulf(q.b21 + mulf(q.b22, A), A);
         if (LAP) {
           const long long ad = mulf(u1 + 2 * u2, A);
 #pragma unroll
-          for (int x = 0; x < 3; ++x) fe[x] += mulh(ad, q.g[x]);
+          for (int x = 0; x < 3; ++x) fe[x] += mulh<3>(ad, q.g[x]);
           l0 += mulf(q.L[0][0] + mulf(q.L[0][1], A), A);
           l1 += mulf(q.L[1][0] + mulf(q.L[1][1], A), A);
           l2 += mulf(q.L[2][0] + mulf(q.L[2][1], A), A);
