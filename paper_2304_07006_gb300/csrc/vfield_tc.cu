@@ -697,7 +697,7 @@ unsigned tile_ctas(const VfieldArgs& a) {
 // CTAs per launch of a GEMM of n CTAs along x.  The CTAs resident at one time stream the same panels of A and
 // B and meet in L2 only while they are at about the same k.  Nothing keeps them there: each new tile starts when
 // some other one ends, and after ten waves of the N = 120 build the starts are spread over a third of a tile's time,
-// with 58.6 GB read from HBM where the panels of its waves are 17 GB.  The board is at its power cap, so that
+// with 58.6 GB read from HBM (1,184 outer points) where the panels of its waves are 17 GB (21 now).  The board is at its power cap, so that
 // traffic is paid for in clock rate.  Launches of whole waves line the CTAs up again: step (b) of that build 1,060 -> 925 ms,
 // of a piece of the N = 200 build 169 -> 134 ms (one wave a launch; two 134, four 139).  A launch costs a few
 // microseconds and the tail of its last wave, so it lasts at least LAUNCH_RANGES ranges of 64 values (2 ms;
