@@ -16,7 +16,8 @@
 // brought to the same largest value), taken out of rho and multiplied into the pair functions: a row of those is then weighted as in the sum, and its
 // maximum is not set by points that contribute nothing (a neighbour of the outer point, a far point
 // with no density).  With seven digits and no such scales the error of the water-sized build was 1,500
-// times that of the FP64 pipe's sums.  Step (d) uses the same scales for rho and A.
+// times that of the FP64 pipe's sums.  Step (d) uses the same scales for rho and A, and the
+// contraction of K scales of its own (point_scale_k_kernel).
 //
 // Why: the FP64 pipe does 2 FMA per SM and clock on this GPU, the 128 x 32 x 64 FMA of one range of a
 // tile take 131,072 of its cycles; the same range is 36 fp16 products of 4 k-steps.  They are bound by shared
@@ -317,13 +318,6 @@ struct LrSrc {
     return sj[i] == D64_NO_SCALE ? D64_NO_SCALE : sign * sj[i];
   }
 };
-// FP64 rows as they are.
-struct RowSrc {
-  const double* p;
-  int64_t ld;
-  __device__ double at(int64_t row, int64_t k) const { return p[row * ld + k]; }
-  __device__ int scale(int64_t) const { return 0; }
-};
 // rho^T[pq][j] = w_j phi_p(j) phi_q(j), times 2^-sj[j]
 struct RhoSrc {
   const double* phiT;
@@ -337,25 +331,43 @@ struct RhoSrc {
   }
   __device__ int scale(int64_t k) const { return sj[k] == D64_NO_SCALE ? D64_NO_SCALE : -sj[k]; }
 };
-// Left operand of the contraction of K: row pq = p N + q, k = c ncp + i: c = 0: w phi_p phi_q / 2;
-// c = 1..3: w phi_p d_x phi_q (dphiT row 3 q + x); 0 past the chunk's points.  No point scales here: the orbital
-// gradients are an input of their own, not bounded by the orbitals' values.
+// Operands of the contraction of K, k = c ncp + i, i < n_i a point of the chunk (zero past them).  Left: row
+// pq = p N + q, c = 0: w phi_p phi_q / 2, c = 1..3: w phi_p d_x phi_q (dphiT row 3 q + x).  Right: W, V_x.  W grows as 1/r
+// next to a nucleus, where the weight is as small, so the points carry the scales of point_scale_k_kernel,
+// taken out of the left operand and multiplied into the right one.  Without them a point 1e-12 bohr from a
+// nucleus cost every row the bits of 1/r: 1e-10 of max |K| where FP64 sums give 1e-14.
+__device__ __forceinline__ int k_component(int64_t k, int64_t ncp) { return (k >= ncp) + (k >= 2 * ncp) + (k >= 3 * ncp); }
 struct PsiSrc {
   const double* phiT;
   const double* dphiT;
   int64_t ld;
   const double* w;
+  const int* si;
   int64_t i0, n_i, ncp;
   int n_orb;
   __device__ double at(int64_t row, int64_t k) const {
-    const int c = static_cast<int>(k / ncp);
+    const int c = k_component(k, ncp);
     const int64_t i = k - c * ncp, g = i0 + i;
     if (i >= n_i) return 0.0;
     const int64_t p = row / n_orb, q = row - p * n_orb;
     const double wp = w[g] * phiT[p * ld + g];
     return c == 0 ? 0.5 * wp * phiT[q * ld + g] : wp * dphiT[(3 * q + c - 1) * ld + g];
   }
-  __device__ int scale(int64_t) const { return 0; }
+  __device__ int scale(int64_t k) const {
+    const int64_t i = k - k_component(k, ncp) * ncp;
+    if (i >= n_i) return 0;
+    return si[i0 + i] == D64_NO_SCALE ? D64_NO_SCALE : -si[i0 + i];
+  }
+};
+struct WvSrc {
+  const double* p;
+  const int* si;
+  int64_t i0, n_i, ncp;
+  __device__ double at(int64_t row, int64_t k) const { return p[row * 4 * ncp + k]; }
+  __device__ int scale(int64_t k) const {
+    const int64_t i = k - k_component(k, ncp) * ncp;
+    return i < n_i ? si[i0 + i] : 0;
+  }
 };
 
 // One CTA per row: the row's largest exponent, then the digits of four consecutive k per thread.  The
@@ -407,6 +419,30 @@ __global__ void point_scale_kernel(const double* __restrict__ phiT, int64_t ld, 
   }
   const int kw = d64_key(w[j], 0);
   sj[j] = m == D64_NO_SCALE || kw == 0 ? D64_NO_SCALE : kw - D64_BIAS - 1022 + 2 * m;
+}
+
+// si[i]: the exponent of |w_i| max_p (|phi_p(i)| / max |phi_p|) max_q (|phi_q(i)|, |d_x phi_q(i)|, / max of both), which the
+// left operand of K is of at point i; D64_NO_SCALE where that operand is 0.  orb[n_orb], dorb[3 n_orb]: largest keys.
+__global__ void point_scale_k_kernel(const double* __restrict__ phiT, const double* __restrict__ dphiT, int64_t ld,
+                                     const double* __restrict__ w, int64_t n, int n_orb, const int* __restrict__ orb,
+                                     const int* __restrict__ dorb, int* __restrict__ si) {
+  const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (i >= n) return;
+  int mp = D64_NO_SCALE, mq = D64_NO_SCALE;
+#pragma unroll 2
+  for (int q = 0; q < n_orb; ++q) {
+    const int k = d64_key(phiT[q * ld + i], 0);
+    int kd = k, top = orb[q];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      kd = max(kd, d64_key(dphiT[(3 * q + x) * ld + i], 0));
+      top = max(top, dorb[3 * q + x]);
+    }
+    if (k) mp = max(mp, k - orb[q]);
+    if (kd) mq = max(mq, kd - top);
+  }
+  const int kw = d64_key(w[i], 0);
+  si[i] = mp == D64_NO_SCALE || kw == 0 ? D64_NO_SCALE : kw - D64_BIAS - 1022 + mp + mq;
 }
 
 }  // namespace
@@ -464,10 +500,6 @@ void launch_digits_lr(const double* src, int64_t rows, int64_t ld, int64_t k0, i
                                                                     planes, rows * K, exps);
 }
 
-void launch_digits_rows(const double* src, int64_t rows, int64_t K, uint16_t* planes, int* exps, cudaStream_t st) {
-  digits_kernel<<<static_cast<unsigned>(rows), DG_THREADS, 0, st>>>(RowSrc{src, K}, K, K, planes, rows * K, exps);
-}
-
 void launch_digits_rho(const double* phiT, int64_t ld, const double* w, int64_t n_j, int64_t Kp, int n_orb,
                        const int* pair_p, const int* pair_q, const int* sj, uint16_t* planes, int* exps,
                        cudaStream_t st) {
@@ -482,11 +514,25 @@ void launch_point_scale(const double* phiT, int64_t ld, const double* w, int64_t
   point_scale_kernel<<<static_cast<unsigned>((n_grid + 127) / 128), 128, 0, st>>>(phiT, ld, w, n_grid, n_orb, orb, sj);
 }
 
-void launch_digits_psi(const double* phiT, const double* dphiT, int64_t ld, const double* w, int64_t i0, int64_t n_i,
-                       int64_t ncp, int n_orb, uint16_t* planes, int* exps, cudaStream_t st) {
+void launch_point_scale_k(const double* phiT, const double* dphiT, int64_t ld, const double* w, int64_t n_grid,
+                          int n_orb, int* orb, int* si, cudaStream_t st) {
+  orbital_key_kernel<<<n_orb, DG_THREADS, 0, st>>>(phiT, ld, n_grid, orb);
+  orbital_key_kernel<<<3 * n_orb, DG_THREADS, 0, st>>>(dphiT, ld, n_grid, orb + n_orb);
+  point_scale_k_kernel<<<static_cast<unsigned>((n_grid + 127) / 128), 128, 0, st>>>(phiT, dphiT, ld, w, n_grid, n_orb, orb,
+                                                                                 orb + n_orb, si);
+}
+
+void launch_digits_psi(const double* phiT, const double* dphiT, int64_t ld, const double* w, const int* si, int64_t i0,
+                       int64_t n_i, int64_t ncp, int n_orb, uint16_t* planes, int* exps, cudaStream_t st) {
   const int64_t rows = static_cast<int64_t>(n_orb) * n_orb;
   digits_kernel<<<static_cast<unsigned>(rows), DG_THREADS, 0, st>>>(
-      PsiSrc{phiT, dphiT, ld, w, i0, n_i, ncp, n_orb}, 4 * ncp, 4 * ncp, planes, rows * 4 * ncp, exps);
+      PsiSrc{phiT, dphiT, ld, w, si, i0, n_i, ncp, n_orb}, 4 * ncp, 4 * ncp, planes, rows * 4 * ncp, exps);
+}
+
+void launch_digits_wv(const double* src, int64_t rows, const int* si, int64_t i0, int64_t n_i, int64_t ncp,
+                      uint16_t* planes, int* exps, cudaStream_t st) {
+  digits_kernel<<<static_cast<unsigned>(rows), DG_THREADS, 0, st>>>(WvSrc{src, si, i0, n_i, ncp}, 4 * ncp, 4 * ncp,
+                                                                    planes, rows * 4 * ncp, exps);
 }
 
 }  // namespace xtc
