@@ -209,8 +209,10 @@ XTC_API int xtc_vfield(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* gr
 /* Self-test of failure detection (no counterpart in the paper): every wait inside the library's
  * tensor-core kernels is bounded; when it runs out, the kernel records an error code and returns,
  * and the call reports XTC_ERR_TIMEOUT.  This call runs one such wait on a barrier that nothing
- * completes, with a limit of limit_ms (1..4000), and returns what a timed-out build would:
- * XTC_ERR_TIMEOUT.  The context stays usable.  XTC_ERR_ARG for a limit out of range. */
+ * completes, and beside it a warp's wait on one that completes for half of its lanes only, with a limit of
+ * limit_ms (1..4000), and returns what a timed-out build would:
+ * XTC_ERR_TIMEOUT (XTC_OK if the lanes of the warp came to different verdicts).  The context stays
+ * usable.  XTC_ERR_ARG for a limit out of range. */
 XTC_API int xtc_selftest_wait_timeout(xtc_ctx* ctx, int limit_ms);
 
 /* Frozen-core folding of the xTC corrections, xTC-FC (Results section "Frozen core

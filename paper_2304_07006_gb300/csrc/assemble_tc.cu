@@ -136,10 +136,10 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int kb0 = r * kd, kb1 = min(n_kb, kb0 + kd);
       const int b = r & 1, u = r >> 1;
       const uint32_t d = tmem + b * AS_BN;
-      if (u >= 1 && !mbar_spin(&d_free[b], (u - 1) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS)) break;
+      if (u >= 1 && !mbar_spin_warp(&d_free[b], (u - 1) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS)) break;
       // cross products of each stage as it lands, then the hi x hi products of the range
       for (int kb = kb0; kb < kb1; ++kb) {
-        if (!(alive = mbar_spin(&full[kb % STAGES], (kb / STAGES) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS))) break;
+        if (!(alive = mbar_spin_warp(&full[kb % STAGES], (kb / STAGES) & 1, abort_flag, err, DEV_ERR_TIMEOUT_AS))) break;
         tc_fence_after();
         const uint64_t sa = desc0 + ((smem_base + (kb % STAGES) * STAGE_BYTES) >> 4), sb = sa + (PARTS * A_TILE >> 4);
 #pragma unroll

@@ -168,12 +168,12 @@ __global__ void __launch_bounds__(THREADS, 1)
     int s = 0, lap = 0;   // slot of the next A plane and its use
     for (int r = 0; r < n_ranges && ok; ++r) {
       const int b = r & 1, u = r >> 1;
-      if (u >= 1 && !(ok = mbar_spin(&e_free[b], (u - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_G64))) break;
-      if (!(ok = mbar_spin(&b_full[b], u & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_G64))) break;
+      if (u >= 1 && !(ok = mbar_spin_warp(&e_free[b], (u - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_G64))) break;
+      if (!(ok = mbar_spin_warp(&b_full[b], u & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_G64))) break;
       const uint64_t db = db0 + b * (B_SLOT >> 4);
 #pragma unroll
       for (int i = 0; i < DIG; ++i) {
-        if (!(ok = mbar_spin(&a_full[s], lap & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_G64))) break;
+        if (!(ok = mbar_spin_warp(&a_full[s], lap & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_G64))) break;
         tc_fence_after();
         const uint64_t da = da0 + s * (A_SLOT >> 4);
         const uint32_t d = tmem + b * SET_COLS + i * BN;
@@ -205,9 +205,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     bool ok = true;
     for (int r = 0; r < n_ranges; ++r) {
       const int b = r & 1;
-      ok = __all_sync(0xffffffffu,
-                      mbar_spin(&rdone[b], (r >> 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_G64));
-      __syncwarp();
+      ok = mbar_spin_warp(&rdone[b], (r >> 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_G64);
       if (!ok) break;
       tc_fence_after();
       const uint32_t src = base + b * SET_COLS;

@@ -66,9 +66,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return true;
 }
 
-// The same with a non-suspending test in a tight loop: for the threads that issue MMAs and the
-// warps that drain their accumulators, where the wake-up latency of a suspended wait sits on the
-// critical path.
+// The same with a non-suspending test in a tight loop, where the wake-up latency of a suspended wait sits on the critical
+// path: mbar_spin_warp below, for the warps that issue MMAs or drain their accumulators.
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -96,6 +95,14 @@ __device__ __forceinline__ bool mbar_spin(uint64_t* bar, uint32_t parity, volati
     }
   }
   return true;
+}
+
+// A warp's wait: every lane polls, and all take one verdict.  Without the vote a wait that runs out in one lane while
+// the barrier completes for another would send the lanes to different warp-wide instructions (elect.sync, tcgen05.ld), which
+// then wait for each other without a bound.
+__device__ __forceinline__ bool mbar_spin_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err, int code,
+                                               unsigned long long limit_ns = TIMEOUT_NS) {
+  return __all_sync(0xffffffffu, mbar_spin(bar, parity, abort_flag, err, code, limit_ns));
 }
 
 // ------------------------------------------------------------------ proxies / TMA

@@ -9,18 +9,25 @@
 namespace xtc {
 namespace {
 
+// Warp 0: one thread's wait.  Warp 1: a warp's wait in which the barrier of the even lanes has completed and that of the odd
+// lanes never does; it must run out for all of them (an error word of 0 says that the lanes did not agree).
 __global__ void wait_timeout_selftest_kernel(int* err, unsigned long long limit_ns) {
-  __shared__ uint64_t bar;
-  __shared__ int abort_flag;
+  __shared__ uint64_t bars[2];   // the phase of parity 0 completes on bars[0] alone
+  __shared__ int abort_flags[2], split;
   if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
-    abort_flag = 0;
+    mbar_init(&bars[0], 1);
+    mbar_init(&bars[1], 1);
+    abort_flags[0] = abort_flags[1] = split = 0;
     fence_mbar_init();
+    mbar_arrive(&bars[0]);
   }
   __syncthreads();
-  // the phase of parity 0 never completes: no thread arrives on bar
-  if (threadIdx.x == 0) mbar_wait(&bar, 0, &abort_flag, err, DEV_ERR_TIMEOUT_SELFTEST, limit_ns);
+  if (threadIdx.x == 0) mbar_wait(&bars[1], 0, &abort_flags[0], err, DEV_ERR_TIMEOUT_SELFTEST, limit_ns);
+  if (threadIdx.x >= 32 &&
+      mbar_spin_warp(&bars[threadIdx.x & 1], 0, &abort_flags[1], err, DEV_ERR_TIMEOUT_SELFTEST, limit_ns))
+    split = 1;
   __syncthreads();
+  if (threadIdx.x == 0 && split) *err = 0;
 }
 
 __global__ void recip_selftest_kernel(const float* __restrict__ x, int64_t n, float* __restrict__ y_rsqrt,
@@ -42,7 +49,7 @@ __global__ void recip_selftest_kernel(const float* __restrict__ x, int64_t n, fl
 }  // namespace
 
 void launch_wait_timeout_selftest(int* err, unsigned long long limit_ns, cudaStream_t st) {
-  wait_timeout_selftest_kernel<<<1, 32, 0, st>>>(err, limit_ns);
+  wait_timeout_selftest_kernel<<<1, 64, 0, st>>>(err, limit_ns);
 }
 
 void launch_recip_selftest(const float* x, int64_t n, float* y_rsqrt, float* y_rcp, cudaStream_t st) {

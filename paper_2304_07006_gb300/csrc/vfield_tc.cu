@@ -243,8 +243,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(XB_THREADS, 1)
           const int s = (it >> 1) % XB_STAGES;
           // the stage first: it landed long ago as a rule, the set is what the issuer waits for
           if (!(it & 1) || it == it0)
-            alive = mbar_spin(&full[s], ((it >> 1) / XB_STAGES) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
-          if (it == it0) alive = alive && mbar_spin(&e_free[k], u & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
+            alive = mbar_spin_warp(&full[s], ((it >> 1) / XB_STAGES) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
+          if (it == it0) alive = alive && mbar_spin_warp(&e_free[k], u & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF);
           if (!alive) break;
           tc_fence_after();
           // the block's 32 values are half of the 128-byte rows; k-steps of 16 values advance 32 bytes
@@ -507,10 +507,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(BF_THREADS, 1)
         const int it0 = r * kd, it1 = min(n_it, it0 + kd);
         const int b = r & 1, u = r >> 1;
         const uint32_t d_tmem = tmem + b * BF_BN;
-        if (u >= 1 && !mbar_spin(&d_free[b], (u - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF)) break;
+        if (u >= 1 && !mbar_spin_warp(&d_free[b], (u - 1) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF)) break;
         for (int it = it0; it < it1; ++it) {
           const int s = it % BF_STAGES;
-          if (!(alive = mbar_spin(&full[s], (it / BF_STAGES) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF))) break;
+          if (!(alive = mbar_spin_warp(&full[s], (it / BF_STAGES) & 1, abort_flag, args.err, DEV_ERR_TIMEOUT_VF))) break;
           tc_fence_after();
           const uint64_t sa = desc0 + ((smem_base + s * BF_STAGE) >> 4);
           const uint64_t sb = sa + (BF_PARTS * BF_A_TILE >> 4);

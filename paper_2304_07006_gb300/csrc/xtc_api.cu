@@ -481,8 +481,9 @@ int xtc_set_outer_range(xtc_ctx* ctx, int64_t begin, int64_t end) {
 // 4: step (d) on an fp16 plane of R as well (three products), drains waiting without suspending;
 // 5: tiles ordered in groups of 16 row tiles (8 before);
 // 6: CTA pairs on 256 x 128 tiles, hi_a x [hi_b | lo_b] in one MMA, 64-value stages;
-// 7: launches of whole waves, step (d) in slices of K when its tiles are few.
-int xtc_engine_revision(void) { return 7; }
+// 7: launches of whole waves, step (d) in slices of K when its tiles are few;
+// 8: the issuing warps' waits end with one verdict.
+int xtc_engine_revision(void) { return 8; }
 
 int xtc_get_timings(xtc_ctx* ctx, double* ms, int64_t* launches, int n) {
   if (!ctx || n < XTC_N_KERNELS) return XTC_ERR_ARG;

@@ -51,7 +51,8 @@ constexpr int DEV_ERR_TIMEOUT_AS = 2;
 constexpr int DEV_ERR_TIMEOUT_SELFTEST = 3;
 constexpr int DEV_ERR_TIMEOUT_G64 = 4;
 // Self-test of the bounded waits: one CTA waits on an mbarrier that nothing arrives on, with the
-// kernels' own wait routine and a limit of limit_ns, and records DEV_ERR_TIMEOUT_SELFTEST in err.
+// kernels' own wait routines (a thread's and a warp's) and a limit of limit_ns, and records
+// DEV_ERR_TIMEOUT_SELFTEST in err, or 0 when the warp's lanes do not agree.
 void launch_wait_timeout_selftest(int* err, unsigned long long limit_ns, cudaStream_t st);
 // Self-test of the gradient kernel's refined 1/sqrt(x) and 1/x (simt_pack.cuh) on x[0..n).
 void launch_recip_selftest(const float* x, int64_t n, float* y_rsqrt, float* y_rcp, cudaStream_t st);
