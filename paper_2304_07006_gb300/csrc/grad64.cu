@@ -5,7 +5,10 @@
 // u = sum_I sum_t c (a1^m a2^n + a1^n a2^m) b^o with a = r/(1+r) for the electron-nucleus distances and b
 // the same for r12 (jastrow_coef.cuh).  With the first electron's factors taken into coefficients,
 //   grad_1 u = E + H b' e12,   E = K0 + b K1 + b^2 K2 + sum_I a2 t_I(a2, b) g_I,   H = h1 + b h2 = du/db,
-//   lap_1 u  = L0 + b L1 + b^2 L2 + h2 b'^2 + 2 H b' (1/r12 - 1/(1+r12)) + 2 b' e12 . dE/db,
+//   lap_1 u  = L0 + b L1 + b^2 L2 + h2 b'^2 + 2 H b' (1/r12 - 1/(1+r12)) + 2 b' e12 . dE/db
+//            = L0 + b L1 + b^2 L2 + 3 h2 b'^2 + 2 h1 b' / (r12 (1+r12)) + 2 b' e12 . dE/db,
+// (b (1/r12 - 1/(1+r12)) = b'; so 1/r12 meets h1 alone, which has a scale of its own and is exactly 0 where du/db
+// vanishes at r12 = 0: with H / r12 from one fixed-point H a pair 1e-7 bohr apart lost 1e-11 of F with terms in b^2 only)
 // where L_o holds a'^2 d2/da1^2 + (a'' + 2 a'/r1) d/da1 of the terms in b^o (a polynomial in a2 per
 // nucleus), b' = (1 + r12)^-2, b'' = -2 b'/(1 + r12).  A zero-length unit vector (a point on a nucleus,
 // r12 = 0) and the 1/r terms that go with it contribute zero; everything else is kept.
@@ -157,13 +160,14 @@ __device__ __forceinline__ double from_fixed(long long v, int s) {
 }
 // x t, t a fraction from unit_fixed.
 __device__ __forceinline__ long long mulf(long long x, long long t) { return mulh<2>(x, t); }
-// Exponent e with |x| < 2^e (x finite).
+// Exponent e with |x| < 2^e (x finite); 0 for 0, so that sums of no terms stay clear of the rare forms.
 __device__ __forceinline__ int exponent_above(double x) {
-  return max(static_cast<int>((__double_as_longlong(x) >> 52) & 0x7ff), 1) - 1022;
+  return x == 0.0 ? 0 : max(static_cast<int>((__double_as_longlong(x) >> 52) & 0x7ff), 1) - 1022;
 }
 
 // The fixed-point coefficients of an outer point.  Scales: a.. of nucleus I by 2^(61 - e_I), e_I bounding the sum of their
-// magnitudes; g of nucleus I so that their products, and K, carry 2^sE; b.. and Hc 2^sH, L 2^sL.
+// magnitudes; g of nucleus I so that their products, and K, carry 2^sE; b1. and Hc1 2^sH1, b2. and Hc2 2^sH2 (one scale
+// where F is not asked for), L 2^sL.
 struct NucFix {
   long long a01, a02, a11, a12, a21, a22, g[3];
   long long b11, b12, b21, b22;
@@ -171,12 +175,13 @@ struct NucFix {
 };
 struct PointFix {
   long long K[3][3], Hc1, Hc2, L[3];
-  int sE, sH, sL;
+  int sE, sH1, sH2, sL;
 };
 __device__ __forceinline__ double bound_a(const NucCoef& q) {
   return fabs(q.a01) + fabs(q.a02) + fabs(q.a11) + fabs(q.a12) + 2.0 * (fabs(q.a21) + fabs(q.a22));
 }
 // Threads 0, 1, 2: the scales of E, H and L.
+template <bool LAP>
 __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef* nuc, int n_nuc, int k, PointFix& f) {
   double s = 0.0, s2 = 0.0, s3 = 0.0;
   if (k == 0) {
@@ -191,7 +196,8 @@ __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef*
       s += fabs(nuc[I].b11) + fabs(nuc[I].b12);
       s2 += fabs(nuc[I].b21) + fabs(nuc[I].b22);
     }
-    f.sH = 60 - exponent_above(fmax(s, s2));
+    f.sH1 = 60 - exponent_above(LAP ? s : fmax(s, s2));
+    f.sH2 = 60 - exponent_above(LAP ? s2 : fmax(s, s2));
   } else {
     s = fabs(pt.L[0]);
     s2 = fabs(pt.L[1]);
@@ -213,10 +219,10 @@ __device__ __forceinline__ void nuc_fix(const NucCoef& q, const PointFix& p, Nuc
   f.a21 = to_fixed(q.a21, sa);
   f.a22 = to_fixed(q.a22, sa);
   for (int x = 0; x < 3; ++x) f.g[x] = halves(to_fixed(q.g[x], sg));
-  f.b11 = to_fixed(q.b11, p.sH);
-  f.b12 = to_fixed(q.b12, p.sH);
-  f.b21 = to_fixed(q.b21, p.sH);
-  f.b22 = to_fixed(q.b22, p.sH);
+  f.b11 = to_fixed(q.b11, p.sH1);
+  f.b12 = to_fixed(q.b12, p.sH1);
+  f.b21 = to_fixed(q.b21, p.sH2);
+  f.b22 = to_fixed(q.b22, p.sH2);
   for (int o = 0; o < 3; ++o)
     for (int k = 0; k < 2; ++k) f.L[o][k] = to_fixed(q.L[o][k], p.sL);
 }
@@ -275,7 +281,7 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
       (k < 9 ? pt.K[k / 3][k % 3] : (k == 9 ? pt.Hc1 : (k == 10 ? pt.Hc2 : pt.L[k - 11]))) = s;
     }
     __syncthreads();
-    if (threadIdx.x < 3) point_scales(pt, nuc, n_nuc, threadIdx.x, pf);
+    if (threadIdx.x < 3) point_scales<LAP>(pt, nuc, n_nuc, threadIdx.x, pf);
     __syncthreads();
     for (int I = threadIdx.x; I < n_nuc; I += THREADS) nuc_fix(nuc[I], pf, nf[I]);
     if (threadIdx.x < 14) {
@@ -283,12 +289,12 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
       if (k < 9)
         pf.K[k / 3][k % 3] = to_fixed(pt.K[k / 3][k % 3], pf.sE);
       else if (k < 11)
-        (k == 9 ? pf.Hc1 : pf.Hc2) = to_fixed(k == 9 ? pt.Hc1 : pt.Hc2, pf.sH);
+        (k == 9 ? pf.Hc1 : pf.Hc2) = to_fixed(k == 9 ? pt.Hc1 : pt.Hc2, k == 9 ? pf.sH1 : pf.sH2);
       else
         pf.L[k - 11] = to_fixed(pt.L[k - 11], pf.sL);
     }
     __syncthreads();
-    const int sE = pf.sE, sH = pf.sH, sL = pf.sL;
+    const int sE = pf.sE, sH1 = pf.sH1, sH2 = pf.sH2, sL = pf.sL;
     // ------------------------------------------------------------ the row in FP64, and its largest exponents
     int mx[NC];
 #pragma unroll
@@ -329,7 +335,8 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
           l2 += mulf(q.L[2][0] + mulf(q.L[2][1], A), A);
         }
       }
-      const double h = from_fixed(h1 + mulf(h2, B), sH);
+      const double h1d = LAP ? from_fixed(h1, sH1) : 0.0;
+      const double h = LAP ? fma(b, from_fixed(h2, sH2), h1d) : from_fixed(h1 + mulf(h2, B), sH1);
       const double s = bp * i12, hs = h * s;   // b' e12 = s d
       const double gx = fma(hs, dx, from_fixed(e[0], sE)), gy = fma(hs, dy, from_fixed(e[1], sE)),
                    gz = fma(hs, dz, from_fixed(e[2], sE));
@@ -337,8 +344,9 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
       if (LAP) {
         const double fx = from_fixed(fe[0], sE), fy = from_fixed(fe[1], sE), fz = from_fixed(fe[2], sE);
         double f = from_fixed(l0 + mulf(l1 + mulf(l2, B), B), sL);
-        f = fma(from_fixed(h2, sH) * bp, bp, f);
-        const double t = fma(s, fma(dx, fx, fma(dy, fy, dz * fz)), (h * bp) * (i12 - s12));
+        // where 1/r12 counts as 0: h2 b'^2 - 2 H b' / (1+r12)
+        f = fma(from_fixed(apart ? 3 * h2 : h2, sH2) * bp, bp, f);
+        const double t = fma(s, fma(dx, fx, fma(dy, fy, dz * fz)), (apart ? h1d * s : -(h * bp)) * s12);
         f = fma(2.0, t, f);
         f = fma(gx, gx, fma(gy, gy, fma(gz, gz, f)));
         v[NC == 1 ? 0 : 3] = f;
