@@ -110,6 +110,9 @@ __device__ __forceinline__ void nuc_coef(const JastrowParams& jp, int I, double 
 }
 
 // ------------------------------------------------------------------ fixed point
+// Scale of coefficients whose magnitudes do not add up to a finite number (infinities, NaN, sums beyond the FP64
+// range): what is evaluated from them is NaN (from_fixed_rare, which every value of such a scale goes through).
+constexpr int NO_RANGE = 1 << 20;
 // x 2^s as an integer, rounded to nearest (|x| 2^s < 2^63).
 __device__ __forceinline__ long long to_fixed(double x, int s) {
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
@@ -143,7 +146,9 @@ __device__ __forceinline__ long long unit_fixed(double x) {
 }
 // The rare forms out of line: inlined they are predicated, and their FP64 instructions issue for every pair (45 of
 // 81 a pair before).
-__device__ __noinline__ double from_fixed_rare(long long v, int s) { return scalbn(static_cast<double>(v), -s); }
+__device__ __noinline__ double from_fixed_rare(long long v, int s) {
+  return s == NO_RANGE ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(static_cast<double>(v), -s);
+}
 __device__ __noinline__ double sqrt_rare(double x) { return sqrt(x); }
 __device__ __noinline__ double rsqrt_rare(double x) { return 1.0 / sqrt(x); }
 __device__ __noinline__ double rcp_rare(double x) { return 1.0 / x; }
@@ -180,15 +185,20 @@ struct PointFix {
 __device__ __forceinline__ double bound_a(const NucCoef& q) {
   return fabs(q.a01) + fabs(q.a02) + fabs(q.a11) + fabs(q.a12) + 2.0 * (fabs(q.a21) + fabs(q.a22));
 }
+__device__ __forceinline__ int scale_of(double sum, int bits) {
+  return sum < INFINITY ? bits - exponent_above(sum) : NO_RANGE;   // NaN is not below
+}
+// The larger of two magnitudes, NaN if either is (fmax would drop it).
+__device__ __forceinline__ double nan_max(double a, double b) { return b <= a ? a : (a <= b ? b : a + b); }
 // Threads 0, 1, 2: the scales of E, H and L.
 template <bool LAP>
 __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef* nuc, int n_nuc, int k, PointFix& f) {
   double s = 0.0, s2 = 0.0, s3 = 0.0;
   if (k == 0) {
-    for (int x = 0; x < 3; ++x) s = fmax(s, fabs(pt.K[0][x]) + fabs(pt.K[1][x]) + 2.0 * fabs(pt.K[2][x]));
+    for (int x = 0; x < 3; ++x) s = nan_max(s, fabs(pt.K[0][x]) + fabs(pt.K[1][x]) + 2.0 * fabs(pt.K[2][x]));
     for (int I = 0; I < n_nuc; ++I)
-      s += bound_a(nuc[I]) * fmax(fabs(nuc[I].g[0]), fmax(fabs(nuc[I].g[1]), fabs(nuc[I].g[2])));
-    f.sE = 61 - exponent_above(s);
+      s += bound_a(nuc[I]) * nan_max(fabs(nuc[I].g[0]), nan_max(fabs(nuc[I].g[1]), fabs(nuc[I].g[2])));
+    f.sE = scale_of(s, 61);
   } else if (k == 1) {
     s = fabs(pt.Hc1);
     s2 = fabs(pt.Hc2);
@@ -196,8 +206,8 @@ __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef*
       s += fabs(nuc[I].b11) + fabs(nuc[I].b12);
       s2 += fabs(nuc[I].b21) + fabs(nuc[I].b22);
     }
-    f.sH1 = 60 - exponent_above(LAP ? s : fmax(s, s2));
-    f.sH2 = 60 - exponent_above(LAP ? s2 : fmax(s, s2));
+    f.sH1 = scale_of(LAP ? s : nan_max(s, s2), 60);
+    f.sH2 = scale_of(LAP ? s2 : nan_max(s, s2), 60);
   } else {
     s = fabs(pt.L[0]);
     s2 = fabs(pt.L[1]);
@@ -207,7 +217,7 @@ __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef*
       s2 += fabs(nuc[I].L[1][0]) + fabs(nuc[I].L[1][1]);
       s3 += fabs(nuc[I].L[2][0]) + fabs(nuc[I].L[2][1]);
     }
-    f.sL = 59 - exponent_above(fmax(s, fmax(s2, s3)));
+    f.sL = scale_of(nan_max(s, nan_max(s2, s3)), 59);
   }
 }
 __device__ __forceinline__ void nuc_fix(const NucCoef& q, const PointFix& p, NucFix& f) {
