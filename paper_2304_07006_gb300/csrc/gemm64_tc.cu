@@ -31,11 +31,10 @@
 // B tile is loaded plane after plane, so its rows are contiguous), and writes diagonals i..7, which
 // are adjacent columns of the accumulator set.  Warp 0 loads (A planes through a ring of ten 16 KB
 // slots, B tiles through two of 32 KB), warp 1 issues the MMAs, warps 2..9 drain.  Every wait is bounded.
-#include <algorithm>
-
 #include <cuda_fp16.h>
 
 #include "digits64.cuh"
+#include "gemm_rules.h"
 #include "ptx_sm100.cuh"
 #include "xtc_internal.cuh"
 
@@ -444,27 +443,6 @@ __global__ void point_scale_k_kernel(const double* __restrict__ phiT, const doub
 }
 
 }  // namespace
-
-int gemm64_splits(int m_tiles, int n_tiles, int n_ranges, int n_sm) {
-  // Few tiles: slices of k (of at least 8 ranges) so that the waves of CTAs are full, the count with the
-  // least (waves x ranges of a slice), a CTA's start and end counted as 6 ranges; with eight waves or
-  // more the last one matters little.  At most 8,192 ranges per slice: the 64-bit sums cannot overflow.
-  const int64_t tiles = static_cast<int64_t>(m_tiles) * n_tiles;
-  int best = 1;
-  if (tiles < 8 * static_cast<int64_t>(n_sm)) {
-    int64_t best_cost = -1;
-    for (int s = 1; s <= std::max(1, std::min(n_ranges / 8, 2 * n_sm)); ++s) {
-      const int64_t cost = (tiles * s + n_sm - 1) / n_sm * ((n_ranges + s - 1) / s + 6);
-      if (best_cost < 0 || cost < best_cost) {
-        best_cost = cost;
-        best = s;
-      }
-    }
-  }
-  best = std::max(best, (n_ranges + 8191) / 8192);
-  const int per = (n_ranges + best - 1) / best;
-  return (n_ranges + per - 1) / per;
-}
 
 size_t gemm64_tile_bytes(int m_tiles, int n_tiles, int splits) {
   return static_cast<size_t>(m_tiles) * n_tiles * splits * BM * BN * sizeof(double);

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/xtc.h"
+#include "gemm_rules.h"
 #include "xtc_internal.cuh"
 
 using namespace xtc;

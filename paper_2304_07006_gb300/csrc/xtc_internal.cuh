@@ -230,7 +230,6 @@ struct Gemm64Out {
   const int* pair_p;
   const int* pair_q;
 };
-int gemm64_splits(int m_tiles, int n_tiles, int n_ranges, int n_sm);
 size_t gemm64_tile_bytes(int m_tiles, int n_tiles, int splits);
 void launch_gemm64(const CUtensorMap* tm_a, const CUtensorMap* tm_b, const Gemm64Args& a, int splits,
                    cudaStream_t st);
