@@ -33,4 +33,31 @@ inline int gemm64_splits(int m_tiles, int n_tiles, int n_ranges, int n_sm) {
   return (n_ranges + per - 1) / per;
 }
 
+// Slices of a step (d) GEMM's K of n ranges, when its tiles leave pairs of SMs idle (10 of 76 pairs at N = 23).  Its sums are
+// FP32 chains between FP64 flushes, column c of a thread's `cols` being flushed after the ranges r with r % flush = c: a
+// slice that starts at a multiple of the flush interval and runs `cols` ranges past its end holds whole chains of every
+// column, and whole periods of the cross-product accumulators (x_period ranges), so that every FP32 sum is the unsliced
+// one.  The price is the overlap, `cols` ranges a slice.  The count with the least (waves of tiles on `slots` x (ranges of a
+// slice + 30 for its start and end)), at most 16, if that saves 5 %; *flushes receives the flush intervals of a slice.
+// Measured, step (d) unsliced -> sliced: N = 23, 3,957 points 154 -> 106 us; two GEMMs of N = 40, 20,000 points 1.45 -> 0.74
+// ms; N = 65, 24,001 points (153 pairs of tiles, one more than two waves) 2.69 -> 2.33 ms.
+inline int chain_slices(int n, int flush, int x_period, int cols, int tiles, int slots, int* flushes) {
+  int best = 1;
+  if (flush < cols || flush % cols || cols % x_period) return best;
+  int64_t best_cost = static_cast<int64_t>((tiles + slots - 1) / slots) * (n + 30);
+  for (int q = (n - 1) / flush; q >= 1; --q) {
+    const int z = (n + q * flush - 1) / (q * flush);
+    if (z > 16) break;
+    if (n - (z - 1) * q * flush <= cols) continue;   // the last slice holds the end of every column's chains
+    const int64_t cost =
+        (static_cast<int64_t>(tiles) * z + slots - 1) / slots * (std::min(n, q * flush + cols) + 30);
+    if (cost < best_cost - best_cost / 20) {
+      best_cost = cost;
+      best = z;
+      *flushes = q;
+    }
+  }
+  return best;
+}
+
 }  // namespace xtc

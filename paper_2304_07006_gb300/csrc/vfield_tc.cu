@@ -54,6 +54,7 @@
 // Its accumulation is not exact: the truncation bias is only kept small by the short ranges.
 #include <algorithm>
 
+#include "gemm_rules.h"
 #include "ptx_sm100.cuh"
 #include "xtc_internal.cuh"
 
@@ -712,33 +713,14 @@ int launch_ctas(const VfieldArgs& a, int n, int splits) {
 
 }  // namespace
 
-// Slices of a step (d) GEMM's K, when its tiles leave pairs of SMs idle (10 of 76 pairs at N = 23).  Its sums are FP32
-// chains between FP64 flushes, column c of a thread being flushed after the ranges r with r % flush = c: a slice that
-// starts at a multiple of the flush interval and runs XB_HC ranges past its end holds whole chains of every column, and
-// whole periods of the cross-product accumulators, so that every FP32 sum is the unsliced one.  The price is
-// the overlap, XB_HC ranges a slice.  The count with the least (waves x (ranges of a slice + 30 for its start and
-// end)); measured,
-// step (d) unsliced -> sliced: N = 23, 3,957 points 154 -> 106 us; two GEMMs of N = 40, 20,000 points 1.45 -> 0.74
-// ms; N = 65, 24,001 points (153 pairs of tiles, one more than two waves) 2.69 -> 2.33 ms.
 int chain_slices(const VfieldArgs& a, int* kb_per_slice) {
-  const int n = a.n_kb / a.kd, tiles = static_cast<int>(tile_ctas(a) / 2), slots = std::max(1, a.n_sm / 2);
-  int best = 1;
   *kb_per_slice = a.n_kb;
-  const int x_period = 2 * std::max(1, a.xper / (2 * a.kd));
-  if (a.mode != 1 || a.n_kb % a.kd || a.flush < XB_HC || a.flush % XB_HC || XB_HC % x_period || a.kd < 2) return best;
-  int64_t best_cost = static_cast<int64_t>((tiles + slots - 1) / slots) * (n + 30);
-  for (int q = (n - 1) / a.flush; q >= 1; --q) {   // flush intervals of a slice
-    const int z = (n + q * a.flush - 1) / (q * a.flush);
-    if (z > 16) break;
-    if (n - (z - 1) * q * a.flush <= XB_HC) continue;   // the last slice holds the end of every column's chains
-    const int64_t cost = (static_cast<int64_t>(tiles) * z + slots - 1) / slots * (std::min(n, q * a.flush + XB_HC) + 30);
-    if (cost < best_cost - best_cost / 20) {
-      best_cost = cost;
-      best = z;
-      *kb_per_slice = q * a.flush * a.kd;
-    }
-  }
-  return best;
+  if (a.mode != 1 || a.n_kb % a.kd || a.kd < 2) return 1;
+  int flushes = 0;
+  const int z = chain_slices(a.n_kb / a.kd, a.flush, 2 * std::max(1, a.xper / (2 * a.kd)), XB_HC,
+                             static_cast<int>(tile_ctas(a) / 2), std::max(1, a.n_sm / 2), &flushes);
+  if (z > 1) *kb_per_slice = flushes * a.flush * a.kd;
+  return z;
 }
 
 bool vfield_tc_supported(int n_nuc) { return n_nuc >= 1 && n_nuc <= 8; }
