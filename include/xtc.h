@@ -287,8 +287,11 @@ XTC_API int xtc_three_body_L(xtc_ctx* ctx, int64_t n_grid, int n_orb, const doub
  *   K    [n_orb]^4 FP64, host or device memory (n_orb = 120: 1.66 GB)
  * The vector pair field V (steps a and b) is formed in the context's precision; the Laplacian
  * term, its product with the pair densities and the contraction are FP64 (as XTC_PREC_FP64).  Workspace:
- * n_orb^2 x n_pair doubles, up to 32 GB of digits of the operands of the pair fields, and about 10 GB per
- * chunk of outer points (the context's grid_chunk, else chosen by the budgets).  Synchronous.  Requires xtc_set_jastrow.  Errors: XTC_ERR_ARG,
+ * n_orb^2 x n_pair doubles and about as many again per slice of the contraction (its tile sums), up to 32 GB
+ * of digits of the operands of the pair fields, and about 10 GB per chunk of outer points (the context's
+ * grid_chunk, else chosen by the budgets); where that does not fit, the digits are formed in smaller blocks
+ * (so in XTC_PREC_FP64 builds), and XTC_ERR_OOM is returned only when the smallest do not fit either.
+ * Synchronous.  Requires xtc_set_jastrow.  Errors: XTC_ERR_ARG,
  * XTC_ERR_STATE, XTC_ERR_NONFINITE (grid, weights, orbitals or their gradients), XTC_ERR_OOM,
  * XTC_ERR_CUDA and those of xtc_vfield. */
 #define XTC_TWO_BODY_K_MAX_ORB 200

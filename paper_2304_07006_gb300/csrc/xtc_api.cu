@@ -515,6 +515,24 @@ int check_device_error(xtc_ctx* ctx) {
   return XTC_OK;
 }
 
+// Runs a call that cuts operands into digits (`digits`); when its workspace does not fit the memory that is left, again with
+// blocks an eighth the size, down to the smallest (128 points), and reports XTC_ERR_OOM when those do not fit either.  The
+// context keeps the size that fitted.  The default blocks (up to 38 GB) are many times what the FP64 tables would take: without
+// this, calls on a nearly full GPU that ran with FP64 tables were refused (4,000 points, 12 orbitals: 0.8 GB for 2.5 MB).
+// Every call starts from its inputs and zeroed sums.
+template <typename F>
+int fit_blocks(xtc_ctx* ctx, bool digits, F&& call) {
+  const double budget = ctx->d64_budget;
+  int rc = call();
+  while (rc == XTC_ERR_OOM && digits && ctx->d64_budget > 1e-6) {
+    for (DBuf* b : {&ctx->d_rho, &ctx->d_G, &ctx->d_tmp, &ctx->d_L, &ctx->d_R, &ctx->k_W, &ctx->Vacc}) release(*b);
+    ctx->d64_budget *= 0.125;
+    rc = call();
+  }
+  if (rc == XTC_ERR_OOM) ctx->d64_budget = budget;
+  return rc;
+}
+
 // Tables of the FP64 contractions over the inner points: per-point table, digits of rho^T when the whole
 // grid is one block (else they are formed block by block), room for the digits of `comps` pair functions.
 int prepare64(xtc_ctx* ctx, Plan& pl, int comps, const double* d_grid, const double* d_w) {
@@ -862,7 +880,7 @@ struct Pass {
   DBuf* M2;
 };
 
-int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, const double* weights,
+int build_once(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, const double* weights,
                const double* phi, const double* const* gammas, const BuildOut& out) {
   NvtxRange nvtx_build(out.n_spin == 2 ? "xtc build (spin)" : "xtc build");
   CUDA_OK(cudaSetDevice(ctx->prm.device));
@@ -1211,6 +1229,12 @@ int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
   return XTC_OK;
 }
 
+int build_impl(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, const double* weights,
+               const double* phi, const double* const* gammas, const BuildOut& out) {
+  return fit_blocks(ctx, ctx->prm.precision == XTC_PREC_FP64,
+                    [&] { return build_once(ctx, n_grid, n_orb, grid_xyz, weights, phi, gammas, out); });
+}
+
 }  // namespace
 
 extern "C" int xtc_build_1b2b(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, const double* weights,
@@ -1271,9 +1295,10 @@ extern "C" int xtc_jastrow_grad(xtc_ctx* ctx, int64_t n, const double* r1, const
   return XTC_OK;
 }
 
-extern "C" int xtc_vfield(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, const double* weights,
-                          const double* phi, int64_t outer_begin, int64_t outer_end, double* V) {
-  if (!ctx) return XTC_ERR_ARG;
+namespace {
+
+int vfield_once(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, const double* weights,
+                const double* phi, int64_t outer_begin, int64_t outer_end, double* V) {
   if (!V || outer_begin < 0 || outer_end < outer_begin || outer_end > n_grid)
     return fail(ctx, XTC_ERR_ARG, "bad outer range or null output");
   CUDA_OK(cudaSetDevice(ctx->prm.device));
@@ -1311,6 +1336,16 @@ extern "C" int xtc_vfield(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double*
   if ((rc = check_device_error(ctx))) return rc;
   finish_timers(ctx);
   return XTC_OK;
+}
+
+}  // namespace
+
+extern "C" int xtc_vfield(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, const double* weights,
+                          const double* phi, int64_t outer_begin, int64_t outer_end, double* V) {
+  if (!ctx) return XTC_ERR_ARG;
+  return fit_blocks(ctx, ctx->prm.precision == XTC_PREC_FP64, [&] {
+    return vfield_once(ctx, n_grid, n_orb, grid_xyz, weights, phi, outer_begin, outer_end, V);
+  });
 }
 
 // ====================================================================== bounded-wait self-test
@@ -1497,9 +1532,10 @@ extern "C" int xtc_three_body_L(xtc_ctx* ctx, int64_t n_grid, int n_orb, const d
 // K_pr^qs of the Theory section on the grid: per chunk of outer points V (steps a+b, the
 // context's precision), W (the FP64 contraction with F = lap_1 u + |grad_1 u|^2) and the FP64 sum S
 // of two_body_k.cu; then K[p][q][r][s] = S[pq][rs] + S[rs][pq].
-extern "C" int xtc_two_body_K(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz,
-                              const double* weights, const double* phi, const double* dphi, double* K) {
-  if (!ctx) return XTC_ERR_ARG;
+namespace {
+
+int two_body_K_once(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, const double* weights,
+                    const double* phi, const double* dphi, double* K) {
   if (!K || !dphi || n_orb < 1 || n_orb > XTC_TWO_BODY_K_MAX_ORB || n_grid < 1 || !grid_xyz || !weights || !phi)
     return fail(ctx, XTC_ERR_ARG, "two_body_K: null pointer, n_grid < 1 or n_orb outside 1..%d",
                 XTC_TWO_BODY_K_MAX_ORB);
@@ -1581,6 +1617,15 @@ extern "C" int xtc_two_body_K(xtc_ctx* ctx, int64_t n_grid, int n_orb, const dou
   if (!out_dev) CUDA_OK(cudaMemcpyAsync(K, Kd, n4 * 8, cudaMemcpyDeviceToHost, st));
   if ((rc = check_device_error(ctx))) return rc;
   return XTC_OK;
+}
+
+}  // namespace
+
+extern "C" int xtc_two_body_K(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz,
+                              const double* weights, const double* phi, const double* dphi, double* K) {
+  if (!ctx) return XTC_ERR_ARG;
+  return fit_blocks(ctx, true,
+                    [&] { return two_body_K_once(ctx, n_grid, n_orb, grid_xyz, weights, phi, dphi, K); });
 }
 
 // ====================================================================== internal accessors
