@@ -395,7 +395,11 @@ int xtc_create(xtc_ctx** out, const xtc_params* p) {
   if (const char* s = std::getenv("XTC_VF_KD")) ctx->vf_kd = std::max(1, std::atoi(s));
   if (const char* s = std::getenv("XTC_AS_KD")) ctx->as_kd = std::max(1, std::atoi(s));
   if (const char* s = std::getenv("XTC_VF_FLUSH")) ctx->vf_flush = std::max(0, std::atoi(s));
-  if (const char* s = std::getenv("XTC_D64_BUDGET")) ctx->d64_budget = std::atof(s);
+  if (const char* s = std::getenv("XTC_D64_BUDGET")) {
+    // a scale of the budgets; what is not one (text, NaN, zero, sizes beyond any GPU) leaves the default
+    const double v = std::strtod(s, nullptr);
+    if (v > 0.0 && v <= 1024.0) ctx->d64_budget = v;
+  }
   if (const char* s = std::getenv("XTC_X_PERIOD")) ctx->x_period = std::max(1, std::atoi(s));
   if (p->range_stages > 0) ctx->vf_kd = ctx->as_kd = p->range_stages;
   if (!ensure(ctx->jp_dev, sizeof(JastrowParams)) || !ensure(ctx->err_dev, 16) || !ensure(ctx->flag_dev, 16)) {

@@ -81,3 +81,17 @@ def test_memory_too_small_for_any_block_is_refused(problem):
     with _ctx(p, "fp64") as c:
         want = c.build(p.grid, p.weights, p.phi, p.gamma)
     assert np.abs(out["dU"] - want["dU"]).max() <= 1e-14 * np.abs(want["dU"]).max()
+
+
+@pytest.mark.parametrize("text", ["nan", "inf", "-1", "0", "1e300", "junk", ""])
+def test_a_budget_scale_that_is_none_leaves_the_default(monkeypatch, problem, text):
+    p, _ = problem
+    peaks = []
+    for value in (None, text):
+        if value is not None:
+            monkeypatch.setenv("XTC_D64_BUDGET", value)
+        a = _Allocator(8 << 30)
+        with _ctx(p, "fp64", a) as c:
+            c.vfield(p.grid, p.weights, p.phi, 0, 256)
+        peaks.append(a.peak)
+    assert peaks[0] == peaks[1]
