@@ -66,8 +66,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return true;
 }
 
-// The same with a non-suspending test in a tight loop, where the wake-up latency of a suspended wait sits on the critical
-// path: mbar_spin_warp below, for the warps that issue MMAs or drain their accumulators.
+// A non-suspending test, for loops where the wake-up latency of a suspended wait sits on the critical path
+// (mbar_spin_warp below: the warps that issue MMAs or drain their accumulators).
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -79,15 +79,18 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool mbar_spin(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err,
-                                          int code, unsigned long long limit_ns = TIMEOUT_NS) {
+// A warp's wait: every lane polls, and the warp votes on every poll, so that all take one verdict and stay together.  With a
+// verdict for each lane a wait that runs out in one while the barrier completes for another would send the lanes
+// to different warp-wide instructions (elect.sync, tcgen05.ld), which then wait for each other without a bound.
+__device__ __forceinline__ bool mbar_spin_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err, int code,
+                                               unsigned long long limit_ns = TIMEOUT_NS) {
   unsigned long long t0 = 0;
   uint32_t it = 0;
-  while (!mbar_test(bar, parity)) {
+  while (!__all_sync(0xffffffffu, mbar_test(bar, parity))) {
     if ((++it & 255u) == 0) {
-      if (*abort_flag) return false;
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
       if (t0 == 0) t0 = global_timer_ns();  // not on the first failures: reading the timer is slow
-      if (global_timer_ns() - t0 > limit_ns) {
+      if (__any_sync(0xffffffffu, global_timer_ns() - t0 > limit_ns)) {
         *abort_flag = 1;
         atomicExch(err, code);
         return false;
@@ -97,12 +100,23 @@ __device__ __forceinline__ bool mbar_spin(uint64_t* bar, uint32_t parity, volati
   return true;
 }
 
-// A warp's wait: every lane polls, and all take one verdict.  Without the vote a wait that runs out in one lane while
-// the barrier completes for another would send the lanes to different warp-wide instructions (elect.sync, tcgen05.ld), which
-// then wait for each other without a bound.
-__device__ __forceinline__ bool mbar_spin_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err, int code,
-                                               unsigned long long limit_ns = TIMEOUT_NS) {
-  return __all_sync(0xffffffffu, mbar_spin(bar, parity, abort_flag, err, code, limit_ns));
+// The same with one vote at the end, each lane polling by itself until then: a wait that sees a little later.
+__device__ __forceinline__ bool mbar_spin_vote(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* err, int code) {
+  unsigned long long t0 = 0;
+  uint32_t it = 0;
+  bool ok;
+  while (!(ok = mbar_test(bar, parity))) {
+    if ((++it & 255u) == 0) {
+      if (*abort_flag) break;
+      if (t0 == 0) t0 = global_timer_ns();
+      if (global_timer_ns() - t0 > TIMEOUT_NS) {
+        *abort_flag = 1;
+        atomicExch(err, code);
+        break;
+      }
+    }
+  }
+  return __all_sync(0xffffffffu, ok);
 }
 
 // ------------------------------------------------------------------ proxies / TMA
