@@ -21,13 +21,16 @@ __device__ __forceinline__ int block_max(int v, int* scratch) {
   return v;
 }
 
-// Biased exponent of x 2^s, to be maximised over a row: 0 for x = 0, D64_NONFINITE for infinities and NaN.
+// Biased exponent of x 2^s, to be maximised over a row: 0 for x = 0, D64_NONFINITE for infinities and NaN.  That of a
+// subnormal value is its own, down to -51: a density of 1e-320 at a far point, brought up by its point's scale, would
+// otherwise count for up to 2^52 times its size, and its row lose as many bits.
 constexpr int D64_BIAS = 1 << 16;
 __device__ __forceinline__ int d64_key(double x, int s) {
-  const int hi = __double2hiint(x) & 0x7fffffff;
-  if ((hi | __double2loint(x)) == 0 || s == D64_NO_SCALE) return 0;
+  const int hi = __double2hiint(x) & 0x7fffffff, lo = __double2loint(x);
+  if ((hi | lo) == 0 || s == D64_NO_SCALE) return 0;
   const int ex = hi >> 20;
-  return ex == 0x7ff ? D64_NONFINITE : max(ex, 1) + s + D64_BIAS;
+  if (ex == 0) return (hi ? 12 - __clz(hi) : -20 - __clz(lo)) + s + D64_BIAS;
+  return ex == 0x7ff ? D64_NONFINITE : ex + s + D64_BIAS;
 }
 // Exponent e of a row (every |x 2^s| < 2^e) from the largest key.
 __device__ __forceinline__ int d64_exponent(int key) {
@@ -46,9 +49,11 @@ __device__ __forceinline__ Fixed72 d64_fixed(double x, int s, int e) {
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
   const int ex = static_cast<int>(b >> 52) & 0x7ff;
   const unsigned long long m = (b & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
-  const int sh = max(ex, 1) - 1004 - e + s;   // at most 18
+  const int sh = max(ex, 1) - 1004 - e + s;   // at most 18, subnormal values at most 70 (the value is below 2^71)
   unsigned long long lo = 0, hi = 0;
-  if (sh > 0) {
+  if (sh >= 64) {
+    hi = m << (sh - 64);
+  } else if (sh > 0) {
     lo = m << sh;
     hi = m >> (64 - sh);
   } else if (sh > -54) {
