@@ -16,8 +16,8 @@
 // brought to the same largest value), taken out of rho and multiplied into the pair functions: a row of those is then weighted as in the sum, and its
 // maximum is not set by points that contribute nothing (a neighbour of the outer point, a far point
 // with no density).  With seven digits and no such scales the error of the water-sized build was 1,500
-// times that of the FP64 pipe's sums.  Step (d) uses the same scales for rho and A, and the
-// contraction of K scales of its own (point_scale_k_kernel).
+// times that of the FP64 pipe's sums.  Step (d) uses the same scales for rho and A, others for
+// V and B (v_scale_kernel), and the contraction of K scales of its own (point_scale_k_kernel).
 //
 // Why: the FP64 pipe does 2 FMA per SM and clock on this GPU, the 128 x 32 x 64 FMA of one range of a
 // tile take 131,072 of its cycles; the same range is 36 fp16 products of 4 k-steps.  They are bound by shared
@@ -300,19 +300,23 @@ constexpr int DG_THREADS = 256;
 // at index k carry (and the other operand's do not): with s_j, the point scale, rho is of order 2^s_j at
 // point j, and what it multiplies is weighted by it.
 
-// Operand of step (d) from FP64 rows, k = 4 i + c: L = (rho, V) and R = (A, B) with A ~ V^2 and B ~ rho V, so
-// rho goes without its scale into L (sign -1) and A with it into R (sign +1).
+// Operand of step (d) from FP64 rows, k = 4 i + c: L = (rho, V) and R = (A, B).  Both parts of L go without their scales
+// (sign -1), sj for rho and sv for V (v_scale_kernel), which bring them to the heights of the pair's orbitals, and
+// those of R with them (sign +1).  With rho alone scaled, V kept what bits its size beside phi^2 left it: none of the
+// result's was right with weights of 1e-40 (sums of w phi^2 are 1 for orthonormal orbitals, but no input has to be).
 struct LrSrc {
   const double* p;
   int64_t ld, k0;           // first k of the block
   const int* sj;            // of the chunk's first point
+  const int* sv;
   int64_t n_i;
   int sign;
   __device__ double at(int64_t row, int64_t k) const { return p[row * ld + k]; }
   __device__ int scale(int64_t k) const {
     const int64_t i = (k0 + k) >> 2;
-    if (((k0 + k) & 3) || i >= n_i) return 0;
-    return sj[i] == D64_NO_SCALE ? D64_NO_SCALE : sign * sj[i];
+    if (i >= n_i) return 0;
+    const int s = (k0 + k) & 3 ? sv[i] : sj[i];
+    return s <= D64_NO_SCALE ? D64_NO_SCALE : sign * s;
   }
 };
 // rho^T[pq][j] = w_j phi_p(j) phi_q(j), times 2^-sj[j]
@@ -418,6 +422,26 @@ __global__ void point_scale_kernel(const double* __restrict__ phiT, int64_t ld, 
   sj[j] = m == D64_NO_SCALE || kw == 0 ? D64_NO_SCALE : kw - D64_BIAS - 1022 + 2 * m;
 }
 
+// sv[i], initially below D64_NO_SCALE: the exponent of max_pq,x |V_x,pq(i)| / (max phi_p max phi_q), from the rows of L; stays
+// below where V is 0.  One thread per point and VS_PAIRS pairs.
+constexpr int VS_PAIRS = 16;
+__global__ void __launch_bounds__(128) v_scale_kernel(const double* __restrict__ L, int64_t ld, int64_t n_i, int n_pair,
+                                                      const int* __restrict__ pair_p, const int* __restrict__ pair_q,
+                                                      const int* __restrict__ orb, int* __restrict__ sv) {
+  const int64_t i = blockIdx.x * 128ll + threadIdx.x;
+  if (i >= n_i) return;
+  const int pq0 = blockIdx.y * VS_PAIRS, pq1 = min(n_pair, pq0 + VS_PAIRS);
+  int m = D64_NO_SCALE;
+#pragma unroll 4
+  for (int pq = pq0; pq < pq1; ++pq) {
+    const double2* v = reinterpret_cast<const double2*>(L + pq * ld + 4 * i);
+    const double2 v0 = v[0], v1 = v[1];
+    const int k = max(d64_key(v0.y, 0), max(d64_key(v1.x, 0), d64_key(v1.y, 0)));
+    if (k && k < D64_NONFINITE) m = max(m, k - orb[pair_p[pq]] - orb[pair_q[pq]] + D64_BIAS + 1022);
+  }
+  if (m > D64_NO_SCALE) atomicMax(sv + i, m);
+}
+
 // si[i]: the exponent of |w_i| max_p (|phi_p(i)| / max |phi_p|) max_q (|phi_q(i)|, |d_x phi_q(i)|, / max of both), which the
 // left operand of K is of at point i; D64_NO_SCALE where that operand is 0.  orb[n_orb], dorb[3 n_orb]: largest keys.
 __global__ void point_scale_k_kernel(const double* __restrict__ phiT, const double* __restrict__ dphiT, int64_t ld,
@@ -469,10 +493,17 @@ void launch_gemm64_finalize(const Gemm64Args& a, int splits, const Gemm64Out& o,
     gemm64_finalize_kernel<ADD><<<g, BM, 0, st>>>(a, splits, o);
 }
 
-void launch_digits_lr(const double* src, int64_t rows, int64_t ld, int64_t k0, int64_t K, const int* sj, int64_t n_i,
-                      int sign, uint16_t* planes, int* exps, cudaStream_t st) {
+void launch_v_scale(const double* L, int64_t ld, int64_t n_i, int n_pair, const int* pair_p, const int* pair_q,
+                    const int* orb, int* sv, cudaStream_t st) {
+  cudaMemsetAsync(sv, 0x80, n_i * sizeof(int), st);   // below D64_NO_SCALE
+  v_scale_kernel<<<dim3(static_cast<unsigned>((n_i + 127) / 128), static_cast<unsigned>((n_pair + VS_PAIRS - 1) / VS_PAIRS)), 128,
+                   0, st>>>(L, ld, n_i, n_pair, pair_p, pair_q, orb, sv);
+}
+
+void launch_digits_lr(const double* src, int64_t rows, int64_t ld, int64_t k0, int64_t K, const int* sj, const int* sv,
+                      int64_t n_i, int sign, uint16_t* planes, int* exps, cudaStream_t st) {
   if (rows <= 0) return;
-  digits_kernel<<<static_cast<unsigned>(rows), DG_THREADS, 0, st>>>(LrSrc{src + k0, ld, k0, sj, n_i, sign}, K, K,
+  digits_kernel<<<static_cast<unsigned>(rows), DG_THREADS, 0, st>>>(LrSrc{src + k0, ld, k0, sj, sv, n_i, sign}, K, K,
                                                                     planes, rows * K, exps);
 }
 

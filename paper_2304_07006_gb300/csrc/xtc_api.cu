@@ -103,7 +103,7 @@ struct xtc_ctx {
   DBuf k_si;                       // and its point scales
   // digit planes and row exponents of the FP64 contractions: rho^T, the pair functions (with their
   // scratch rows), and the operands of step (d) or of the contraction of K
-  DBuf d_rho, d_rhoe, d_sj, d_G, d_Ge, d_tmp, d_L, d_Le, d_R, d_Re;
+  DBuf d_rho, d_rhoe, d_sj, d_sv, d_G, d_Ge, d_tmp, d_L, d_Le, d_R, d_Re;
   cudaStream_t st2 = nullptr;  // created on first use
   cudaEvent_t ev_g[2] = {nullptr, nullptr};  // gradient table b written
   cudaEvent_t ev_b[2] = {nullptr, nullptr};  // step (b) GEMM that read table b done
@@ -129,7 +129,7 @@ struct xtc_ctx {
     return {&jp_dev, &err_dev, &flag_dev, &grid, &w, &phi, &gamma, &phiT, &phi32, &pair_p, &pair_q, &jtab, &jtab64,
             &rho, &colmax, &colexp, &G, &gcoef, &V, &Vacc, &L, &R, &L32, &R32, &eL, &eR, &M, &evec, &lam, &dU_tmp,
             &dh_tmp, &e0_tmp, &vout, &r1, &r2, &lamd, &gamma_b, &M2, &M3, &lam2, &R2, &R32b, &eR2, &Lv, &T3,
-            &h_tmp, &fc_U, &fc_h, &fc_hout, &fc_Uout, &G2, &k_dphi, &k_dphiT, &k_W, &k_S, &k_si, &d_rho, &d_rhoe, &d_sj,
+            &h_tmp, &fc_U, &fc_h, &fc_hout, &fc_Uout, &G2, &k_dphi, &k_dphiT, &k_W, &k_S, &k_si, &d_rho, &d_rhoe, &d_sj, &d_sv,
             &d_G, &d_Ge, &d_tmp, &d_L, &d_Le, &d_R, &d_Re};
   }
 };
@@ -991,7 +991,7 @@ int build_once(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
   const int64_t kblk = block_of(ctx->d64_budget * D64_LR_BYTES, 2.0 * D64_BYTES * NP, kdim);
   if (pl.f64 && (!ensure(ctx->d_L, static_cast<size_t>(D64_BYTES) * kblk * NP) ||
                  !ensure(ctx->d_R, static_cast<size_t>(D64_BYTES) * kblk * NP) || !ensure(ctx->d_Le, 4ull * NP) ||
-                 !ensure(ctx->d_Re, 4ull * NP)))
+                 !ensure(ctx->d_Re, 4ull * NP) || !ensure(ctx->d_sv, 4ull * pl.gc)))
     return fail(ctx, XTC_ERR_OOM, "step (d) digits (%.2f GB)", 2.0 * D64_BYTES * kblk * NP / 1e9);
   VfMaps maps{};
   CUtensorMap tm_L{}, tm_R{}, tm_R2{}, tm_R16{}, tm_R216{};
@@ -1149,15 +1149,19 @@ int build_once(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_xyz, 
         }
       } else if (pl.f64) {
         // per block of k: the digits of L once, those of R and the contraction for each accumulator
+        timed(ctx, XTC_K_AUX, 1, [&] {
+          launch_v_scale(ctx->L.as<double>(), kdim, n_i, NP, ctx->pair_p.as<int>(), ctx->pair_q.as<int>(),
+                         ctx->d_sj.as<int>() + pl.NGp, ctx->d_sv.as<int>(), st);
+        });
         for (int64_t k0 = 0; k0 < kdim; k0 += kblk) {
           const int64_t kp = std::min(kblk, kdim - k0);
           timed(ctx, XTC_K_AUX, 1, [&] {
-            launch_digits_lr(ctx->L.as<double>(), NP, kdim, k0, kp, ctx->d_sj.as<int>() + c0, n_i, -1,
+            launch_digits_lr(ctx->L.as<double>(), NP, kdim, k0, kp, ctx->d_sj.as<int>() + c0, ctx->d_sv.as<int>(), n_i, -1,
                              ctx->d_L.as<uint16_t>(), ctx->d_Le.as<int>(), st);
           });
           for (int e = 0; e < (M2 ? 2 : 1); ++e) {
             timed(ctx, XTC_K_AUX, 1, [&] {
-              launch_digits_lr((e ? ctx->R2 : ctx->R).as<double>(), NP, kdim, k0, kp, ctx->d_sj.as<int>() + c0, n_i,
+              launch_digits_lr((e ? ctx->R2 : ctx->R).as<double>(), NP, kdim, k0, kp, ctx->d_sj.as<int>() + c0, ctx->d_sv.as<int>(), n_i,
                                1, ctx->d_R.as<uint16_t>(), ctx->d_Re.as<int>(), st);
             });
             Gemm64Out o{};

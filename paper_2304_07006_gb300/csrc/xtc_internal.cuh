@@ -234,18 +234,22 @@ size_t gemm64_tile_bytes(int m_tiles, int n_tiles, int splits);
 void launch_gemm64(const CUtensorMap* tm_a, const CUtensorMap* tm_b, const Gemm64Args& a, int splits,
                    cudaStream_t st);
 void launch_gemm64_finalize(const Gemm64Args& a, int splits, const Gemm64Out& o, int mode, cudaStream_t st);
-// Digits: FP64 rows of L (sign -1) or R (+1) from value k0 on, K of them, with the point scales of rho and A
-// (gemm64_tc.cu; sj: launch_point_scale, of the chunk's first point);
+// Digits: FP64 rows of L (sign -1) or R (+1) from value k0 on, K of them, with the point scales of rho and A (sj:
+// launch_point_scale, of the chunk's first point) and of V and B (sv: launch_v_scale);
 // rho^T[pq][j] 2^-sj[j] of n_j inner points; the operands of the contraction of K (left: rows p N + q from phi and
 // dphiT[3 q + x][j], right: rows of 4 ncp values, W and V) with the scales si of launch_point_scale_k, k = c ncp + i, point i0 + i.
-void launch_digits_lr(const double* src, int64_t rows, int64_t ld, int64_t k0, int64_t K, const int* sj, int64_t n_i,
-                      int sign, uint16_t* planes, int* exps, cudaStream_t st);
+void launch_digits_lr(const double* src, int64_t rows, int64_t ld, int64_t k0, int64_t K, const int* sj, const int* sv,
+                      int64_t n_i, int sign, uint16_t* planes, int* exps, cudaStream_t st);
 void launch_digits_rho(const double* phiT, int64_t ld, const double* w, int64_t n_j, int64_t Kp, int n_orb,
                        const int* pair_p, const int* pair_q, const int* sj, uint16_t* planes, int* exps,
                        cudaStream_t st);
 // sj[j]: exponent of |w_j| max_p (phi_p(j) / max phi_p)^2, the common scale of inner point j; orb[n_orb]: scratch.
 void launch_point_scale(const double* phiT, int64_t ld, const double* w, int64_t n_grid, int n_orb, int* orb, int* sj,
                         cudaStream_t st);
+// sv[i]: exponent of max |V_x,pq(i)| / (max phi_p max phi_q) over the rows of L (n_pair rows of ld, k = 4 i + c), at or
+// below D64_NO_SCALE where V is 0; orb: as written by launch_point_scale.
+void launch_v_scale(const double* L, int64_t ld, int64_t n_i, int n_pair, const int* pair_p, const int* pair_q,
+                    const int* orb, int* sv, cudaStream_t st);
 // si[i]: the exponent of the largest entry of K's left operand at point i, every orbital at one height; orb[4 n_orb]: scratch.
 void launch_point_scale_k(const double* phiT, const double* dphiT, int64_t ld, const double* w, int64_t n_grid,
                           int n_orb, int* orb, int* si, cudaStream_t st);
