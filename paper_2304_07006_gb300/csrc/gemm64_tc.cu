@@ -17,7 +17,8 @@
 // maximum is not set by points that contribute nothing (a neighbour of the outer point, a far point
 // with no density).  With seven digits and no such scales the error of the water-sized build was 1,500
 // times that of the FP64 pipe's sums.  Step (d) uses the same scales for rho and A, others for
-// V and B (v_scale_kernel), and the contraction of K scales of its own (point_scale_k_kernel).
+// V and B (v_scale_kernel), and the contraction of K those of rho and others for the
+// gradients (gradient_scale_kernel).
 //
 // Why: the FP64 pipe does 2 FMA per SM and clock on this GPU, the 128 x 32 x 64 FMA of one range of a
 // tile take 131,072 of its cycles; the same range is 36 fp16 products of 4 k-steps.  They are bound by shared
@@ -334,16 +335,26 @@ struct RhoSrc {
 };
 // Operands of the contraction of K, k = c ncp + i, i < n_i a point of the chunk (zero past them).  Left: row
 // pq = p N + q, c = 0: w phi_p phi_q / 2, c = 1..3: w phi_p d_x phi_q (dphiT row 3 q + x).  Right: W, V_x.  W grows as 1/r
-// next to a nucleus, where the weight is as small, so the points carry the scales of point_scale_k_kernel,
-// taken out of the left operand and multiplied into the right one.  Without them a point 1e-12 bohr from a
-// nucleus cost every row the bits of 1/r: 1e-10 of max |K| where FP64 sums give 1e-14.
+// next to a nucleus, where the weight is as small, and gradients have a length in them, so both kinds of k carry scales of their
+// own, sj (as in step (b)) and sg (gradient_scale_kernel), taken out of the left operand and multiplied into the right one.
+// Without any a point 1e-12 bohr from a nucleus cost every row the bits of 1/r, 1e-10 of max |K| where FP64 sums give
+// 1e-14; with one for both, a grid 1e-12 bohr across did.
 __device__ __forceinline__ int k_component(int64_t k, int64_t ncp) { return (k >= ncp) + (k >= 2 * ncp) + (k >= 3 * ncp); }
+// Scale of index k: sj and sg of the chunk's first point.
+__device__ __forceinline__ int k_scale(int64_t k, int64_t ncp, int64_t n_i, const int* sj, const int* sg, int sign) {
+  const int c = k_component(k, ncp);
+  const int64_t i = k - c * ncp;
+  if (i >= n_i) return 0;
+  const int s = c ? sg[i] : sj[i];
+  return s == D64_NO_SCALE ? D64_NO_SCALE : sign * s;
+}
 struct PsiSrc {
   const double* phiT;
   const double* dphiT;
   int64_t ld;
   const double* w;
-  const int* si;
+  const int* sj;
+  const int* sg;
   int64_t i0, n_i, ncp;
   int n_orb;
   __device__ double at(int64_t row, int64_t k) const {
@@ -354,21 +365,15 @@ struct PsiSrc {
     const double wp = w[g] * phiT[p * ld + g];
     return c == 0 ? 0.5 * wp * phiT[q * ld + g] : wp * dphiT[(3 * q + c - 1) * ld + g];
   }
-  __device__ int scale(int64_t k) const {
-    const int64_t i = k - k_component(k, ncp) * ncp;
-    if (i >= n_i) return 0;
-    return si[i0 + i] == D64_NO_SCALE ? D64_NO_SCALE : -si[i0 + i];
-  }
+  __device__ int scale(int64_t k) const { return k_scale(k, ncp, n_i, sj + i0, sg + i0, -1); }
 };
 struct WvSrc {
   const double* p;
-  const int* si;
+  const int* sj;
+  const int* sg;
   int64_t i0, n_i, ncp;
   __device__ double at(int64_t row, int64_t k) const { return p[row * 4 * ncp + k]; }
-  __device__ int scale(int64_t k) const {
-    const int64_t i = k - k_component(k, ncp) * ncp;
-    return i < n_i ? si[i0 + i] : 0;
-  }
+  __device__ int scale(int64_t k) const { return k_scale(k, ncp, n_i, sj + i0, sg + i0, 1); }
 };
 
 // One CTA per row: the row's largest exponent, then the digits of four consecutive k per thread.  The
@@ -442,28 +447,29 @@ __global__ void __launch_bounds__(128) v_scale_kernel(const double* __restrict__
   if (m > D64_NO_SCALE) atomicMax(sv + i, m);
 }
 
-// si[i]: the exponent of |w_i| max_p (|phi_p(i)| / max |phi_p|) max_q (|phi_q(i)|, |d_x phi_q(i)|, / max of both), which the
-// left operand of K is of at point i; D64_NO_SCALE where that operand is 0.  orb[n_orb], dorb[3 n_orb]: largest keys.
-__global__ void point_scale_k_kernel(const double* __restrict__ phiT, const double* __restrict__ dphiT, int64_t ld,
-                                     const double* __restrict__ w, int64_t n, int n_orb, const int* __restrict__ orb,
-                                     const int* __restrict__ dorb, int* __restrict__ si) {
+// sg[i]: the exponent of |w_i| max_p (|phi_p(i)| / max |phi_p|) max_q,x (|d_x phi_q(i)| / max |phi_q|), every orbital at one
+// height (an orbital that is 0 everywhere: at that of its gradient); D64_NO_SCALE where that is 0.  orb[n_orb],
+// dorb[3 n_orb]: largest keys of the orbitals and of their gradients.
+__global__ void gradient_scale_kernel(const double* __restrict__ phiT, const double* __restrict__ dphiT, int64_t ld,
+                                      const double* __restrict__ w, int64_t n, int n_orb, const int* __restrict__ orb,
+                                      const int* __restrict__ dorb, int* __restrict__ sg) {
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   int mp = D64_NO_SCALE, mq = D64_NO_SCALE;
 #pragma unroll 2
   for (int q = 0; q < n_orb; ++q) {
     const int k = d64_key(phiT[q * ld + i], 0);
-    int kd = k, top = orb[q];
+    int kd = 0, top = 0;
 #pragma unroll
     for (int x = 0; x < 3; ++x) {
       kd = max(kd, d64_key(dphiT[(3 * q + x) * ld + i], 0));
       top = max(top, dorb[3 * q + x]);
     }
     if (k) mp = max(mp, k - orb[q]);
-    if (kd) mq = max(mq, kd - top);
+    if (kd) mq = max(mq, kd - (orb[q] ? orb[q] : top));
   }
   const int kw = d64_key(w[i], 0);
-  si[i] = mp == D64_NO_SCALE || kw == 0 ? D64_NO_SCALE : kw - D64_BIAS - 1022 + mp + mq;
+  sg[i] = mp == D64_NO_SCALE || mq == D64_NO_SCALE || kw == 0 ? D64_NO_SCALE : kw - D64_BIAS - 1022 + mp + mq;
 }
 
 }  // namespace
@@ -521,24 +527,23 @@ void launch_point_scale(const double* phiT, int64_t ld, const double* w, int64_t
   point_scale_kernel<<<static_cast<unsigned>((n_grid + 127) / 128), 128, 0, st>>>(phiT, ld, w, n_grid, n_orb, orb, sj);
 }
 
-void launch_point_scale_k(const double* phiT, const double* dphiT, int64_t ld, const double* w, int64_t n_grid,
-                          int n_orb, int* orb, int* si, cudaStream_t st) {
-  orbital_key_kernel<<<n_orb, DG_THREADS, 0, st>>>(phiT, ld, n_grid, orb);
-  orbital_key_kernel<<<3 * n_orb, DG_THREADS, 0, st>>>(dphiT, ld, n_grid, orb + n_orb);
-  point_scale_k_kernel<<<static_cast<unsigned>((n_grid + 127) / 128), 128, 0, st>>>(phiT, dphiT, ld, w, n_grid, n_orb, orb,
-                                                                                 orb + n_orb, si);
+void launch_gradient_scale(const double* phiT, const double* dphiT, int64_t ld, const double* w, int64_t n_grid,
+                           int n_orb, const int* orb, int* dorb, int* sg, cudaStream_t st) {
+  orbital_key_kernel<<<3 * n_orb, DG_THREADS, 0, st>>>(dphiT, ld, n_grid, dorb);
+  gradient_scale_kernel<<<static_cast<unsigned>((n_grid + 127) / 128), 128, 0, st>>>(phiT, dphiT, ld, w, n_grid, n_orb,
+                                                                                  orb, dorb, sg);
 }
 
-void launch_digits_psi(const double* phiT, const double* dphiT, int64_t ld, const double* w, const int* si, int64_t i0,
-                       int64_t n_i, int64_t ncp, int n_orb, uint16_t* planes, int* exps, cudaStream_t st) {
+void launch_digits_psi(const double* phiT, const double* dphiT, int64_t ld, const double* w, const int* sj, const int* sg,
+                       int64_t i0, int64_t n_i, int64_t ncp, int n_orb, uint16_t* planes, int* exps, cudaStream_t st) {
   const int64_t rows = static_cast<int64_t>(n_orb) * n_orb;
   digits_kernel<<<static_cast<unsigned>(rows), DG_THREADS, 0, st>>>(
-      PsiSrc{phiT, dphiT, ld, w, si, i0, n_i, ncp, n_orb}, 4 * ncp, 4 * ncp, planes, rows * 4 * ncp, exps);
+      PsiSrc{phiT, dphiT, ld, w, sj, sg, i0, n_i, ncp, n_orb}, 4 * ncp, 4 * ncp, planes, rows * 4 * ncp, exps);
 }
 
-void launch_digits_wv(const double* src, int64_t rows, const int* si, int64_t i0, int64_t n_i, int64_t ncp,
+void launch_digits_wv(const double* src, int64_t rows, const int* sj, const int* sg, int64_t i0, int64_t n_i, int64_t ncp,
                       uint16_t* planes, int* exps, cudaStream_t st) {
-  digits_kernel<<<static_cast<unsigned>(rows), DG_THREADS, 0, st>>>(WvSrc{src, si, i0, n_i, ncp}, 4 * ncp, 4 * ncp,
+  digits_kernel<<<static_cast<unsigned>(rows), DG_THREADS, 0, st>>>(WvSrc{src, sj, sg, i0, n_i, ncp}, 4 * ncp, 4 * ncp,
                                                                     planes, rows * 4 * ncp, exps);
 }
 

@@ -100,7 +100,7 @@ struct xtc_ctx {
   DBuf fc_U, fc_h, fc_hout, fc_Uout;  // frozen-core folding: staged host inputs and outputs
   DBuf G2;                     // second gradient table: step (a) of the next chunk on stream st2
   DBuf k_dphi, k_dphiT, k_W, k_S;  // two-body integrals K: staged and transposed gradients, rows of W and V, S
-  DBuf k_si;                       // and its point scales
+  DBuf k_sg;                       // and the point scales of the gradients
   // digit planes and row exponents of the FP64 contractions: rho^T, the pair functions (with their
   // scratch rows), and the operands of step (d) or of the contraction of K
   DBuf d_rho, d_rhoe, d_sj, d_sv, d_G, d_Ge, d_tmp, d_L, d_Le, d_R, d_Re;
@@ -129,7 +129,7 @@ struct xtc_ctx {
     return {&jp_dev, &err_dev, &flag_dev, &grid, &w, &phi, &gamma, &phiT, &phi32, &pair_p, &pair_q, &jtab, &jtab64,
             &rho, &colmax, &colexp, &G, &gcoef, &V, &Vacc, &L, &R, &L32, &R32, &eL, &eR, &M, &evec, &lam, &dU_tmp,
             &dh_tmp, &e0_tmp, &vout, &r1, &r2, &lamd, &gamma_b, &M2, &M3, &lam2, &R2, &R32b, &eR2, &Lv, &T3,
-            &h_tmp, &fc_U, &fc_h, &fc_hout, &fc_Uout, &G2, &k_dphi, &k_dphiT, &k_W, &k_S, &k_si, &d_rho, &d_rhoe, &d_sj, &d_sv,
+            &h_tmp, &fc_U, &fc_h, &fc_hout, &fc_Uout, &G2, &k_dphi, &k_dphiT, &k_W, &k_S, &k_sg, &d_rho, &d_rhoe, &d_sj, &d_sv,
             &d_G, &d_Ge, &d_tmp, &d_L, &d_Le, &d_R, &d_Re};
   }
 };
@@ -1581,16 +1581,16 @@ int two_body_K_once(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_
     const int64_t NN = static_cast<int64_t>(N) * N;
     const size_t s_bytes = static_cast<size_t>(NN) * NP * 8;
     if (!ensure(ctx->k_S, s_bytes) || !ensure(ctx->k_W, static_cast<size_t>(4) * ch * NP * 8) ||
-        !ensure(ctx->k_dphiT, static_cast<size_t>(3) * N * pl.NGp * 8) || !ensure(ctx->k_si, 4ull * (pl.NGp + 4 * N)) ||
+        !ensure(ctx->k_dphiT, static_cast<size_t>(3) * N * pl.NGp * 8) || !ensure(ctx->k_sg, 4ull * (pl.NGp + 3 * N)) ||
         !ensure(ctx->d_L, static_cast<size_t>(D64_BYTES) * NN * 4 * ch) || !ensure(ctx->d_Le, 4ull * NN) ||
         !ensure(ctx->d_R, static_cast<size_t>(D64_BYTES) * NP * 4 * ch) || !ensure(ctx->d_Re, 4ull * NP))
       return fail(ctx, XTC_ERR_OOM, "two_body_K workspace (%.2f GB)", (s_bytes + ch * per_point) * 1e-9);
     VfMaps maps{};
     if ((rc = make_vfield_maps(ctx, pl, maps))) return rc;
     launch_transpose_phi(d_dphi, n_grid, pl.NGp, 3 * N, ctx->k_dphiT.as<double>(), st);  // row 3 q + x
-    const int* si = ctx->k_si.as<int>();
-    launch_point_scale_k(ctx->phiT.as<double>(), ctx->k_dphiT.as<double>(), pl.NGp, d_w, pl.NG, N,
-                         ctx->k_si.as<int>() + pl.NGp, ctx->k_si.as<int>(), st);
+    const int *sj = ctx->d_sj.as<int>(), *sg = ctx->k_sg.as<int>();
+    launch_gradient_scale(ctx->phiT.as<double>(), ctx->k_dphiT.as<double>(), pl.NGp, d_w, pl.NG, N, sj + pl.NGp,
+                          ctx->k_sg.as<int>() + pl.NGp, ctx->k_sg.as<int>(), st);
     CUDA_OK(cudaMemsetAsync(ctx->k_S.p, 0, s_bytes, st));
     for (int64_t c0 = pl.ob; c0 < pl.oe; c0 += ch) {
       const int64_t n_c = std::min<int64_t>(ch, pl.oe - c0), ncp = round_up(n_c, D64_BK);
@@ -1608,8 +1608,8 @@ int two_body_K_once(xtc_ctx* ctx, int64_t n_grid, int n_orb, const double* grid_
                       ncp, rows, st);
       }
       if ((rc = run_vfield64(ctx, pl, d_grid, d_w, c0, n_c, o, D64_TO_ROWS))) return rc;
-      launch_digits_wv(rows, NP, si, c0, n_c, ncp, ctx->d_R.as<uint16_t>(), ctx->d_Re.as<int>(), st);
-      launch_digits_psi(ctx->phiT.as<double>(), ctx->k_dphiT.as<double>(), pl.NGp, d_w, si, c0, n_c, ncp, N,
+      launch_digits_wv(rows, NP, sj, sg, c0, n_c, ncp, ctx->d_R.as<uint16_t>(), ctx->d_Re.as<int>(), st);
+      launch_digits_psi(ctx->phiT.as<double>(), ctx->k_dphiT.as<double>(), pl.NGp, d_w, sj, sg, c0, n_c, ncp, N,
                         ctx->d_L.as<uint16_t>(), ctx->d_Le.as<int>(), st);
       Gemm64Out so{};
       so.out = ctx->k_S.as<double>();

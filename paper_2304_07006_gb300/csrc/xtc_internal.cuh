@@ -237,7 +237,7 @@ void launch_gemm64_finalize(const Gemm64Args& a, int splits, const Gemm64Out& o,
 // Digits: FP64 rows of L (sign -1) or R (+1) from value k0 on, K of them, with the point scales of rho and A (sj:
 // launch_point_scale, of the chunk's first point) and of V and B (sv: launch_v_scale);
 // rho^T[pq][j] 2^-sj[j] of n_j inner points; the operands of the contraction of K (left: rows p N + q from phi and
-// dphiT[3 q + x][j], right: rows of 4 ncp values, W and V) with the scales si of launch_point_scale_k, k = c ncp + i, point i0 + i.
+// dphiT[3 q + x][j], right: rows of 4 ncp values, W and V) with the scales sj (c = 0) and sg (launch_gradient_scale), k = c ncp + i, point i0 + i.
 void launch_digits_lr(const double* src, int64_t rows, int64_t ld, int64_t k0, int64_t K, const int* sj, const int* sv,
                       int64_t n_i, int sign, uint16_t* planes, int* exps, cudaStream_t st);
 void launch_digits_rho(const double* phiT, int64_t ld, const double* w, int64_t n_j, int64_t Kp, int n_orb,
@@ -250,12 +250,13 @@ void launch_point_scale(const double* phiT, int64_t ld, const double* w, int64_t
 // below D64_NO_SCALE where V is 0; orb: as written by launch_point_scale.
 void launch_v_scale(const double* L, int64_t ld, int64_t n_i, int n_pair, const int* pair_p, const int* pair_q,
                     const int* orb, int* sv, cudaStream_t st);
-// si[i]: the exponent of the largest entry of K's left operand at point i, every orbital at one height; orb[4 n_orb]: scratch.
-void launch_point_scale_k(const double* phiT, const double* dphiT, int64_t ld, const double* w, int64_t n_grid,
-                          int n_orb, int* orb, int* si, cudaStream_t st);
-void launch_digits_psi(const double* phiT, const double* dphiT, int64_t ld, const double* w, const int* si, int64_t i0,
-                       int64_t n_i, int64_t ncp, int n_orb, uint16_t* planes, int* exps, cudaStream_t st);
-void launch_digits_wv(const double* src, int64_t rows, const int* si, int64_t i0, int64_t n_i, int64_t ncp,
+// sg[i]: exponent of |w_i| max_p (|phi_p(i)| / max |phi_p|) max_q,x (|d_x phi_q(i)| / max |phi_q|); orb: as written by
+// launch_point_scale; dorb[3 n_orb]: scratch.
+void launch_gradient_scale(const double* phiT, const double* dphiT, int64_t ld, const double* w, int64_t n_grid,
+                           int n_orb, const int* orb, int* dorb, int* sg, cudaStream_t st);
+void launch_digits_psi(const double* phiT, const double* dphiT, int64_t ld, const double* w, const int* sj, const int* sg,
+                       int64_t i0, int64_t n_i, int64_t ncp, int n_orb, uint16_t* planes, int* exps, cudaStream_t st);
+void launch_digits_wv(const double* src, int64_t rows, const int* sj, const int* sg, int64_t i0, int64_t n_i, int64_t ncp,
                       uint16_t* planes, int* exps, cudaStream_t st);
 // Pair functions of the Jastrow factor in FP64 as digit rows (grad64.cu): comps = 3: the three components
 // of grad_1 u, 4: those and F = lap_1 u + |grad_1 u|^2, 1: F alone; row c * c_rows + il for outer point

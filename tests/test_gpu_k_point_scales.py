@@ -48,3 +48,16 @@ def test_scaled_orbitals_scale_k_exactly():
     p.phi = p.phi * s
     Ks = _k(p, dphi * s[:, None])
     assert np.array_equal(Ks, K * np.einsum("p,q,r,s->pqrs", s, s, s, s))
+
+
+@pytest.mark.parametrize("length", [1e-12, 1e-6, 1e6])
+def test_grids_of_other_lengths(length):
+    """W and the gradients have a length in them, V and the orbitals do not: neither part of an operand row takes bits from the
+    other, whatever their sizes."""
+    rng = np.random.default_rng(5)
+    p = synth.make_small(n_orb=5, n_rad=5, n_theta=4, n_phi=5, n_atoms=1, seed=14)   # 100 points around one nucleus
+    p.nuc_xyz = np.zeros((1, 3))
+    p.grid = rng.normal(size=p.grid.shape) * length
+    dphi = rng.normal(size=(p.n_grid, p.n_orb, 3)) * np.abs(p.phi).max() / length
+    want = two_body_k.k_integrals(p.grid, p.weights, p.phi, dphi, p.nuc_xyz, p.nuc_set, p.terms, p.coef)
+    assert np.abs(_k(p, dphi) - want).max() <= TOL * np.abs(want).max()
