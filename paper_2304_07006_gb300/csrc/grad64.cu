@@ -181,6 +181,7 @@ struct NucFix {
 struct PointFix {
   long long K[3][3], Hc1, Hc2, L[3];
   int sE, sH1, sH2, sL;
+  int uE, uH1, uH2, uL;   // exponents of their units; NO_UNIT where the sum is empty, and exact
 };
 __device__ __forceinline__ double bound_a(const NucCoef& q) {
   return fabs(q.a01) + fabs(q.a02) + fabs(q.a11) + fabs(q.a12) + 2.0 * (fabs(q.a21) + fabs(q.a22));
@@ -188,6 +189,8 @@ __device__ __forceinline__ double bound_a(const NucCoef& q) {
 __device__ __forceinline__ int scale_of(double sum, int bits) {
   return sum < INFINITY ? bits - exponent_above(sum) : NO_RANGE;   // NaN is not below
 }
+constexpr int NO_UNIT = -(1 << 20);
+__device__ __forceinline__ int unit_of(double sum, int scale) { return sum == 0.0 ? NO_UNIT : -scale; }
 // The larger of two magnitudes, NaN if either is (fmax would drop it).
 __device__ __forceinline__ double nan_max(double a, double b) { return b <= a ? a : (a <= b ? b : a + b); }
 // Threads 0, 1, 2: the scales of E, H and L.
@@ -199,6 +202,7 @@ __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef*
     for (int I = 0; I < n_nuc; ++I)
       s += bound_a(nuc[I]) * nan_max(fabs(nuc[I].g[0]), nan_max(fabs(nuc[I].g[1]), fabs(nuc[I].g[2])));
     f.sE = scale_of(s, 61);
+    f.uE = unit_of(s, f.sE);
   } else if (k == 1) {
     s = fabs(pt.Hc1);
     s2 = fabs(pt.Hc2);
@@ -206,8 +210,11 @@ __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef*
       s += fabs(nuc[I].b11) + fabs(nuc[I].b12);
       s2 += fabs(nuc[I].b21) + fabs(nuc[I].b22);
     }
-    f.sH1 = scale_of(LAP ? s : nan_max(s, s2), 60);
-    f.sH2 = scale_of(LAP ? s2 : nan_max(s, s2), 60);
+    if (!LAP) s = s2 = nan_max(s, s2);
+    f.sH1 = scale_of(s, 60);
+    f.sH2 = scale_of(s2, 60);
+    f.uH1 = unit_of(s, f.sH1);
+    f.uH2 = unit_of(s2, f.sH2);
   } else {
     s = fabs(pt.L[0]);
     s2 = fabs(pt.L[1]);
@@ -217,7 +224,9 @@ __device__ __forceinline__ void point_scales(const PointCoef& pt, const NucCoef*
       s2 += fabs(nuc[I].L[1][0]) + fabs(nuc[I].L[1][1]);
       s3 += fabs(nuc[I].L[2][0]) + fabs(nuc[I].L[2][1]);
     }
-    f.sL = scale_of(nan_max(s, nan_max(s2, s3)), 59);
+    s = nan_max(s, nan_max(s2, s3));
+    f.sL = scale_of(s, 59);
+    f.uL = unit_of(s, f.sL);
   }
 }
 __device__ __forceinline__ void nuc_fix(const NucCoef& q, const PointFix& p, NucFix& f) {
@@ -261,6 +270,91 @@ __device__ __forceinline__ double rcp64(double x) {
   return fma(y, fma(e, e, e), y);
 }
 
+// Exponent e with x < 2^e for x >= 0 of the given high word.
+__device__ __forceinline__ int exponent_of_hi(int hi) { return (hi >> 20) - 1022; }
+
+// Largest values of the CTA for M values a thread, to every thread; scratch: M ints a warp.
+template <int M>
+__device__ __forceinline__ void block_max_n(int* v, int* scratch) {
+  constexpr int W = THREADS / 32;
+#pragma unroll
+  for (int c = 0; c < M; ++c) v[c] = __reduce_max_sync(0xffffffffu, v[c]);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int c = 0; c < M; ++c) scratch[c * W + (threadIdx.x >> 5)] = v[c];
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < M; ++c)
+#pragma unroll
+    for (int w = 0; w < W; ++w) v[c] = max(v[c], scratch[c * W + w]);
+}
+
+// The pair functions in FP64 throughout, for rows that the fixed point does not resolve: v[0..2] the gradient, v[3] F.
+__device__ __forceinline__ void pair_fp64(const JastrowParams& jp, const PointCoef& pt, const NucCoef* nuc, double dx,
+                                       double dy, double dz, double xj, double yj, double zj, double (&v)[4]) {
+  const double r2 = dx * dx + dy * dy + dz * dz, r = sqrt(r2);
+  const bool apart = r2 > EPS2;
+  const double i12 = apart ? 1.0 / r : 0.0, s12 = 1.0 / (1.0 + r), b = r * s12, bp = s12 * s12, s = bp * i12;
+  double e[3], fe[3], h1 = pt.Hc1, h2 = pt.Hc2, l[3] = {pt.L[0], pt.L[1], pt.L[2]};
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    e[x] = pt.K[0][x] + b * (pt.K[1][x] + b * pt.K[2][x]);
+    fe[x] = pt.K[1][x] + 2.0 * b * pt.K[2][x];
+  }
+  for (int I = 0; I < jp.n_nuc; ++I) {
+    const NucCoef& q = nuc[I];
+    const double ux = xj - jp.nuc[I][0], uy = yj - jp.nuc[I][1], uz = zj - jp.nuc[I][2];
+    const double d = sqrt(ux * ux + uy * uy + uz * uz), a = d / (1.0 + d);
+    const double u1 = q.a11 + q.a12 * a, u2 = (q.a21 + q.a22 * a) * b;
+    const double at = a * (q.a01 + q.a02 * a + b * (u1 + u2)), ad = a * (u1 + 2.0 * u2);
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      e[x] += at * q.g[x];
+      fe[x] += ad * q.g[x];
+      l[x] += a * (q.L[x][0] + q.L[x][1] * a);
+    }
+    h1 += a * (q.b11 + q.b12 * a);
+    h2 += a * (q.b21 + q.b22 * a);
+  }
+  const double h = h1 + b * h2, hs = h * s;
+  v[0] = hs * dx + e[0];
+  v[1] = hs * dy + e[1];
+  v[2] = hs * dz + e[2];
+  const double t = s * (dx * fe[0] + dy * fe[1] + dz * fe[2]) + (apart ? h1 * s : -(h * bp)) * s12;
+  v[3] = l[0] + b * (l[1] + b * l[2]) + (apart ? 3.0 : 1.0) * (h2 * bp) * bp + 2.0 * t + v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+}
+
+// This thread's part of a row, and its largest exponents.
+template <int NC>
+__device__ __noinline__ void row_fp64(const JastrowParams& jp, const PointCoef& pt, const NucCoef* nuc, double px,
+                                      double py, double pz, const double* jt, int64_t ld, int64_t n_j, int64_t Kp,
+                                      const int* sj, double* rows, int* mx) {
+  for (int c = 0; c < NC; ++c) mx[c] = 0;
+  for (int64_t j = threadIdx.x; j < n_j; j += THREADS) {
+    const double xj = jt[j], yj = jt[ld + j], zj = jt[2 * ld + j];
+    double v[4];
+    pair_fp64(jp, pt, nuc, px - xj, py - yj, pz - zj, xj, yj, zj, v);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      rows[c * Kp + j] = v[NC == 1 ? 3 : c];
+      mx[c] = max(mx[c], d64_key(v[NC == 1 ? 3 : c], sj[j]));
+    }
+  }
+}
+
+// Bits that the largest entry of a row (with its points' scales) has to stand above the largest error unit of the fixed point
+// for the row to be kept; else it is evaluated again in FP64.  Rows of molecules stand 54 and more above it
+// (gradient) and 47 and more (F, whose unit is bounded less closely: far outer points).  Rows below are those of
+// outer points whose coefficients meet only small powers of a2 or b where the weight is: grids far smaller than a bohr,
+// densities within 1e-6 bohr of a nucleus.  They lost up to half of their bits.
+constexpr int BITS_GRAD = 50, BITS_F = 46;
+
+// Does the row of largest key `key` stand less than `bits` above the unit 2^unit (some error, not infinite or NaN)?
+__device__ __forceinline__ bool short_of(int key, int unit, int bits) {
+  return unit > NO_UNIT / 2 && key < D64_NONFINITE && (key == 0 || key - D64_BIAS - 1022 - unit < bits);
+}
+
 template <int NC>
 __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
     grad64_kernel(const double* __restrict__ grid, const JastrowParams* __restrict__ jp, int n_nuc,
@@ -270,11 +364,14 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
   constexpr bool GRAD = NC >= 3, LAP = NC == 1 || NC == 4;
   extern __shared__ __align__(16) uint8_t smem_raw[];
   __shared__ PointCoef pt;
-  __shared__ int red[32];
+  __shared__ int red[(NC + 1) * (THREADS / 32)];
   __shared__ PointFix pf;
   NucCoef* nuc = reinterpret_cast<NucCoef*>(smem_raw);
   NucFix* nf = reinterpret_cast<NucFix*>(nuc + n_nuc);
   double* rows = scratch + static_cast<int64_t>(blockIdx.x) * NC * Kp;
+  int s_max = 2 * NO_UNIT;   // the largest point scale
+  for (int64_t j = threadIdx.x; j < n_j; j += THREADS) s_max = max(s_max, __ldg(sj + j));
+  block_max_n<1>(&s_max, red);
   for (int64_t il = blockIdx.x; il < n_i; il += gridDim.x) {
     const double px = grid[3 * (i0 + il)], py = grid[3 * (i0 + il) + 1], pz = grid[3 * (i0 + il) + 2];
     __syncthreads();  // the previous point's coefficients and rows are no longer read
@@ -306,9 +403,10 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
     __syncthreads();
     const int sE = pf.sE, sH1 = pf.sH1, sH2 = pf.sH2, sL = pf.sL;
     // ------------------------------------------------------------ the row in FP64, and its largest exponents
-    int mx[NC];
+    int mx[NC + 1];   // and of b' max(1, 1/r12 if F is asked for) with the points' scales
 #pragma unroll
     for (int c = 0; c < NC; ++c) mx[c] = 0;
+    mx[NC] = 2 * NO_UNIT;
     for (int64_t j = threadIdx.x; j < n_j; j += THREADS) {
       const double dx = px - __ldg(jt + j), dy = py - __ldg(jt + ld + j), dz = pz - __ldg(jt + 2 * ld + j);
       const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
@@ -362,16 +460,31 @@ __global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
         v[NC == 1 ? 0 : 3] = f;
       }
       const int s_j = __ldg(sj + j);
+      mx[NC] = max(mx[NC], s_j + exponent_of_hi(LAP ? max(__double2hiint(s), __double2hiint(bp)) : __double2hiint(bp)));
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         rows[c * Kp + j] = v[c];
         mx[c] = max(mx[c], d64_key(v[c], s_j));
       }
     }
+    block_max_n<NC + 1>(mx, red);  // the barriers also publish the FP64 row
+    // the largest error unit of the row: of the gradient max(2^uE, b' 2^uH), of F also (the gradient's) times twice the gradient,
+    // and h1's times b' / r12
+    const int uE = pf.uE, uH = max(pf.uH1, pf.uH2), top = max(max(uE + 61, uH + 60) + 1, 0);
+    bool again = false;
+    if (GRAD) again = short_of(max(mx[0], max(mx[1], mx[2])), max(s_max + uE, mx[NC] + uH), BITS_GRAD);
+    if (LAP) again |= short_of(mx[NC - 1], max(s_max + max(pf.uL, uE + top + 1), mx[NC] + uH + top + 2), BITS_F);
+    if (again) {   // the same for all threads
+      int m[NC];
+      row_fp64<NC>(*jp, pt, nuc, px, py, pz, jt, ld, n_j, Kp, sj, rows, m);
+      block_max_n<NC>(m, red);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) mx[c] = m[c];
+    }
     // ------------------------------------------------------------ digits of the rows
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      const int e = d64_exponent(block_max(mx[c], red));  // the barriers also publish the FP64 row
+      const int e = d64_exponent(mx[c]);
       const int64_t row = (GRAD ? c : 0) * c_rows + il;
       if (threadIdx.x == 0) exps[row] = e;
       for (int64_t k = 4 * threadIdx.x; k < Kp; k += 4 * THREADS) {
