@@ -18,7 +18,7 @@
 // with no density).  With seven digits and no such scales the error of the water-sized build was 1,500
 // times that of the FP64 pipe's sums.  Step (d) uses the same scales for rho and A, others for
 // V and B (v_scale_kernel), and the contraction of K those of rho and others for the
-// gradients (gradient_scale_kernel).
+// gradients.
 //
 // Why: the FP64 pipe does 2 FMA per SM and clock on this GPU, the 128 x 32 x 64 FMA of one range of a
 // tile take 131,072 of its cycles; the same range is 36 fp16 products of 4 k-steps.  They are bound by shared
@@ -306,22 +306,30 @@ constexpr int DG_THREADS = 256;
 // those of R with them (sign +1).  With rho alone scaled, V kept what bits its size beside phi^2 left it: none of the
 // result's was right with weights of 1e-40 (sums of w phi^2 are 1 for orthonormal orbitals, but no input has to be).
 struct LrSrc {
+  static constexpr bool GROUPED = true;
   const double* p;
   int64_t ld, k0;           // first k of the block
   const int* sj;            // of the chunk's first point
   const int* sv;
   int64_t n_i;
   int sign;
-  __device__ double at(int64_t row, int64_t k) const { return p[row * ld + k]; }
-  __device__ int scale(int64_t k) const {
+  // four values from k on, k a multiple of 4: one point's
+  __device__ void load4(int64_t row, int64_t k, double (&v)[4], int (&s)[4]) const {
+    const double2* q = reinterpret_cast<const double2*>(p + row * ld + k);
+    const double2 a = q[0], b = q[1];
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = b.x;
+    v[3] = b.y;
     const int64_t i = (k0 + k) >> 2;
-    if (i >= n_i) return 0;
-    const int s = (k0 + k) & 3 ? sv[i] : sj[i];
-    return s <= D64_NO_SCALE ? D64_NO_SCALE : sign * s;
+    const int j = i < n_i ? sj[i] : 0, g = i < n_i ? sv[i] : 0;
+    s[0] = j <= D64_NO_SCALE ? D64_NO_SCALE : sign * j;
+    s[1] = s[2] = s[3] = g <= D64_NO_SCALE ? D64_NO_SCALE : sign * g;
   }
 };
 // rho^T[pq][j] = w_j phi_p(j) phi_q(j), times 2^-sj[j]
 struct RhoSrc {
+  static constexpr bool GROUPED = false;
   const double* phiT;
   int64_t ld;
   const double* w;
@@ -336,19 +344,12 @@ struct RhoSrc {
 // Operands of the contraction of K, k = c ncp + i, i < n_i a point of the chunk (zero past them).  Left: row
 // pq = p N + q, c = 0: w phi_p phi_q / 2, c = 1..3: w phi_p d_x phi_q (dphiT row 3 q + x).  Right: W, V_x.  W grows as 1/r
 // next to a nucleus, where the weight is as small, and gradients have a length in them, so both kinds of k carry scales of their
-// own, sj (as in step (b)) and sg (gradient_scale_kernel), taken out of the left operand and multiplied into the right one.
+// own, sj (as in step (b)) and sg (point_scale_kernel), taken out of the left operand and multiplied into the right one.
 // Without any a point 1e-12 bohr from a nucleus cost every row the bits of 1/r, 1e-10 of max |K| where FP64 sums give
 // 1e-14; with one for both, a grid 1e-12 bohr across did.
 __device__ __forceinline__ int k_component(int64_t k, int64_t ncp) { return (k >= ncp) + (k >= 2 * ncp) + (k >= 3 * ncp); }
-// Scale of index k: sj and sg of the chunk's first point.
-__device__ __forceinline__ int k_scale(int64_t k, int64_t ncp, int64_t n_i, const int* sj, const int* sg, int sign) {
-  const int c = k_component(k, ncp);
-  const int64_t i = k - c * ncp;
-  if (i >= n_i) return 0;
-  const int s = c ? sg[i] : sj[i];
-  return s == D64_NO_SCALE ? D64_NO_SCALE : sign * s;
-}
 struct PsiSrc {
+  static constexpr bool GROUPED = false;
   const double* phiT;
   const double* dphiT;
   int64_t ld;
@@ -365,15 +366,32 @@ struct PsiSrc {
     const double wp = w[g] * phiT[p * ld + g];
     return c == 0 ? 0.5 * wp * phiT[q * ld + g] : wp * dphiT[(3 * q + c - 1) * ld + g];
   }
-  __device__ int scale(int64_t k) const { return k_scale(k, ncp, n_i, sj + i0, sg + i0, -1); }
+  __device__ int scale(int64_t k) const {
+    const int c = k_component(k, ncp);
+    const int64_t i = k - c * ncp;
+    const int s = i < n_i ? (c ? sg : sj)[i0 + i] : 0;
+    return s == D64_NO_SCALE ? D64_NO_SCALE : -s;
+  }
 };
 struct WvSrc {
+  static constexpr bool GROUPED = true;
   const double* p;
   const int* sj;
   const int* sg;
   int64_t i0, n_i, ncp;
-  __device__ double at(int64_t row, int64_t k) const { return p[row * 4 * ncp + k]; }
-  __device__ int scale(int64_t k) const { return k_scale(k, ncp, n_i, sj + i0, sg + i0, 1); }
+  __device__ void load4(int64_t row, int64_t k, double (&v)[4], int (&s)[4]) const {
+    const double2* q = reinterpret_cast<const double2*>(p + row * 4 * ncp + k);
+    const double2 a = q[0], b = q[1];
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = b.x;
+    v[3] = b.y;
+    const int c = k_component(k, ncp);   // of all four: ncp is a multiple of 64
+    const int64_t i = k - c * ncp;
+    const int* sc = (c ? sg : sj) + i0 + i;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) s[t] = i + t < n_i ? sc[t] : 0;
+  }
 };
 
 // One CTA per row: the row's largest exponent, then the digits of four consecutive k per thread.  The
@@ -385,7 +403,18 @@ __global__ void __launch_bounds__(DG_THREADS) digits_kernel(const Src src, int64
                                                             int* __restrict__ exps) {
   const int64_t row = blockIdx.x;
   int m = 0;
-  for (int64_t k = threadIdx.x; k < K; k += DG_THREADS) m = max(m, d64_key(src.at(row, k), src.scale(k)));
+  if constexpr (Src::GROUPED) {   // K is a multiple of 4
+#pragma unroll 2
+    for (int64_t k = 4 * threadIdx.x; k < K; k += 4 * DG_THREADS) {
+      double v[4];
+      int s[4];
+      src.load4(row, k, v, s);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) m = max(m, d64_key(v[t], s[t]));
+    }
+  } else {
+    for (int64_t k = threadIdx.x; k < K; k += DG_THREADS) m = max(m, d64_key(src.at(row, k), src.scale(k)));
+  }
   __shared__ int red[32];
   const int e = d64_exponent(block_max(m, red));
   if (threadIdx.x == 0) exps[row] = e;
@@ -393,38 +422,79 @@ __global__ void __launch_bounds__(DG_THREADS) digits_kernel(const Src src, int64
   for (int64_t k = 4 * threadIdx.x; k < Kp; k += 4 * DG_THREADS) {
     double v[4];
     int s[4];
+    if constexpr (Src::GROUPED) {
+      src.load4(row, k, v, s);
+    } else {
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      v[t] = k + t < K ? src.at(row, k + t) : 0.0;
-      s[t] = k + t < K ? src.scale(k + t) : 0;
+      for (int t = 0; t < 4; ++t) {
+        v[t] = k + t < K ? src.at(row, k + t) : 0.0;
+        s[t] = k + t < K ? src.scale(k + t) : 0;
+      }
     }
     d64_store_digits(v, s, e, out + k, plane);
   }
 }
 
-// orb[p]: the largest key of orbital p over the grid.
+// orb[p] (initially 0): the largest key of row p over the grid, OK_POINTS points a CTA.
+constexpr int OK_POINTS = 8 * DG_THREADS;
 __global__ void __launch_bounds__(DG_THREADS) orbital_key_kernel(const double* __restrict__ phiT, int64_t ld,
                                                                  int64_t n_grid, int* __restrict__ orb) {
   __shared__ int red[32];
+  const int64_t j0 = static_cast<int64_t>(blockIdx.x) * OK_POINTS + threadIdx.x;
+  double v[OK_POINTS / DG_THREADS];
+#pragma unroll
+  for (int t = 0; t < OK_POINTS / DG_THREADS; ++t) {
+    const int64_t j = j0 + t * DG_THREADS;
+    v[t] = j < n_grid ? phiT[blockIdx.y * ld + j] : 0.0;
+  }
   int m = 0;
-  for (int64_t j = threadIdx.x; j < n_grid; j += DG_THREADS) m = max(m, d64_key(phiT[blockIdx.x * ld + j], 0));
+#pragma unroll
+  for (int t = 0; t < OK_POINTS / DG_THREADS; ++t) m = max(m, d64_key(v[t], 0));
   m = block_max(m, red);
-  if (threadIdx.x == 0) orb[blockIdx.x] = m;
+  if (threadIdx.x == 0 && m) atomicMax(orb + blockIdx.y, m);
 }
 
 // sj[j]: the exponent of |w_j| max_p (phi_p(j) / max phi_p)^2, the largest pair product of inner point j with
-// every orbital brought to the same height; D64_NO_SCALE where that is 0 (every pair product is 0 then).
-__global__ void point_scale_kernel(const double* __restrict__ phiT, int64_t ld, const double* __restrict__ w,
-                                   int64_t n_j, int n_orb, const int* __restrict__ orb, int* __restrict__ sj) {
-  const int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (j >= n_j) return;
-  int m = D64_NO_SCALE;
-  for (int p = 0; p < n_orb; ++p) {
-    const int k = d64_key(phiT[p * ld + j], 0);
-    if (k) m = max(m, k - orb[p]);
+// every orbital brought to the same height; D64_NO_SCALE where that is 0 (every pair product is 0 then).  With dphiT, sg[j]
+// instead: |w_j| max_p (|phi_p(j)| / max |phi_p|) max_q,x (|d_x phi_q(j)| / max |phi_q|), for the operands of K (an orbital
+// that is 0 everywhere: at the height of its gradient).  orb[n_orb], dorb[3 n_orb]: largest keys of the orbitals and of their
+// gradients.  Latency-bound: PS_GROUPS threads share a point's orbitals.
+constexpr int PS_GROUPS = 8;
+__global__ void __launch_bounds__(32 * PS_GROUPS)
+    point_scale_kernel(const double* __restrict__ phiT, const double* __restrict__ dphiT, int64_t ld,
+                       const double* __restrict__ w, int64_t n_j, int n_orb, const int* __restrict__ orb,
+                       const int* __restrict__ dorb, int* __restrict__ sj) {
+  __shared__ int red[2][PS_GROUPS][32];
+  const int64_t j = blockIdx.x * 32ll + threadIdx.x;
+  int m = D64_NO_SCALE, mg = D64_NO_SCALE;
+  if (j < n_j) {
+#pragma unroll 2
+    for (int p = threadIdx.y; p < n_orb; p += PS_GROUPS) {
+      const int k = d64_key(phiT[p * ld + j], 0);
+      if (k) m = max(m, k - orb[p]);
+      if (dphiT) {
+        int kd = 0, top = 0;
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+          kd = max(kd, d64_key(dphiT[(3 * p + x) * ld + j], 0));
+          top = max(top, dorb[3 * p + x]);
+        }
+        if (kd) mg = max(mg, kd - (orb[p] ? orb[p] : top));
+      }
+    }
   }
+  red[0][threadIdx.y][threadIdx.x] = m;
+  red[1][threadIdx.y][threadIdx.x] = mg;
+  __syncthreads();
+  if (threadIdx.y || j >= n_j) return;
+#pragma unroll
+  for (int g = 1; g < PS_GROUPS; ++g) {
+    m = max(m, red[0][g][threadIdx.x]);
+    mg = max(mg, red[1][g][threadIdx.x]);
+  }
+  if (!dphiT) mg = m;
   const int kw = d64_key(w[j], 0);
-  sj[j] = m == D64_NO_SCALE || kw == 0 ? D64_NO_SCALE : kw - D64_BIAS - 1022 + 2 * m;
+  sj[j] = m == D64_NO_SCALE || mg == D64_NO_SCALE || kw == 0 ? D64_NO_SCALE : kw - D64_BIAS - 1022 + m + mg;
 }
 
 // sv[i], initially below D64_NO_SCALE: the exponent of max_pq,x |V_x,pq(i)| / (max phi_p max phi_q), from the rows of L; stays
@@ -433,43 +503,21 @@ constexpr int VS_PAIRS = 16;
 __global__ void __launch_bounds__(128) v_scale_kernel(const double* __restrict__ L, int64_t ld, int64_t n_i, int n_pair,
                                                       const int* __restrict__ pair_p, const int* __restrict__ pair_q,
                                                       const int* __restrict__ orb, int* __restrict__ sv) {
+  __shared__ int height[VS_PAIRS];
   const int64_t i = blockIdx.x * 128ll + threadIdx.x;
-  if (i >= n_i) return;
   const int pq0 = blockIdx.y * VS_PAIRS, pq1 = min(n_pair, pq0 + VS_PAIRS);
+  if (pq0 + threadIdx.x < pq1) height[threadIdx.x] = orb[pair_p[pq0 + threadIdx.x]] + orb[pair_q[pq0 + threadIdx.x]];
+  __syncthreads();
+  if (i >= n_i) return;
   int m = D64_NO_SCALE;
 #pragma unroll 4
   for (int pq = pq0; pq < pq1; ++pq) {
     const double2* v = reinterpret_cast<const double2*>(L + pq * ld + 4 * i);
     const double2 v0 = v[0], v1 = v[1];
     const int k = max(d64_key(v0.y, 0), max(d64_key(v1.x, 0), d64_key(v1.y, 0)));
-    if (k && k < D64_NONFINITE) m = max(m, k - orb[pair_p[pq]] - orb[pair_q[pq]] + D64_BIAS + 1022);
+    if (k && k < D64_NONFINITE) m = max(m, k - height[pq - pq0] + D64_BIAS + 1022);
   }
   if (m > D64_NO_SCALE) atomicMax(sv + i, m);
-}
-
-// sg[i]: the exponent of |w_i| max_p (|phi_p(i)| / max |phi_p|) max_q,x (|d_x phi_q(i)| / max |phi_q|), every orbital at one
-// height (an orbital that is 0 everywhere: at that of its gradient); D64_NO_SCALE where that is 0.  orb[n_orb],
-// dorb[3 n_orb]: largest keys of the orbitals and of their gradients.
-__global__ void gradient_scale_kernel(const double* __restrict__ phiT, const double* __restrict__ dphiT, int64_t ld,
-                                      const double* __restrict__ w, int64_t n, int n_orb, const int* __restrict__ orb,
-                                      const int* __restrict__ dorb, int* __restrict__ sg) {
-  const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (i >= n) return;
-  int mp = D64_NO_SCALE, mq = D64_NO_SCALE;
-#pragma unroll 2
-  for (int q = 0; q < n_orb; ++q) {
-    const int k = d64_key(phiT[q * ld + i], 0);
-    int kd = 0, top = 0;
-#pragma unroll
-    for (int x = 0; x < 3; ++x) {
-      kd = max(kd, d64_key(dphiT[(3 * q + x) * ld + i], 0));
-      top = max(top, dorb[3 * q + x]);
-    }
-    if (k) mp = max(mp, k - orb[q]);
-    if (kd) mq = max(mq, kd - (orb[q] ? orb[q] : top));
-  }
-  const int kw = d64_key(w[i], 0);
-  sg[i] = mp == D64_NO_SCALE || mq == D64_NO_SCALE || kw == 0 ? D64_NO_SCALE : kw - D64_BIAS - 1022 + mp + mq;
 }
 
 }  // namespace
@@ -523,15 +571,20 @@ void launch_digits_rho(const double* phiT, int64_t ld, const double* w, int64_t 
 
 void launch_point_scale(const double* phiT, int64_t ld, const double* w, int64_t n_grid, int n_orb, int* orb, int* sj,
                         cudaStream_t st) {
-  orbital_key_kernel<<<n_orb, DG_THREADS, 0, st>>>(phiT, ld, n_grid, orb);
-  point_scale_kernel<<<static_cast<unsigned>((n_grid + 127) / 128), 128, 0, st>>>(phiT, ld, w, n_grid, n_orb, orb, sj);
+  cudaMemsetAsync(orb, 0, n_orb * sizeof(int), st);
+  orbital_key_kernel<<<dim3(static_cast<unsigned>((n_grid + OK_POINTS - 1) / OK_POINTS), n_orb), DG_THREADS, 0, st>>>(
+      phiT, ld, n_grid, orb);
+  point_scale_kernel<<<static_cast<unsigned>((n_grid + 31) / 32), dim3(32, PS_GROUPS), 0, st>>>(phiT, nullptr, ld, w, n_grid,
+                                                                                             n_orb, orb, nullptr, sj);
 }
 
 void launch_gradient_scale(const double* phiT, const double* dphiT, int64_t ld, const double* w, int64_t n_grid,
                            int n_orb, const int* orb, int* dorb, int* sg, cudaStream_t st) {
-  orbital_key_kernel<<<3 * n_orb, DG_THREADS, 0, st>>>(dphiT, ld, n_grid, dorb);
-  gradient_scale_kernel<<<static_cast<unsigned>((n_grid + 127) / 128), 128, 0, st>>>(phiT, dphiT, ld, w, n_grid, n_orb,
-                                                                                  orb, dorb, sg);
+  cudaMemsetAsync(dorb, 0, 3 * n_orb * sizeof(int), st);
+  orbital_key_kernel<<<dim3(static_cast<unsigned>((n_grid + OK_POINTS - 1) / OK_POINTS), 3 * n_orb), DG_THREADS, 0, st>>>(
+      dphiT, ld, n_grid, dorb);
+  point_scale_kernel<<<static_cast<unsigned>((n_grid + 31) / 32), dim3(32, PS_GROUPS), 0, st>>>(phiT, dphiT, ld, w, n_grid,
+                                                                                             n_orb, orb, dorb, sg);
 }
 
 void launch_digits_psi(const double* phiT, const double* dphiT, int64_t ld, const double* w, const int* sj, const int* sg,
