@@ -115,8 +115,8 @@ class Clocks:
 # dram__bytes_read.sum + dram__bytes_write.sum of one step (b) GEMM (fp16x2, the sum over its launches) captured with
 # ncu on the first VFIELD_CAPTURE_OUTER outer points of the workload (`--ncu-case`), for GEMM
 # engine revision VFIELD_CAPTURE_REVISION; with another revision the traffic is reported as null
-VFIELD_CAPTURE_REVISION = 7
-VFIELD_DRAM_BYTES_CAPTURED = 21_236_646_656 + 2_783_462_656
+VFIELD_CAPTURE_REVISION = 8
+VFIELD_DRAM_BYTES_CAPTURED = 21_375_324_160 + 2_796_734_720
 VFIELD_CAPTURE_OUTER = 1184
 
 

@@ -82,9 +82,14 @@ typedef enum {
 } xtc_status;
 
 typedef enum {
-  XTC_PREC_FP64 = 0,   /* all four steps to FP64 accuracy: step (a) and (c) on the FP64 pipe, the
-                          contractions (b) and (d) on the tensor cores from eight 9-bit integer digits per
-                          value (71 bits below an operand row's maximum), summed in 64-bit integers */
+  XTC_PREC_FP64 = 0,   /* all four steps to FP64 accuracy.  Step (a): distances and last products in FP64,
+                          the polynomials of u in 64-bit fixed point with scales per outer point (2^-59 of
+                          the sum of its coefficients' magnitudes), outer points that this does not resolve
+                          in FP64 throughout; step (c) in FP64; the contractions (b) and (d) on the tensor
+                          cores from eight 9-bit integer digits per value (71 bits below the largest value
+                          of an operand's row, values at each grid point weighted by what they multiply),
+                          summed in 64-bit integers.  Errors are relative to the largest terms of a sum over
+                          the grid, for orbitals of comparable norm.  xtc_vfield_noalloc keeps to plain FP64 */
   XTC_PREC_FP16X2 = 1, /* steps (b) and (d): range-exact 2-term FP16 split with power-of-2 scaling
                           (per pair column of rho in step b, per row of L and R in step d): per
                           accumulation range (range_stages blocks of 32 inner values, default 2)

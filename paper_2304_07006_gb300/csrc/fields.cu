@@ -26,13 +26,13 @@
 // density of more factors than one pass holds runs several passes: the first writes L and R, the
 // next ones add their R (FP32 and FP64 outputs).
 // Points past the chunk end are written as zeros.
-#include <cuda_bf16.h>
-
 //
 // What bounds it: instructions, shared loads first (the V traffic is a quarter of the time at rank 16).  So
 // the factor loops are unrolled to the rank's bucket (4, 8, 16), phase 1 loads four factors of c in one access, and
 // phase 2 keeps lam H_p of a row in registers.  Step (c), before -> now (one GB300): N = 65, 24,001 points, 65 factors
 // 10.1 -> 8.7 ms; N = 120, 100,000 points, 7 factors 26 -> 19 ms; N = 23, 3,957 points 52 -> 43 us.
+#include <cuda_bf16.h>
+
 #include "xtc_internal.cuh"
 
 namespace xtc {

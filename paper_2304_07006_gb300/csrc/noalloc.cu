@@ -203,8 +203,8 @@ extern "C" XTC_API int xtc_vfield_noalloc(xtc_ctx* ctx, int64_t n_grid, int n_or
     launch_transpose_phi(phi, n_grid, NGp, N, phiT, st);
     launch_jtab(grid_xyz, n_grid, NGp, cv.jp_dev, n_nuc, jtab_stride(n_nuc), jtab, st);
     launch_rho_split(phiT, weights, n_grid, NGp, N, parts, kd_b, pair_p, pair_q, colmax, colexp, phi32, rho, st);
-    // rho^T (box rows vf_bn) and the gradient table [part][x * gc + il][j] (boxes 32 x 32
-    // for the step (a) stores and 32 x 128 for the step (b) loads)
+    // rho^T (box rows vf_bn, bf16 half of that) and the gradient table, rows x * gc + il (boxes of GFIELD_ROWS rows
+    // for the step (a) stores and of VF_BM rows for the step (b) loads; 64 values wide, bf16 32)
     auto encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(cv.encode_tiled);
     // (fp16: 128-byte runs of 64 values of one part; bf16: one plane per part)
     const bool wide = parts == 2;

@@ -27,9 +27,9 @@ constexpr int PT_COEF = 14;     // x y z, K0[3] K1[3] K2[3], Hc1 Hc2
 // Tile shapes of the tensor-core kernels.
 constexpr int VF_BM = 128;      // outer points per tile (TMEM lanes)
 // orbital pairs per tensor-core tile (B rows): the fp16 engine keeps two sets of TMEM accumulators
-// of 2 x 128 columns (exact hi x hi and cross products); the bf16
-// engine two accumulators of 160 columns, 4 stages of 54 KB; each drain thread holds a running sum
-// of half a tile row in registers
+// of 2 x 128 columns (exact hi x hi and cross products), 4 stages of 56 KB, a quarter of a tile row's running
+// sums in the registers of each drain thread; the bf16 engine two accumulators of 160 columns, 5 stages of 39 KB,
+// half a tile row
 __host__ __device__ constexpr int vf_bn(int parts) { return parts == 2 ? 128 : 160; }
 constexpr int VF_BK = 32;       // inner points per pipeline stage (64-byte rows, SWIZZLE_64B)
 constexpr int AS_BM = 128;      // step (d) tile rows (pairs pq)
@@ -133,12 +133,12 @@ void launch_check_finite(const double* x, int64_t n, int* flag, cudaStream_t st)
 
 // Step (a), tensor-core path: the split Jastrow gradient of the outer points [i0, i0 + n_i) and every
 // padded inner point, K-major, row x * gcp + il: fp16 (2 parts) G[row][j / 64][part][j % 64] stored
-// as 128-byte-swizzled TMA tiles (box 64 x 32); bf16 (3 parts) G[part][row][j] as 64-byte-swizzled
-// tiles (box 32 x 32).  Rows up to n_tiles * 32 are written (past n_i they repeat the last point).
+// as 128-byte-swizzled TMA tiles (box 64 x GFIELD_ROWS); bf16 (3 parts) G[part][row][j] as 64-byte-swizzled
+// tiles (box 32 x GFIELD_ROWS).  Rows past n_i, up to `rows`, repeat the last point.
 struct GfieldArgs {
   const double* grid;          // outer-point coordinates (global index space)
   const JastrowParams* jp;
-  const float* jtab;           // pair-interleaved inner-point table (launch_jtab, 12 floats per point)
+  const float* jtab;           // pair-interleaved inner-point table (launch_jtab)
   int64_t i0, n_i;             // outer range of this chunk
   int64_t gcp;                 // padded chunk length (rows per component)
   int64_t rows;                // rows to write per component: n_i rounded up to 128
