@@ -21,6 +21,10 @@ __device__ __forceinline__ int block_max(int v, int* scratch) {
   return v;
 }
 
+// Biased exponent of a subnormal value.  Out of line: inlined it is predicated and issues for every value (464 us and not
+// 435 for the left operand of K at 30 orbitals and 8,000 points).
+static __device__ __noinline__ int d64_subnormal_exponent(int hi, int lo) { return hi ? 12 - __clz(hi) : -20 - __clz(lo); }
+
 // Biased exponent of x 2^s, to be maximised over a row: 0 for x = 0, D64_NONFINITE for infinities and NaN.  That of a
 // subnormal value is its own, down to -51: a density of 1e-320 at a far point, brought up by its point's scale, would
 // otherwise count for up to 2^52 times its size, and its row lose as many bits.
@@ -29,7 +33,7 @@ __device__ __forceinline__ int d64_key(double x, int s) {
   const int hi = __double2hiint(x) & 0x7fffffff, lo = __double2loint(x);
   if ((hi | lo) == 0 || s == D64_NO_SCALE) return 0;
   const int ex = hi >> 20;
-  if (ex == 0) return (hi ? 12 - __clz(hi) : -20 - __clz(lo)) + s + D64_BIAS;
+  if (ex == 0) return d64_subnormal_exponent(hi, lo) + s + D64_BIAS;
   return ex == 0x7ff ? D64_NONFINITE : ex + s + D64_BIAS;
 }
 // Exponent e of a row (every |x 2^s| < 2^e) from the largest key.

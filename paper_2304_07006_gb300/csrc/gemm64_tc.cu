@@ -369,8 +369,9 @@ struct PsiSrc {
   }
   __device__ int scale(int64_t k) const {
     const int c = k_component(k, ncp);
-    const int64_t i = k - c * ncp;
-    const int s = i < n_i ? (c ? sg : sj)[i0 + i] : 0;
+    const int64_t i = k - c * ncp, g = i0 + i;
+    if (i >= n_i) return 0;
+    const int s = c ? sg[g] : sj[g];
     return s == D64_NO_SCALE ? D64_NO_SCALE : -s;
   }
 };
@@ -500,7 +501,7 @@ __global__ void __launch_bounds__(32 * PS_GROUPS)
 
 // sv[i], initially below D64_NO_SCALE: the exponent of max_pq,x |V_x,pq(i)| / (max phi_p max phi_q), from the rows of L; stays
 // below where V is 0.  One thread per point and VS_PAIRS pairs.
-constexpr int VS_PAIRS = 16;
+constexpr int VS_PAIRS = 8;
 __global__ void __launch_bounds__(128) v_scale_kernel(const double* __restrict__ L, int64_t ld, int64_t n_i, int n_pair,
                                                       const int* __restrict__ pair_p, const int* __restrict__ pair_q,
                                                       const int* __restrict__ orb, int* __restrict__ sv) {
@@ -511,12 +512,17 @@ __global__ void __launch_bounds__(128) v_scale_kernel(const double* __restrict__
   __syncthreads();
   if (i >= n_i) return;
   int m = D64_NO_SCALE;
-#pragma unroll 4
-  for (int pq = pq0; pq < pq1; ++pq) {
-    const double2* v = reinterpret_cast<const double2*>(L + pq * ld + 4 * i);
-    const double2 v0 = v[0], v1 = v[1];
-    const int k = max(d64_key(v0.y, 0), max(d64_key(v1.x, 0), d64_key(v1.y, 0)));
-    if (k && k < D64_NONFINITE) m = max(m, k - height[pq - pq0] + D64_BIAS + 1022);
+  double2 v[VS_PAIRS][2];   // all in flight
+#pragma unroll
+  for (int t = 0; t < VS_PAIRS; ++t) {
+    const double2* p = reinterpret_cast<const double2*>(L + static_cast<int64_t>(min(pq0 + t, n_pair - 1)) * ld + 4 * i);
+    v[t][0] = p[0];
+    v[t][1] = p[1];
+  }
+#pragma unroll
+  for (int t = 0; t < VS_PAIRS; ++t) {
+    const int k = max(d64_key(v[t][0].y, 0), max(d64_key(v[t][1].x, 0), d64_key(v[t][1].y, 0)));
+    if (pq0 + t < pq1 && k && k < D64_NONFINITE) m = max(m, k - height[t] + D64_BIAS + 1022);
   }
   if (m > D64_NO_SCALE) atomicMax(sv + i, m);
 }

@@ -25,7 +25,7 @@
 // Calls, all FP64 -> fixed point (one GB300): K with 30 orbitals, 8,000 points and 3 nuclei 18.8 -> 10.6 ms, K on an H2-sized input
 // 1,168 -> 770 us, its FP64 build 847 -> 659 us, 512 points of a water-sized build 9.7 -> 8.3 ms.  Rows that it does not
 // resolve are evaluated in FP64 (BITS_GRAD), so the errors against 64 bits are those of the FP64 pipe; with that check, the
-// scale of its own for h1 and the points' scales of K and V those calls take 10.7 ms, 831 us, 682 us and (with the waits
+// scale of its own for h1 and the points' scales of K and V those calls take 10.6 ms, 834 us, 680 us and (with the waits
 // of gemm64_tc.cu) 7.8 ms.
 #include <algorithm>
 
